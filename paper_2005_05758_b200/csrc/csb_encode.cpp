@@ -43,11 +43,13 @@ static uint16_t f32_to_f16_rne(float f) {
 
 // binary32 -> 16-bit fixed point with `frac_bits` fraction bits: the nearest integer to w * 2^frac_bits,
 // halves to the even one, saturated to the int16 range; NaN becomes 0.  (The scaling by a power of
-// two is exact in double precision, nearbyint rounds to nearest-even in the default rounding mode.)
-static int16_t f32_to_q16(float w, int frac_bits) {
+// two is exact in double precision.  After the clamp the sum with 1.5 * 2^52 has a unit in the last
+// place of 1, so adding and subtracting it rounds to nearest-even in the default rounding mode.)
+static int16_t f32_to_q16(float w, double scale) {
     if (w != w) return 0;
-    const double q = std::nearbyint(std::ldexp((double)w, frac_bits));
-    return (int16_t)(q < -32768.0 ? -32768.0 : q > 32767.0 ? 32767.0 : q);
+    const double q = std::min(32767.0, std::max(-32768.0, (double)w * scale));
+    constexpr double kRound = 6755399441055744.0;
+    return (int16_t)((q + kRound) - kRound);
 }
 
 int encode_host(const float* dense, int64_t rows, int64_t cols, int64_t ld, int br, int bc,
@@ -83,6 +85,7 @@ int encode_host(const float* dense, int64_t rows, int64_t cols, int64_t ld, int 
         A->nnz = (int64_t)vo;
         A->row_idx.resize(ro); A->col_idx.resize(co); A->val.resize(vo * vs);
         // pass 2: indices and values
+        const double scale = std::ldexp(1.0, A->q_frac_bits);
         for (int64_t bi = 0; bi < A->nbr; ++bi) {
             const int rlim = (int)std::min<int64_t>(br, rows - bi * br);
             for (int64_t bj = 0; bj < A->nbc; ++bj) {
@@ -99,7 +102,7 @@ int encode_host(const float* dense, int64_t rows, int64_t cols, int64_t ld, int 
                     for (int k = 0; k < n; ++k) {
                         const float w = src[ci[k]];
                         if (vs == 4) std::memcpy(v, &w, 4);
-                        else if (val_dtype == CSB_Q16) { const int16_t q = f32_to_q16(w, A->q_frac_bits); std::memcpy(v, &q, 2); }
+                        else if (val_dtype == CSB_Q16) { const int16_t q = f32_to_q16(w, scale); std::memcpy(v, &q, 2); }
                         else { const uint16_t h = f32_to_f16_rne(w); std::memcpy(v, &h, 2); }
                         v += vs;
                     }

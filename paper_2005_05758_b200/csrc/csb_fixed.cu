@@ -6,7 +6,12 @@
 // result is exact and does not depend on the order of summation.  That is what lets this kernel
 // add through atomics in shared memory without giving up bit-reproducibility.
 //
-// The kernel reads the canonical arrays of Section 3.1.1 as they are (m{}, n{}, RowIdx{}, ColIdx{},
+// Matrices of up to 16384 columns run the panel kernel of the batch-1 product (csb_panel.cu), whose
+// layout moves 16-bit values whatever they mean; it streams every value once with 16-byte loads.
+// Measured, 8192 x 8192 at 4x: 12.7 us against 55.2 us for the kernel below.  This file's kernel
+// serves what the panel layout does not take (wider matrices, panels beyond its limits).
+//
+// It reads the canonical arrays of Section 3.1.1 as they are (m{}, n{}, RowIdx{}, ColIdx{},
 // Val{} and the offsets), uploaded once.  A CTA works for one block-row and a range of its
 // block-columns (enough ranges to fill the GPU several times over: what a warp does per block is a
 // chain of dependent loads); its warps take the blocks of the range in turn, and the CTAs of a
@@ -131,7 +136,13 @@ int plan_fixed(csb_matrix* A) {
     FixedPlan* P = new (std::nothrow) FixedPlan();
     if (!P) { set_error("out of host memory"); return CSB_ERR_ALLOC; }
     A->fixed = P;
+    ProductPlan& Q = A->product;                          // the status word that bounded waits raise; nothing else of it is used
+    CSB_CUDA(cudaHostAlloc((void**)&Q.h_status, 4, cudaHostAllocMapped));
+    *Q.h_status = 0;
+    CSB_CUDA(cudaHostGetDevicePointer((void**)&Q.d_status, Q.h_status, 0));
     int rc;
+    if ((rc = plan_panels(A)) != CSB_OK) return rc;
+    if (A->panel) return CSB_OK;
     if ((rc = upload_arr(A->m.data(), A->m.size(), &P->d_m)) != CSB_OK) return rc;
     if ((rc = upload_arr(A->n.data(), A->n.size(), &P->d_n)) != CSB_OK) return rc;
     if ((rc = upload_arr(A->row_idx.data(), A->row_idx.size(), &P->d_ridx)) != CSB_OK) return rc;
@@ -158,6 +169,7 @@ void free_fixed(csb_matrix* A) {
 }
 
 int launch_fixed(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch, int64_t* acc, int64_t ldy, void* stream) {
+    if (A->panel) return launch_panels_q16(A, Xq, ldx, batch, acc, ldy, stream);
     int prev = 0;
     CSB_CUDA(cudaGetDevice(&prev));
     if (prev != A->device) CSB_CUDA(cudaSetDevice(A->device));

@@ -32,8 +32,10 @@ namespace csb {
 
 struct PanelArgs {
     const uint8_t* panels;
-    const float* x;
-    float* y;
+    const void* x;                     // float [cols], or int16 [nb, ldx]
+    void* y;                           // float [rows], or int64 [nb, ldy]
+    long long ldx, ldy;                // fixed point only
+    int nb;                            // fixed point: batch columns of this pass, 1..BT
     uint32_t* status;
     int rows, cols;
     int log2_stage, log2_slots;        // ring = 2^log2_slots stages of 2^log2_stage bytes
@@ -53,16 +55,18 @@ struct PanelArgs {
 
 __host__ __device__ inline size_t panel_align(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Shared-memory carve-up, identical on host and device.
+// Shared-memory carve-up, identical on host and device.  BT = 0: fp32 inputs and per-warp fp32
+// sums; BT > 0: fixed point, BT int16 inputs per matrix column, one 64-bit sum per row and batch column.
 struct PanelSmem {
-    size_t ring, xs, xg, zs, meta, bars, done, issued, dead, total;
-    __host__ __device__ PanelSmem(int W, int log2_stage, int log2_slots, int cols, int max_xg, int max_rows, int max_meta) {
+    size_t ring, xs, xs_row, xg, zs, meta, bars, done, issued, dead, total;
+    __host__ __device__ PanelSmem(int BT, int W, int log2_stage, int log2_slots, int cols, int max_xg, int max_rows, int max_meta) {
         const int slots = 1 << log2_slots;
         ring = 0;
         xs = (size_t)slots << log2_stage;
-        xg = panel_align(xs + (size_t)cols * 4, 16);
-        zs = panel_align(xg + (size_t)max_xg * 4, 16);
-        meta = panel_align(zs + (size_t)W * max_rows * 4, 128);
+        xs_row = panel_align((size_t)cols * (BT ? 2 : 4), 16);
+        xg = xs + xs_row * (BT ? BT : 1);
+        zs = panel_align(xg + (size_t)max_xg * (BT ? 2 * BT : 4), 16);
+        meta = panel_align(zs + (BT ? (size_t)BT * max_rows * 8 : (size_t)W * max_rows * 4), 128);
         bars = panel_align(meta + (size_t)max_meta, 16);
         done = bars + (size_t)(slots + 2) * 8;
         issued = done + (size_t)slots * 4;
@@ -126,10 +130,94 @@ __device__ __forceinline__ bool panel_wait_stage(uint64_t* full, volatile uint32
     return panel_wait(&full[slot], use & 1u, dead);
 }
 
+// Two 16-bit weights times the signed / unsigned bytes 0, 1 (lo) or 2, 3 (hi) of b, added to c.
+__device__ __forceinline__ int dp2a_lo_s(uint32_t w, uint32_t b, int c) { int d; asm("dp2a.lo.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(b), "r"(c)); return d; }
+__device__ __forceinline__ int dp2a_hi_s(uint32_t w, uint32_t b, int c) { int d; asm("dp2a.hi.s32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(b), "r"(c)); return d; }
+__device__ __forceinline__ int dp2a_lo_u(uint32_t w, uint32_t b, int c) { int d; asm("dp2a.lo.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(b), "r"(c)); return d; }
+__device__ __forceinline__ int dp2a_hi_u(uint32_t w, uint32_t b, int c) { int d; asm("dp2a.hi.s32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(w), "r"(b), "r"(c)); return d; }
+
+// The lane's share of one item in fixed point, added into the CTA's 64-bit sums.  An input is split
+// into its signed high and unsigned low byte, x = 256 xh + xl, so that a pair of weights costs one
+// dp2a per half and nothing is converted; the gathered inputs lie in quads of columns, per batch
+// column four high bytes and four low bytes.  Neither 32-bit sum can overflow: an item has at most
+// 128 columns, |w xh| <= 2^22 and |w xl| < 2^23, so the sums stay below 2^29 and 2^30.  Integer sums
+// do not depend on their order, hence the shared-memory atomics.
+template <int BT>
+__device__ __forceinline__ void panel_item_q16(const uint8_t* ring, uint32_t ring_mask, uint32_t off, const uint2* __restrict__ xq4, int n, int m,
+                                               int gl, int logp, int logg, int my_row, bool live, unsigned long long* zs) {
+    int hi[BT], lo[BT];
+#pragma unroll
+    for (int b = 0; b < BT; ++b) { hi[b] = 0; lo[b] = 0; }
+    const int r = gl & ((1 << logp) - 1), sub = gl >> logp, S = 32 >> (logg + logp);
+    const int noct = n >> 3;
+    uint32_t q = off + ((uint32_t)(sub * m + r) << 4);
+    const uint32_t qstep = (uint32_t)(S * m) << 4;
+    const uint2* xq = xq4 + (size_t)2 * sub * BT;
+#pragma unroll 2
+    for (int o = sub; o < noct; o += S) {
+        const uint4 w = *reinterpret_cast<const uint4*>(ring + (q & ring_mask));
+#pragma unroll
+        for (int b = 0; b < BT; ++b) {
+            const uint2 x0 = xq[b], x1 = xq[BT + b];
+            hi[b] = dp2a_lo_s(w.x, x0.x, hi[b]); lo[b] = dp2a_lo_u(w.x, x0.y, lo[b]);
+            hi[b] = dp2a_hi_s(w.y, x0.x, hi[b]); lo[b] = dp2a_hi_u(w.y, x0.y, lo[b]);
+            hi[b] = dp2a_lo_s(w.z, x1.x, hi[b]); lo[b] = dp2a_lo_u(w.z, x1.y, lo[b]);
+            hi[b] = dp2a_hi_s(w.w, x1.x, hi[b]); lo[b] = dp2a_hi_u(w.w, x1.y, lo[b]);
+        }
+        q += qstep;
+        xq += 2 * S * BT;
+    }
+    if ((n & 7) && gl < m) {
+        // the last n % 8 columns: [row][4], [row][2], [row][1] behind the octets
+        uint32_t tb = off + ((uint32_t)(noct * m) << 4);
+        const uint2* xt = xq4 + (size_t)2 * noct * BT;
+        if (n & 4) {
+            const uint2 w = *reinterpret_cast<const uint2*>(ring + ((tb + 8u * gl) & ring_mask));
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                const uint2 x0 = xt[b];
+                hi[b] = dp2a_lo_s(w.x, x0.x, hi[b]); lo[b] = dp2a_lo_u(w.x, x0.y, lo[b]);
+                hi[b] = dp2a_hi_s(w.y, x0.x, hi[b]); lo[b] = dp2a_hi_u(w.y, x0.y, lo[b]);
+            }
+            tb += 8u * m; xt += BT;
+        }
+        if (n & 2) {
+            const uint32_t w = *reinterpret_cast<const uint32_t*>(ring + ((tb + 4u * gl) & ring_mask));
+#pragma unroll
+            for (int b = 0; b < BT; ++b) { hi[b] = dp2a_lo_s(w, xt[b].x, hi[b]); lo[b] = dp2a_lo_u(w, xt[b].y, lo[b]); }
+            tb += 4u * m;
+        }
+        if (n & 1) {
+            const uint32_t w = *reinterpret_cast<const uint16_t*>(ring + ((tb + 2u * gl) & ring_mask));   // upper weight 0
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                if (n & 2) { hi[b] = dp2a_hi_s(w, xt[b].x, hi[b]); lo[b] = dp2a_hi_u(w, xt[b].y, lo[b]); }
+                else { hi[b] = dp2a_lo_s(w, xt[b].x, hi[b]); lo[b] = dp2a_lo_u(w, xt[b].y, lo[b]); }
+            }
+        }
+    }
+    // join the lanes that split the columns of a row
+    const int pmin = logg ? (int)__reduce_min_sync(0xffffffffu, 1u << logp) : 1 << logp;
+    for (int o = 16 >> logg; o >= pmin; o >>= 1)
+#pragma unroll
+        for (int b = 0; b < BT; ++b) {
+            const int th = __shfl_xor_sync(0xffffffffu, hi[b], o), tl = __shfl_xor_sync(0xffffffffu, lo[b], o);
+            if (o >= (1 << logp)) { hi[b] += th; lo[b] += tl; }
+        }
+    if (live)
+#pragma unroll
+        for (int b = 0; b < BT; ++b) {
+            const long long v = ((long long)hi[b] << 8) + (long long)lo[b];
+            if (v) atomicAdd(zs + (size_t)my_row * BT + b, (unsigned long long)v);
+        }
+}
+
+// BT = 0: fp16 values, fp32 input and output.  BT = 1, 2, 4: 16-bit fixed point, BT batch columns a pass.
+template <int BT>
 __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constant__ PanelArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const int W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const PanelSmem L(W, a.log2_stage, a.log2_slots, a.cols, a.max_xg, a.max_rows, a.max_meta);
+    const PanelSmem L(BT, W, a.log2_stage, a.log2_slots, a.cols, a.max_xg, a.max_rows, a.max_meta);
     const uint4 ct = a.cta[blockIdx.x];
     const uint8_t* panel = a.panels + (size_t)ct.x * 16;
     const uint32_t meta_bytes = ct.y, value_bytes = ct.z;
@@ -149,7 +237,8 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
     volatile uint32_t* issued = reinterpret_cast<volatile uint32_t*>(smem + L.issued);
     volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(smem + L.dead);
 
-    const bool x_bulk = (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols & 3) == 0;
+    const bool x_bulk = BT ? (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols & 7) == 0 && (a.nb == 1 || (a.ldx & 7) == 0)
+                           : (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols & 3) == 0;
     // Launched with programmatic stream serialization, this grid may start while the kernel in
     // front of it on the stream is still draining: whatever comes next may be scheduled as early
     // as the hardware likes, and this grid touches x and y only behind grid_dependency_wait().
@@ -172,10 +261,12 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
         }
         if (s == slots + 1u && x_bulk) {
             grid_dependency_wait();
-            const uint32_t xb = (uint32_t)a.cols * 4u;
-            mbar_expect_tx(xbar, xb);
-            for (uint32_t off = 0; off < xb; off += 16384u)
-                bulk_g2s(smem + L.xs + off, reinterpret_cast<const uint8_t*>(a.x) + off, min(16384u, xb - off), xbar);
+            const uint32_t xb = (uint32_t)a.cols * (BT ? 2u : 4u);
+            const int nb = BT ? a.nb : 1;
+            mbar_expect_tx(xbar, xb * (uint32_t)nb);
+            for (int b = 0; b < nb; ++b)
+                for (uint32_t off = 0; off < xb; off += 16384u)
+                    bulk_g2s(smem + L.xs + b * L.xs_row + off, reinterpret_cast<const uint8_t*>(a.x) + (BT ? (size_t)b * a.ldx * 2 : 0) + off, min(16384u, xb - off), xbar);
         }
         __syncwarp(slots + 2u >= 32u ? 0xffffffffu : (1u << (slots + 2u)) - 1u);
         if (s < slots && s < n_stages) {
@@ -185,10 +276,14 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
             bulk_g2s(ring + ((size_t)s << a.log2_stage), values + ((size_t)s << a.log2_stage), bytes, &full[s]);
         }
     }
-    for (int i = threadIdx.x; i < W * a.max_rows; i += blockDim.x) zs_all[i] = 0.f;
+    for (int i = threadIdx.x; i < (BT ? 2 * BT : W) * a.max_rows; i += blockDim.x) zs_all[i] = 0.f;
     if (!x_bulk) {
         grid_dependency_wait();
-        for (int i = threadIdx.x; i < a.cols; i += blockDim.x) xs[i] = __ldg(a.x + i);
+        if (BT == 0)
+            for (int i = threadIdx.x; i < a.cols; i += blockDim.x) xs[i] = __ldg(reinterpret_cast<const float*>(a.x) + i);
+        for (int b = 0; b < (BT ? a.nb : 0); ++b)
+            for (int i = threadIdx.x; i < a.cols; i += blockDim.x)
+                reinterpret_cast<int16_t*>(smem + L.xs + b * L.xs_row)[i] = __ldg(reinterpret_cast<const int16_t*>(a.x) + (long long)b * a.ldx + i);
     }
     __syncthreads();                                       // barriers initialised, counters and sums cleared
     PANEL_STAMP(1);
@@ -215,6 +310,24 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
                 const uint32_t xbase = gd.x & 0xffffu, n = gd.x >> 16, xoff = gd.y;
                 for (uint32_t k = (uint32_t)(lane & 7) * 4u; k < n; k += 32u) {
                     const uint32_t c4 = *reinterpret_cast<const uint32_t*>(cidx + xoff + k);
+                    if (BT) {
+                        const int16_t* xr = reinterpret_cast<const int16_t*>(xs) + xbase;
+                        uint2* dst = reinterpret_cast<uint2*>(xg) + (size_t)((xoff + k) >> 2) * BT;
+#pragma unroll
+                        for (int b = 0; b < BT; ++b) {
+                            // two inputs to a word, then the bytes sorted into high and low ones; a column past nb stays 0
+                            uint2 h = make_uint2(0u, 0u);
+                            if (b < a.nb) {
+                                const uint32_t v0 = (uint16_t)xr[c4 & 0xffu], v1 = (uint16_t)xr[(c4 >> 8) & 0xffu];
+                                const uint32_t v2 = (uint16_t)xr[(c4 >> 16) & 0xffu], v3 = (uint16_t)xr[c4 >> 24];
+                                const uint32_t p0 = v0 | (v1 << 16), p1 = v2 | (v3 << 16);
+                                h = make_uint2(__byte_perm(p0, p1, 0x7531), __byte_perm(p0, p1, 0x6420));
+                            }
+                            dst[b] = h;
+                            xr += L.xs_row >> 1;
+                        }
+                        continue;
+                    }
                     float4 v;
                     v.x = xs[xbase + (c4 & 0xffu)]; v.y = xs[xbase + ((c4 >> 8) & 0xffu)];
                     v.z = xs[xbase + ((c4 >> 16) & 0xffu)]; v.w = xs[xbase + (c4 >> 24)];
@@ -249,6 +362,10 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
             const uint32_t st = off >> a.log2_stage;          // the same for every member of the bundle
             if (__any_sync(0xffffffffu, !panel_wait_stage(full, issued, st, a.log2_slots, s_dead))) { *s_dead = 1u; break; }
 
+            if (BT) {
+                panel_item_q16<BT ? BT : 1>(ring, ring_mask, off, reinterpret_cast<const uint2*>(xg) + (size_t)xoff4 * BT, n, m, gl, logp, logg, my_row, gl < m,
+                                            reinterpret_cast<unsigned long long*>(zs_all));
+            } else {
             const int r = gl & ((1 << logp) - 1), sub = gl >> logp, S = 32 >> (logg + logp);
             const int noct = n >> 3;
             float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
@@ -322,6 +439,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
                     __syncwarp();
                 }
             }
+            }
             __syncwarp();
             // ---- the bundle is done with its stage; the last one out refills the slot
             if (lane == 0) {
@@ -361,10 +479,17 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
 
     // ---- add the warps' copies in warp order and store the CTA's rows
     const int n_rows = (int)H->n_rows, row0 = (int)H->row0;
+    if (BT) {
+        for (int t = threadIdx.x; t < n_rows * a.nb; t += blockDim.x) {
+            const int b = t / n_rows, r = t - b * n_rows;
+            reinterpret_cast<long long*>(a.y)[(long long)b * a.ldy + row0 + r] = reinterpret_cast<const long long*>(zs_all)[r * BT + b];
+        }
+        return;
+    }
     for (int t = threadIdx.x; t < n_rows; t += blockDim.x) {
         float v = 0.f;
         for (int w = 0; w < W; ++w) v += zs_all[(size_t)w * a.max_rows + t];
-        a.y[row0 + t] = v;
+        reinterpret_cast<float*>(a.y)[row0 + t] = v;
     }
     PANEL_STAMP(5);
     PANEL_STAMP(7);
@@ -386,7 +511,7 @@ static int env_int(const char* name, int dflt) {
 static int log2_floor(int v) { int l = 0; while ((2 << l) <= v) ++l; return l; }
 
 int plan_panels(csb_matrix* A) {
-    if (A->val_dtype != CSB_F16 || env_int("CSB_NO_PANEL", 0)) return CSB_OK;
+    if ((A->val_dtype != CSB_F16 && A->val_dtype != CSB_Q16) || env_int("CSB_NO_PANEL", 0)) return CSB_OK;
     const int warps = std::min(32, std::max(1, env_int("CSB_PANEL_WARPS", 32)));
     int stage = env_int("CSB_PANEL_STAGE", 16384);
     stage = 1 << std::min(15, std::max(13, log2_floor(stage)));
@@ -399,12 +524,17 @@ int plan_panels(csb_matrix* A) {
     P->ctas = (int)H.cta.size(); P->warps = warps; P->stage_bytes = stage;
     P->max_xg = (int)H.max_xg; P->max_meta = (int)H.max_meta; P->max_rows = (int)std::max<size_t>(H.max_rows, 1);
     const int want_ring = std::min(17, std::max(log2_floor(stage) + 1, env_int("CSB_PANEL_RING_LOG2", 17)));
-    P->log2_ring = 0;
-    for (int lr = want_ring; lr > log2_floor(stage); --lr) {
-        const PanelSmem L(warps, log2_floor(stage), lr - log2_floor(stage), (int)A->cols, P->max_xg, P->max_rows, P->max_meta);
-        if (L.total <= A->smem_optin) { P->log2_ring = lr; P->smem_bytes = L.total; break; }
+    // the deepest ring that leaves room for the rest, per variant of the kernel
+    for (int v = 0; v < PanelPlan::kVariants; ++v) {
+        P->log2_ring[v] = 0;
+        if ((PanelPlan::bt(v) != 0) != (A->val_dtype == CSB_Q16)) continue;
+        for (int lr = want_ring; lr > log2_floor(stage); --lr) {
+            const PanelSmem L(PanelPlan::bt(v), warps, log2_floor(stage), lr - log2_floor(stage), (int)A->cols, P->max_xg, P->max_rows, P->max_meta);
+            if (L.total <= A->smem_optin) { P->log2_ring[v] = lr; P->smem_bytes[v] = L.total; break; }
+        }
     }
-    if (!P->log2_ring) { delete P; return CSB_OK; }        // does not fit: the other path serves this matrix
+    // the variant that takes one vector does not fit: the other path serves this matrix
+    if (!P->log2_ring[A->val_dtype == CSB_Q16 ? 1 : 0]) { delete P; return CSB_OK; }
     int prev = 0;
     CSB_CUDA(cudaGetDevice(&prev));
     CSB_CUDA(cudaSetDevice(A->device));
@@ -414,7 +544,8 @@ int plan_panels(csb_matrix* A) {
     P->balance = H.balance; P->warp_balance = H.warp_balance;
     CSB_CUDA(cudaMalloc((void**)&P->d_panels, std::max<size_t>(H.bytes.size(), 16)));
     CSB_CUDA(cudaMemcpy(P->d_panels, H.bytes.data(), H.bytes.size(), cudaMemcpyHostToDevice));
-    CSB_CUDA(cudaFuncSetAttribute(csb_panel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
+    for (const void* k : {(const void*)csb_panel_kernel<0>, (const void*)csb_panel_kernel<1>, (const void*)csb_panel_kernel<2>, (const void*)csb_panel_kernel<4>})
+        CSB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
     CSB_CUDA(cudaDeviceSynchronize());
     CSB_CUDA(cudaSetDevice(prev));
     P->built = true;
@@ -440,7 +571,7 @@ extern "C" int csb_debug_panel_clocks(unsigned long long* host_out, int ctas) {
 }
 #endif
 
-int launch_panels(const csb_matrix* A, const float* x, float* y, void* stream) {
+static int launch_variant(const csb_matrix* A, int v, const void* x, int64_t ldx, int nb, void* y, int64_t ldy, void* stream) {
     const PanelPlan& P = *A->panel;
     const ProductPlan& Q = A->product;
     if (Q.h_status && *Q.h_status != 0) { set_error("an earlier product on this handle gave up waiting on the device (code %u)", *Q.h_status); return CSB_ERR_TIMEOUT; }
@@ -448,9 +579,9 @@ int launch_panels(const csb_matrix* A, const float* x, float* y, void* stream) {
     CSB_CUDA(cudaGetDevice(&prev));
     if (prev != A->device) CSB_CUDA(cudaSetDevice(A->device));
     PanelArgs a{};
-    a.panels = P.d_panels; a.x = x; a.y = y; a.status = Q.d_status;
+    a.panels = P.d_panels; a.x = x; a.y = y; a.ldx = ldx; a.ldy = ldy; a.nb = nb; a.status = Q.d_status;
     a.rows = (int)A->rows; a.cols = (int)A->cols;
-    a.log2_stage = log2_floor(P.stage_bytes); a.log2_slots = P.log2_ring - a.log2_stage;
+    a.log2_stage = log2_floor(P.stage_bytes); a.log2_slots = P.log2_ring[v] - a.log2_stage;
     a.max_rows = P.max_rows; a.max_xg = P.max_xg; a.max_meta = P.max_meta;
     for (int c = 0; c < P.ctas; ++c) a.cta[c] = make_uint4(P.cta[c].off16, P.cta[c].meta_bytes, P.cta[c].value_bytes, P.cta[c].n_rows);
 #ifdef CSB_PANEL_CLOCKS
@@ -465,15 +596,33 @@ int launch_panels(const csb_matrix* A, const float* x, float* y, void* stream) {
     const int use_pdl = env_int("CSB_PANEL_PDL", 1);      // read at every launch, so a caller can compare both kinds
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)P.ctas); cfg.blockDim = dim3((unsigned)P.warps * 32u);
-    cfg.dynamicSmemBytes = P.smem_bytes; cfg.stream = (cudaStream_t)stream;
+    cfg.dynamicSmemBytes = P.smem_bytes[v]; cfg.stream = (cudaStream_t)stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = use_pdl ? 1u : 0u;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, csb_panel_kernel, a);
+    cudaError_t e = v == 0 ? cudaLaunchKernelEx(&cfg, csb_panel_kernel<0>, a) : v == 1 ? cudaLaunchKernelEx(&cfg, csb_panel_kernel<1>, a)
+                  : v == 2 ? cudaLaunchKernelEx(&cfg, csb_panel_kernel<2>, a) : cudaLaunchKernelEx(&cfg, csb_panel_kernel<4>, a);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (prev != A->device) cudaSetDevice(prev);
     if (e != cudaSuccess) { set_error("panel kernel launch failed: %s", cudaGetErrorString(e)); return CSB_ERR_CUDA; }
+    return CSB_OK;
+}
+
+int launch_panels(const csb_matrix* A, const float* x, float* y, void* stream) {
+    return launch_variant(A, 0, x, A->cols, 1, y, A->rows, stream);
+}
+
+int launch_panels_q16(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch, int64_t* acc, int64_t ldy, void* stream) {
+    for (int b0 = 0; b0 < batch;) {
+        // as many batch columns a pass as are left and as leave room for a ring
+        int v = batch - b0 >= 3 ? 3 : batch - b0;
+        while (v > 1 && !A->panel->log2_ring[v]) --v;
+        const int nb = std::min(batch - b0, PanelPlan::bt(v));
+        const int rc = launch_variant(A, v, Xq + (int64_t)b0 * ldx, ldx, nb, acc + (int64_t)b0 * ldy, ldy, stream);
+        if (rc != CSB_OK) return rc;
+        b0 += nb;
+    }
     return CSB_OK;
 }
 

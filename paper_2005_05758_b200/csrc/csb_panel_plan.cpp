@@ -24,7 +24,11 @@
 // longest first and dealt to the CTA's warps in that order, each to the warp with the least
 // work so far; the deal is part of the plan, so the summation order is fixed.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
+#include <new>
+#include <system_error>
+#include <thread>
 
 #include "csb_internal.hpp"
 
@@ -69,7 +73,7 @@ struct PanelItemSrc {
 int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, int max_xg_floats, int max_rows,
                      PanelHostPlan* out) {
     *out = PanelHostPlan{};
-    if (A->val_dtype != CSB_F16) return 1;
+    if (A->val_dtype != CSB_F16 && A->val_dtype != CSB_Q16) return 1;   // 16-bit values, moved as they are
     if (A->block_c > 128 || A->cols > 16384) return 1;
     if (stage_bytes < 8192 || (stage_bytes & (stage_bytes - 1))) return 1;
     const int BR = A->block_r, BC = A->block_c;
@@ -103,7 +107,15 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
     // followed row by row: rows are packed into a CTA until a limit T would be passed, and T is
     // the smallest limit (by bisection) that needs no more than n_ctas CTAs.
     std::vector<uint16_t> cnt(A->nblk, 0);                 // rows of the block in the CTA being filled
-    auto block_cost = [&](int m, int n) { double c = 0.0; for (int r0 = 0; r0 < m; r0 += 32) c += panel_item_cost(std::min(32, m - r0), n); return c; };
+    // the bisection asks for the cost of a block many times per row: a table of all (rows, columns) it can have
+    std::vector<double> cost_table((size_t)(BR + 1) * (BC + 1), 0.0);
+    for (int n = 1; n <= BC; ++n)
+        for (int m = 1; m <= BR; ++m) {
+            double c = 0.0;
+            for (int r0 = 0; r0 < m; r0 += 32) c += panel_item_cost(std::min(32, m - r0), n);
+            cost_table[(size_t)n * (BR + 1) + m] = c;
+        }
+    auto block_cost = [&](int m, int n) { return cost_table[(size_t)n * (BR + 1) + m]; };
     auto pack = [&](double T, std::vector<int64_t>* cuts, double* worst) -> int {
         int used = 1;
         double cur = 0.0;
@@ -147,7 +159,11 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
     out->stage_bytes = stage_bytes;
     out->cta.resize(n_ctas);
     double max_cta_cost = 0.0, max_warp_cost = 0.0, sum_cta_cost = 0.0;
-    for (int c = 0; c < n_ctas; ++c) {
+    // The panels are independent of one another: a few host threads build them, and they are then
+    // appended in CTA order, so the result does not depend on the number of threads.
+    struct PanelBuild { std::vector<uint8_t> bytes; size_t meta_bytes = 0, value_bytes = 0, n_xg = 0; double cost = 0.0, warp_cost = 0.0; };
+    std::vector<PanelBuild> built(n_ctas);
+    auto build_panel = [&](int c) -> int {
         const int64_t R0 = cut[c], R1 = cut[c + 1];
         if (R1 - R0 > max_rows) return 1;
         std::vector<PanelItemSrc> items;
@@ -260,10 +276,8 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
         }
         if (cidx.size() > (size_t)max_xg_floats || cidx.size() / 4 > 0xffff || ridx.size() > 0xffff || values.size() / 16 > 0xffffffffull)
             return 1;                                            // beyond the kernel's limits: the caller keeps the other path
-        double cta_cost = 0.0;
-        for (int w = 0; w < warps; ++w) { cta_cost += load[w]; max_warp_cost = std::max(max_warp_cost, load[w]); }
-        sum_cta_cost += cta_cost;
-        max_cta_cost = std::max(max_cta_cost, cta_cost);
+        PanelBuild& out_c = built[c];
+        for (int w = 0; w < warps; ++w) { out_c.cost += load[w]; out_c.warp_cost = std::max(out_c.warp_cost, load[w]); }
         // descriptors in the order the warps take them: a bundle's members side by side, missing
         // members as empty descriptors (no rows, no columns) that point at the bundle's stage
         std::vector<PanelItem> table;
@@ -300,9 +314,9 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
         h.cidx_off = (uint32_t)off; off = pad_to(off + cidx.size(), 16);
         h.ridx_off = (uint32_t)off; off = pad_to(off + ridx.size(), 128);
         const size_t meta_bytes = off;
-        const size_t base = pad_to(out->bytes.size(), 128);
-        out->bytes.resize(base + meta_bytes + pad_to(values.size(), 128), 0);
-        uint8_t* p = out->bytes.data() + base;
+        out_c.bytes.assign(meta_bytes + pad_to(values.size(), 128), 0);
+        out_c.meta_bytes = meta_bytes; out_c.value_bytes = values.size(); out_c.n_xg = cidx.size();
+        uint8_t* p = out_c.bytes.data();
         std::memcpy(p, &h, sizeof h);
         std::memcpy(p + h.warp_off, wbegin.data(), wbegin.size() * 2);
         if (!wlist.empty()) std::memcpy(p + h.list_off, wlist.data(), wlist.size() * 2);
@@ -312,12 +326,43 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
         if (!cidx.empty()) std::memcpy(p + h.cidx_off, cidx.data(), cidx.size());
         if (!ridx.empty()) std::memcpy(p + h.ridx_off, ridx.data(), ridx.size());
         if (!values.empty()) std::memcpy(p + meta_bytes, values.data(), values.size());
+        return CSB_OK;
+    };
+    {
+        const unsigned hw = std::thread::hardware_concurrency();
+        const int n_threads = (int)std::min<int64_t>(std::min<int64_t>(hw ? hw : 1, 8), std::max<int64_t>(1, (int64_t)(total_bytes >> 18)));   // 256 KB of values and more per thread
+        std::atomic<int> next{0}, status{CSB_OK};
+        auto work = [&]() {
+            for (int c; status.load() == CSB_OK && (c = next.fetch_add(1)) < n_ctas;) {
+                int rc;
+                try { rc = build_panel(c); } catch (const std::bad_alloc&) { rc = CSB_ERR_ALLOC; }
+                if (rc != CSB_OK) status.store(rc);
+            }
+        };
+        std::vector<std::thread> pool;
+        try { for (int t = 1; t < n_threads; ++t) pool.emplace_back(work); } catch (const std::system_error&) {}   // fewer threads then
+        work();
+        for (auto& t : pool) t.join();
+        if (status.load() == CSB_ERR_ALLOC) throw std::bad_alloc();
+        if (status.load() != CSB_OK) return status.load();
+    }
+    size_t total = 0;
+    for (const PanelBuild& b : built) total += pad_to(b.bytes.size(), 128);
+    out->bytes.resize(total);
+    size_t base = 0;
+    for (int c = 0; c < n_ctas; ++c) {
+        PanelBuild& b = built[c];
+        std::memcpy(out->bytes.data() + base, b.bytes.data(), b.bytes.size());
         PanelCta& ct = out->cta[c];
-        ct.off16 = (uint32_t)(base / 16); ct.meta_bytes = (uint32_t)meta_bytes; ct.value_bytes = (uint32_t)values.size();
-        ct.n_rows = (uint32_t)(R1 - R0);
-        out->max_meta = std::max(out->max_meta, meta_bytes);
-        out->max_xg = std::max(out->max_xg, cidx.size());
-        out->max_rows = std::max<size_t>(out->max_rows, (size_t)(R1 - R0));
+        ct.off16 = (uint32_t)(base / 16); ct.meta_bytes = (uint32_t)b.meta_bytes; ct.value_bytes = (uint32_t)b.value_bytes;
+        ct.n_rows = (uint32_t)(cut[c + 1] - cut[c]);
+        out->max_meta = std::max(out->max_meta, b.meta_bytes);
+        out->max_xg = std::max(out->max_xg, b.n_xg);
+        out->max_rows = std::max<size_t>(out->max_rows, (size_t)(cut[c + 1] - cut[c]));
+        sum_cta_cost += b.cost;
+        max_cta_cost = std::max(max_cta_cost, b.cost); max_warp_cost = std::max(max_warp_cost, b.warp_cost);
+        base += b.bytes.size();
+        std::vector<uint8_t>().swap(b.bytes);
     }
     if (out->bytes.size() / 16 > 0xffffffffull) return 1;
     out->balance = max_cta_cost > 0.0 ? (sum_cta_cost / n_ctas) / max_cta_cost : 1.0;

@@ -41,6 +41,29 @@ def test_random_masks_exact(shape):
     run(mat, rng.standard_normal((B, C)).astype(np.float32), 16, 12)
 
 
+@pytest.mark.parametrize("C,bc,B", [(16384, 64, 1), (16392, 64, 1), (16384, 128, 3), (1001, 7, 4), (1000, 100, 2), (264, 33, 6), (16383, 128, 5)])
+def test_panel_kernel_and_its_limits(C, bc, B):
+    # the panel kernel takes up to 16384 columns (one more block-column goes to the other kernel); every remainder of
+    # the kept columns modulo 8, passes of 1, 2 and 4 vectors, inputs that do and do not start on 16 bytes
+    rng = np.random.default_rng(C + B)
+    R, br = 90, 40
+    nblk = -(-R // br) * -(-C // bc)
+    mat = workloads.MatrixSpec((rng.standard_normal((R, C)) * 0.1).astype(np.float32), br, bc, (rng.random(nblk * br) < 0.5).astype(np.uint8),
+                               (rng.random(nblk * bc) < rng.random(nblk).repeat(bc)).astype(np.uint8), "f16")
+    X = np.clip(rng.standard_normal((B, C)), -7, 7).astype(np.float32)
+    X[:, ::5] = 7.99
+    X[:, 1::7] = -8.0
+    want = run(mat, X, 16, 12)
+    A = binding.csb_encode_q16(mat.dense, br, bc, mat.row_keep, mat.col_keep, 16, 0)
+    wide = torch.zeros((B, C + 3), dtype=torch.int16, device="cuda")
+    wide[:, 1:C + 1] = torch.from_numpy(F.quantize(X, 12).astype(np.int16)).cuda()
+    acc = torch.full((B, R + 5), -7, dtype=torch.int64, device="cuda")
+    binding.csb_spmm_q16(A, wide[:, 1:C + 1], acc[:, 2:R + 2])
+    torch.cuda.synchronize()
+    assert np.array_equal(acc[:, 2:R + 2].cpu().numpy(), want) and bool((acc[:, :2] == -7).all()) and bool((acc[:, R + 2:] == -7).all())
+    A.free()
+
+
 def test_saturating_values_and_full_range_inputs():
     rng = np.random.default_rng(3)
     R, C = 128, 256
