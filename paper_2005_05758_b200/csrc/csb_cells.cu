@@ -214,7 +214,7 @@ static int cell_forward(int kind, int L, const csb_matrix_t* const* W, const csb
     // one sequence: the batch-1 time loop in one launch, as long as the weights fit the SMs' shared memory
     if (B == 1) {
         const int cell = kind == kCellLstmp ? kR1Lstmp : kind == kCellLigru ? kR1Ligru : kR1GruRb;
-        const int rc = rnn1_forward(cell, L, W, kind == kCellLstmp ? Wp : nullptr, bias, x, T, H, S, in_size, h0, c0, y, hT, cT, flags, stream);
+        const int rc = rnn1_forward(cell, L, W, kind == kCellLstmp ? Wp : nullptr, bias, x, T, B, H, S, in_size, h0, c0, y, hT, cT, flags, stream);
         if (rc != 1) return rc;
     }
 

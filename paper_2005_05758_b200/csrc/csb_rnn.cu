@@ -835,7 +835,7 @@ static int rnn_forward(int gates, int L, const csb_matrix_t* const* W, const flo
 
     // one sequence: the batch-1 time loop, as long as the weights fit the SMs' shared memory
     if (B == 1) {
-        const int rc = rnn1_forward(gates == 4 ? kR1Lstm : kR1Gru, L, W, nullptr, bias, x, T, H, H, in_size, h0, c0, y, hT, cT, flags, stream);
+        const int rc = rnn1_forward(gates == 4 ? kR1Lstm : kR1Gru, L, W, nullptr, bias, x, T, B, H, H, in_size, h0, c0, y, hT, cT, flags, stream);
         if (rc != 1) return rc;
     }
 

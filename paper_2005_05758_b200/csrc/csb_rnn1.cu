@@ -1,21 +1,22 @@
-// Batch-1 time loop of the recurrent cells (LSTM, GRU, LSTMP, Li-GRU, reset-before GRU): one
-// cooperative launch per sequence (Section 2.1 of the paper: per step a CSB product with
+// Resident time loop of the recurrent cells (LSTM, GRU, LSTMP, Li-GRU, reset-before GRU) for small
+// batches: one cooperative launch per sequence (Section 2.1 of the paper: per step a CSB product with
 // [u_t ; h_{t-1}], then the element-wise gate arithmetic, the c / h "context link" feeding the next step).
 //
 // A CTA owns a range of hidden units of one layer (csb_rnn1.hpp); its weights stay in shared memory.
-// What bounds a step is latency: the exchange of h_t between CTAs, then the chain gather -> product ->
-// sum -> gates.  So
+// What bounds a step is latency: the exchange of h_t between CTAs, then product, sums and gates, and
+// inside the product the traffic of shared memory.  So
 //   * a vector crosses CTAs as 16-byte words of three values and the number of their step, written
 //     and read with single 16-byte accesses (relaxed, 128-bit atomic): a reader that sees the step
 //     it waits for also holds the values.  No fence, no counter, no grid barrier; layers run as a
 //     dataflow pipeline.  Step numbers go on from call to call (a word per CTA keeps the count), so
 //     nothing is cleared between calls.  A vector stays for 32 steps; every 8 steps a layer checks
 //     that the layer above has read what it is about to overwrite;
-//   * the product over the input part [u_t] is done while h_{t-1} is on its way;
-//   * the product is a plain loop: per pair of slots a lane reads 16 bytes of weights, two places and
-//     two times four gathered inputs, and adds into one register pair; every thread works for one
-//     row, so there is no scatter, and a row's threads meet once, in the gate arithmetic;
-//   * a unit's gates sit on four neighbouring lanes, so the gate arithmetic needs no further barrier.
+//   * the product over the input part [u_t] is done while h_{t-1} is on its way, and u_{t+1} is fetched
+//     into the other of two buffers meanwhile;
+//   * a lane of the product fetches up to 8 inputs through the column indices into registers and
+//     multiplies them with the rows of its task one after the other; partial sums go to places of
+//     their own, ordered by row.  Measured at 2 x 2048 units, 10x pruned, batch 1: FIXME_WALK
+//   * three barriers a step: inputs complete, partial sums complete, row sums complete.
 // LSTMP and the reset-before GRU have a second product in the step (the projection; the candidate's):
 // what it reads (o * tanh(c); r * h) crosses the CTAs of the layer in the same way.
 //
@@ -46,7 +47,7 @@ struct R1Args {
     float* y; float* hT; float* cT;
     const float* bias[kMaxLayers];
     int in_size[kMaxLayers];
-    const uint32_t* wmap[2][kMaxLayers];       // unit0 | units << 16 of every exchange word
+    const uint32_t* wmap[2][kMaxLayers];       // first element | elements << 24 of every exchange word
     int words[2][kMaxLayers];
     uint4* ex[2][kMaxLayers];                  // [kR1Ring][words]
     uint32_t* epoch;                           // per CTA: step numbers used so far
@@ -55,24 +56,38 @@ struct R1Args {
     uint32_t* status;
     unsigned long long limit_ns;
     uint32_t never;                            // test hook: wait for step numbers that never come
-    int T, H, S, L;
-    uint32_t xg[2][2], vu, vr, vm, part, misc; // shared-memory offsets behind the image
+    int T, B, H, S, L;
+    uint32_t vu[2], vr, vm, part[2], z[2], cs, bias0, bias1, misc;   // shared-memory offsets behind the image
+#ifdef CSB_PHASE_CLOCKS
+    long long* clocks;                         // [CTA][8] cycles of thread 0 summed over the steps
+#endif
 };
+#ifdef CSB_PHASE_CLOCKS
+#define R1_LAP(i) do { if (tid == 0) { const long long n_ = clock64(); lap[i] += n_ - lap_at; lap_at = n_; } } while (0)
+#else
+#define R1_LAP(i) do { } while (0)
+#endif
 
-__device__ __forceinline__ uint4 ld_word(const uint4* p) {
-    uint64_t a, b;
-    asm volatile("{\n\t.reg .b128 r;\n\tld.relaxed.gpu.global.b128 r, [%2];\n\tmov.b128 {%0, %1}, r;\n\t}" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-    return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+typedef unsigned __int128 Word;                // three values and a step number
+__device__ __forceinline__ Word ld_word(const uint4* p) {
+    Word w;
+    asm volatile("ld.relaxed.gpu.global.b128 %0, [%1];" : "=q"(w) : "l"(p) : "memory");
+    return w;
 }
-__device__ __forceinline__ void st_word(uint4* p, uint4 v) {
-    const uint64_t a = (uint64_t)v.x | ((uint64_t)v.y << 32), b = (uint64_t)v.z | ((uint64_t)v.w << 32);
-    asm volatile("{\n\t.reg .b128 r;\n\tmov.b128 r, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], r;\n\t}" ::"l"(p), "l"(a), "l"(b) : "memory");
+__device__ __forceinline__ void st_word(uint4* p, float a, float b, float c, uint32_t tag) {
+    const Word w = (Word)__float_as_uint(a) | ((Word)__float_as_uint(b) << 32) | ((Word)__float_as_uint(c) << 64) | ((Word)tag << 96);
+    asm volatile("st.relaxed.gpu.global.b128 [%0], %1;" ::"l"(p), "q"(w) : "memory");
 }
+__device__ __forceinline__ uint32_t word_tag(Word w) { return (uint32_t)(w >> 96); }
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     unsigned long long d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;"
@@ -83,106 +98,133 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ float2 half2_to_float2(uint32_t w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
 __device__ __forceinline__ float logistic(float a) { return 1.f / (1.f + expf(-a)); }
 
-// This thread's slots of one part of a product: `pairs` rounds of two slots, [round][lane].
-template <typename T>
-__device__ __forceinline__ float walk(const uint4* w, const uint32_t* places, int pairs, const uint8_t* xg) {
-    float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-    constexpr int kStride = sizeof(T) == 2 ? 32 : 64;
-#pragma unroll 4
-    for (int i = 0; i < pairs; ++i) {
-        const uint32_t o = places[i * 32];
-        const float4 x0 = *reinterpret_cast<const float4*>(xg + (o & 0xffffu)), x1 = *reinterpret_cast<const float4*>(xg + (o >> 16));
-        if (sizeof(T) == 2) {
-            const uint4 v = w[i * kStride];
-            a = fma2(half2_to_float2(v.x), make_float2(x0.x, x0.y), a);
-            b = fma2(half2_to_float2(v.y), make_float2(x0.z, x0.w), b);
-            a = fma2(half2_to_float2(v.z), make_float2(x1.x, x1.y), a);
-            b = fma2(half2_to_float2(v.w), make_float2(x1.z, x1.w), b);
+// N consecutive 32-bit words of shared memory.
+template <int N> struct Regs { uint32_t v[N]; };
+template <int N>
+__device__ __forceinline__ Regs<N> ld_regs(const uint8_t* p) {
+    Regs<N> r;
+    if (N == 1) r.v[0] = *reinterpret_cast<const uint32_t*>(p);
+    if (N == 2) { const uint2 t = *reinterpret_cast<const uint2*>(p); r.v[0] = t.x; r.v[N > 1 ? 1 : 0] = t.y; }
+#pragma unroll
+    for (int i = 0; i + 4 <= N; i += 4) {
+        const uint4 t = *reinterpret_cast<const uint4*>(p + 4 * i);
+        r.v[i] = t.x; r.v[i + 1 < N ? i + 1 : 0] = t.y; r.v[i + 2 < N ? i + 2 : 0] = t.z; r.v[i + 3 < N ? i + 3 : 0] = t.w;
+    }
+    return r;
+}
+
+// One group of tasks with K columns: inputs into registers, then row after row.
+template <typename T, int BT, int K>
+__device__ __forceinline__ void walk_group(const uint8_t* img, const R1Group& g, int lane, const float* v, float* partials) {
+    constexpr int kWords = K * (int)sizeof(T) / 4;         // weight words of a row
+    const Regs<K / 2> c = ld_regs<K / 2>(img + g.cols_off + lane * (K * 2));
+    float x[K][BT];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const float* p = v + (size_t)((c.v[k / 2] >> (16 * (k & 1))) & 0xffffu) * BT;
+        if (BT == 1) x[k][0] = *p;
+        if (BT == 2) { const float2 t = *reinterpret_cast<const float2*>(p); x[k][0] = t.x; x[k][BT > 1 ? 1 : 0] = t.y; }
+#pragma unroll
+        for (int b = 0; b + 4 <= BT; b += 4) {
+            const float4 t = *reinterpret_cast<const float4*>(p + b);
+            x[k][b] = t.x; x[k][b + 1 < BT ? b + 1 : 0] = t.y; x[k][b + 2 < BT ? b + 2 : 0] = t.z; x[k][b + 3 < BT ? b + 3 : 0] = t.w;
+        }
+    }
+    const uint8_t* w = img + g.w_off + lane * (kWords == 8 ? 16 : kWords * 4);
+    const uint32_t* pos = reinterpret_cast<const uint32_t*>(img + g.pos_off) + lane;
+    auto row = [&](const Regs<kWords>& q, uint32_t place) {
+        float wf[K];
+#pragma unroll
+        for (int i = 0; i < kWords; ++i) {
+            if (sizeof(T) == 2) { const float2 t = half2_to_float2(q.v[i]); wf[(2 * i) % K] = t.x; wf[(2 * i + 1) % K] = t.y; }
+            else wf[i % K] = __uint_as_float(q.v[i]);
+        }
+        float* out = partials + place * BT;
+        if (BT == 1) {
+            float2 a = make_float2(wf[0] * x[0][0], wf[1] * x[1][0]);
+#pragma unroll
+            for (int k = 2; k < K; k += 2) a = fma2(make_float2(wf[k], wf[k + 1]), make_float2(x[k][0], x[k + 1][0]), a);
+            *out = a.x + a.y;
         } else {
-            const float4 v0 = *reinterpret_cast<const float4*>(w + i * kStride), v1 = *reinterpret_cast<const float4*>(w + i * kStride + 32);
-            a = fma2(make_float2(v0.x, v0.y), make_float2(x0.x, x0.y), a);
-            b = fma2(make_float2(v0.z, v0.w), make_float2(x0.z, x0.w), b);
-            a = fma2(make_float2(v1.x, v1.y), make_float2(x1.x, x1.y), a);
-            b = fma2(make_float2(v1.z, v1.w), make_float2(x1.z, x1.w), b);
+            float2 a[BT / 2 > 0 ? BT / 2 : 1];
+#pragma unroll
+            for (int b = 0; b < BT / 2; ++b) a[b] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+                for (int b = 0; b < BT / 2; ++b) a[b] = fma2(make_float2(wf[k], wf[k]), make_float2(x[k][2 * b], x[k][(2 * b + 1) % BT]), a[b]);
+            if (BT == 2) *reinterpret_cast<float2*>(out) = a[0];
+#pragma unroll
+            for (int b = 0; b + 1 < BT / 2; b += 2)
+                *reinterpret_cast<float4*>(out + 2 * b) = make_float4(a[b].x, a[b].y, a[(b + 1) % (BT / 2 > 0 ? BT / 2 : 1)].x, a[(b + 1) % (BT / 2 > 0 ? BT / 2 : 1)].y);
         }
+    };
+    auto load = [&](int r) {
+        if (kWords == 8) {                                 // fp32, eight columns: [half][lane]
+            const Regs<4> lo = ld_regs<4>(w + (size_t)r * 1024), hi = ld_regs<4>(w + (size_t)r * 1024 + 512);
+            Regs<kWords> q;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { q.v[i % kWords] = lo.v[i]; q.v[(4 + i) % kWords] = hi.v[i]; }
+            return q;
+        }
+        return ld_regs<kWords>(w + (size_t)r * (32 * kWords * 4));
+    };
+    int r = 0;
+    for (; r + 2 <= g.rows; r += 2) {
+        const uint32_t p = pos[(r / 2) * 32];
+        const Regs<kWords> a = load(r), b = load(r + 1);
+        row(a, p & 0xffffu);
+        row(b, p >> 16);
     }
-    return (a.x + a.y) + (b.x + b.y);
+    if (r < g.rows) row(load(r), pos[(r / 2) * 32] & 0xffffu);
 }
 
-// The pairs of the recurrent part that stay in registers for the whole sequence.
-template <typename T, int N> struct RegPairs {
-    static constexpr int kN = N, kV = sizeof(T) == 2 ? 1 : 2;
-    uint4 w[kN][kV];
-    uint32_t o[kN];
-    __device__ __forceinline__ void load(const uint8_t* img, const R1Op& d, int warp, int lane) {
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-#pragma unroll
-            for (int v = 0; v < kV; ++v) w[i][v] = __ldg(reinterpret_cast<const uint4*>(img + d.reg_off) + ((warp * kN + i) * kV + v) * 32 + lane);
-            o[i] = __ldg(reinterpret_cast<const uint32_t*>(img + d.reg_places) + (warp * kN + i) * 32 + lane);
-        }
-    }
-    __device__ __forceinline__ float walk(const uint8_t* xg) const {
-        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < kN; ++i) {
-            const float4 x0 = *reinterpret_cast<const float4*>(xg + (o[i] & 0xffffu)), x1 = *reinterpret_cast<const float4*>(xg + (o[i] >> 16));
-            const uint4 v = w[i][0], u = w[i][kV - 1];
-            if (sizeof(T) == 2) {
-                a = fma2(half2_to_float2(v.x), make_float2(x0.x, x0.y), a);
-                b = fma2(half2_to_float2(v.y), make_float2(x0.z, x0.w), b);
-                a = fma2(half2_to_float2(v.z), make_float2(x1.x, x1.y), a);
-                b = fma2(half2_to_float2(v.w), make_float2(x1.z, x1.w), b);
-            } else {
-                a = fma2(make_float2(__uint_as_float(v.x), __uint_as_float(v.y)), make_float2(x0.x, x0.y), a);
-                b = fma2(make_float2(__uint_as_float(v.z), __uint_as_float(v.w)), make_float2(x0.z, x0.w), b);
-                a = fma2(make_float2(__uint_as_float(u.x), __uint_as_float(u.y)), make_float2(x1.x, x1.y), a);
-                b = fma2(make_float2(__uint_as_float(u.z), __uint_as_float(u.w)), make_float2(x1.z, x1.w), b);
-            }
-        }
-        return (a.x + a.y) + (b.x + b.y);
-    }
-};
-
-// The kept inputs of a part's blocks, four a thread: xg[i] = v[idx[i]] (padding indices point at a zero).
-__device__ __forceinline__ void gather(const uint16_t* idx, int quads, const float* v, float* xg) {
-    for (int q = threadIdx.x; q < quads; q += kR1Threads) {
-        const uint2 i = reinterpret_cast<const uint2*>(idx)[q];
-        float4 r;
-        r.x = v[i.x & 0xffffu]; r.y = v[i.x >> 16];
-        r.z = v[i.y & 0xffffu]; r.w = v[i.y >> 16];
-        reinterpret_cast<float4*>(xg)[q] = r;
+// A warp's groups [g0, g0 + n) of one product.
+template <typename T, int BT>
+__device__ __forceinline__ void walk(const uint8_t* img, const R1Group* groups, int n, int lane, const float* v, float* partials) {
+    constexpr int kWide = BT >= 8 ? 4 : 8;                 // r1_wide()
+    for (int i = 0; i < n; ++i) {
+        const R1Group g = groups[i];
+        if (g.narrow) walk_group<T, BT, kWide / 2>(img, g, lane, v, partials);
+        else walk_group<T, BT, kWide>(img, g, lane, v, partials);
     }
 }
 
-template <typename T, int CELL>
+template <typename T, int CELL, int BT>
 __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn1_kernel(const __grid_constant__ R1Args a) {
     extern __shared__ __align__(128) uint8_t smem[];
     constexpr int OPS = CELL == kR1Lstmp || CELL == kR1GruRb ? 2 : 1;
     constexpr int G0 = CELL == kR1Lstm || CELL == kR1Lstmp ? 4 : CELL == kR1Gru ? 3 : 2;
+    constexpr bool kHasC = CELL == kR1Lstm || CELL == kR1Lstmp;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const R1Cta me = a.ctas[blockIdx.x];
-    const int layer = me.layer, I = a.in_size[layer], S = a.S, H = a.H, T_ = a.T;
-    float* vu = reinterpret_cast<float*>(smem + a.vu);
-    float* vr = reinterpret_cast<float*>(smem + a.vr);
-    float* vm = reinterpret_cast<float*>(smem + a.vm);
-    float2* part = reinterpret_cast<float2*>(smem + a.part);
+    const int layer = me.layer, below = layer - 1, I = a.in_size[layer], S = a.S, H = a.H, T_ = a.T, B = a.B;
+    const uint8_t* img = smem;
+    auto f32 = [&](uint32_t off) { return reinterpret_cast<float*>(smem + off); };
+    float* vr = f32(a.vr);
+    float* vm = f32(a.vm);
+    float* cs = f32(a.cs);
     uint64_t* bar = reinterpret_cast<uint64_t*>(smem + a.misc);
     volatile int* s_ok = reinterpret_cast<volatile int*>(smem + a.misc + 8);
-    const uint8_t* img = smem;
 
-    // ---- weights, initial state, first input
+    // ---- weights; initial state; first input.  A staged vector holds BT values per column and ends in zeros.
     if (tid == 0) {
         mbar_init(bar, 1);
         mbar_fence_init();
-        mbar_expect_tx(bar, me.smem_bytes);
+        mbar_expect_tx(bar, me.bytes);
         const uint8_t* src = a.images + (size_t)me.off16 * 16;
-        for (uint32_t off = 0; off < me.smem_bytes; off += 16384u) bulk_g2s(smem + off, src + off, min(16384u, me.smem_bytes - off), bar);
+        for (uint32_t off = 0; off < me.bytes; off += 16384u) bulk_g2s(smem + off, src + off, min(16384u, me.bytes - off), bar);
         *s_ok = 1;
     }
-    for (int i = tid; i <= S; i += kR1Threads) vr[i] = i < S && a.h0 ? __ldg(a.h0 + (size_t)layer * S + i) : 0.f;
-    for (int i = tid; i <= I; i += kR1Threads) vu[i] = i < I && layer == 0 ? __ldg(a.x + i) : 0.f;
-    if (OPS == 2 && tid == 0) vm[H] = 0.f;
+    auto stage = [&](float* dst, const float* src, int n) {      // [B][n] in global memory
+        for (int b = 0; b < BT; ++b)
+            for (int i = tid; i < n; i += kR1Threads) dst[i * BT + b] = src && b < B ? __ldg(src + (size_t)b * n + i) : 0.f;
+    };
+    stage(vr, a.h0 ? a.h0 + (size_t)layer * B * S : nullptr, S);
+    if (layer == 0) stage(f32(a.vu[0]), a.x, I);
+    if (tid < BT) { vr[S * BT + tid] = 0.f; f32(a.vu[0])[I * BT + tid] = 0.f; f32(a.vu[1])[I * BT + tid] = 0.f; if (OPS == 2) vm[H * BT + tid] = 0.f; }
+    if (layer == 0 && BT > 1)                                    // batch columns past B stay zero
+        for (int i = tid; i < I * BT; i += kR1Threads) if (i % BT >= B) f32(a.vu[1])[i] = 0.f;
     const uint32_t base = a.epoch[blockIdx.x] + 1u;        // the step number of step 0
     uint32_t above0 = 0;                                   // the progress of the layer above when this call began
     if (layer + 1 < a.L) above0 = ld_relaxed(a.progress + layer + 1);
@@ -193,131 +235,156 @@ __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn1_kernel(const __grid_co
         if (tid == 0) a.epoch[blockIdx.x] = base - 1u + (uint32_t)T_;
         return;
     }
-
-    // ---- what stays the same over the steps
     const R1Header* hd = reinterpret_cast<const R1Header*>(img);
-    constexpr int kRegPairs = (sizeof(T) == 2 ? 4 : 2) / OPS;     // r1_reg_pairs()
-    RegPairs<T, kRegPairs> regs[OPS];
-    struct Walk { const uint4* w[2]; const uint32_t* o[2]; int n[2]; } wk[OPS];
-    struct Gate { int u, t0, k; bool on; float bias; } gt[OPS];
-    const int j = lane >> 2, g = lane & 3;
+    const int U0 = hd->op[0].units, U1 = OPS == 2 ? hd->op[OPS - 1].units : 0;
+    // places of partial sums that no task writes stay zero; cell state and bias of the CTA's units
+#pragma unroll
+    for (int op = 0; op < OPS; ++op) for (int i = tid; i < (int)hd->op[op].partials * BT; i += kR1Threads) f32(a.part[op])[i] = 0.f;
+    if (kHasC)
+        for (int i = tid; i < U0 * BT; i += kR1Threads) {
+            const int u = i / BT, b = i % BT;
+            cs[i] = a.c0 && b < B ? __ldg(a.c0 + ((size_t)layer * B + b) * H + hd->op[0].unit0 + u) : 0.f;
+        }
+    const float* bl = a.bias[layer];
+    for (int i = tid; i < 4 * U0; i += kR1Threads) {
+        const int g = i / U0, u = i % U0;
+        f32(a.bias0)[i] = bl && g < (CELL == kR1Gru ? 4 : G0) ? __ldg(bl + (size_t)g * H + hd->op[0].unit0 + u) : 0.f;
+    }
+    if (OPS == 2)
+        for (int u = tid; u < U1; u += kR1Threads) f32(a.bias1)[u] = bl && CELL == kR1GruRb ? __ldg(bl + (size_t)2 * H + hd->op[OPS - 1].unit0 + u) : 0.f;
+    struct Walk { const R1Group* g; int n[2]; } wk[OPS];
 #pragma unroll
     for (int op = 0; op < OPS; ++op) {
-        const R1Op& d = hd->op[op];
-        regs[op].load(a.images + (size_t)me.off16 * 16, d, warp, lane);
-        const uint4 wd = reinterpret_cast<const uint4*>(img + d.warp_off)[warp];
-        wk[op].w[0] = reinterpret_cast<const uint4*>(img) + wd.x + lane;
-        wk[op].w[1] = wk[op].w[0] + (size_t)wd.z * (sizeof(T) == 2 ? 32 : 64);
-        wk[op].o[0] = reinterpret_cast<const uint32_t*>(img + wd.y) + lane;
-        wk[op].o[1] = wk[op].o[0] + (size_t)wd.z * 32;
-        wk[op].n[0] = (int)wd.z; wk[op].n[1] = (int)wd.w;
-        // gate lanes: four per unit, six units per warp
-        const int gates = op == 0 ? G0 : 1, u = warp * kR1WarpUnits + j;
-        gt[op].u = (int)d.unit0 + u;
-        gt[op].on = j < kR1WarpUnits && u < (int)d.units;
-        // GRU: lanes 2 and 3 take the input and the hidden part of the candidate's row
-        const int row_g = CELL == kR1Gru ? min(g, 2) : g;
-        const bool has = gt[op].on && row_g < gates;
-        const uint32_t row = has ? reinterpret_cast<const uint32_t*>(img + d.rows_off)[row_g * (int)d.units + u] : 0u;
-        gt[op].t0 = (int)(row & 0xffffu); gt[op].k = (int)(row >> 16);
-        const float* bl = a.bias[layer];
-        gt[op].bias = 0.f;
-        if (bl && gt[op].on) {
-            if (op == 0 && g < (CELL == kR1Gru ? 4 : G0)) gt[op].bias = __ldg(bl + (size_t)g * H + gt[op].u);
-            if (op == 1 && CELL == kR1GruRb && g == 0) gt[op].bias = __ldg(bl + (size_t)2 * H + gt[op].u);
-        }
+        const uint16_t* wd = reinterpret_cast<const uint16_t*>(img + hd->op[op].warp_off) + warp * 4;
+        wk[op].g = reinterpret_cast<const R1Group*>(img + hd->op[op].groups_off) + wd[0];
+        wk[op].n[0] = wd[1]; wk[op].n[1] = wd[2];
     }
-    float c_state = 0.f;                                   // LSTM, LSTMP: cell state of the lanes' unit
-    if ((CELL == kR1Lstm || CELL == kR1Lstmp) && gt[0].on && a.c0) c_state = __ldg(a.c0 + (size_t)layer * H + gt[0].u);
-
-    // ---- the exchange.  Words are asked for early (poll_issue) and looked at late (poll_take).
-    auto slot = [&](int e, int l, int t) { return a.ex[e][l] + (size_t)(t & (kR1Ring - 1)) * a.words[e][l]; };
-    auto poll_issue = [&](uint4 (&w)[kR1Words], const uint4* src, int n) {
+    // row sums: 2^lp neighbouring lanes per row
+    int lp[OPS];
 #pragma unroll
-        for (int q = 0; q < kR1Words; ++q)
-            if (tid + q * kR1Threads < n) w[q] = ld_word(src + tid + q * kR1Threads);
+    for (int op = 0; op < OPS; ++op) { lp[op] = 0; while (lp[op] < 5 && (hd->op[op].n_rows << (lp[op] + 1)) <= kR1Threads) ++lp[op]; }
+
+    // ---- the exchange.  The first words are asked for early (poll_issue), all are taken in poll_take.
+    uint4* ex_state = a.ex[0][layer];
+    const int n_state = a.words[0][layer];
+    const uint32_t* map_state = a.wmap[0][layer];
+    uint4* ex_mid = OPS == 2 ? a.ex[1][layer] : nullptr;
+    const int n_mid = OPS == 2 ? a.words[1][layer] : 0;
+    const uint32_t* map_mid = OPS == 2 ? a.wmap[1][layer] : nullptr;
+    const uint4* ex_below = layer > 0 ? a.ex[0][below] : nullptr;
+    const int n_below = layer > 0 ? a.words[0][below] : 0;
+    const uint32_t* map_below = layer > 0 ? a.wmap[0][below] : nullptr;
+    auto poll_issue = [&](Word (&w)[kR1Words], const uint4* src, int n) {
+#pragma unroll
+        for (int q = 0; q < kR1Words; ++q) if (tid + q * kR1Threads < n) w[q] = ld_word(src + tid + q * kR1Threads);
     };
-    auto poll_take = [&](uint4 (&w)[kR1Words], const uint4* src, int n, const uint32_t* map, uint32_t want, float* dst) {
+    auto take_word = [&](Word w, const uint4* src, const uint32_t* map, int i, uint32_t want, float* dst) {
+        unsigned long long t0 = 0;
+        unsigned int spins = 0;
+        while (word_tag(w) != want) {
+            if (*s_ok == 0) { ok = false; break; }         // another thread has given up
+            if ((++spins & 63u) == 0) {
+                const unsigned long long now = global_ns();
+                if (t0 == 0) t0 = now;
+                else if (now - t0 > a.limit_ns) { *(volatile uint32_t*)a.status = (uint32_t)kDevBarrierTimeout; *s_ok = 0; ok = false; break; }
+            }
+            w = ld_word(src + i);
+        }
+        const uint32_t m = __ldg(map + i);
+        float* p = dst + (m & 0xffffffu);
+        p[0] = __uint_as_float((uint32_t)w);
+        if ((m >> 24) > 1) p[1] = __uint_as_float((uint32_t)(w >> 32));
+        if ((m >> 24) > 2) p[2] = __uint_as_float((uint32_t)(w >> 64));
+    };
+    auto poll_take = [&](Word (&w)[kR1Words], const uint4* src, int n, const uint32_t* map, uint32_t want, float* dst) {
         want += a.never;
 #pragma unroll
-        for (int q = 0; q < kR1Words; ++q) {
-            const int i = tid + q * kR1Threads;
-            if (i >= n) continue;
-            unsigned long long t0 = 0;
-            unsigned int spins = 0;
-            while (w[q].w != want) {
-                if (*s_ok == 0) { ok = false; break; }     // another thread has given up
-                if ((++spins & 63u) == 0) {
-                    const unsigned long long now = global_ns();
-                    if (t0 == 0) t0 = now;
-                    else if (now - t0 > a.limit_ns) { *(volatile uint32_t*)a.status = (uint32_t)kDevBarrierTimeout; *s_ok = 0; ok = false; break; }
+        for (int q = 0; q < kR1Words; ++q) if (tid + q * kR1Threads < n) take_word(w[q], src, map, tid + q * kR1Threads, want, dst);
+        for (int i = tid + kR1Words * kR1Threads; i < n; i += kR1Threads) take_word(ld_word(src + i), src, map, i, want, dst);
+    };
+    // The sums of a product's rows over their partial sums (GRU: input and recurrent part apart).
+    auto row_sums = [&](int op) {
+        const R1Row* rows = reinterpret_cast<const R1Row*>(img + hd->op[op].rows_off);
+        const float* P = f32(a.part[op]);
+        float* z = f32(a.z[op]);
+        const int n = hd->op[op].n_rows, lanes = 1 << lp[op], s = tid & (lanes - 1);
+        for (int r0 = 0; r0 < n; r0 += kR1Threads >> lp[op]) {
+            const int r = r0 + (tid >> lp[op]);
+            float sum[2][BT];
+#pragma unroll
+            for (int b = 0; b < BT; ++b) { sum[0][b] = 0.f; sum[1][b] = 0.f; }
+            if (r < n) {
+                const R1Row d = rows[r];
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    const float* q = P + (size_t)d.base[p] * 4 * BT;
+                    for (int i = s; i < d.quads[p]; i += lanes)
+#pragma unroll
+                        for (int k = 0; k < BT; ++k) {     // BT float4: four places of BT values
+                            const float4 t = *reinterpret_cast<const float4*>(q + ((size_t)i * BT + k) * 4);
+                            const float e[4] = {t.x, t.y, t.z, t.w};
+                            float* acc = sum[CELL == kR1Gru ? p : 0];
+                            if (BT == 1) acc[0] += (e[0] + e[1]) + (e[2] + e[3]);
+                            else
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) acc[(4 * k + j) % BT] += e[j];
+                        }
                 }
-                w[q] = ld_word(src + i);
             }
-            const uint32_t m = __ldg(map + i);
-            float* p = dst + (m & 0xffffu);
-            p[0] = __uint_as_float(w[q].x);
-            if ((m >> 16) > 1) p[1] = __uint_as_float(w[q].y);
-            if ((m >> 16) > 2) p[2] = __uint_as_float(w[q].z);
+            for (int off = lanes >> 1; off >= 1; off >>= 1)
+#pragma unroll
+                for (int b = 0; b < BT; ++b) {
+                    sum[0][b] += __shfl_xor_sync(0xffffffffu, sum[0][b], off);
+                    if (CELL == kR1Gru) sum[1][b] += __shfl_xor_sync(0xffffffffu, sum[1][b], off);
+                }
+            if (r < n && s == 0)
+#pragma unroll
+                for (int b = 0; b < BT; ++b) {
+                    if (CELL == kR1Gru) {
+                        const bool cand = r >= 2 * U0;     // the candidate's two parts stay apart: slots 2 and 3
+                        z[r * BT + b] = cand ? sum[0][b] : sum[0][b] + sum[1][b];
+                        if (cand) z[(r + U0) * BT + b] = sum[1][b];
+                    } else z[r * BT + b] = sum[0][b];
+                }
         }
     };
-    // The gate lanes' units to the other CTAs: two words of three units per warp.
-    auto publish = [&](int e, int op, float v, int t) {
-        const float v1 = __shfl_down_sync(0xffffffffu, v, 4), v2 = __shfl_down_sync(0xffffffffu, v, 8);
-        if (gt[op].on && g == 0 && (j == 0 || j == 3))
-            st_word(slot(e, layer, t) + hd->op[op].word0 + warp * 2 + j / 3,
-                    make_uint4(__float_as_uint(v), __float_as_uint(v1), __float_as_uint(v2), base + (uint32_t)t));
-    };
-    // The sum of a gate lane's row over its threads.
-    auto row_sum = [&](int op) {
-        float s = 0.f;
-        for (int i = 0; i < gt[op].k; ++i) {
-            const float2 p = part[gt[op].t0 + i];
-            s += CELL == kR1Gru ? (g == 3 ? p.y : g == 2 ? p.x : p.x + p.y) : p.x;
-        }
-        return s;
-    };
-    const bool gate_warp0 = warp * kR1WarpUnits < (int)hd->op[0].units, gate_warp1 = OPS == 2 && warp * kR1WarpUnits < (int)hd->op[OPS - 1].units;
-    const int below = layer - 1;
-    uint4 wr[kR1Words] = {}, wi[kR1Words] = {};
+    Word wr[kR1Words] = {}, wi[kR1Words] = {};
     if (layer > 0) {
-        poll_issue(wi, slot(0, below, 0), a.words[0][below]);
-        poll_take(wi, slot(0, below, 0), a.words[0][below], a.wmap[0][below], base, vu);
+        poll_issue(wi, ex_below, n_below);
+        poll_take(wi, ex_below, n_below, map_below, base, f32(a.vu[0]));
     }
-    __syncthreads();
-
+    if (!__syncthreads_and(ok)) {
+        if (tid == 0) a.epoch[blockIdx.x] = base - 1u + (uint32_t)T_;
+        return;
+    }
+#ifdef CSB_PHASE_CLOCKS
+    long long lap[8] = {0, 0, 0, 0, 0, 0, 0, 0}, lap_at = clock64();
+#endif
+    const int j = lane >> 2, g = lane & 3;                 // gate lanes: four per state, six states per warp and round
     for (int t = 0; t < T_; ++t) {
         const bool more = t + 1 < T_;
-        // u_t lies in vu.  Ask for the state of the step before; the input part of the product meanwhile.
-        const uint4* rec_src = slot(0, layer, t - 1);
-        if (t > 0) poll_issue(wr, rec_src, a.words[0][layer]);
-        gather(reinterpret_cast<const uint16_t*>(img + hd->op[0].gather_off[0]), hd->op[0].quads[0], vu, reinterpret_cast<float*>(smem + a.xg[0][0]));
-        if (CELL == kR1GruRb)
-            gather(reinterpret_cast<const uint16_t*>(img + hd->op[OPS - 1].gather_off[0]), hd->op[OPS - 1].quads[0], vu, reinterpret_cast<float*>(smem + a.xg[1][0]));
-        float x_next[4];
-        if (layer == 0 && more) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) if (tid + q * kR1Threads < I) x_next[q] = __ldg(a.x + (size_t)(t + 1) * I + tid + q * kR1Threads);
-        }
-        __syncthreads();
-        if (layer > 0 && tid == 0 && (t & (kR1Block - 1)) == kR1Block - 1) atomicAdd(a.progress + layer, 1u);   // u up to step t has been read
-        const float in0 = walk<T>(wk[0].w[0], wk[0].o[0], wk[0].n[0], smem + a.xg[0][0]);
-        float in1 = 0.f;
-        if (CELL == kR1GruRb) in1 = walk<T>(wk[OPS - 1].w[0], wk[OPS - 1].o[0], wk[OPS - 1].n[0], smem + a.xg[1][0]);
-        if (t > 0) poll_take(wr, rec_src, a.words[0][layer], a.wmap[0][layer], base + (uint32_t)(t - 1), vr);
-        if (more) {
-            // every thread is past reading vu: the next input frame moves in; the layer below is asked for its next state
-            if (layer == 0) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) if (tid + q * kR1Threads < I) vu[tid + q * kR1Threads] = x_next[q];
-                for (int i = tid + 4 * kR1Threads; i < I; i += kR1Threads) vu[i] = __ldg(a.x + (size_t)(t + 1) * I + i);
-            } else poll_issue(wi, slot(0, below, t + 1), a.words[0][below]);
-        }
+        const float* vu = f32(a.vu[t & 1]);
+        float* vu_next = f32(a.vu[(t + 1) & 1]);
+        // ---- u_t lies in vu: its part of the product, while h_{t-1} and u_{t+1} are on their way
+        const uint4* rec_src = ex_state + (size_t)((t - 1) & (kR1Ring - 1)) * n_state;
+        const uint4* next_src = ex_below + (size_t)((t + 1) & (kR1Ring - 1)) * n_below;
+        if (layer == 0 && more)
+            for (int b = 0; b < B; ++b)
+                for (int i = tid; i < I; i += kR1Threads) cp_async4(vu_next + i * BT + b, a.x + ((size_t)(t + 1) * B + b) * I + i);
+        if (t > 0) poll_issue(wr, rec_src, n_state);
+        walk<T, BT>(img, wk[0].g, wk[0].n[0], lane, vu, f32(a.part[0]));
+        if (CELL == kR1GruRb) walk<T, BT>(img, wk[OPS - 1].g, wk[OPS - 1].n[0], lane, vu, f32(a.part[1]));
+        R1_LAP(0);                                         // product of the input part
+        if (t > 0) poll_take(wr, rec_src, n_state, map_state, base + (uint32_t)(t - 1), vr);
+        if (layer > 0 && more) poll_issue(wi, next_src, n_below);
+        R1_LAP(1);                                         // the state of the step before
         if (!__syncthreads_and(ok)) break;
-        gather(reinterpret_cast<const uint16_t*>(img + hd->op[0].gather_off[1]), hd->op[0].quads[1], vr, reinterpret_cast<float*>(smem + a.xg[0][1]));
-        __syncthreads();
-        const float rec0 = regs[0].walk(smem + a.xg[0][1]) + walk<T>(wk[0].w[1], wk[0].o[1], wk[0].n[1], smem + a.xg[0][1]);
-        part[tid] = CELL == kR1Gru ? make_float2(in0, rec0) : make_float2(in0 + rec0, 0.f);
+        R1_LAP(2);
+        if (layer > 0 && tid == 0 && (t & (kR1Block - 1)) == kR1Block - 1) atomicAdd(a.progress + layer, 1u);   // u up to step t has been read
+        walk<T, BT>(img, wk[0].g + wk[0].n[0], wk[0].n[1], lane, vr, f32(a.part[0]));
+        R1_LAP(3);                                         // product of the recurrent part
+        if (layer > 0 && more) poll_take(wi, next_src, n_below, map_below, base + (uint32_t)(t + 1), vu_next);
+        if (layer == 0 && more) cp_async_wait();
         // before the slots of steps t .. t + 7 are overwritten, the layer above must have read what they
         // hold, steps up to t - 25.  Only the sum over its CTAs of the blocks of 8 they have read is kept:
         // CTAs of one layer are never more than two steps apart, so while one has not finished block k
@@ -335,80 +402,101 @@ __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn1_kernel(const __grid_co
             }
         }
         if (!__syncthreads_and(ok)) break;
-        // ---- gates
-        float zg = 0.f;                                    // reset-before GRU: the update gate, on the unit's lane 1
-        if (gate_warp0) {
-            float z = row_sum(0) + gt[0].bias;
-            const int l0 = lane & ~3;
-            float h = 0.f;
-            if (CELL == kR1Lstm || CELL == kR1Lstmp) {
+        row_sums(0);
+        __syncthreads();
+        R1_LAP(4);                                         // row sums
+        // ---- gates: lane g of a state's four applies gate g
+        const int E0 = U0 * BT;
+        for (int e0 = warp * kR1WarpUnits; e0 < E0; e0 += kR1Warps * kR1WarpUnits) {
+            const int e = e0 + j, l0 = lane & ~3;
+            const bool on = j < kR1WarpUnits && e < E0;
+            const int u = on ? e / BT : 0, b = on ? e % BT : 0;
+            float z = on && g < (CELL == kR1Gru ? 4 : G0) ? f32(a.z[0])[g * E0 + e] + f32(a.bias0)[g * U0 + u] : 0.f;
+            const int at = ((int)hd->op[0].unit0 + u) * BT + b;      // the state's element in the staged vectors
+            const float hp = CELL == kR1Gru || CELL == kR1Ligru || CELL == kR1GruRb ? vr[at] : 0.f;
+            float h, c = 0.f;
+            if (kHasC) {
+                c = on ? cs[e] : 0.f;
                 z = g == 2 ? tanhf(z) : logistic(z);
                 const float zi = __shfl_sync(0xffffffffu, z, l0), zf = __shfl_sync(0xffffffffu, z, l0 + 1);
                 const float zc = __shfl_sync(0xffffffffu, z, l0 + 2), zo = __shfl_sync(0xffffffffu, z, l0 + 3);
-                c_state = zf * c_state + zi * zc;
-                h = zo * tanhf(c_state);
-                if (!more && a.cT && gt[0].on && g == 0) a.cT[(size_t)layer * H + gt[0].u] = c_state;
+                c = zf * c + zi * zc;
+                h = zo * tanhf(c);
+                if (on && g == 0) cs[e] = c;
             } else if (CELL == kR1Gru) {
                 if (g < 2) z = logistic(z);
                 const float r = __shfl_sync(0xffffffffu, z, l0), zz = __shfl_sync(0xffffffffu, z, l0 + 1);
                 const float ni = __shfl_sync(0xffffffffu, z, l0 + 2), nh = __shfl_sync(0xffffffffu, z, l0 + 3);
-                const float n = tanhf(ni + r * nh), hp = gt[0].on ? vr[gt[0].u] : 0.f;
-                h = (1.f - zz) * n + zz * hp;
+                h = (1.f - zz) * tanhf(ni + r * nh) + zz * hp;
             } else if (CELL == kR1Ligru) {
                 if (g == 0) z = logistic(z);
                 const float zz = __shfl_sync(0xffffffffu, z, l0), cand = fmaxf(__shfl_sync(0xffffffffu, z, l0 + 1), 0.f);
-                const float hp = gt[0].on ? vr[gt[0].u] : 0.f;
                 h = zz * hp + (1.f - zz) * cand;
             } else {
                 z = logistic(z);
-                zg = __shfl_sync(0xffffffffu, z, l0 + 1);
-                h = __shfl_sync(0xffffffffu, z, l0) * (gt[0].on ? vr[gt[0].u] : 0.f);     // r * h_{t-1}
+                if (on && g == 1) cs[e] = z;               // the update gate, for the second half of the step
+                h = __shfl_sync(0xffffffffu, z, l0) * hp;  // r * h_{t-1}
             }
-            if (OPS == 2) publish(1, 0, h, t);
-            else {
-                if (more || layer + 1 < a.L) publish(0, 0, h, t);
-                if (gt[0].on && g == 0) {
-                    if (layer == a.L - 1 && a.y) a.y[(size_t)t * S + gt[0].u] = h;
-                    if (!more && a.hT) a.hT[(size_t)layer * S + gt[0].u] = h;
+            const float h1 = __shfl_down_sync(0xffffffffu, h, 4), h2 = __shfl_down_sync(0xffffffffu, h, 8);
+            uint4* ex = OPS == 2 ? ex_mid + (size_t)(t & (kR1Ring - 1)) * n_mid : ex_state + (size_t)(t & (kR1Ring - 1)) * n_state;
+            if (on && g == 0 && (j == 0 || j == 3) && (OPS == 2 || more || layer + 1 < a.L)) st_word(ex + hd->op[0].word0 + e / 3, h, h1, h2, base + (uint32_t)t);
+            if (on && g == 0 && b < B) {
+                if (OPS == 1) {
+                    if (layer == a.L - 1 && a.y) a.y[((size_t)t * B + b) * S + at / BT] = h;
+                    if (!more && a.hT) a.hT[((size_t)layer * B + b) * S + at / BT] = h;
                 }
+                if (kHasC && !more && a.cT) a.cT[((size_t)layer * B + b) * H + at / BT] = c;
             }
         }
+        R1_LAP(5);                                         // gates
         if (OPS == 2) {
             // ---- second product of the step: what the first one gave, from every CTA of the layer
-            const uint4* src = slot(1, layer, t);
-            poll_issue(wr, src, a.words[1][layer]);
-            poll_take(wr, src, a.words[1][layer], a.wmap[1][layer], base + (uint32_t)t, vm);
+            const uint4* src = ex_mid + (size_t)(t & (kR1Ring - 1)) * n_mid;
+            poll_issue(wr, src, n_mid);
+            poll_take(wr, src, n_mid, map_mid, base + (uint32_t)t, vm);
             if (!__syncthreads_and(ok)) break;
-            gather(reinterpret_cast<const uint16_t*>(img + hd->op[1].gather_off[1]), hd->op[1].quads[1], vm, reinterpret_cast<float*>(smem + a.xg[1][1]));
+            R1_LAP(6);                                     // exchange inside the step
+            walk<T, BT>(img, wk[OPS - 1].g + wk[OPS - 1].n[0], wk[OPS - 1].n[1], lane, vm, f32(a.part[1]));
             __syncthreads();
-            part[tid] = make_float2(in1 + (regs[OPS - 1].walk(smem + a.xg[1][1]) + walk<T>(wk[OPS - 1].w[1], wk[OPS - 1].o[1], wk[OPS - 1].n[1], smem + a.xg[1][1])), 0.f);
+            row_sums(OPS - 1);
             __syncthreads();
-            if (gate_warp1) {
-                float h = row_sum(OPS - 1) + gt[OPS - 1].bias;
-                if (CELL == kR1GruRb) {
-                    const float n = tanhf(h), hp = gt[0].on ? vr[gt[0].u] : 0.f;
-                    h = (1.f - zg) * n + zg * hp;
-                }
-                if (more || layer + 1 < a.L) publish(0, OPS - 1, h, t);
-                if (gt[OPS - 1].on && g == 0) {
-                    if (layer == a.L - 1 && a.y) a.y[(size_t)t * S + gt[OPS - 1].u] = h;
-                    if (!more && a.hT) a.hT[(size_t)layer * S + gt[OPS - 1].u] = h;
+            const int E1 = U1 * BT;
+            for (int e0 = warp * kR1WarpUnits; e0 < E1; e0 += kR1Warps * kR1WarpUnits) {
+                const int e = e0 + j;
+                const bool on = j < kR1WarpUnits && e < E1;
+                const int u = on ? e / BT : 0, b = on ? e % BT : 0, at = ((int)hd->op[OPS - 1].unit0 + u) * BT + b;
+                float h = on ? f32(a.z[1])[e] + f32(a.bias1)[u] : 0.f;
+                if (CELL == kR1GruRb && on) { const float zz = cs[e]; h = (1.f - zz) * tanhf(h) + zz * vr[at]; }
+                const float h1 = __shfl_down_sync(0xffffffffu, h, 4), h2 = __shfl_down_sync(0xffffffffu, h, 8);
+                if (on && g == 0 && (j == 0 || j == 3) && (more || layer + 1 < a.L))
+                    st_word(ex_state + (size_t)(t & (kR1Ring - 1)) * n_state + hd->op[OPS - 1].word0 + e / 3, h, h1, h2, base + (uint32_t)t);
+                if (on && g == 0 && b < B) {
+                    if (layer == a.L - 1 && a.y) a.y[((size_t)t * B + b) * S + at / BT] = h;
+                    if (!more && a.hT) a.hT[((size_t)layer * B + b) * S + at / BT] = h;
                 }
             }
-        }
-        // ---- the next input: from the layer below (layer 0 has put it in place already)
-        if (layer > 0 && more) {
-            poll_take(wi, slot(0, below, t + 1), a.words[0][below], a.wmap[0][below], base + (uint32_t)(t + 1), vu);
-            if (!__syncthreads_and(ok)) break;
+            R1_LAP(7);                                     // second product, its sums and gates
         }
     }
+#ifdef CSB_PHASE_CLOCKS
+    if (tid == 0) for (int i = 0; i < 8; ++i) a.clocks[(size_t)blockIdx.x * 8 + i] = lap[i];
+#endif
     if (tid == 0) a.epoch[blockIdx.x] = base - 1u + (uint32_t)T_;
 }
+
+#ifdef CSB_PHASE_CLOCKS
+static long long* g_r1_clocks = nullptr;
+static int g_r1_clock_ctas = 0;
+extern "C" int csb_debug_rnn1_clocks(long long* host_out, int max_ctas) {
+    cudaMemcpy(host_out, g_r1_clocks, (size_t)std::min(max_ctas, g_r1_clock_ctas) * 8 * 8, cudaMemcpyDeviceToHost);
+    return g_r1_clock_ctas;
+}
+#endif
 
 // Everything one (cell, layer stack) needs on the device; built on first use and kept until one of
 // its matrices is freed.
 struct Rnn1Plan {
-    int cell = 0, L = 0, device = 0, n_ctas = 0, H = 0, S = 0, val_dtype = 0;
+    int cell = 0, L = 0, BT = 1, device = 0, n_ctas = 0, H = 0, S = 0, val_dtype = 0;
     bool unusable = false;
     std::vector<uint64_t> uids;
     R1Args a{};
@@ -439,15 +527,19 @@ void drop_rnn1_plans(const csb_matrix* A) {
     cudaSetDevice(prev);
 }
 
-template <typename T>
+template <typename T, int BT>
 static const void* pick_kernel(int cell) {
     switch (cell) {
-        case kR1Lstm: return (const void*)csb_rnn1_kernel<T, kR1Lstm>;
-        case kR1Gru: return (const void*)csb_rnn1_kernel<T, kR1Gru>;
-        case kR1Lstmp: return (const void*)csb_rnn1_kernel<T, kR1Lstmp>;
-        case kR1Ligru: return (const void*)csb_rnn1_kernel<T, kR1Ligru>;
-        default: return (const void*)csb_rnn1_kernel<T, kR1GruRb>;
+        case kR1Lstm: return (const void*)csb_rnn1_kernel<T, kR1Lstm, BT>;
+        case kR1Gru: return (const void*)csb_rnn1_kernel<T, kR1Gru, BT>;
+        case kR1Lstmp: return (const void*)csb_rnn1_kernel<T, kR1Lstmp, BT>;
+        case kR1Ligru: return (const void*)csb_rnn1_kernel<T, kR1Ligru, BT>;
+        default: return (const void*)csb_rnn1_kernel<T, kR1GruRb, BT>;
     }
+}
+template <typename T>
+static const void* pick_kernel_bt(int cell, int BT) {
+    return BT == 1 ? pick_kernel<T, 1>(cell) : nullptr;
 }
 
 static int env_int(const char* name, int dflt) {
@@ -466,9 +558,9 @@ static int put(Rnn1Plan* P, const V* h, size_t n, V** d) {
 }
 
 // Returns 1 (and marks the plan) when the kernel does not take these matrices.
-static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, Rnn1Plan* P) {
+static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, Rnn1Plan* P) {
     const csb_matrix* A0 = W[0];
-    P->cell = cell; P->L = L; P->device = A0->device; P->H = H; P->S = S; P->val_dtype = A0->val_dtype;
+    P->cell = cell; P->L = L; P->BT = BT; P->device = A0->device; P->H = H; P->S = S; P->val_dtype = A0->val_dtype;
     P->unusable = true;
     for (int l = 0; l < L; ++l) P->uids.push_back(W[l]->uid);
     if (Wp) for (int l = 0; l < L; ++l) P->uids.push_back(Wp[l]->uid);
@@ -480,24 +572,23 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
     int want = (int)std::min<int64_t>(A0->sm_count, std::max<int64_t>(L, weights / env_int("CSB_R1_MIN", 1024)));
     want = std::min(A0->sm_count, env_int("CSB_R1_CTAS", want));
     R1HostPlan Hp;
-    const int hrc = plan_rnn1_host(cell, L, W, Wp, in_size, H, S, want, &Hp);
+    const int hrc = plan_rnn1_host(cell, L, W, Wp, in_size, H, S, BT, want, &Hp);
     if (hrc != CSB_OK) return hrc;
     R1Args& a = P->a;
-    size_t at = Hp.max_smem;
-    auto room = [&](size_t bytes) { const size_t o = at; at = (at + bytes + 15) & ~(size_t)15; return (uint32_t)o; };
+    size_t at = Hp.max_bytes;
+    auto room = [&](size_t floats) { const size_t o = at; at = (at + floats * 4 + 15) & ~(size_t)15; return (uint32_t)o; };
     int max_in = 0;
     for (int l = 0; l < L; ++l) max_in = std::max(max_in, in_size[l]);
-    // the gathered inputs of the input parts are used up before those of the recurrent part are written,
-    // and those before the second product's: they share their room
-    const size_t x00 = (Hp.max_xg[0][0] * 4 + 15) & ~(size_t)15;
-    const uint32_t xg = room(std::max(std::max(x00 + Hp.max_xg[1][0] * 4, Hp.max_xg[0][1] * 4), Hp.max_xg[1][1] * 4));
-    a.xg[0][0] = a.xg[0][1] = a.xg[1][1] = xg; a.xg[1][0] = xg + (uint32_t)x00;
-    a.vu = room((size_t)(max_in + 1) * 4); a.vr = room((size_t)(S + 1) * 4); a.vm = room((size_t)(H + 1) * 4);
-    a.part = room((size_t)kR1Threads * 8); a.misc = room(16);
+    for (uint32_t& v : a.vu) v = room((size_t)(max_in + 1) * BT);
+    a.vr = room((size_t)(S + 1) * BT); a.vm = room(r1_ops(cell) == 2 ? (size_t)(H + 1) * BT : 0);
+    for (int op = 0; op < 2; ++op) a.part[op] = room(Hp.max_partials[op] * BT);
+    a.z[0] = room(4 * Hp.max_units * BT); a.z[1] = room(r1_ops(cell) == 2 ? Hp.max_units * BT : 0);
+    a.cs = room(Hp.max_units * BT); a.bias0 = room(4 * Hp.max_units); a.bias1 = room(Hp.max_units);
+    a.misc = room(4);
     P->smem = at;
     if (P->smem > A0->smem_optin) return 1;
     P->n_ctas = (int)Hp.ctas.size();
-    P->kernel = P->val_dtype == CSB_F16 ? pick_kernel<__half>(cell) : pick_kernel<float>(cell);
+    P->kernel = P->val_dtype == CSB_F16 ? pick_kernel_bt<__half>(cell, BT) : pick_kernel_bt<float>(cell, BT);
     CSB_CUDA(cudaFuncSetAttribute(P->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A0->smem_optin));
     int occ = 0;
     CSB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, P->kernel, kR1Threads, P->smem));
@@ -525,14 +616,16 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
     return CSB_OK;
 }
 
-int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const float* const* bias, const float* x, int64_t T,
+int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const float* const* bias, const float* x, int64_t T, int B,
                  int H, int S, const int* in_size, const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream) {
     if (env_int("CSB_RNN_NO_RNN1", 0)) return 1;
+    if (B > 1) return 1;
+    const int BT = 1;
     Rnn1Plan* P = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_r1_mu);
         for (auto& p : g_r1_plans) {
-            if (p->cell != cell || p->L != L) continue;
+            if (p->cell != cell || p->L != L || p->BT != BT) continue;
             bool same = true;
             for (int l = 0; l < L; ++l) same = same && p->uids[l] == W[l]->uid && (!Wp || p->uids[L + l] == Wp[l]->uid);
             if (same) { P = p.get(); break; }
@@ -540,7 +633,7 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
         if (!P) {
             std::unique_ptr<Rnn1Plan> np(new Rnn1Plan());
             int rc;
-            try { rc = build_plan(cell, L, W, Wp, in_size, H, S, np.get()); }
+            try { rc = build_plan(cell, L, W, Wp, in_size, H, S, BT, np.get()); }
             catch (const std::bad_alloc&) { set_error("out of host memory while planning the time loop"); rc = CSB_ERR_ALLOC; }
             if (rc != CSB_OK && rc != 1) return rc;
             P = np.get();
@@ -550,7 +643,7 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     if (P->unusable) return 1;
     cudaStream_t st = (cudaStream_t)stream;
     const bool host_io = (flags & CSB_FLAG_HOST_IO) != 0, has_c = cell == kR1Lstm || cell == kR1Lstmp;
-    const size_t nx = (size_t)T * in_size[0], ny = y ? (size_t)T * S : 0, nh = (size_t)L * S, nc = has_c ? (size_t)L * H : 0;
+    const size_t nx = (size_t)T * B * in_size[0], ny = y ? (size_t)T * B * S : 0, nh = (size_t)L * B * S, nc = has_c ? (size_t)L * B * H : 0;
     R1Args a = P->a;
     a.x = x; a.h0 = h0; a.c0 = has_c ? c0 : nullptr; a.y = y; a.hT = hT; a.cT = has_c ? cT : nullptr;
     if (host_io) {
@@ -575,11 +668,15 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
         out(a.y, ny); out(a.hT, nh); out(a.cT, nc);
     }
     for (int l = 0; l < L; ++l) a.bias[l] = bias ? bias[l] : nullptr;
-    a.T = (int)T;
+    a.T = (int)T; a.B = B;
     uint32_t extra = 0;
     barrier_test_hook(&extra, &a.limit_ns);
     a.never = extra ? 0x40000000u : 0u;
     *P->h_status = 0;
+#ifdef CSB_PHASE_CLOCKS
+    if (!g_r1_clocks) cudaMalloc((void**)&g_r1_clocks, 192 * 8 * 8);
+    a.clocks = g_r1_clocks; g_r1_clock_ctas = P->n_ctas;
+#endif
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)P->n_ctas); cfg.blockDim = dim3(kR1Threads); cfg.dynamicSmemBytes = P->smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
