@@ -1,6 +1,7 @@
 """ctypes binding of libcsb: argument marshalling only.
 
-Every function mirrors one entry point of include/csb.h under the same name.
+Every function mirrors one entry point of include/csb.h under the same name; the calls of a
+model's hot path (products, recurrent calls) marshal their arguments in _csb_py (csrc/csb_py.c).
 Device buffers are torch CUDA tensors (torch is used for device memory and
 streams only); host buffers are numpy arrays.
 """
@@ -18,6 +19,10 @@ if not os.path.exists(_LIB_PATH):
     raise ImportError("libcsb.so is not built: run `python -m paper_2005_05758_b200.build` "
                       "(there is no CPU fallback)")
 lib = C.CDLL(_LIB_PATH)
+try:
+    from . import _csb_py                  # marshalling of the calls below in native code (csrc/csb_py.c)
+except ImportError as e:
+    raise ImportError("_csb_py is not built: run `python -m paper_2005_05758_b200.build`") from e
 
 CSB_F32, CSB_F16 = 0, 1
 CSB_FLAG_ASYNC, CSB_FLAG_HOST_IO = 1, 2
@@ -92,10 +97,20 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_current = None                            # (raw stream of a device, current device) of torch, once CUDA is up
+
+
 def _stream(stream) -> Optional[int]:
+    global _current
     if stream is None:
+        if _current is not None:
+            return _current[0](_current[1]())
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        st = torch.cuda.current_stream().cuda_stream           # initialises CUDA
+        raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if raw is not None and dev is not None and raw(dev()) == st:
+            _current = (raw, dev)                              # the same two steps without torch's stream object
+        return st
     return getattr(stream, "cuda_stream", stream)
 
 
@@ -193,10 +208,7 @@ def csb_encode_q16(dense: np.ndarray, block_r: int, block_c: int, row_keep: np.n
 
 def csb_spmm_q16(A: CsbMatrix, Xq, acc, stream=None) -> None:
     """acc[b, :] = A_q . Xq[b, :] in integers: Xq torch int16 [batch, cols], acc torch int64 [batch, rows]."""
-    lib.csb_spmm_q16.argtypes = [_P, _P, C.c_int64, C.c_int, _P, C.c_int64, _P]
-    lib.csb_spmm_q16.restype = C.c_int
-    batch = Xq.shape[0]
-    _check(lib.csb_spmm_q16(A.handle, _ptr(Xq), Xq.stride(0) if batch else 0, batch, _ptr(acc), acc.stride(0) if batch else 0, _stream(stream)))
+    _check(_csb_py.spmm(_FN["csb_spmm_q16"], A, Xq, acc, _stream(stream)))
 
 
 def csb_spmm_plan_dump(A: CsbMatrix, batch: int, sm_count: int) -> dict:
@@ -257,68 +269,45 @@ def csb_project(W, block_r: int, block_c: int, prune_fraction: float, row_keep=N
     return row_keep, col_keep, workspace
 
 
+#: Addresses of the library's functions that the native marshalling calls.
+_FN = {name: C.cast(getattr(lib, name), C.c_void_p).value
+       for name in ("csb_spmv", "csb_spmv_static_scratch", "csb_spmm", "csb_spmm_q16", "csb_lstm_forward", "csb_gru_forward",
+                    "csb_lstmp_forward", "csb_ligru_forward", "csb_gru_reset_before_forward")}
+_LSTM, _GRU, _LSTMP = 0, 1, 2              # argument lists: with cell states, without, with projections
+
+
 def csb_spmv(A: CsbMatrix, x, y, stream=None) -> None:
-    _check(lib.csb_spmv(A.handle, _ptr(x), _ptr(y), _stream(stream)))
+    _check(_csb_py.spmv(_FN["csb_spmv"], A, x, y, _stream(stream)))
 
 
 def csb_spmv_static_scratch(A: CsbMatrix, x, y, stream=None) -> None:
     """csb_spmv for callers that may not allocate device memory: the kernel's scratch is a fixed
     array inside the library (4 MiB per GPU), shared by all handles -- do not overlap calls."""
-    _check(lib.csb_spmv_static_scratch(A.handle, _ptr(x), _ptr(y), _stream(stream)))
+    _check(_csb_py.spmv(_FN["csb_spmv_static_scratch"], A, x, y, _stream(stream)))
 
 
 def csb_spmm(A: CsbMatrix, X, Y, stream=None) -> None:
-    batch = X.shape[0]
-    _check(lib.csb_spmm(A.handle, _ptr(X), X.stride(0) if batch else 0, batch, _ptr(Y),
-                        Y.stride(0) if batch else 0, _stream(stream)))
-
-
-def _ptr_array(items: Sequence, n: int):
-    arr = (_P * n)()
-    for i in range(n):
-        arr[i] = _ptr(items[i]) if not isinstance(items[i], CsbMatrix) else items[i].handle
-    return arr
+    _check(_csb_py.spmm(_FN["csb_spmm"], A, X, Y, _stream(stream)))
 
 
 def csb_lstm_forward(W: Sequence[CsbMatrix], bias, x, h0, c0, y, hT, cT, flags: int = 0, stream=None) -> None:
-    L = len(W)
-    T, B = (x.shape[0], x.shape[1])
-    b = _ptr_array(bias, L) if bias is not None else None
-    _check(lib.csb_lstm_forward(L, _ptr_array(W, L), b, _ptr(x), T, B, _ptr(h0), _ptr(c0), _ptr(y), _ptr(hT),
-                                _ptr(cT), flags, _stream(stream)))
+    _check(_csb_py.recurrent(_FN["csb_lstm_forward"], _LSTM, W, None, bias, x, h0, c0, y, hT, cT, flags, _stream(stream)))
 
 
 def csb_gru_forward(W: Sequence[CsbMatrix], bias, x, h0, y, hT, flags: int = 0, stream=None) -> None:
-    L = len(W)
-    T, B = (x.shape[0], x.shape[1])
-    b = _ptr_array(bias, L) if bias is not None else None
-    _check(lib.csb_gru_forward(L, _ptr_array(W, L), b, _ptr(x), T, B, _ptr(h0), _ptr(y), _ptr(hT), flags,
-                               _stream(stream)))
+    _check(_csb_py.recurrent(_FN["csb_gru_forward"], _GRU, W, None, bias, x, h0, None, y, hT, None, flags, _stream(stream)))
 
 
 def csb_lstmp_forward(W: Sequence[CsbMatrix], Wp: Sequence[CsbMatrix], bias, x, h0, c0, y, hT, cT, flags: int = 0, stream=None) -> None:
-    L = len(W)
-    lib.csb_lstmp_forward.argtypes = [C.c_int, C.POINTER(_P), C.POINTER(_P), C.POINTER(_P), _P, C.c_int64, C.c_int, _P, _P, _P, _P, _P, C.c_uint, _P]
-    lib.csb_lstmp_forward.restype = C.c_int
-    b = _ptr_array(bias, L) if bias is not None else None
-    _check(lib.csb_lstmp_forward(L, _ptr_array(W, L), _ptr_array(Wp, L), b, _ptr(x), x.shape[0], x.shape[1], _ptr(h0), _ptr(c0), _ptr(y),
-                                 _ptr(hT), _ptr(cT), flags, _stream(stream)))
-
-
-def _gru_like(fn, W, bias, x, h0, y, hT, flags, stream):
-    L = len(W)
-    fn.argtypes = [C.c_int, C.POINTER(_P), C.POINTER(_P), _P, C.c_int64, C.c_int, _P, _P, _P, C.c_uint, _P]
-    fn.restype = C.c_int
-    b = _ptr_array(bias, L) if bias is not None else None
-    _check(fn(L, _ptr_array(W, L), b, _ptr(x), x.shape[0], x.shape[1], _ptr(h0), _ptr(y), _ptr(hT), flags, _stream(stream)))
+    _check(_csb_py.recurrent(_FN["csb_lstmp_forward"], _LSTMP, W, Wp, bias, x, h0, c0, y, hT, cT, flags, _stream(stream)))
 
 
 def csb_ligru_forward(W: Sequence[CsbMatrix], bias, x, h0, y, hT, flags: int = 0, stream=None) -> None:
-    _gru_like(lib.csb_ligru_forward, W, bias, x, h0, y, hT, flags, stream)
+    _check(_csb_py.recurrent(_FN["csb_ligru_forward"], _GRU, W, None, bias, x, h0, None, y, hT, None, flags, _stream(stream)))
 
 
 def csb_gru_reset_before_forward(W: Sequence[CsbMatrix], bias, x, h0, y, hT, flags: int = 0, stream=None) -> None:
-    _gru_like(lib.csb_gru_reset_before_forward, W, bias, x, h0, y, hT, flags, stream)
+    _check(_csb_py.recurrent(_FN["csb_gru_reset_before_forward"], _GRU, W, None, bias, x, h0, None, y, hT, None, flags, _stream(stream)))
 
 
 # shorter aliases

@@ -4,12 +4,27 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcsb.so")
 SOURCES = ["csb_api.cpp", "csb_encode.cpp", "csb_plan.cpp", "csb_schedule.cpp", "csb_spmm_plan.cpp", "csb_panel_plan.cpp", "csb_product.cu", "csb_panel.cu", "csb_spmm_mma.cu", "csb_rnn.cu", "csb_rnn_step.cu", "csb_rnn1_plan.cpp", "csb_rnn1.cu", "csb_cells.cu", "csb_fixed.cu", "csb_project.cu"]
 HEADERS = ["csb_internal.hpp", "csb_device.cuh", "csb_rnn1.hpp", "csb_gates.cuh", os.path.join("..", "..", "include", "csb.h")]
+
+
+PY_MODULE = os.path.join(HERE, "_csb_py" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+
+
+def build_py_module() -> str:
+    """Compile the marshalling module (a CPython extension, plain C) if it is missing or older than its source."""
+    src = os.path.join(CSRC, "csb_py.c")
+    if not os.path.exists(PY_MODULE) or os.path.getmtime(PY_MODULE) < os.path.getmtime(src):
+        res = subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-fPIC", "-shared", "-I" + sysconfig.get_paths()["include"], "-o", PY_MODULE, src],
+                             capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("gcc failed:\n" + res.stdout + res.stderr)
+    return PY_MODULE
 
 
 def _stale() -> bool:
@@ -34,6 +49,7 @@ def build(force: bool = False, verbose: bool = False, defines=(), out: str = Non
     instrumented library, so that the normal libcsb.so is never replaced by one."""
     if defines and not out:
         raise ValueError("an instrumented build needs its own output path")
+    build_py_module()
     if not defines and not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
