@@ -1,16 +1,18 @@
 """Build libcsb.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
 from __future__ import annotations
 
+import concurrent.futures
 import os
 import subprocess
 import sys
 import sysconfig
+import tempfile
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcsb.so")
-SOURCES = ["csb_api.cpp", "csb_encode.cpp", "csb_plan.cpp", "csb_schedule.cpp", "csb_spmm_plan.cpp", "csb_panel_plan.cpp", "csb_product.cu", "csb_panel.cu", "csb_spmm_mma.cu", "csb_rnn.cu", "csb_rnn_step.cu", "csb_rnn1_plan.cpp", "csb_rnn1.cu", "csb_cells.cu", "csb_fixed.cu", "csb_project.cu"]
-HEADERS = ["csb_internal.hpp", "csb_device.cuh", "csb_rnn1.hpp", "csb_gates.cuh", os.path.join("..", "..", "include", "csb.h")]
+SOURCES = ["csb_api.cpp", "csb_encode.cpp", "csb_plan.cpp", "csb_schedule.cpp", "csb_spmm_plan.cpp", "csb_panel_plan.cpp", "csb_product.cu", "csb_panel.cu", "csb_spmm_mma.cu", "csb_rnn.cu", "csb_rnn_step.cu", "csb_rnn1_plan.cpp", "csb_rnn1.cu", "csb_rnn1_b1.cu", "csb_rnn1_b4.cu", "csb_rnn1_b8.cu", "csb_cells.cu", "csb_fixed.cu", "csb_project.cu"]
+HEADERS = ["csb_internal.hpp", "csb_device.cuh", "csb_rnn1.hpp", "csb_rnn1_args.hpp", "csb_rnn1_kernel.cuh", "csb_gates.cuh", os.path.join("..", "..", "include", "csb.h")]
 
 
 PY_MODULE = os.path.join(HERE, "_csb_py" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
@@ -52,17 +54,22 @@ def build(force: bool = False, verbose: bool = False, defines=(), out: str = Non
     build_py_module()
     if not defines and not force and not _stale():
         return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    cmd = [nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-           "-Xcompiler", "-fPIC", "-shared", "-o", out or LIB] + ["-D" + d for d in defines] + [os.path.join(CSRC, s) for s in SOURCES]
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
-    if verbose:
-        sys.stderr.write(res.stderr)
+    nvcc = [os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-Xcompiler", "-fPIC"]
+    flags = ["-lineinfo", "-O3", "-std=c++17"] + ["-D" + d for d in defines] + (["-Xptxas", "-v"] if verbose else [])
+
+    def run(cmd):
+        res = subprocess.run(cmd, capture_output=True, text=True)
+        if res.returncode != 0:
+            raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+        if verbose:
+            sys.stderr.write(res.stderr)
+
+    # one object per source, compiled side by side
+    with tempfile.TemporaryDirectory() as tmp:
+        objects = [os.path.join(tmp, f + ".o") for f in SOURCES]
+        with concurrent.futures.ThreadPoolExecutor(os.cpu_count() or 1) as pool:
+            list(pool.map(run, [nvcc + flags + ["-c", "-o", o, os.path.join(CSRC, f)] for f, o in zip(SOURCES, objects)]))
+        run(nvcc + ["-shared", "-o", out or LIB] + objects)
     return out or LIB
 
 

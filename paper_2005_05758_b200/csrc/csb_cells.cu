@@ -211,8 +211,8 @@ static int cell_forward(int kind, int L, const csb_matrix_t* const* W, const csb
     if (prev != W[0]->device) CSB_CUDA(cudaSetDevice(W[0]->device));
     struct Restore { int prev, cur; ~Restore() { if (prev != cur) cudaSetDevice(prev); } } restore{prev, W[0]->device};
 
-    // one sequence: the batch-1 time loop in one launch, as long as the weights fit the SMs' shared memory
-    if (B == 1) {
+    // small batches: the resident time loop in one launch, as long as weights and vectors fit the SMs' shared memory
+    if (B <= 8) {
         const int cell = kind == kCellLstmp ? kR1Lstmp : kind == kCellLigru ? kR1Ligru : kR1GruRb;
         const int rc = rnn1_forward(cell, L, W, kind == kCellLstmp ? Wp : nullptr, bias, x, T, B, H, S, in_size, h0, c0, y, hT, cT, flags, stream);
         if (rc != 1) return rc;

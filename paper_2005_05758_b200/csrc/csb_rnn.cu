@@ -827,15 +827,15 @@ static int rnn_forward(int gates, int L, const csb_matrix_t* const* W, const flo
     CSB_CUDA(cudaSetDevice(W[0]->device));
     struct Restore { int d; ~Restore() { cudaSetDevice(d); } } restore{prev};
 
-    // larger batches with fp16 values: step by step, the products on tensor cores
-    if (rnn_stepwise_wanted(gates, L, W, B)) {
-        const int rc = rnn_forward_stepwise(gates, L, W, bias, x, T, B, H, in_size, h0, c0, y, hT, cT, flags, stream);
+    // small batches: the resident time loop, as long as weights and vectors fit the SMs' shared memory
+    if (B <= 8) {
+        const int rc = rnn1_forward(gates == 4 ? kR1Lstm : kR1Gru, L, W, nullptr, bias, x, T, B, H, H, in_size, h0, c0, y, hT, cT, flags, stream);
         if (rc != 1) return rc;
     }
 
-    // one sequence: the batch-1 time loop, as long as the weights fit the SMs' shared memory
-    if (B == 1) {
-        const int rc = rnn1_forward(gates == 4 ? kR1Lstm : kR1Gru, L, W, nullptr, bias, x, T, B, H, H, in_size, h0, c0, y, hT, cT, flags, stream);
+    // larger batches with fp16 values: step by step, the products on tensor cores
+    if (rnn_stepwise_wanted(gates, L, W, B)) {
+        const int rc = rnn_forward_stepwise(gates, L, W, bias, x, T, B, H, in_size, h0, c0, y, hT, cT, flags, stream);
         if (rc != 1) return rc;
     }
 

@@ -22,7 +22,6 @@ enum { kR1Threads = 512, kR1Warps = kR1Threads / 32,
        kR1WarpUnits = 6,                       // states whose gates a warp applies at a time: four lanes each, two words of three
        kR1MaxUnits = 255,
        kR1MaxRows = 16,                        // rows of a task
-       kR1Words = 2,                           // exchange words a thread asks for ahead
        kR1Ring = 32, kR1Block = 8 };           // steps a published vector stays; steps between two looks at the readers' progress
 
 // Columns of a wide task for a batch tile: its inputs stay in registers.

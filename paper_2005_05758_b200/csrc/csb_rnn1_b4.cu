@@ -1,0 +1,10 @@
+// The resident time loop's kernels for batch tiles of 4 (a file of their own: they compile for a while).
+#include "csb_rnn1_kernel.cuh"
+
+namespace csb {
+
+const void* r1_kernel_b4(int cell, int val_dtype) {
+    return val_dtype == CSB_F16 ? pick_kernel<__half, 4>(cell) : pick_kernel<float, 4>(cell);
+}
+
+}  // namespace csb
