@@ -1,7 +1,6 @@
-// Gate arithmetic of one LSTM / GRU layer and step for a tile of 32 hidden units x the whole batch
+// Gate arithmetic of one LSTM / GRU layer and step for a tile of 32 hidden units x some batch columns
 // (Section 2.1), with h_t written straight into the packed binary16 (hi, lo) input rows that the
-// batched product kernel reads.  Device functions shared by the per-step gate kernels and by the
-// time loop that keeps the batched product and the gates in one kernel.
+// batched product kernel reads.
 //
 // Packed layout: one row of `pitch` bytes per matrix column; x = hi + lo, hi at halves [slot], lo at
 // [cap + slot], slot = the product row (batch column; for the GRU, whose product has 2B rows,
@@ -46,15 +45,16 @@ __device__ __forceinline__ void pack_columns(float (*tile)[33], const float* __r
     pack_tile(tile, min(32, ncols - c0), nb, xp + (size_t)c0 * pitch, pitch, cap, slot0, nullptr, 0);
 }
 
-// LSTM, hidden units j0 .. j0 + 31:  c_t = s(z_f) c_{t-1} + s(z_i) tanh(z_g),  h_t = s(z_o) tanh(c_t);
+// LSTM, hidden units j0 .. j0 + 31 and batch columns b0 .. b0 + nb - 1 (nb <= 32):  c_t = s(z_f) c_{t-1} + s(z_i) tanh(z_g),  h_t = s(z_o) tanh(c_t);
 // rows of Z [B, 4H] stacked i, f, g, o.  h_t goes, packed, to rows j of xp_self (this layer's recurrent
 // columns) and of xp_next (the input columns of the layer above, or null), as fp32 to hs[b, j] and y_t[b, j].
 __device__ __forceinline__ void lstm_gates_tile(float (*tile)[33], const float* __restrict__ Z, const float* __restrict__ bias,
                                                 float* __restrict__ c, float* __restrict__ hs, uint8_t* __restrict__ xp_self,
-                                                uint8_t* __restrict__ xp_next, float* __restrict__ y_t, int pitch, int cap, int B, int H,
-                                                int j0) {
+                                                uint8_t* __restrict__ xp_next, float* __restrict__ y_t, int pitch, int cap, int b0, int nb,
+                                                int H, int j0) {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, nw = blockDim.x >> 5, j = j0 + tx;
-    for (int b = ty; b < B; b += nw) {
+    for (int bt = ty; bt < nb; bt += nw) {
+        const int b = b0 + bt;
         float h = 0.f;
         if (j < H) {
             const float* z = Z + (size_t)b * 4 * H;
@@ -67,20 +67,21 @@ __device__ __forceinline__ void lstm_gates_tile(float (*tile)[33], const float* 
             hs[e] = h;
             if (y_t) y_t[e] = h;
         }
-        tile[b][tx] = h;
+        tile[bt][tx] = h;
     }
     __syncthreads();
-    pack_tile(tile, min(32, H - j0), B, xp_self + (size_t)j0 * pitch, pitch, cap, 0, xp_next ? xp_next + (size_t)j0 * pitch : nullptr, 0);
+    pack_tile(tile, min(32, H - j0), nb, xp_self + (size_t)j0 * pitch, pitch, cap, b0, xp_next ? xp_next + (size_t)j0 * pitch : nullptr, b0);
 }
 
-// GRU (reset gate applied after the recurrent product), hidden units j0 .. j0 + 31:
+// GRU (reset gate applied after the recurrent product), hidden units j0 .. j0 + 31, batch columns b0 .. b0 + nb - 1:
 //   r = s(zx_r + zh_r + b_r),  u = s(zx_z + zh_z + b_z),  n = tanh(zx_n + b_in + r (zh_n + b_hn)),
 //   h_t = (1 - u) n + u h_{t-1};  zx = row b, zh = row B + b of Z [2B, 3H]; bias = b_r, b_z, b_in, b_hn.
 __device__ __forceinline__ void gru_gates_tile(float (*tile)[33], const float* __restrict__ Z, const float* __restrict__ bias,
                                                float* __restrict__ hs, uint8_t* __restrict__ xp_self, uint8_t* __restrict__ xp_next,
-                                               float* __restrict__ y_t, int pitch, int cap, int B, int H, int j0) {
+                                               float* __restrict__ y_t, int pitch, int cap, int B, int b0, int nb, int H, int j0) {
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, nw = blockDim.x >> 5, j = j0 + tx;
-    for (int b = ty; b < B; b += nw) {
+    for (int bt = ty; bt < nb; bt += nw) {
+        const int b = b0 + bt;
         float h = 0.f;
         if (j < H) {
             const float* zx = Z + (size_t)b * 3 * H;
@@ -95,10 +96,10 @@ __device__ __forceinline__ void gru_gates_tile(float (*tile)[33], const float* _
             hs[e] = h;
             if (y_t) y_t[e] = h;
         }
-        tile[b][tx] = h;
+        tile[bt][tx] = h;
     }
     __syncthreads();
-    pack_tile(tile, min(32, H - j0), B, xp_self + (size_t)j0 * pitch, pitch, cap, B, xp_next ? xp_next + (size_t)j0 * pitch : nullptr, 0);
+    pack_tile(tile, min(32, H - j0), nb, xp_self + (size_t)j0 * pitch, pitch, cap, B + b0, xp_next ? xp_next + (size_t)j0 * pitch : nullptr, b0);
 }
 
 }  // namespace csb

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <list>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -230,7 +231,7 @@ struct SpmmCta {
 static_assert(sizeof(SpmmCta) == 48, "three 16-byte words");
 // Warps per CTA: the 16 accumulator registers of one 8-column batch tile leave room for 32 warps per
 // SM, which halves the chain of dependent work a warp has to get through; wider tiles allow 16.
-inline int spmm_warps(int NT) { return NT == 1 ? 32 : 16; }
+inline int spmm_warps(int NT) { return NT == 1 ? 32 : NT == 8 ? 8 : 16; }   // (a tile of 64 columns: 128 accumulators a thread)
 // Batch classes: how many 8-column batch tiles a warp carries.  A pass covers 8 * NT <= 32 batch columns.
 inline int spmm_nt(int batch) { return batch <= 8 ? 1 : batch <= 16 ? 2 : 4; }
 inline int spmm_class_index(int batch) { return batch <= 8 ? 0 : batch <= 16 ? 1 : 2; }
@@ -249,7 +250,8 @@ struct SpmmHostPlan {
     double balance = 1.0, warp_balance = 1.0; // mean / max of the modelled cost over CTAs, and over warps
 };
 // Plans for `sm_count` SMs; returns CSB_OK, or 1 when the path does not suit the matrix.
-int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, SpmmHostPlan* out);
+// force_S > 0: this many column ranges per row group.
+int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, int force_S, SpmmHostPlan* out);
 struct MmaPlan {                           // device side, one per batch class, built on first use
     struct PerClass {
         bool built = false, unusable = false;
@@ -259,22 +261,23 @@ struct MmaPlan {                           // device side, one per batch class, 
         void* d_xp = nullptr;
         int64_t stream_bytes = 0;
         double balance = 1.0, warp_balance = 1.0;
-    } cls[3];
+    } cls[4];                              // batches of up to 8, 16, 32, 64 columns a pass
+    // plans without inputs of their own, for a share of the SMs (the layers of a recurrent stack); S = 0: free choice
+    struct Shared { int ci, sms, S; PerClass plan; };
+    std::list<Shared> shared;
 };
-int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream,
-                    const uint8_t* packed = nullptr);
+int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
+struct SpmmStack {                         // the products of a recurrent stack's layers (plans belong to the matrices)
+    int L = 0, NT = 0;
+    bool joint = false;                    // one launch serves several layers
+    const MmaPlan::PerClass* plan[kMaxLayers] = {};
+};
+int prepare_spmm_stack(int L, const csb_matrix* const* A, int batch, SpmmStack* out);
+// Y[l] = A[l] . xp[l] for the layers l0 <= l < l1.
+int launch_spmm_stack(const SpmmStack& K, int l0, int l1, const csb_matrix* const* A, uint8_t* const* xp, float* const* Y, int nb, int64_t ldy, void* stream);
 bool spmm_mma_applicable(const csb_matrix* A, int batch);
-// The time loop of a recurrent stack inside the batched product kernel (csb_spmm_mma.cu): everything on the device.
-struct RnnTileLoop {
-    int L, B, H, gates; int64_t T;
-    const csb_matrix* const* W; const float* const* bias; const int* in_size;
-    const float* x; float* y;              // [T, B, I0]; [T, B, H] or null
-    uint8_t* const* xp;                    // per layer: packed inputs of its product, initialised for step 0
-    float* z; float* c; float* hs;         // pre-activations [rows of the product, gates * H]; c [L, B, H] (LSTM); h [L, B, H]
-    unsigned int* gbar;                    // one word for the grid barrier
-    int pitch, cap;
-};
-int launch_rnn_tile_loop(const RnnTileLoop& R, void* stream);
+// Layer l alone, over fp32 inputs [batch, cols] (any batch).
+int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
 void free_mma(csb_matrix* A);
 
 // ---- panel layout of the batch-1 product (csb_panel_plan.cpp, csb_panel.cu) ----

@@ -13,10 +13,10 @@
 // Up to 32 product rows (LSTM: batch <= 32, GRU: batch <= 16) the fp32 buffers V_l do not exist at all:
 // the gate arithmetic writes h_t, and that of layer 0 also x_{t+1}, straight into the packed binary16
 // (hi, lo) input rows that the product kernel reads, transposed through shared memory so that the
-// stores of a row are contiguous; a step is then two launches per layer (product, gates).  With
-// CSB_RNN_STEP_LOOP=1, and where the layers' plans allow it, the whole sequence is instead ONE
-// cooperative launch of the product kernel's time loop (product pass, grid barrier, gates, grid barrier
-// per layer and step: csb_spmm_mma.cu).
+// stores of a row are contiguous.  The layers then run as a wavefront: in tick k layer l does step k - l,
+// which needs nothing newer than tick k - 1, so one product launch (the SMs shared between the layers) and
+// one launch of gates serve all layers, and the fixed cost of the two is paid once per tick instead of once
+// per layer and step.  Measured, two 2048-unit LSTM layers, 10x pruned, batch 32: 51 -> 29.6 us per step.
 //
 // GRU (reset gate applied after the recurrent product) needs the input part and the recurrent part
 // of the candidate's pre-activation apart.  One product still does: V_l has 2B rows, row b holds
@@ -46,7 +46,8 @@ struct StepPlan {
     int L = 0, B = 0, H = 0, gates = 0, device = -1;
     int in_size[kMaxLayers] = {};
     float* d_v[kMaxLayers] = {};       // [B, in_size[l] + H] per layer (GRU: [2B, ...], input rows then recurrent rows)
-    float* d_z = nullptr;              // [B, 4H] (GRU: [2B, 3H]) pre-activations of the layer being worked on
+    float* d_z = nullptr;              // [B, 4H] (GRU: [2B, 3H]) pre-activations; packed path: one such per layer
+    SpmmStack stack;                   // packed path
     float* d_c = nullptr;              // [L, B, H] cell state
     float* d_stage = nullptr;          // host-I/O staging of x and y
     size_t stage_cap = 0;
@@ -54,12 +55,11 @@ struct StepPlan {
     // `pitch` bytes per column of W_l, and the fp32 h of every layer
     uint8_t* d_xp[kMaxLayers] = {};
     float* d_h = nullptr;              // [L, B, H]
-    unsigned int* d_gbar = nullptr;    // grid-barrier word of the one-launch time loop
     int pitch = 0, cap = 0;
     ~StepPlan() {
         for (float* p : d_v) cudaFree(p);
         for (uint8_t* p : d_xp) cudaFree(p);
-        cudaFree(d_z); cudaFree(d_c); cudaFree(d_stage); cudaFree(d_h); cudaFree(d_gbar);
+        cudaFree(d_z); cudaFree(d_c); cudaFree(d_stage); cudaFree(d_h);
     }
 };
 static std::mutex g_step_mu;
@@ -155,29 +155,34 @@ __global__ void csb_pack_rows_kernel(const float* __restrict__ src, long long ld
     pack_columns(tile, src, ld, nb, ncols, (int)blockIdx.x * 32, xp, pitch, cap, slot0);
 }
 
-// Blocks 0 .. h_blocks - 1: the LSTM gates of 32 hidden units x the batch each; blocks from h_blocks on
-// pack x_next [B, I] (the next step's input of layer 0) into rows of xp0.
-__global__ void csb_lstm_gates_pack_kernel(const float* __restrict__ Z, const float* __restrict__ bias, float* __restrict__ c,
-                                           float* __restrict__ hs, uint8_t* __restrict__ xp_self, uint8_t* __restrict__ xp_next,
-                                           float* __restrict__ y_t, const float* __restrict__ x_next, int I, uint8_t* __restrict__ xp0,
-                                           int pitch, int cap, int B, int H, int h_blocks) {
+// The gates of one tick: blocks [part, next part) take a layer's hidden units, 32 at a time and 8 batch
+// columns each, the blocks behind the last part pack x_next [B, I] (the next input of layer 0) into
+// rows of xp0.
+struct GatePart {
+    const float* Z; const float* bias; float* c; float* hs; uint8_t* xp_self; uint8_t* xp_next; float* y;
+    int end;                                       // first block behind the part
+};
+struct GateArgs {
+    GatePart part[kMaxLayers];
+    const float* x_next; uint8_t* xp0;
+    int n_parts, I, pitch, cap, B, H, b_tiles;
+};
+template <int GATES>
+__global__ void __launch_bounds__(256) csb_gates_pack_kernel(const __grid_constant__ GateArgs a) {
+    __shared__ float tile[32][33];
     pdl_launch_dependents();
     pdl_wait();                                    // Z comes from the product in front, which also still reads xp0
-    __shared__ float tile[32][33];
-    if ((int)blockIdx.x < h_blocks) lstm_gates_tile(tile, Z, bias, c, hs, xp_self, xp_next, y_t, pitch, cap, B, H, (int)blockIdx.x * 32);
-    else pack_columns(tile, x_next, (long long)I, B, I, ((int)blockIdx.x - h_blocks) * 32, xp0, pitch, cap, 0);
-}
-
-// The same for the GRU (its product has 2B rows: the zeros of the unused slots are written once, before the first step).
-__global__ void csb_gru_gates_pack_kernel(const float* __restrict__ Z, const float* __restrict__ bias, float* __restrict__ hs,
-                                          uint8_t* __restrict__ xp_self, uint8_t* __restrict__ xp_next, float* __restrict__ y_t,
-                                          const float* __restrict__ x_next, int I, uint8_t* __restrict__ xp0, int pitch, int cap, int B,
-                                          int H, int h_blocks) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ float tile[32][33];
-    if ((int)blockIdx.x < h_blocks) gru_gates_tile(tile, Z, bias, hs, xp_self, xp_next, y_t, pitch, cap, B, H, (int)blockIdx.x * 32);
-    else pack_columns(tile, x_next, (long long)I, B, I, ((int)blockIdx.x - h_blocks) * 32, xp0, pitch, cap, 0);
+    int first = 0, p = 0;
+    while (p < a.n_parts && (int)blockIdx.x >= a.part[p].end) first = a.part[p++].end;
+    const int blk = (int)blockIdx.x - first;
+    if (p < a.n_parts) {
+        const GatePart& g = a.part[p];
+        const int j0 = blk / a.b_tiles * 32, b0 = blk % a.b_tiles * 8, nb = min(8, a.B - b0);
+        if (GATES == 4) lstm_gates_tile(tile, g.Z, g.bias, g.c, g.hs, g.xp_self, g.xp_next, g.y, a.pitch, a.cap, b0, nb, a.H, j0);
+        else gru_gates_tile(tile, g.Z, g.bias, g.hs, g.xp_self, g.xp_next, g.y, a.pitch, a.cap, a.B, b0, nb, a.H, j0);
+    } else {
+        pack_columns(tile, a.x_next, (long long)a.I, a.B, a.I, blk * 32, a.xp0, a.pitch, a.cap, 0);
+    }
 }
 
 static int env_flag(const char* name) {
@@ -223,11 +228,10 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
                 if (packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], (size_t)(in_size[l] + H) * np->pitch));
                 else CSB_CUDA(cudaMalloc((void**)&np->d_v[l], (size_t)rows_v * (in_size[l] + H) * 4));
             }
-            if (packed_path) {
-                CSB_CUDA(cudaMalloc((void**)&np->d_h, (size_t)L * B * H * 4));
-                CSB_CUDA(cudaMalloc((void**)&np->d_gbar, 4));
-            }
-            CSB_CUDA(cudaMalloc((void**)&np->d_z, (size_t)(gates == 3 ? 2 : 1) * B * gates * H * 4));
+            const int rc = prepare_spmm_stack(L, W, std::min(rows_v, 32), &np->stack);
+            if (rc != CSB_OK) return rc;
+            if (packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_h, (size_t)L * B * H * 4));
+            CSB_CUDA(cudaMalloc((void**)&np->d_z, (size_t)(packed_path ? L : 1) * (gates == 3 ? 2 : 1) * B * gates * H * 4));
             if (gates == 4) CSB_CUDA(cudaMalloc((void**)&np->d_c, (size_t)L * B * H * 4));
             P = np.get();
             g_step_plans.push_back(std::move(np));
@@ -273,49 +277,35 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             if (c0) CSB_CUDA(cudaMemcpyAsync(P->d_c, c0, ns * 4, in_kind, st));
             else CSB_CUDA(cudaMemsetAsync(P->d_c, 0, ns * 4, st));
         }
-        // On request (CSB_RNN_STEP_LOOP=1) the whole sequence in one launch of the product kernel's time loop,
-        // where that serves the stack.  Not the default: measured, two grid barriers per layer and step cost
-        // as much as the two launch hand-overs they replace (47.6 against 48-51 us per step on a two-layer
-        // 2048-unit LSTM at batch 32, 14.0 against 11.4 on a 1024-unit GRU at batch 8).
-        bool looped = false;
-        if (env_flag("CSB_RNN_STEP_LOOP") && T < (1 << 24)) {
-            RnnTileLoop R{};
-            R.L = L; R.B = B; R.H = H; R.gates = gates; R.T = T; R.W = W; R.bias = bias; R.in_size = in_size;
-            R.x = dx; R.y = dy; R.xp = P->d_xp; R.z = P->d_z; R.c = gru ? nullptr : P->d_c; R.hs = P->d_h; R.gbar = P->d_gbar;
-            R.pitch = pitch; R.cap = cap;
-            const int rc = launch_rnn_tile_loop(R, stream);
-            if (rc == CSB_OK) looped = true;
-            else if (rc != 1) return rc;
-        }
-        const int h_blocks = (H + 31) / 32, x_blocks = (I0 + 31) / 32;
-        for (int64_t t = 0; t < T && !looped; ++t) {
-            for (int l = 0; l < L; ++l) {
-                const int rc = launch_spmm_mma(W[l], nullptr, 0, vrows, P->d_z, (int64_t)gates * H, stream, P->d_xp[l]);
-                if (rc != CSB_OK) {
-                    if (rc == 1 && t > 0) { set_error("the tensor-core plan of layer %d became unusable in mid-sequence", l); return CSB_ERR_CUDA; }
-                    return rc;
-                }
-                const bool top = l == L - 1;
-                const float* x_next = (l == 0 && t + 1 < T) ? dx + (size_t)(t + 1) * B * I0 : nullptr;
-                cudaLaunchAttribute attr[1];
-                attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-                attr[0].val.programmaticStreamSerializationAllowed = 1;
-                cudaLaunchConfig_t cfg{};
-                cfg.gridDim = dim3((unsigned)(h_blocks + (x_next ? x_blocks : 0))); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = 0;
-                cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
-                const float* bl = bias ? bias[l] : nullptr;
-                float* hs = P->d_h + (size_t)l * B * H;
-                uint8_t* xp_self = P->d_xp[l] + (size_t)in_size[l] * pitch;
-                uint8_t* xp_next = top ? nullptr : P->d_xp[l + 1];
-                float* yt = (top && dy) ? dy + (size_t)t * B * H : nullptr;
-                if (gru)
-                    CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_gru_gates_pack_kernel, (const float*)P->d_z, bl, hs, xp_self, xp_next, yt, x_next, I0,
-                                                P->d_xp[0], pitch, cap, B, H, h_blocks));
-                else
-                    CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_lstm_gates_pack_kernel, (const float*)P->d_z, bl, P->d_c + (size_t)l * B * H, hs, xp_self,
-                                                xp_next, yt, x_next, I0, P->d_xp[0], pitch, cap, B, H, h_blocks));
-                CSB_CUDA(cudaGetLastError());
+        const int h_tiles = (H + 31) / 32, b_tiles = (B + 7) / 8, x_blocks = (I0 + 31) / 32;
+        float* Z[kMaxLayers];
+        for (int l = 0; l < L; ++l) Z[l] = P->d_z + (size_t)l * vrows * gates * H;
+        for (int64_t k = 0; k < T + L - 1; ++k) {
+            // the layers with a step in this tick are neighbours
+            const int l0 = (int)std::max<int64_t>(0, k - T + 1), l1 = (int)std::min<int64_t>(L, k + 1);
+            const int rc = launch_spmm_stack(P->stack, l0, l1, W, P->d_xp, Z, vrows, (int64_t)gates * H, stream);
+            if (rc != CSB_OK) return rc;
+            GateArgs a{};
+            a.n_parts = l1 - l0; a.I = I0; a.pitch = pitch; a.cap = cap; a.B = B; a.H = H; a.b_tiles = b_tiles;
+            int blocks = 0;
+            for (int l = l0; l < l1; ++l) {
+                GatePart& g = a.part[l - l0];
+                const int64_t t = k - l;
+                g.Z = Z[l]; g.bias = bias ? bias[l] : nullptr; g.c = gru ? nullptr : P->d_c + (size_t)l * B * H; g.hs = P->d_h + (size_t)l * B * H;
+                g.xp_self = P->d_xp[l] + (size_t)in_size[l] * pitch; g.xp_next = l + 1 < L ? P->d_xp[l + 1] : nullptr;
+                g.y = (l == L - 1 && dy) ? dy + (size_t)t * B * H : nullptr;
+                blocks += h_tiles * b_tiles;
+                g.end = blocks;
             }
+            if (k + 1 < T) { a.x_next = dx + (size_t)(k + 1) * B * I0; a.xp0 = P->d_xp[0]; blocks += x_blocks; }
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)blocks); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = 0;
+            cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
+            CSB_CUDA(cudaLaunchKernelEx(&cfg, gru ? csb_gates_pack_kernel<3> : csb_gates_pack_kernel<4>, a));
+            CSB_CUDA(cudaGetLastError());
         }
         if (hT) CSB_CUDA(cudaMemcpyAsync(hT, P->d_h, ns * 4, out_kind, st));
         if (cT && !gru) CSB_CUDA(cudaMemcpyAsync(cT, P->d_c, ns * 4, out_kind, st));
@@ -350,12 +340,8 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     for (int64_t t = 0; t < T; ++t) {
         for (int l = 0; l < L; ++l) {
             const int ld = in_size[l] + H;
-            const int rc = launch_spmm_mma(W[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
-            if (rc != CSB_OK) {
-                // in step 0 only scratch has been written so far (y is written behind the top layer's product)
-                if (rc == 1 && t > 0) { set_error("the tensor-core plan of layer %d became unusable in mid-sequence", l); return CSB_ERR_CUDA; }
-                return rc;
-            }
+            const int rc = launch_spmm_stack_fp32(P->stack, l, W[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
+            if (rc != CSB_OK) return rc;
             const bool top = l == L - 1;
             const float* x_next = (l == 0 && t + 1 < T) ? dx + (size_t)(t + 1) * B * I0 : nullptr;
             cudaLaunchAttribute attr[1];

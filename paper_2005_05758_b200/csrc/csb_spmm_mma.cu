@@ -34,51 +34,32 @@
 
 #include "csb_internal.hpp"
 #include "csb_device.cuh"
-#include "csb_gates.cuh"
 
 namespace csb {
 
 constexpr uint32_t kOffMaskM = 0x3fffffffu;
 constexpr uint32_t kNoRow = 0xffffffffu;
-constexpr size_t kLoopTileBytes = 32 * 33 * 4;  // the time loop's transposition tile of the gate arithmetic
 constexpr size_t kSpmmStaticSmem = 256;       // the kernel's statically allocated shared memory (CTA descriptor, row table), rounded up
 
-struct SpmmArgs {
+// One product of a launch: the layers of a recurrent stack that work on different steps at the same
+// time share a launch, each with the CTAs of its own plan.
+struct SpmmPart {
     const uint8_t* stream;
     const uint4* warp_desc;    // per warp: first chunk's offset, chunk count, sizes of its first three chunks
     const SpmmCta* ctas;
     const uint8_t* xp;         // packed inputs: one row of `pitch` bytes per matrix column
     float* Y;
+    int rows, cols, RG, cta_end;   // cta_end: the part's CTAs end here in the grid
+};
+struct SpmmArgs {
+    SpmmPart part[kMaxLayers];
     long long ldy;
     uint32_t* status;
-    int nb, rows, cols, block_r, block_c, tile_cols, RG, S, x_depth, w_stages, pitch, tile_bytes;   // tile_cols: matrix columns per input tile
+    int n_parts, nb, block_r, block_c, tile_cols, S, x_depth, w_stages, pitch, tile_bytes;   // tile_cols: matrix columns per input tile
     int q_rows;                // rows of the largest row group the shared-memory carve-up must hold (RG * block_r of one product)
 #ifdef CSB_SPMM_CLOCKS
     long long* clocks;         // instrumented build only: [CTA][warp][16] cycles per phase
 #endif
-};
-
-// The recurrent time loop around the product (batches of 8 and more, up to 32 product rows): one
-// cooperative launch runs all steps of all layers.  Per layer and step: the product pass of that
-// layer's matrix over its packed inputs into Z, a grid barrier, the gate arithmetic (tiles of 32 hidden
-// units dealt to the CTAs; h_t goes straight into the packed inputs of the next products), a grid barrier.
-struct SpmmLoopLayer {
-    const uint8_t* stream; const uint4* warp_desc; const SpmmCta* ctas;
-    const uint8_t* xp;         // packed inputs of this layer's product, rows 0 .. in_size + H - 1
-    const float* bias; float* c; float* hs;
-    uint8_t* xp_self;          // = xp + in_size * pitch: where h_t of this layer goes
-    uint8_t* xp_next;          // the input rows of the layer above, or null
-    int rows, cols, n_ctas, RG;
-};
-struct SpmmLoop {
-    SpmmLoopLayer layer[kMaxLayers];
-    float* Z; long long ldz;   // pre-activations of the layer being worked on: [product rows][gates * H]
-    const float* x;            // [T, B, I0]
-    float* y;                  // [T, B, H] or null
-    uint8_t* xp0;              // packed inputs of layer 0 (x_{t+1} is packed into its first I0 rows)
-    unsigned int* gbar;        // grid barrier counter, zero at launch
-    unsigned long long barrier_ns;
-    int T, L, B, H, I0, gates, cap;
 };
 
 #ifdef CSB_SPMM_CLOCKS
@@ -95,11 +76,9 @@ __host__ __device__ constexpr int spmm_sum_pitch(int NT) { return NT == 1 ? 8 : 
 __host__ __device__ constexpr size_t spmm_q_bytes(int NT, int group_rows) { return (size_t)8 * NT * (group_rows + 1) * 4; }
 
 struct SpmmSmem {
-    size_t wfull, xfull, wcnt, xcnt, dead, zero, extra, rings, wring, xring, qsums, total;
-    // q_bytes: room for the CTA's own sums of its row group; extra_bytes: a region outside the rings (the time
-    // loop's tile of the gate arithmetic, which runs while the next pass's first weights are on their way)
-    __host__ __device__ SpmmSmem(int n_warps, int w_stages, int x_depth, int tile_bytes, int pitch, int MT, int NT, size_t q_bytes,
-                                 size_t extra_bytes = 0) {
+    size_t wfull, xfull, wcnt, xcnt, dead, zero, rings, wring, xring, qsums, total;
+    // q_bytes: room for the CTA's own sums of its row group
+    __host__ __device__ SpmmSmem(int n_warps, int w_stages, int x_depth, int tile_bytes, int pitch, int MT, int NT, size_t q_bytes) {
         const int n_streams = n_warps;
         wfull = 0;
         xfull = wfull + (size_t)n_streams * w_stages * 8;
@@ -107,8 +86,7 @@ struct SpmmSmem {
         xcnt = wcnt + (size_t)n_streams * w_stages * 4;
         dead = xcnt + (size_t)x_depth * 4;
         zero = (dead + 4 + 127) & ~(size_t)127;
-        extra = (zero + (size_t)pitch + 127) & ~(size_t)127;
-        rings = (extra + extra_bytes + 127) & ~(size_t)127;
+        rings = (zero + (size_t)pitch + 127) & ~(size_t)127;
         wring = rings;
         xring = wring + (size_t)n_streams * w_stages * kSpmmStageBytes;
         const size_t ring_end = xring + (size_t)x_depth * tile_bytes;
@@ -123,7 +101,7 @@ struct SpmmSmem {
 __global__ void csb_pack_x_kernel(const float* __restrict__ X, long long ldx, int nb, int cols, uint8_t* __restrict__ xp, int pitch, int NT) {
     pdl_launch_dependents();
     pdl_wait();                                    // X may come from the kernel in front; xp may still be read by it
-    __shared__ float tile[32][33];
+    __shared__ float tile[64][33];
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, c0 = blockIdx.x * 32;
     const int cap = 8 * NT;
     for (int b = ty; b < cap; b += 8) tile[b][tx] = (b < nb && c0 + tx < cols) ? X[(long long)b * ldx + c0 + tx] : 0.f;
@@ -141,7 +119,7 @@ __global__ void csb_pack_x_kernel(const float* __restrict__ X, long long ldx, in
 }
 
 __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
@@ -189,20 +167,16 @@ __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
     return v;
 }
 
-__device__ __forceinline__ unsigned int ld_acquire_gpu_u32(const unsigned int* p) {
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
+// Warps per CTA and with them the registers a thread may have (spmm_warps()).
+template <int NT> constexpr int kWarpsOf = NT == 1 ? 32 : NT == 8 ? 8 : 16;
 
-// One product pass (LOOP = false: the whole kernel), or the time loop of a recurrent stack around it.
-template <int MT, int NT, bool LOOP>
-__device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
-    constexpr int kSpmmWarps = NT == 1 ? 32 : 16;
-    if (!LOOP) pdl_launch_dependents();
+template <int MT, int NT>
+__global__ void __launch_bounds__(kWarpsOf<NT> * 32, 1) csb_spmm_tile_kernel(const __grid_constant__ SpmmArgs a) {
+    constexpr int kSpmmWarps = kWarpsOf<NT>;
+    pdl_launch_dependents();
     extern __shared__ __align__(128) uint8_t smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const SpmmSmem L(kSpmmWarps, a.w_stages, a.x_depth, a.tile_bytes, a.pitch, MT, NT, spmm_q_bytes(NT, a.q_rows), LOOP ? kLoopTileBytes : 0);
+    const SpmmSmem L(kSpmmWarps, a.w_stages, a.x_depth, a.tile_bytes, a.pitch, MT, NT, spmm_q_bytes(NT, a.q_rows));
     uint64_t* wfull = reinterpret_cast<uint64_t*>(smem + L.wfull) + warp * a.w_stages;
     uint64_t* xfull = reinterpret_cast<uint64_t*>(smem + L.xfull);
     uint32_t* xcnt = reinterpret_cast<uint32_t*>(smem + L.xcnt);
@@ -225,21 +199,17 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
         mbar_fence_init();
     }
     for (int i = threadIdx.x; i < (a.pitch + 16) / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(smem + L.zero)[i] = 0u;
-    // ring positions: they run on from pass to pass of the time loop (every use of a slot is one phase of its barrier)
+    int p_idx = 0, cta0 = 0;                       // which product this CTA works for, and its first CTA
+    while (p_idx + 1 < a.n_parts && (int)blockIdx.x >= a.part[p_idx].cta_end) { cta0 = a.part[p_idx].cta_end; ++p_idx; }
+    const SpmmPart& pt = a.part[p_idx];
+    const int cta = (int)blockIdx.x - cta0;
     int xs = 0, s = 0;                             // slot of the input ring the warp is at; stage of its weight ring
     uint32_t xpar = 0u, parity = 0u;               // and the parities of their current uses
-    unsigned int gbar_round = 0;                   // grid barriers passed (time loop)
-    // time loop: what the next pass starts with is fetched while this one ends
-    bool primed = false;
-    uint4 wd_next = make_uint4(0u, 0u, 0u, 0u);
-    uint32_t me_word_next = 0u, issue_off_next = 0u;
-    // The first chunks of a warp's weight stream go out, into the stages in ring order from where the warp
-    // stands; returns where the next chunk to be fetched starts.  (A warp's chunks lie back to back.)
+    // The first chunks of a warp's weight stream go out, into the stages in ring order; returns where the
+    // next chunk to be fetched starts.  (A warp's chunks lie back to back.)
     auto first_weights = [&](const uint8_t* stream, const uint4& d) -> uint32_t {
         const uint32_t first[3] = {d.z & 0xffffu, d.z >> 16, d.w};
         uint32_t off = d.x;
-        // (time loop: the rings were last touched by ordinary loads and stores, the sums of the pass in front,
-        // which a CTA barrier separates from these copies)
         int si = s;
         for (int k = 0; k < a.w_stages && k < (int)d.y; ++k) {
             if (lane == 0) {
@@ -251,31 +221,18 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
         }
         return off;
     };
-    const int n_pass = LOOP ? lp->T * lp->L : 1;
-    for (int pass = 0; pass < n_pass; ++pass) {
-    const int layer = LOOP ? pass % lp->L : 0, step = LOOP ? pass / lp->L : 0;
-    bool pass_dead = false;
-    if (LOOP) {
-        const SpmmLoopLayer& ly = lp->layer[layer];
-        a.stream = ly.stream; a.warp_desc = ly.warp_desc; a.ctas = ly.ctas; a.xp = ly.xp;
-        a.rows = ly.rows; a.cols = ly.cols; a.RG = ly.RG; a.Y = lp->Z; a.ldy = lp->ldz;
-    }
-    if (!LOOP || (int)blockIdx.x < lp->layer[layer].n_ctas) {
-    // (time loop: descriptors and first weights of this pass were fetched during the pass in front, where there was one)
-    const bool was_primed = LOOP && primed;
-    primed = false;
     if (threadIdx.x < sizeof(SpmmCta) / 4)
-        reinterpret_cast<uint32_t*>(&s_me)[threadIdx.x] = was_primed ? me_word_next : reinterpret_cast<const uint32_t*>(a.ctas + blockIdx.x)[threadIdx.x];
-    const uint4 wd = was_primed ? wd_next : __ldg(a.warp_desc + (size_t)blockIdx.x * kSpmmWarps + warp);
+        reinterpret_cast<uint32_t*>(&s_me)[threadIdx.x] = reinterpret_cast<const uint32_t*>(pt.ctas + cta)[threadIdx.x];
+    const uint4 wd = __ldg(pt.warp_desc + (size_t)cta * kSpmmWarps + warp);
     const uint32_t n_chunks = wd.y;
     __syncthreads();
     const SpmmCta* me = &s_me;
     const int ntiles = me->ntiles, tile0 = me->tile0;
-    auto tile_bytes_of = [&](int tl) { return (uint32_t)min(a.tile_cols, a.cols - (tile0 * a.block_c + tl * a.tile_cols)) * (uint32_t)a.pitch; };
-    auto tile_src = [&](int tl) { return a.xp + (size_t)(tile0 * a.block_c + tl * a.tile_cols) * a.pitch; };
+    auto tile_bytes_of = [&](int tl) { return (uint32_t)min(a.tile_cols, pt.cols - (tile0 * a.block_c + tl * a.tile_cols)) * (uint32_t)a.pitch; };
+    auto tile_src = [&](int tl) { return pt.xp + (size_t)(tile0 * a.block_c + tl * a.tile_cols) * a.pitch; };
     // the weights were written at plan time: their first copies go out before the work in front is waited for
     // (a warp's chunks lie back to back; issue_off is where the next one to be fetched starts)
-    uint32_t issue_off = was_primed ? issue_off_next : first_weights(a.stream, wd);
+    uint32_t issue_off = first_weights(pt.stream, wd);
     if (threadIdx.x == 0) {
         int rr = 0;
         s_first[0] = 0;
@@ -283,10 +240,7 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
             while (rr < (int)me->warp_row[w]) s_first[++rr] = w;
         while (rr < 4) s_first[++rr] = kSpmmWarps;
     }
-    if (!LOOP) pdl_wait();                         // the packed inputs and Y belong to the work in front on the stream
-    // (time loop: the packed inputs were written with ordinary stores by other CTAs, before the grid barrier;
-    // every lane that may issue a copy of them orders that behind its view of the barrier, once per pass)
-    if (LOOP && lane == 0) fence_proxy_async_all();
+    pdl_wait();                                    // the packed inputs and Y belong to the work in front on the stream
     // One lane fetches a tile with one bulk copy.  (No proxy fence in front of a refill: the slot's
     // readers have their data in registers by the time they release it, and the release orders them
     // before this copy is issued.)
@@ -437,7 +391,7 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
         if (refill_bytes) {
             if (lane == 0) {
                 mbar_expect_tx(&wfull[s], refill_bytes);
-                bulk_g2s(wring + (size_t)s * kSpmmStageBytes, a.stream + (size_t)issue_off * 16, refill_bytes, &wfull[s]);
+                bulk_g2s(wring + (size_t)s * kSpmmStageBytes, pt.stream + (size_t)issue_off * 16, refill_bytes, &wfull[s]);
             }
             issue_off += refill_bytes >> 4;
         }
@@ -449,15 +403,6 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
         release_x();
     }
     SPMM_LAP(5);                                   // the tiles behind this warp's last item
-    if (LOOP && pass + 1 < n_pass) {
-        // descriptors of this CTA in the next pass: asked for now, used once the sums below are done
-        const SpmmLoopLayer& nx = lp->layer[(pass + 1) % lp->L];
-        if ((int)blockIdx.x < nx.n_ctas) {
-            wd_next = __ldg(nx.warp_desc + (size_t)blockIdx.x * kSpmmWarps + warp);
-            if (threadIdx.x < sizeof(SpmmCta) / 4) me_word_next = __ldg(reinterpret_cast<const uint32_t*>(nx.ctas + blockIdx.x) + threadIdx.x);
-            primed = true;
-        }
-    }
     __syncthreads();
     SPMM_LAP(6);                                   // waiting for the other warps of the CTA
     const bool dead = *s_dead != 0u;
@@ -466,8 +411,7 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
         // time to land before the CTA's shared memory goes away, and write nothing
         const unsigned long long t0 = global_ns();
         while (global_ns() - t0 < 200000ull) __nanosleep(1000);
-        if (!LOOP && a.S == 1) return;             // (a CTA of a cluster still has to keep the cluster's barriers company)
-        pass_dead = true;
+        if (a.S == 1) return;                      // (a CTA of a cluster still has to keep the cluster's barriers company)
     }
 
     // ---- the warps' sums meet in shared memory (the rings are no longer in use)
@@ -486,8 +430,8 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
     }
     __syncthreads();
     SPMM_LAP(7);                                   // accumulators to shared memory
-    const int group_rows = a.RG * a.block_r, row0 = me->group * group_rows;
-    const int nrows = min(group_rows, a.rows - row0);
+    const int group_rows = pt.RG * a.block_r, row0 = me->group * group_rows;
+    const int nrows = min(group_rows, pt.rows - row0);
     // this CTA's sums over its range: [batch column][row of the group], one float of padding per column
     // (written four columns at a time without bank conflicts, read by the cluster in runs of consecutive rows)
     float* part = reinterpret_cast<float*>(smem + L.qsums);
@@ -565,7 +509,7 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
                     float sum = v[j][0];
 #pragma unroll
                     for (int s2 = 1; s2 < 8; ++s2) sum += v[j][s2];
-                    if (b < a.nb && r < r_n) a.Y[(long long)b * a.ldy + row0 + r_lo + r] = sum;
+                    if (b < a.nb && r < r_n) pt.Y[(long long)b * a.ldy + row0 + r_lo + r] = sum;
                 }
             }
     }
@@ -575,77 +519,9 @@ __device__ __forceinline__ void spmm_tile_body(SpmmArgs a, const SpmmLoop* lp) {
         cluster_barrier();
     }
     SPMM_LAP(11);                                  // until every CTA of the cluster has read
-    // (time loop) the rings are free again: the next pass's first weights go out and land while the gates are done
-    if (LOOP) {
-        __syncthreads();                           // every thread is done reading the sums that lie where the rings are
-        if (primed && !pass_dead) issue_off_next = first_weights(lp->layer[(pass + 1) % lp->L].stream, wd_next);
-        else primed = false;
-    }
-    }                                              // (CTAs beyond this layer's plan sit the pass out)
-    if (LOOP) {
-        // ---- every CTA's part of Z is written: gate arithmetic of (layer, step), then on to the next pass.
-        // A CTA that gave up does not come here; the others then run into the bound of the barrier.
-        if (pass_dead) break;
-        auto grid_sync = [&]() -> bool {
-            __syncthreads();
-            ++gbar_round;
-            if (threadIdx.x == 0) {
-                __threadfence();
-                atomicAdd(lp->gbar, 1u);
-                const unsigned int target = gbar_round * gridDim.x;
-                unsigned long long t0 = 0;
-                unsigned int spins = 0;
-                while (ld_acquire_gpu_u32(lp->gbar) < target) {
-                    if ((++spins & 63u) == 0) {
-                        const unsigned long long now = global_ns();
-                        if (t0 == 0) t0 = now;
-                        else if (now - t0 > lp->barrier_ns) { *s_dead = 1u; *(volatile uint32_t*)a.status = (uint32_t)kDevBarrierTimeout; break; }
-                    }
-                }
-            }
-            __syncthreads();
-            return *s_dead == 0u;
-        };
-        SPMM_LAP(15);                              // (time loop) next pass's first weights out
-        if (!grid_sync()) break;
-        SPMM_LAP(12);                              // (time loop) grid barrier behind the product pass
-        {
-            const SpmmLoopLayer& ly = lp->layer[layer];
-            float (*tile)[33] = reinterpret_cast<float (*)[33]>(smem + L.extra);
-            const int B = lp->B, H = lp->H, h_tiles = (H + 31) / 32;
-            const bool pack_x = layer == 0 && step + 1 < lp->T;
-            const int n_tiles = h_tiles + (pack_x ? (lp->I0 + 31) / 32 : 0);
-            float* y_t = (layer == lp->L - 1 && lp->y) ? lp->y + (size_t)step * B * H : nullptr;
-            for (int tl = blockIdx.x; tl < n_tiles; tl += gridDim.x) {
-                if (tl < h_tiles) {
-                    if (lp->gates == 4) lstm_gates_tile(tile, lp->Z, ly.bias, ly.c, ly.hs, ly.xp_self, ly.xp_next, y_t, a.pitch, lp->cap, B, H, tl * 32);
-                    else gru_gates_tile(tile, lp->Z, ly.bias, ly.hs, ly.xp_self, ly.xp_next, y_t, a.pitch, lp->cap, B, H, tl * 32);
-                } else {
-                    pack_columns(tile, lp->x + (size_t)(step + 1) * B * lp->I0, (long long)lp->I0, B, lp->I0, (tl - h_tiles) * 32, lp->xp0,
-                                 a.pitch, lp->cap, 0);
-                }
-                __syncthreads();                   // the tile is free again
-            }
-        }
-        SPMM_LAP(13);                              // (time loop) gate arithmetic
-        if (pass + 1 < n_pass && !grid_sync()) break;
-        SPMM_LAP(14);                              // (time loop) grid barrier behind the gates
-    }
-    }                                              // passes
 #ifdef CSB_SPMM_CLOCKS
     if (lane == 0) for (int i = 0; i < 16; ++i) a.clocks[((size_t)blockIdx.x * kSpmmWarps + warp) * 16 + i] = sprof[i];
 #endif
-}
-
-template <int MT, int NT>
-__global__ void __launch_bounds__((NT == 1 ? 32 : 16) * 32, 1) csb_spmm_tile_kernel(const SpmmArgs a) {
-    spmm_tile_body<MT, NT, false>(a, nullptr);
-}
-
-// The recurrent time loop (see SpmmLoop): launched cooperatively, so that the bounded grid barriers can be passed.
-template <int MT, int NT>
-__global__ void __launch_bounds__((NT == 1 ? 32 : 16) * 32, 1) csb_rnn_tile_kernel(const SpmmArgs a, const __grid_constant__ SpmmLoop lp) {
-    spmm_tile_body<MT, NT, true>(a, &lp);
 }
 
 #define CSB_CUDA(call)                                                                     \
@@ -673,28 +549,38 @@ static int upload_v(const std::vector<V>& h, V** d) {
 
 static int mt_of(const csb_matrix* A) { return A->block_r <= 16 ? 1 : A->block_r <= 32 ? 2 : 4; }
 
-template <int MT, int NT>
-static cudaError_t set_smem_attr(size_t bytes) {
-    return cudaFuncSetAttribute(csb_spmm_tile_kernel<MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+template <int MT, int NT> struct SetSmem {
+    static cudaError_t call(size_t bytes) { return cudaFuncSetAttribute(csb_spmm_tile_kernel<MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes); }
+};
+template <int MT, int NT> struct MaxClusters {
+    static cudaError_t call(int* n, const cudaLaunchConfig_t* cfg) { return cudaOccupancyMaxActiveClusters(n, csb_spmm_tile_kernel<MT, NT>, cfg); }
+};
+template <int MT, int NT> struct LaunchTile {
+    static cudaError_t call(const cudaLaunchConfig_t* cfg, const SpmmArgs& a) { return cudaLaunchKernelEx(cfg, csb_spmm_tile_kernel<MT, NT>, a); }
+};
+template <template <int, int> class F, int MT, typename... X>
+static cudaError_t spmm_dispatch_nt(int NT, X&&... x) {
+    return NT == 1 ? F<MT, 1>::call(x...) : NT == 2 ? F<MT, 2>::call(x...) : NT == 4 ? F<MT, 4>::call(x...) : F<MT, 8>::call(x...);
 }
-template <int MT, int NT>
-static cudaError_t max_clusters(int* n, const cudaLaunchConfig_t* cfg) {
-    return cudaOccupancyMaxActiveClusters(n, csb_spmm_tile_kernel<MT, NT>, cfg);
+template <template <int, int> class F, typename... X>
+static cudaError_t spmm_dispatch(int MT, int NT, X&&... x) {
+    return MT == 1 ? spmm_dispatch_nt<F, 1>(NT, x...) : MT == 2 ? spmm_dispatch_nt<F, 2>(NT, x...) : spmm_dispatch_nt<F, 4>(NT, x...);
 }
-template <int MT, int NT>
-static cudaError_t launch_tile_kernel(const cudaLaunchConfig_t* cfg, const SpmmArgs& a) {
-    return cudaLaunchKernelEx(cfg, csb_spmm_tile_kernel<MT, NT>, a);
-}
-#define CSB_SPMM_DISPATCH(fn, MT, NT, ...)                                                                        \
-    ((MT) == 1 ? ((NT) == 1 ? fn<1, 1>(__VA_ARGS__) : (NT) == 2 ? fn<1, 2>(__VA_ARGS__) : fn<1, 4>(__VA_ARGS__))  \
-     : (MT) == 2 ? ((NT) == 1 ? fn<2, 1>(__VA_ARGS__) : (NT) == 2 ? fn<2, 2>(__VA_ARGS__) : fn<2, 4>(__VA_ARGS__)) \
-                 : ((NT) == 1 ? fn<4, 1>(__VA_ARGS__) : (NT) == 2 ? fn<4, 2>(__VA_ARGS__) : fn<4, 4>(__VA_ARGS__)))
 
-static int build_spmm_plan(const csb_matrix* A, int ci, MmaPlan::PerClass* P) {
+// Room for packed inputs: whole tiles, so that a tile copy never runs past the end.
+static int alloc_packed(const csb_matrix* A, int NT, MmaPlan::PerClass* P) {
+    const size_t bytes = (size_t)A->nbc * A->block_c * spmm_pitch(NT);
+    CSB_CUDA(cudaMalloc(&P->d_xp, bytes));
+    CSB_CUDA(cudaMemset(P->d_xp, 0, bytes));
+    return CSB_OK;
+}
+
+// The plan of A for batch tiles of 8 * NT columns on `sms` SMs; force_S > 0 fixes the cluster size (the products of
+// one launch share it).
+static int build_spmm_plan(const csb_matrix* A, int ci, int sms, int force_S, bool with_x, MmaPlan::PerClass* P) {
     const int NT = 1 << ci;
     SpmmHostPlan H;
-    const int sms = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
-    int rc = plan_spmm_host(A, NT, sms, &H);
+    int rc = plan_spmm_host(A, NT, sms, force_S, &H);
     if (rc == 1) { P->unusable = true; return CSB_OK; }
     if (rc != CSB_OK) return rc;
     const int MT = mt_of(A), pitch = spmm_pitch(NT);
@@ -714,11 +600,9 @@ static int build_spmm_plan(const csb_matrix* A, int ci, MmaPlan::PerClass* P) {
     if ((rc = upload_v(H.bytes, &P->d_stream)) != CSB_OK) return rc;
     if ((rc = upload_v(H.warp_desc, &P->d_warp_desc)) != CSB_OK) return rc;
     if ((rc = upload_v(H.ctas, &P->d_ctas)) != CSB_OK) return rc;
-    const size_t xp_bytes = (size_t)A->nbc * A->block_c * pitch;          // whole tiles, so that a tile copy never runs past the end
-    CSB_CUDA(cudaMalloc(&P->d_xp, xp_bytes));
-    CSB_CUDA(cudaMemset(P->d_xp, 0, xp_bytes));
+    if (with_x && (rc = alloc_packed(A, NT, P)) != CSB_OK) return rc;
     // (the limit belongs to the kernel, not to this plan: other matrices launch the same instantiation with other sizes)
-    CSB_CUDA(CSB_SPMM_DISPATCH(set_smem_attr, MT, NT, A->smem_optin - kSpmmStaticSmem));
+    CSB_CUDA(spmm_dispatch<SetSmem>(MT, NT, A->smem_optin - kSpmmStaticSmem));
     if (H.S > 1) {
         // the S CTAs of a row group are launched as one cluster: make sure such a cluster can be resident
         cudaLaunchAttribute attr[1];
@@ -728,7 +612,7 @@ static int build_spmm_plan(const csb_matrix* A, int ci, MmaPlan::PerClass* P) {
         cfg.gridDim = dim3((unsigned)H.ctas.size()); cfg.blockDim = dim3((unsigned)spmm_warps(NT) * 32u); cfg.dynamicSmemBytes = smem;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int clusters = 0;
-        CSB_CUDA(CSB_SPMM_DISPATCH(max_clusters, MT, NT, &clusters, &cfg));
+        CSB_CUDA(spmm_dispatch<MaxClusters>(MT, NT, &clusters, &cfg));
         if (clusters < 1) { P->unusable = true; return CSB_OK; }
     }
     CSB_CUDA(cudaDeviceSynchronize());
@@ -741,10 +625,9 @@ void free_mma(csb_matrix* A) {
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(A->device);
-    for (auto& c : A->mma->cls) {
-        cudaFree(c.d_stream); cudaFree(c.d_warp_desc); cudaFree(c.d_ctas);
-        cudaFree(c.d_xp);
-    }
+    auto drop = [](MmaPlan::PerClass& c) { cudaFree(c.d_stream); cudaFree(c.d_warp_desc); cudaFree(c.d_ctas); cudaFree(c.d_xp); };
+    for (auto& c : A->mma->cls) drop(c);
+    for (auto& c : A->mma->shared) drop(c.plan);
     cudaSetDevice(prev);
     delete A->mma;
     A->mma = nullptr;
@@ -759,170 +642,176 @@ extern "C" int csb_debug_spmm_clocks(long long* host_out, int max_warps) {
 }
 #endif
 
-// The plan of A for batch class ci, built on first use (the device of A is current).  CSB_OK, an error, or 1 = the
-// tensor-core layout does not serve this matrix.
-static int ensure_spmm_plan(const csb_matrix* A, int ci) {
-    std::lock_guard<std::mutex> lk(A->mma_mu);
-    if (!A->mma) {
-        A->mma = new (std::nothrow) MmaPlan();
-        if (!A->mma) { set_error("out of host memory"); return CSB_ERR_ALLOC; }
-    }
-    MmaPlan::PerClass& C = A->mma->cls[ci];
-    if (!C.built && !C.unusable) {
+static int make_spmm_plan(const csb_matrix* A, int ci, int sms, int force_S, bool with_x, MmaPlan::PerClass* C) {
+    if (!C->built && !C->unusable) {
         int rc;
-        try { rc = build_spmm_plan(A, ci, &C); }
+        try { rc = build_spmm_plan(A, ci, sms, force_S, with_x, C); }
         catch (const std::bad_alloc&) { set_error("out of host memory while planning the batched product"); rc = CSB_ERR_ALLOC; }
-        if (rc != CSB_OK) { C.unusable = true; return rc; }
+        if (rc != CSB_OK) { C->unusable = true; return rc; }
     }
-    return (C.unusable || !C.built) ? 1 : CSB_OK;
+    return (C->unusable || !C->built) ? 1 : CSB_OK;
+}
+static int ensure_mma(const csb_matrix* A) {
+    if (!A->mma) A->mma = new (std::nothrow) MmaPlan();
+    if (A->mma) return CSB_OK;
+    set_error("out of host memory");
+    return CSB_ERR_ALLOC;
 }
 
-// Returns CSB_OK after launching, or 1 when the caller should use the CUDA-core path.
-// With `packed` (and X == nullptr) the inputs are taken from a buffer the caller has filled in the
-// packed layout of the batch's class (one row of spmm_pitch(NT) bytes per matrix column: the hi parts of
-// 8 * NT batch slots, then the lo parts); a single pass, so at most 32 batch columns.
-int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream, const uint8_t* packed) {
-    if (packed && batch > 32) { set_error("pre-packed inputs serve at most 32 batch columns"); return CSB_ERR_INVALID_ARG; }
+static int gave_up(const csb_matrix* A) {
     const ProductPlan& PP = A->product;
-    if (PP.h_status && *PP.h_status != 0) { set_error("an earlier product on this handle gave up waiting on the device (code %u)", *PP.h_status); return CSB_ERR_TIMEOUT; }
-    int prev = 0;
-    CSB_CUDA(cudaGetDevice(&prev));
-    if (prev != A->device) CSB_CUDA(cudaSetDevice(A->device));
-    struct Restore { int prev, cur; ~Restore() { if (prev != cur) cudaSetDevice(prev); } } restore{prev, A->device};
-    const int ci = spmm_class_index(batch);
-    {
-        const int rc = ensure_spmm_plan(A, ci);
-        if (rc != CSB_OK) return rc;
-    }
-    const MmaPlan::PerClass& P = A->mma->cls[ci];
-    const int NT = 1 << ci, MT = mt_of(A), cap = 8 * NT;
-    cudaStream_t st = (cudaStream_t)stream;
+    if (!PP.h_status || *PP.h_status == 0) return CSB_OK;
+    set_error("an earlier product on this handle gave up waiting on the device (code %u)", *PP.h_status);
+    return CSB_ERR_TIMEOUT;
+}
+
+// Launches the tile kernel over the products (P[i], xp[i], Y[i]) of matrices with the same block shape.
+static int launch_parts(int n, const csb_matrix* const* A, const MmaPlan::PerClass* const* P, const uint8_t* const* xp, float* const* Y, int NT, int nb,
+                        int64_t ldy, cudaStream_t st) {
+    const int MT = mt_of(A[0]);
     SpmmArgs a{};
-    a.stream = P.d_stream; a.warp_desc = (const uint4*)P.d_warp_desc; a.ctas = P.d_ctas;
-    a.xp = packed ? packed : (const uint8_t*)P.d_xp; a.ldy = ldy; a.status = PP.d_status;
-    a.rows = (int)A->rows; a.cols = (int)A->cols; a.block_r = A->block_r; a.block_c = A->block_c;
-    a.RG = P.RG; a.S = P.S; a.x_depth = P.x_depth; a.w_stages = P.w_stages; a.q_rows = P.RG * A->block_r;
-    a.tile_cols = spmm_tile_blocks(A->block_c) * A->block_c;
+    a.n_parts = n; a.nb = nb; a.ldy = ldy; a.status = A[0]->product.d_status;
+    a.block_r = A[0]->block_r; a.block_c = A[0]->block_c; a.S = P[0]->S;
+    a.tile_cols = spmm_tile_blocks(a.block_c) * a.block_c;
     a.pitch = spmm_pitch(NT); a.tile_bytes = (a.tile_cols * a.pitch + 127) & ~127;
+    a.x_depth = P[0]->x_depth; a.w_stages = P[0]->w_stages;
+    int ctas = 0;
+    for (int i = 0; i < n; ++i) {
+        SpmmPart& p = a.part[i];
+        p.stream = P[i]->d_stream; p.warp_desc = (const uint4*)P[i]->d_warp_desc; p.ctas = P[i]->d_ctas; p.xp = xp[i]; p.Y = Y[i];
+        p.rows = (int)A[i]->rows; p.cols = (int)A[i]->cols; p.RG = P[i]->RG;
+        ctas += P[i]->n_ctas;
+        p.cta_end = ctas;
+        a.x_depth = std::min(a.x_depth, P[i]->x_depth); a.w_stages = std::min(a.w_stages, P[i]->w_stages);
+        a.q_rows = std::max(a.q_rows, P[i]->RG * a.block_r);
+    }
+    const SpmmSmem L(spmm_warps(NT), a.w_stages, a.x_depth, a.tile_bytes, a.pitch, MT, NT, spmm_q_bytes(NT, a.q_rows));
 #ifdef CSB_SPMM_CLOCKS
     if (!g_spmm_clocks) cudaMalloc((void**)&g_spmm_clocks, (size_t)1 << 24);
     a.clocks = g_spmm_clocks;
-    g_spmm_clock_warps = P.n_ctas * spmm_warps(NT);
+    g_spmm_clock_warps = ctas * spmm_warps(NT);
 #endif
+    // the kernel orders itself behind the work in front (pdl_wait), so it may be launched with programmatic
+    // stream serialization: its scheduling overlaps that work's tail
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;             // the CTAs that share a row group
+    attr[1].val.clusterDim.x = (unsigned)a.S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = a.S > 1 ? 2 : 1;
+    cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3((unsigned)spmm_warps(NT) * 32u); cfg.dynamicSmemBytes = L.total;
+    CSB_CUDA(spmm_dispatch<LaunchTile>(MT, NT, &cfg, a));
+    CSB_CUDA(cudaGetLastError());
+    return CSB_OK;
+}
+
+// Packs fp32 inputs and launches, 8 * NT batch columns at a time.
+static int pack_and_launch(const csb_matrix* A, const MmaPlan::PerClass* P, int NT, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
+                           cudaStream_t st) {
+    const int cap = 8 * NT;
     for (int b0 = 0; b0 < batch; b0 += cap) {
-        a.nb = std::min(cap, batch - b0);
-        a.Y = Y + (int64_t)b0 * ldy;
-        // both kernels order themselves behind the work in front (pdl_wait), so they may be launched
-        // with programmatic stream serialization: their scheduling overlaps its tail
-        cudaLaunchAttribute attr[2];
+        const int nb = std::min(cap, batch - b0);
+        cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[0].val.programmaticStreamSerializationAllowed = 1;
-        attr[1].id = cudaLaunchAttributeClusterDimension;             // the CTAs that share a row group
-        attr[1].val.clusterDim.x = (unsigned)P.S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
         cudaLaunchConfig_t cfg{};
         cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
         cfg.gridDim = dim3((unsigned)((A->cols + 31) / 32)); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = 0;
-        if (!packed)
-            CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_pack_x_kernel, X + (int64_t)b0 * ldx, (long long)ldx, a.nb, (int)A->cols, (uint8_t*)P.d_xp,
-                                        a.pitch, NT));
-        cfg.gridDim = dim3((unsigned)P.n_ctas); cfg.blockDim = dim3((unsigned)spmm_warps(NT) * 32u); cfg.dynamicSmemBytes = P.smem_bytes;
-        cfg.numAttrs = P.S > 1 ? 2 : 1;
-        CSB_CUDA(CSB_SPMM_DISPATCH(launch_tile_kernel, MT, NT, &cfg, a));
-        CSB_CUDA(cudaGetLastError());
+        CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_pack_x_kernel, X + (int64_t)b0 * ldx, (long long)ldx, nb, (int)A->cols, (uint8_t*)P->d_xp,
+                                    spmm_pitch(NT), NT));
+        const uint8_t* xp = (const uint8_t*)P->d_xp;
+        float* y = Y + (int64_t)b0 * ldy;
+        const int rc = launch_parts(1, &A, &P, &xp, &y, NT, nb, ldy, st);
+        if (rc != CSB_OK) return rc;
     }
     return CSB_OK;
 }
 
-template <int MT, int NT>
-static cudaError_t set_loop_smem_attr(size_t bytes) {
-    return cudaFuncSetAttribute(csb_rnn_tile_kernel<MT, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-template <int MT, int NT>
-static cudaError_t max_loop_clusters(int* n, const cudaLaunchConfig_t* cfg) {
-    return cudaOccupancyMaxActiveClusters(n, csb_rnn_tile_kernel<MT, NT>, cfg);
-}
-template <int MT, int NT>
-static cudaError_t launch_loop_kernel(const cudaLaunchConfig_t* cfg, const SpmmArgs& a, const SpmmLoop& lp) {
-    return cudaLaunchKernelEx(cfg, csb_rnn_tile_kernel<MT, NT>, a, lp);
+// Returns CSB_OK after launching, or 1 when the caller should use the CUDA-core path.
+int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
+    int rc = gave_up(A);
+    if (rc != CSB_OK) return rc;
+    int prev = 0;
+    CSB_CUDA(cudaGetDevice(&prev));
+    if (prev != A->device) CSB_CUDA(cudaSetDevice(A->device));
+    struct Restore { int prev, cur; ~Restore() { if (prev != cur) cudaSetDevice(prev); } } restore{prev, A->device};
+    int ci = spmm_class_index(batch);
+    const int sms = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
+    {
+        std::lock_guard<std::mutex> lk(A->mma_mu);
+        if ((rc = ensure_mma(A)) != CSB_OK) return rc;
+        // more than 32 columns: tiles of 64, so that row maps, weights and bookkeeping are paid once for all of
+        // them (8192 x 8192 at 4x, batch 64: 74.9 -> 59.3 us); where that plan does not fit, passes of 32
+        if (batch > 32 && make_spmm_plan(A, 3, sms, 0, true, &A->mma->cls[3]) == CSB_OK) ci = 3;
+        else if ((rc = make_spmm_plan(A, ci, sms, 0, true, &A->mma->cls[ci])) != CSB_OK) return rc;
+    }
+    return pack_and_launch(A, &A->mma->cls[ci], 1 << ci, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
 }
 
-// The whole sequence of a recurrent stack in one cooperative launch of the product kernel's time loop.
-// Returns CSB_OK after launching, an error, or 1 when the loop does not serve this stack (layers whose
-// plans differ in block shape or cluster size, a plan that does not fit, a grid that cannot be
-// co-resident): the caller then issues the steps as separate launches.  The device of W[0] is current.
-int launch_rnn_tile_loop(const RnnTileLoop& R, void* stream) {
-    const csb_matrix* A0 = R.W[0];
-    const int vrows = R.gates == 3 ? 2 * R.B : R.B;
-    if (vrows > 32 || R.L > kMaxLayers) return 1;
-    const int ci = spmm_class_index(vrows), NT = 1 << ci, MT = mt_of(A0);
-    SpmmArgs a{};
-    SpmmLoop lp{};
-    int S = 0, n_ctas = 0, w_stages = 3, x_depth = 8, q_rows = 0;
-    for (int l = 0; l < R.L; ++l) {
-        const csb_matrix* A = R.W[l];
-        if (A->block_r != A0->block_r || A->block_c != A0->block_c || A->device != A0->device) return 1;
-        const int rc = ensure_spmm_plan(A, ci);
+// The products of a stack's layers over inputs packed by the caller (one row of spmm_pitch(NT) bytes per matrix
+// column: the hi parts of 8 * NT batch slots, then the lo parts), at most 32 batch columns.  Prepared once
+// per stack: the SMs are shared between the layers in proportion to their weights when the layers' blocks
+// have the same shape and one launch can hold all of them (*joint = true), else every layer has all of them.
+int prepare_spmm_stack(int L, const csb_matrix* const* A, int batch, SpmmStack* out) {
+    const int ci = spmm_class_index(batch);
+    *out = SpmmStack{};
+    out->NT = 1 << ci; out->L = L;
+    bool joint = L > 1 && L <= kMaxLayers;
+    int64_t nnz = 0;
+    for (int l = 0; l < L; ++l) {
+        joint = joint && A[l]->block_r == A[0]->block_r && A[l]->block_c == A[0]->block_c && A[l]->nnz > 0;
+        nnz += A[l]->nnz;
+    }
+    const int sms = A[0]->opts.ctas > 0 ? A[0]->opts.ctas : A[0]->sm_count;
+    int S = 0;
+    // (the first layer's plan fixes the cluster size for all; layers above the first have the same shape)
+    for (int pass = joint ? 0 : 1; pass < 2; ++pass) {
+        bool fits = true;
+        for (int l = L - 1; l >= 0 && fits; --l) {
+            const int share = pass == 0 ? std::max(1, (int)(sms * (double)A[l]->nnz / (double)nnz)) : sms, want_S = pass == 0 ? S : 0;
+            std::lock_guard<std::mutex> lk(A[l]->mma_mu);
+            int rc = ensure_mma(A[l]);
+            if (rc != CSB_OK) return rc;
+            MmaPlan::PerClass* C = nullptr;
+            for (auto& q : A[l]->mma->shared) if (q.ci == ci && q.sms == share && q.S == want_S) C = &q.plan;
+            if (!C) {
+                A[l]->mma->shared.push_back({ci, share, want_S, {}});
+                C = &A[l]->mma->shared.back().plan;
+            }
+            rc = make_spmm_plan(A[l], ci, share, want_S, false, C);
+            if (rc == 1) fits = false;
+            else if (rc != CSB_OK) return rc;
+            else { out->plan[l] = C; if (pass == 0 && S == 0) S = C->S; }
+        }
+        if (fits) { out->joint = pass == 0; return CSB_OK; }
+    }
+    return 1;
+}
+
+int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
+    int rc = gave_up(A);
+    if (rc != CSB_OK) return rc;
+    {
+        std::lock_guard<std::mutex> lk(A->mma_mu);
+        MmaPlan::PerClass* C = const_cast<MmaPlan::PerClass*>(K.plan[l]);
+        if (!C->d_xp && (rc = alloc_packed(A, K.NT, C)) != CSB_OK) return rc;
+    }
+    return pack_and_launch(A, K.plan[l], K.NT, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
+}
+
+int launch_spmm_stack(const SpmmStack& K, int l0, int l1, const csb_matrix* const* A, uint8_t* const* xp, float* const* Y, int nb, int64_t ldy, void* stream) {
+    const uint8_t* x[kMaxLayers];
+    for (int l = l0; l < l1; ++l) {
+        const int rc = gave_up(A[l]);
         if (rc != CSB_OK) return rc;
-        if (A->product.h_status && *A->product.h_status != 0) { set_error("an earlier product on a layer's handle gave up waiting on the device"); return CSB_ERR_TIMEOUT; }
-        const MmaPlan::PerClass& P = A->mma->cls[ci];
-        if (l == 0) S = P.S;
-        if (P.S != S) return 1;                              // one cluster shape per launch
-        n_ctas = std::max(n_ctas, P.n_ctas);
-        w_stages = std::min(w_stages, P.w_stages); x_depth = std::min(x_depth, P.x_depth);
-        q_rows = std::max(q_rows, P.RG * A->block_r);
-        SpmmLoopLayer& ly = lp.layer[l];
-        ly.stream = P.d_stream; ly.warp_desc = (const uint4*)P.d_warp_desc; ly.ctas = P.d_ctas; ly.xp = R.xp[l];
-        ly.bias = R.bias ? R.bias[l] : nullptr;
-        ly.c = R.c ? R.c + (size_t)l * R.B * R.H : nullptr;
-        ly.hs = R.hs + (size_t)l * R.B * R.H;
-        ly.xp_self = R.xp[l] + (size_t)R.in_size[l] * R.pitch;
-        ly.xp_next = l + 1 < R.L ? R.xp[l + 1] : nullptr;
-        ly.rows = (int)A->rows; ly.cols = (int)A->cols; ly.n_ctas = P.n_ctas; ly.RG = P.RG;
+        x[l] = xp[l];
     }
-    a.status = A0->product.d_status;
-    a.nb = vrows; a.block_r = A0->block_r; a.block_c = A0->block_c; a.S = S; a.x_depth = x_depth; a.w_stages = w_stages; a.q_rows = q_rows;
-    a.tile_cols = spmm_tile_blocks(A0->block_c) * A0->block_c;
-    a.pitch = spmm_pitch(NT); a.tile_bytes = (a.tile_cols * a.pitch + 127) & ~127;
-    if (a.pitch != R.pitch) { set_error("packed inputs of another batch class"); return CSB_ERR_INVALID_ARG; }
-    // the loop's own tile may cost the input ring a slot
-    while (x_depth > 2 && SpmmSmem(spmm_warps(NT), w_stages, x_depth, a.tile_bytes, a.pitch, MT, NT, spmm_q_bytes(NT, q_rows), kLoopTileBytes).total +
-                                  kSpmmStaticSmem > A0->smem_optin)
-        --x_depth;
-    a.x_depth = x_depth;
-    const SpmmSmem Lay(spmm_warps(NT), w_stages, x_depth, a.tile_bytes, a.pitch, MT, NT, spmm_q_bytes(NT, q_rows), kLoopTileBytes);
-    if (Lay.total + kSpmmStaticSmem > A0->smem_optin) return 1;
-#ifdef CSB_SPMM_CLOCKS
-    if (!g_spmm_clocks) cudaMalloc((void**)&g_spmm_clocks, (size_t)1 << 24);
-    a.clocks = g_spmm_clocks;
-    g_spmm_clock_warps = n_ctas * spmm_warps(NT);
-#endif
-    lp.Z = R.z; lp.ldz = (long long)R.gates * R.H; lp.x = R.x; lp.y = R.y; lp.xp0 = R.xp[0]; lp.gbar = R.gbar;
-    lp.barrier_ns = 2000000000ull;
-    lp.T = (int)R.T; lp.L = R.L; lp.B = R.B; lp.H = R.H; lp.I0 = R.in_size[0]; lp.gates = R.gates; lp.cap = R.cap;
-    cudaStream_t st = (cudaStream_t)stream;
-    CSB_CUDA(CSB_SPMM_DISPATCH(set_loop_smem_attr, MT, NT, A0->smem_optin - kSpmmStaticSmem));
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = S > 1 ? 2 : 1;
-    cfg.gridDim = dim3((unsigned)n_ctas); cfg.blockDim = dim3((unsigned)spmm_warps(NT) * 32u); cfg.dynamicSmemBytes = Lay.total;
-    // every CTA must be resident at once, or the grid barrier cannot be passed
-    int fit = 0;
-    if (S > 1) {
-        int clusters = 0;
-        if (CSB_SPMM_DISPATCH(max_loop_clusters, MT, NT, &clusters, &cfg) != cudaSuccess) { cudaGetLastError(); return 1; }
-        fit = clusters * S;
-    } else {
-        fit = A0->sm_count;                                  // one CTA of this size per SM
+    if (K.joint) return launch_parts(l1 - l0, A + l0, K.plan + l0, x + l0, Y + l0, K.NT, nb, ldy, (cudaStream_t)stream);
+    for (int l = l0; l < l1; ++l) {
+        const int rc = launch_parts(1, A + l, K.plan + l, x + l, Y + l, K.NT, nb, ldy, (cudaStream_t)stream);
+        if (rc != CSB_OK) return rc;
     }
-    if (n_ctas > fit) return 1;
-    if ((unsigned long long)2 * (unsigned long long)R.T * R.L * n_ctas >= (1ull << 32)) return 1;   // the barrier counts arrivals in 32 bits
-    CSB_CUDA(cudaMemsetAsync(R.gbar, 0, 4, st));
-    // a launch that is refused (a grid that cannot be co-resident after all) is no error: the caller issues the steps
-    if (CSB_SPMM_DISPATCH(launch_loop_kernel, MT, NT, &cfg, a, lp) != cudaSuccess) { cudaGetLastError(); return 1; }
     return CSB_OK;
 }
 
@@ -937,7 +826,7 @@ extern "C" int csb_spmm_plan_dump(const csb_matrix_t* A, int batch, int sm_count
     if (!A || !info_out || batch < 1 || sm_count < 1) { set_error("csb_spmm_plan_dump: bad argument"); return CSB_ERR_INVALID_ARG; }
     SpmmHostPlan H;
     int rc;
-    try { rc = plan_spmm_host(A, spmm_nt(batch), sm_count, &H); }
+    try { rc = plan_spmm_host(A, spmm_nt(batch), sm_count, 0, &H); }
     catch (const std::bad_alloc&) { set_error("out of host memory while planning"); return CSB_ERR_ALLOC; }
     if (rc == 1) { set_error("the tensor-core layout does not apply to this matrix (fp16 values, block_r <= 64)"); return CSB_ERR_UNSUPPORTED; }
     if (rc != CSB_OK) return rc;

@@ -58,7 +58,7 @@ static void emit_spmm_item(const csb_matrix* A, int64_t b, int k0, int k1, int t
 
 struct PlannedItem { int64_t block; int k0, k1, tile, col_base; };
 
-int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, SpmmHostPlan* out) {
+int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, int force_S, SpmmHostPlan* out) {
     if (A->val_dtype != CSB_F16 || A->block_r > 64 || A->nbc > 60000) return 1;
     const int64_t nbr = A->nbr, nbc = A->nbc;
     const int MT = A->block_r <= 16 ? 1 : A->block_r <= 32 ? 2 : 4;
@@ -71,7 +71,9 @@ int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, SpmmHostPlan* out)
     for (int RG = 4; RG >= 1; RG /= 2) {
         const int64_t groups = (nbr + RG - 1) / RG;
         int64_t S = std::max<int64_t>(1, sm_count / groups);
-        S = std::min<int64_t>(std::min<int64_t>(S, nbc), 8);      // the CTAs of a row group form one cluster: at most 8
+        if (force_S > 0) S = force_S;
+        if (S > nbc) { if (force_S > 0) return 1; S = nbc; }
+        S = std::min<int64_t>(S, 8);                              // the CTAs of a row group form one cluster: at most 8
         const double ctas = (double)(groups * S);
         const double waves = std::ceil(ctas / sm_count);
         // (a cluster costs two cluster-wide barriers and the wait for its slowest CTA: as much time as about 120 KB of traffic per CTA (measured: a small GRU layer runs faster without, the 8192 x 8192 sweep with))

@@ -28,8 +28,8 @@ ROOT = os.path.dirname(HERE)
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-RNN_PHASES = ["stage input half", "walk items (both halves)", "sync after accumulator sums", "gates + publish",
-              "wait for h of the other CTAs", "activations (thread 0)", "slot-reuse guard", "loads + adds + shuffles of the sums"]
+RNN_PHASES = ["product of the input part", "waiting for the state of the step before", "barrier", "product of the recurrent part",
+              "next input, barrier, row sums", "gates + publish", "exchange inside the step", "second product, sums, gates"]
 PANEL_STAMPS = ["CTA start", "barriers set, first copies out", "bookkeeping + x landed", "inputs gathered", "bundles done",
                 "y stored", "-", "-"]
 
@@ -64,7 +64,7 @@ def rnn(names):
             b.record()
             torch.cuda.synchronize()
         ck = np.zeros((256, 8), np.int64)
-        n = binding.lib.csb_debug_rnn_clocks(C.c_void_p(ck.ctypes.data), 256)
+        n = binding.lib.csb_debug_rnn1_clocks(C.c_void_p(ck.ctypes.data), 256)
         ck = ck[:n] / T
         print("%s: T=%d, %d CTAs, %.2f us per step (instrumented)" % (name, T, n, a.elapsed_time(b) * 1e3 / T))
         for i, nm in enumerate(RNN_PHASES):
@@ -107,9 +107,7 @@ def panel(rates):
 SPMM_PHASES = ["set-up, first copies, wait for the work in front", "waiting for weights", "passing tiles, waiting for the item's tile",
                "row map, operand loads, tensor instructions", "ring bookkeeping, item headers", "tiles behind the last item",
                "waiting for the CTA's other warps", "accumulators to shared memory", "sums over the warps of a block-row",
-               "waiting for the cluster's other CTAs", "sums over the ranges, store", "until the cluster's CTAs have read",
-               "(time loop) grid barrier behind the product pass", "(time loop) gate arithmetic", "(time loop) grid barrier behind the gates",
-               "(time loop) next pass's first weights out"]
+               "waiting for the cluster's other CTAs", "sums over the ranges, store", "until the cluster's CTAs have read"]
 
 
 def spmm(cases):
@@ -132,11 +130,11 @@ def spmm(cases):
         ck = np.zeros((1 << 16, 16), np.int64)
         n = binding.lib.csb_debug_spmm_clocks(C.c_void_p(ck.ctypes.data), 1 << 16)
         ck = ck[:n].astype(np.float64)
-        wpc = 32 if int(B) <= 8 else 16
+        wpc = 32 if int(B) <= 8 else 16 if int(B) <= 32 else 8
         per_cta = ck.reshape(-1, wpc, 16)
         slow = per_cta[np.argmax(per_cta.sum(axis=2).max(axis=1))]
         last = ck[np.argmax(ck[:, :6].sum(axis=1))]      # the warp that reaches the end of its items last
-        print("%s batch %s: %d warps (%d per CTA); cycles per phase, last pass of 32 batch columns"
+        print("%s batch %s: %d warps (%d per CTA); cycles per phase, last pass"
               % (rate if rate.startswith("cfg") else "cfg4 rate %sx" % rate, B, n, wpc))
         for i, nm in enumerate(SPMM_PHASES):
             print("   %-52s mean %8.0f  min %8.0f  max %8.0f   slowest CTA: mean %8.0f  max %8.0f   last warp %8.0f"
@@ -144,40 +142,6 @@ def spmm(cases):
         print("   %-52s mean %8.0f  max %8.0f" % ("all phases", ck.sum(axis=1).mean(), ck.sum(axis=1).max()))
         for a in As:
             a.free()
-
-
-def loop(names):
-    """The one-launch time loop of the batched recurrent path: cycles per phase and pass (layer and step)."""
-    import workloads
-    os.environ["CSB_RNN_STEP_LOOP"] = "1"          # the loop is not the default path
-    torch, binding = _load()
-    for case in names:
-        name, B = case.split(":")
-        w = workloads.CONFIGS[name](B=int(B), T=32)
-        mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in w.layers]
-        L, B, H, T = len(w.layers), w.B, w.hidden_size, w.T
-        x = torch.from_numpy(w.x).cuda()
-        y = torch.empty((T, B, H), device="cuda")
-        hT = torch.empty((L, B, H), device="cuda")
-        cT = torch.empty((L, B, H), device="cuda")
-        for _ in range(3):
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record()
-            if w.cell == "lstm":
-                binding.csb_lstm_forward(mats, None, x, None, None, y, hT, cT, 0)
-            else:
-                binding.csb_gru_forward(mats, None, x, None, y, hT, 0)
-            b.record()
-            torch.cuda.synchronize()
-        ck = np.zeros((1 << 16, 16), np.int64)
-        n = binding.lib.csb_debug_spmm_clocks(C.c_void_p(ck.ctypes.data), 1 << 16)
-        ck = ck[:n].astype(np.float64) / (T * L)
-        print("%s batch %d: T=%d, %d warps, %.2f us per step (instrumented); cycles per phase and pass" % (name, B, T, n, a.elapsed_time(b) * 1e3 / T))
-        for i, nm in enumerate(SPMM_PHASES):
-            print("   %-52s mean %8.0f  min %8.0f  max %8.0f" % (nm, ck[:, i].mean(), ck[:, i].min(), ck[:, i].max()))
-        print("   %-52s mean %8.0f" % ("all phases", ck.sum(axis=1).mean()))
-        for m in mats:
-            m.free()
 
 
 if __name__ == "__main__":
@@ -189,7 +153,5 @@ if __name__ == "__main__":
         panel(rest or ["4", "25"])
     elif what == "spmm":
         spmm(rest or ["4:8", "4:32", "25:8"])
-    elif what == "loop":
-        loop(rest or ["cfg5:32", "cfg3:8"])
     else:
         raise SystemExit(__doc__)
