@@ -33,7 +33,9 @@ struct Rnn1Plan {
     int cell = 0, L = 0, BT = 1, device = 0, n_ctas = 0, H = 0, S = 0, val_dtype = 0;
     bool unusable = false;
     std::vector<uint64_t> uids;
+    bool unit_loop = false;                    // csb_rnn_unit_kernel.cuh, else csb_rnn1_kernel.cuh
     R1Args a{};
+    RuArgs u{};
     size_t smem = 0;
     const void* kernel = nullptr;
     std::vector<void*> owned;                  // device memory
@@ -80,6 +82,68 @@ static int put(Rnn1Plan* P, const V* h, size_t n, V** d) {
     return CSB_OK;
 }
 
+// What both loops need beside images and exchange buffers.
+static int put_common(Rnn1Plan* P, R1Common& c, int L, const int* in_size, const int* layer_ctas, int H, int S) {
+    int rc;
+    if ((rc = put(P, (const uint32_t*)nullptr, (size_t)P->n_ctas, &c.epoch)) != CSB_OK || (rc = put(P, (const uint32_t*)nullptr, (size_t)kMaxLayers, &c.progress)) != CSB_OK) return rc;
+    for (int l = 0; l < L; ++l) { c.in_size[l] = in_size[l]; c.layer_ctas[l] = layer_ctas[l]; }
+    c.H = H; c.S = S; c.L = L;
+    CSB_CUDA(cudaHostAlloc((void**)&P->h_status, 4, cudaHostAllocMapped));
+    *P->h_status = 0;
+    CSB_CUDA(cudaHostGetDevicePointer((void**)&c.status, P->h_status, 0));
+    return CSB_OK;
+}
+// Whether the grid can be resident at once.
+static int fits(Rnn1Plan* P, const csb_matrix* A0, bool* yes) {
+    *yes = false;
+    if (P->smem > A0->smem_optin) return CSB_OK;
+    CSB_CUDA(cudaFuncSetAttribute(P->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A0->smem_optin));
+    int occ = 0;
+    CSB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, P->kernel, kR1Threads, P->smem));
+    *yes = occ >= 1 && P->n_ctas <= occ * A0->sm_count;
+    return CSB_OK;
+}
+
+// The unit loop's plan; 1 when it is not the one for these matrices.
+static int build_unit_plan(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, int64_t weights,
+                           Rnn1Plan* P) {
+    const csb_matrix* A0 = W[0];
+    if (weights > (int64_t)env_int("CSB_RU_MAX", 12000) * A0->sm_count) return 1;
+    const int64_t units = (int64_t)L * H;
+    int want = (int)std::min<int64_t>(A0->sm_count, std::max<int64_t>(L, (units + env_int("CSB_RU_PER", kR1Warps) - 1) / env_int("CSB_RU_PER", kR1Warps)));
+    want = std::min(A0->sm_count, env_int("CSB_R1_CTAS", want));
+    RuHostPlan Hp;
+    const int hrc = plan_unit_host(cell, L, W, Wp, in_size, H, S, BT, want, &Hp);
+    if (hrc != CSB_OK) return hrc;
+    RuArgs& a = P->u;
+    size_t at = Hp.max_bytes;
+    auto room = [&](size_t floats) { const size_t o = at; at = (at + floats * 4 + 15) & ~(size_t)15; return (uint32_t)o; };
+    int max_in = 0;
+    for (int l = 0; l < L; ++l) max_in = std::max(max_in, in_size[l]);
+    const int ops = r1_ops(cell);
+    for (uint32_t& v : a.vu) v = room((size_t)(max_in + 1) * BT);
+    for (uint32_t& v : a.vr) v = room((size_t)(S + 1) * BT);
+    a.vm = room(ops == 2 ? (size_t)(H + 1) * BT : 0);
+    a.misc = room(4);
+    P->smem = at;
+    P->n_ctas = (int)Hp.ctas.size();
+    P->kernel = BT == 1 ? ru_kernel_b1(cell, P->val_dtype) : BT == 4 ? ru_kernel_b4(cell, P->val_dtype) : ru_kernel_b8(cell, P->val_dtype);
+    bool yes = false;
+    int rc = fits(P, A0, &yes);
+    if (rc != CSB_OK) return rc;
+    if (!yes) return 1;
+    uint8_t* d_img = nullptr; RuCta* d_ctas = nullptr;
+    if ((rc = put(P, Hp.bytes.data(), Hp.bytes.size(), &d_img)) != CSB_OK || (rc = put(P, Hp.ctas.data(), Hp.ctas.size(), &d_ctas)) != CSB_OK) return rc;
+    a.images = d_img; a.ctas = d_ctas;
+    for (int l = 0; l < L; ++l) {
+        if ((rc = put(P, (const uint2*)nullptr, (((size_t)S * BT + 1) & ~(size_t)1) * kR1Ring, &a.ex[0][l])) != CSB_OK) return rc;
+        if (ops == 2 && (rc = put(P, (const uint2*)nullptr, (((size_t)H * BT + 1) & ~(size_t)1) * kR1Ring, &a.ex[1][l])) != CSB_OK) return rc;
+    }
+    if ((rc = put_common(P, a, L, in_size, Hp.layer_ctas, H, S)) != CSB_OK) return rc;
+    P->unit_loop = true;
+    return CSB_OK;
+}
+
 // Returns 1 (and marks the plan) when the kernel does not take these matrices.
 static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, Rnn1Plan* P) {
     const csb_matrix* A0 = W[0];
@@ -92,6 +156,12 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
         weights += W[l]->nnz + (Wp ? Wp[l]->nnz : 0);
         if (W[l]->val_dtype != A0->val_dtype || (Wp && Wp[l]->val_dtype != A0->val_dtype)) return 1;
     }
+    {
+        const int rc = build_unit_plan(cell, L, W, Wp, in_size, H, S, BT, weights, P);
+        if (rc == CSB_OK) { CSB_CUDA(cudaDeviceSynchronize()); P->unusable = false; return CSB_OK; }
+        if (rc != 1) return rc;
+    }
+    if (BT == 8 && P->val_dtype != CSB_F16) return 1;      // not built for fp32 values
     int want = (int)std::min<int64_t>(A0->sm_count, std::max<int64_t>(L, weights / env_int("CSB_R1_MIN", 1024)));
     want = std::min(A0->sm_count, env_int("CSB_R1_CTAS", want));
     R1HostPlan Hp;
@@ -109,14 +179,12 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
     a.cs = room(Hp.max_units * BT); a.bias0 = room(4 * Hp.max_units); a.bias1 = room(Hp.max_units);
     a.misc = room(4);
     P->smem = at;
-    if (P->smem > A0->smem_optin) return 1;
     P->n_ctas = (int)Hp.ctas.size();
     P->kernel = pick_kernel_bt(cell, BT, P->val_dtype);
-    CSB_CUDA(cudaFuncSetAttribute(P->kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A0->smem_optin));
-    int occ = 0;
-    CSB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, P->kernel, kR1Threads, P->smem));
-    if (occ < 1 || P->n_ctas > occ * A0->sm_count) return 1;     // the grid must be co-resident
-    int rc;
+    bool yes = false;
+    int rc = fits(P, A0, &yes);
+    if (rc != CSB_OK) return rc;
+    if (!yes) return 1;
     uint8_t* d_img = nullptr; R1Cta* d_ctas = nullptr;
     if ((rc = put(P, Hp.bytes.data(), Hp.bytes.size(), &d_img)) != CSB_OK || (rc = put(P, Hp.ctas.data(), Hp.ctas.size(), &d_ctas)) != CSB_OK) return rc;
     a.images = d_img; a.ctas = d_ctas;
@@ -128,12 +196,7 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
             if ((rc = put(P, (const uint4*)nullptr, m.size() * kR1Ring, &a.ex[e][l])) != CSB_OK) return rc;
             a.wmap[e][l] = d_map; a.words[e][l] = (int)m.size();
         }
-    if ((rc = put(P, (const uint32_t*)nullptr, (size_t)P->n_ctas, &a.epoch)) != CSB_OK || (rc = put(P, (const uint32_t*)nullptr, (size_t)kMaxLayers, &a.progress)) != CSB_OK) return rc;
-    for (int l = 0; l < L; ++l) { a.in_size[l] = in_size[l]; a.layer_ctas[l] = Hp.layer_ctas[l]; }
-    a.H = H; a.S = S; a.L = L;
-    CSB_CUDA(cudaHostAlloc((void**)&P->h_status, 4, cudaHostAllocMapped));
-    *P->h_status = 0;
-    CSB_CUDA(cudaHostGetDevicePointer((void**)&a.status, P->h_status, 0));
+    if ((rc = put_common(P, a, L, in_size, Hp.layer_ctas, H, S)) != CSB_OK) return rc;
     CSB_CUDA(cudaDeviceSynchronize());
     P->unusable = false;
     return CSB_OK;
@@ -143,9 +206,8 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
                  int H, int S, const int* in_size, const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream) {
     if (env_int("CSB_RNN_NO_RNN1", 0)) return 1;
     if (B > 1 && env_int("CSB_RNN_NO_STEPWISE", 0)) return 1;   // asks for the persistent kernel of csb_rnn.cu
-    // tiles of batch columns that the kernel is built for; fp32 values have none of 8
-    const int BT = B == 1 ? 1 : B <= 4 ? 4 : 8;
-    if (B > 8 || (BT == 8 && W[0]->val_dtype != CSB_F16)) return 1;
+    const int BT = B == 1 ? 1 : B <= 4 ? 4 : 8;            // tiles of batch columns that the kernels are built for
+    if (B > 8) return 1;
     Rnn1Plan* P = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_r1_mu);
@@ -169,7 +231,9 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     cudaStream_t st = (cudaStream_t)stream;
     const bool host_io = (flags & CSB_FLAG_HOST_IO) != 0, has_c = cell == kR1Lstm || cell == kR1Lstmp;
     const size_t nx = (size_t)T * B * in_size[0], ny = y ? (size_t)T * B * S : 0, nh = (size_t)L * B * S, nc = has_c ? (size_t)L * B * H : 0;
-    R1Args a = P->a;
+    R1Args a1 = P->a;
+    RuArgs au = P->u;
+    R1Common& a = P->unit_loop ? (R1Common&)au : (R1Common&)a1;
     a.x = x; a.h0 = h0; a.c0 = has_c ? c0 : nullptr; a.y = y; a.hT = hT; a.cT = has_c ? cT : nullptr;
     if (host_io) {
         const size_t need = nx + ny + 2 * nh + 2 * nc;
@@ -208,7 +272,7 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    void* params[] = {(void*)&a};
+    void* params[] = {P->unit_loop ? (void*)&au : (void*)&a1};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, P->kernel, params);
     if (e == cudaErrorCooperativeLaunchTooLarge) { set_error("cooperative launch too large"); return CSB_ERR_LAUNCH; }
     CSB_CUDA(e);

@@ -23,16 +23,10 @@
 // Initial states, bias, x, y and final states are read and written in place, so a call is one launch.
 #pragma once
 
+#include "csb_rnn_exchange.cuh"
 #include "csb_rnn1_args.hpp"
-#include "csb_device.cuh"
 
 namespace csb {
-
-#ifdef CSB_PHASE_CLOCKS
-#define R1_LAP(i) do { if (tid == 0) { const long long n_ = clock64(); lap[i] += n_ - lap_at; lap_at = n_; } } while (0)
-#else
-#define R1_LAP(i) do { } while (0)
-#endif
 
 typedef unsigned __int128 Word;                // three values and a step number
 __device__ __forceinline__ Word ld_word(const uint4* p) {
@@ -45,25 +39,6 @@ __device__ __forceinline__ void st_word(uint4* p, float a, float b, float c, uin
     asm volatile("st.relaxed.gpu.global.b128 [%0], %1;" ::"l"(p), "q"(w) : "memory");
 }
 __device__ __forceinline__ uint32_t word_tag(Word w) { return (uint32_t)(w >> 96); }
-__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(d)
-        : "l"(*reinterpret_cast<unsigned long long*>(&a)), "l"(*reinterpret_cast<unsigned long long*>(&b)), "l"(*reinterpret_cast<unsigned long long*>(&c)));
-    return *reinterpret_cast<float2*>(&d);
-}
-__device__ __forceinline__ float2 half2_to_float2(uint32_t w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
-__device__ __forceinline__ float logistic(float a) { return 1.f / (1.f + expf(-a)); }
-
 // N consecutive 32-bit words of shared memory.
 template <int N> struct Regs { uint32_t v[N]; };
 template <int N>
@@ -388,23 +363,23 @@ __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn1_kernel(const __grid_co
             float h, c = 0.f;
             if (kHasC) {
                 c = on ? cs[e] : 0.f;
-                z = g == 2 ? tanhf(z) : logistic(z);
+                z = activation(z, g == 2);
                 const float zi = __shfl_sync(0xffffffffu, z, l0), zf = __shfl_sync(0xffffffffu, z, l0 + 1);
                 const float zc = __shfl_sync(0xffffffffu, z, l0 + 2), zo = __shfl_sync(0xffffffffu, z, l0 + 3);
                 c = zf * c + zi * zc;
-                h = zo * tanhf(c);
+                h = zo * activation(c, true);
                 if (on && g == 0) cs[e] = c;
             } else if (CELL == kR1Gru) {
-                if (g < 2) z = logistic(z);
+                if (g < 2) z = activation(z, false);
                 const float r = __shfl_sync(0xffffffffu, z, l0), zz = __shfl_sync(0xffffffffu, z, l0 + 1);
                 const float ni = __shfl_sync(0xffffffffu, z, l0 + 2), nh = __shfl_sync(0xffffffffu, z, l0 + 3);
-                h = (1.f - zz) * tanhf(ni + r * nh) + zz * hp;
+                h = (1.f - zz) * activation(ni + r * nh, true) + zz * hp;
             } else if (CELL == kR1Ligru) {
-                if (g == 0) z = logistic(z);
+                if (g == 0) z = activation(z, false);
                 const float zz = __shfl_sync(0xffffffffu, z, l0), cand = fmaxf(__shfl_sync(0xffffffffu, z, l0 + 1), 0.f);
                 h = zz * hp + (1.f - zz) * cand;
             } else {
-                z = logistic(z);
+                z = activation(z, false);
                 if (on && g == 1) cs[e] = z;               // the update gate, for the second half of the step
                 h = __shfl_sync(0xffffffffu, z, l0) * hp;  // r * h_{t-1}
             }
@@ -437,7 +412,7 @@ __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn1_kernel(const __grid_co
                 const bool on = j < kR1WarpUnits && e < E1;
                 const int u = on ? e / BT : 0, b = on ? e % BT : 0, at = ((int)hd->op[OPS - 1].unit0 + u) * BT + b;
                 float h = on ? f32(a.z[1])[e] + f32(a.bias1)[u] : 0.f;
-                if (CELL == kR1GruRb && on) { const float zz = cs[e]; h = (1.f - zz) * tanhf(h) + zz * vr[at]; }
+                if (CELL == kR1GruRb && on) { const float zz = cs[e]; h = (1.f - zz) * activation(h, true) + zz * vr[at]; }
                 const float h1 = __shfl_down_sync(0xffffffffu, h, 4), h2 = __shfl_down_sync(0xffffffffu, h, 8);
                 if (on && g == 0 && (j == 0 || j == 3) && (more || layer + 1 < a.L))
                     st_word(ex_state + (size_t)(t & (kR1Ring - 1)) * n_state + hd->op[OPS - 1].word0 + e / 3, h, h1, h2, base + (uint32_t)t);
