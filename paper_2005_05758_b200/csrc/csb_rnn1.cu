@@ -107,10 +107,20 @@ static int fits(Rnn1Plan* P, const csb_matrix* A0, bool* yes) {
 // The unit loop's plan; 1 when it is not the one for these matrices.
 static int build_unit_plan(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, int64_t weights,
                            Rnn1Plan* P) {
+    if (env_int("CSB_RNN_NO_UNIT", 0)) return 1;           // diagnostics: the other loop, which covers every size of this one
     const csb_matrix* A0 = W[0];
-    if (weights > (int64_t)env_int("CSB_RU_MAX", 12000) * A0->sm_count) return 1;
-    const int64_t units = (int64_t)L * H;
-    int want = (int)std::min<int64_t>(A0->sm_count, std::max<int64_t>(L, (units + env_int("CSB_RU_PER", kR1Warps) - 1) / env_int("CSB_RU_PER", kR1Warps)));
+    int max_in = 0;
+    for (int l = 0; l < L; ++l) max_in = std::max(max_in, in_size[l]);
+    // Taken wherever its lists fit in shared memory: 4 (fp16) or 8 bytes a weight, uneven CTAs and padding one part in
+    // eight (an estimate that spares the planning; fits() decides).  Below that line it was the faster loop at every
+    // size measured except one, level there: 1024 units and 16 k weights a CTA 1.9 against 3.7 us a step, LSTMP
+    // 3.0 / 5.9, 8 batch columns 4.2 / 5.9, 2 x 1024 units on 1024 inputs 3.2 / 3.0, 2048 units on 2048 3.2 / 3.3.
+    const size_t lists = (size_t)weights * (W[0]->val_dtype == CSB_F16 ? 4 : 8) / (size_t)A0->sm_count * 9 / 8;
+    if (lists + (size_t)(2 * (max_in + S) + H) * BT * 4 > A0->smem_optin) return 1;
+    // A unit per warp where a step is a chain of latencies (batch 1: more CTAs make the exchange longer, 2.6 us with 8
+    // units a CTA), as many CTAs as there are where batch columns make it the product's time (4.3 against 6.1 us).
+    const int64_t units = (int64_t)L * H, each = BT == 1 ? kR1Warps : kR1Warps / 4;
+    int want = (int)std::min<int64_t>(A0->sm_count, std::max<int64_t>(L, (units + each - 1) / each));
     want = std::min(A0->sm_count, env_int("CSB_R1_CTAS", want));
     RuHostPlan Hp;
     const int hrc = plan_unit_host(cell, L, W, Wp, in_size, H, S, BT, want, &Hp);
@@ -118,8 +128,6 @@ static int build_unit_plan(int cell, int L, const csb_matrix* const* W, const cs
     RuArgs& a = P->u;
     size_t at = Hp.max_bytes;
     auto room = [&](size_t floats) { const size_t o = at; at = (at + floats * 4 + 15) & ~(size_t)15; return (uint32_t)o; };
-    int max_in = 0;
-    for (int l = 0; l < L; ++l) max_in = std::max(max_in, in_size[l]);
     const int ops = r1_ops(cell);
     for (uint32_t& v : a.vu) v = room((size_t)(max_in + 1) * BT);
     for (uint32_t& v : a.vr) v = room((size_t)(S + 1) * BT);

@@ -6,15 +6,24 @@
 // warp: input part of its rows (while h_{t-1} is on its way), words of h_{t-1}, barrier, recurrent part,
 // sums by shuffle, gates, publication.  Staged vectors are double-buffered, so that the one barrier is
 // enough.
+//
+// What bounds it is the exchange: 0.9 to 1.0 us of a step of 1.9 (1024 LSTM units on 153 inputs, 13x
+// pruned, 64 CTAs; 3.7 us with the other loop, whose sums and gates are phases of their own), the walks
+// take 0.5 and sums and gates 0.4.  Words are asked for as late as they can be: a load that finds a pair not
+// yet written has to be repeated, and many CTAs repeating theirs slow down the arrival itself.  With the
+// loads in front of the input part the same step took 2.8 us.  So nothing is asked for before the input
+// part is done, and pauses stand where a wait is sure to be long: the second exchange of a step (LSTMP 4.6 us
+// without, 3.0 with 200 to 400 ns), and the state of stacked layers, of which two CTA sets read one
+// (2 x 1024 units: 3.6 us without, 2.5 with 150 to 300 ns; a single layer has nothing to gain).  Pauses that
+// adapt themselves, from hits and misses of the first load, did no better (3.3 and 2.5 us).
 #pragma once
 
 #include "csb_rnn_exchange.cuh"
 #include "csb_rnn1_args.hpp"
 
-#ifndef MID_NS
-#define MID_NS 0
-#endif
 namespace csb {
+
+constexpr unsigned kStatePause = 150, kMidPause = 300;     // ns, see above
 
 // s[b] += f * x[b]
 template <int BT>
@@ -222,9 +231,8 @@ __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn_unit_kernel(const __gri
         for (int b = 0; b < BT; ++b) acc[b] = 0.f;
         add_part(0, 0, vu, acc);
         R1_LAP(0);                                         // product of the input part
-        // the state of the step before and the next step's input, so that one barrier covers both.  Nothing is
-        // asked for earlier: a load that finds a pair not yet written makes the line's later arrival slower for
-        // everybody (1024 LSTM units on 64 CTAs: 2.8 us a step with the loads in front of the input part, 1.8 here)
+        // the state of the step before and the next step's input, so that one barrier covers both
+        if (a.L > 1) __nanosleep(kStatePause);
         if (t > 0) take(ex_state + (size_t)((t - 1) & (kR1Ring - 1)) * p_state, n_state, base + (uint32_t)(t - 1), vr);
         if (layer > 0 && more) take(ex_below + (size_t)((t + 1) & (kR1Ring - 1)) * p_state, n_state, base + (uint32_t)(t + 1), vu_next);
         if (layer == 0) cp_async_wait();
@@ -280,7 +288,7 @@ __global__ void __launch_bounds__(kR1Threads, 1) csb_rnn_unit_kernel(const __gri
 #pragma unroll
             for (int b = 0; b < BT; ++b) acc[b] = 0.f;
             if (CELL == kR1GruRb) add_part(OPS - 1, 0, vu, acc);
-            if (MID_NS) __nanosleep(MID_NS);
+            __nanosleep(kMidPause);
             take(ex_mid + (size_t)ring * p_mid, n_mid, base + (uint32_t)t, vm);
             if (!__syncthreads_and(ok)) break;
             R1_LAP(6);                                     // exchange inside the step
