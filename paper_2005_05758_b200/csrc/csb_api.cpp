@@ -25,7 +25,7 @@ int product_any(const csb_matrix* A, const float* X, int64_t ldx, int batch, flo
         const int rc = launch_spmm_mma(A, X, ldx, batch, Y, ldy, stream);
         if (rc != 1) return rc;                       // 1: the tensor-core plan does not fit this matrix
     }
-    if (batch == 1 && A->panel && A->panel->built) return launch_panels(A, X, Y, stream);
+    if (panels_applicable(A, batch)) return launch_panels(A, X, ldx, batch, Y, ldy, stream);
     return launch_product(A, X, ldx, batch, Y, ldy, stream);
 }
 

@@ -319,12 +319,13 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
                      PanelHostPlan* out);
 struct PanelPlan {                         // device side
     bool built = false;
-    // kernel variants: fp16 values with one fp32 vector; 16-bit fixed point with 1, 2 or 4 vectors
-    enum { kVariants = 4 };
-    static int bt(int v) { return v == 3 ? 4 : v; }
+    // kernel variants by value type: 1, 2 or 4 input vectors a pass
+    enum { kVariants = 3 };
+    static int bt(int v) { return 1 << v; }
     int ctas = 0, warps = 0, stage_bytes = 0, max_rows = 0, max_xg = 0, max_meta = 0;
-    int log2_ring[kVariants] = {0, 0, 0, 0};   // 0: the variant does not fit
-    size_t smem_bytes[kVariants] = {0, 0, 0, 0};
+    int log2_ring[kVariants] = {0, 0, 0};   // 0: the variant does not fit
+    bool staged[kVariants] = {true, true, true};   // inputs come to shared memory whole; else the gather reads them where they are
+    size_t smem_bytes[kVariants] = {0, 0, 0};
     uint8_t* d_panels = nullptr;
     std::vector<PanelCta> cta;
     int64_t stream_bytes = 0;
@@ -332,7 +333,8 @@ struct PanelPlan {                         // device side
 };
 int plan_panels(csb_matrix* A);            // after plan_product; leaves A->panel NULL when the path does not apply
 void free_panels(csb_matrix* A);
-int launch_panels(const csb_matrix* A, const float* x, float* y, void* stream);
+bool panels_applicable(const csb_matrix* A, int batch);    // and faster than launch_product
+int launch_panels(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
 int launch_panels_q16(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch, int64_t* acc, int64_t ldy, void* stream);
 
 // csb_product.cu

@@ -32,15 +32,16 @@ namespace csb {
 
 struct PanelArgs {
     const uint8_t* panels;
-    const void* x;                     // float [cols], or int16 [nb, ldx]
-    void* y;                           // float [rows], or int64 [nb, ldy]
-    long long ldx, ldy;                // fixed point only
-    int nb;                            // fixed point: batch columns of this pass, 1..BT
+    const void* x;                     // float or int16 [nb, ldx]
+    void* y;                           // float or int64 [nb, ldy]
+    long long ldx, ldy;
+    int nb;                            // batch columns of this pass, 1..BT
     uint32_t* status;
     int rows, cols;
     int log2_stage, log2_slots;        // ring = 2^log2_slots stages of 2^log2_stage bytes
     int max_rows;                      // accumulators per warp
     int max_xg, max_meta;
+    int staged;                        // PanelPlan::staged
     uint4 cta[kMaxPanelCtas];          // PanelCta per CTA
 #ifdef CSB_PANEL_CLOCKS
     unsigned long long* clocks;        // instrumented build only: [CTA][8] wall-clock stamps in ns
@@ -55,18 +56,18 @@ struct PanelArgs {
 
 __host__ __device__ inline size_t panel_align(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Shared-memory carve-up, identical on host and device.  BT = 0: fp32 inputs and per-warp fp32
-// sums; BT > 0: fixed point, BT int16 inputs per matrix column, one 64-bit sum per row and batch column.
+// Shared-memory carve-up, identical on host and device: BT input vectors, BT gathered values per kept
+// column, BT sums per row.  Float inputs: fp32 sums per warp; fixed point: int16 inputs, one 64-bit sum per CTA.
 struct PanelSmem {
     size_t ring, xs, xs_row, xg, zs, meta, bars, done, issued, dead, total;
-    __host__ __device__ PanelSmem(int BT, int W, int log2_stage, int log2_slots, int cols, int max_xg, int max_rows, int max_meta) {
+    __host__ __device__ PanelSmem(bool q16, bool staged, int BT, int W, int log2_stage, int log2_slots, int cols, int max_xg, int max_rows, int max_meta) {
         const int slots = 1 << log2_slots;
         ring = 0;
         xs = (size_t)slots << log2_stage;
-        xs_row = panel_align((size_t)cols * (BT ? 2 : 4), 16);
-        xg = xs + xs_row * (BT ? BT : 1);
-        zs = panel_align(xg + (size_t)max_xg * (BT ? 2 * BT : 4), 16);
-        meta = panel_align(zs + (BT ? (size_t)BT * max_rows * 8 : (size_t)W * max_rows * 4), 128);
+        xs_row = panel_align((size_t)cols * (q16 ? 2 : 4), 16);
+        xg = xs + (staged ? xs_row * BT : 0);
+        zs = panel_align(xg + (size_t)max_xg * BT * (q16 ? 2 : 4), 16);
+        meta = panel_align(zs + (size_t)max_rows * BT * (q16 ? 8 : 4 * W), 128);
         bars = panel_align(meta + (size_t)max_meta, 16);
         done = bars + (size_t)(slots + 2) * 8;
         issued = done + (size_t)slots * 4;
@@ -212,12 +213,86 @@ __device__ __forceinline__ void panel_item_q16(const uint8_t* ring, uint32_t rin
         }
 }
 
-// BT = 0: fp16 values, fp32 input and output.  BT = 1, 2, 4: 16-bit fixed point, BT batch columns a pass.
-template <int BT>
+// The lane's share of one item of fp16 or fp32 values with BT input vectors.  The gathered inputs lie in
+// quads of columns, BT float4 to a quad; a weight is read and converted once for all vectors.
+template <int VAL, int BT>
+__device__ __forceinline__ void panel_item_float(const uint8_t* ring, uint32_t ring_mask, uint32_t off, const float4* __restrict__ xq4, int n, int m, int gl,
+                                                 int logp, int logg, float (&acc)[BT]) {
+    constexpr int U = VAL == CSB_F32 ? 4 : 8, Q = U / 4;   // columns and quads of 16 bytes
+    float2 lo[BT], hi[BT];
+#pragma unroll
+    for (int b = 0; b < BT; ++b) { lo[b] = make_float2(0.f, 0.f); hi[b] = make_float2(0.f, 0.f); }
+    const int r = gl & ((1 << logp) - 1), sub = gl >> logp, S = 32 >> (logg + logp);
+    const int whole = n / U;
+    uint32_t q = off + ((uint32_t)(sub * m + r) << 4);
+    const uint32_t qstep = (uint32_t)(S * m) << 4;
+    const float4* xq = xq4 + (size_t)Q * sub * BT;
+#pragma unroll 2
+    for (int o = sub; o < whole; o += S) {
+        const uint4 w = *reinterpret_cast<const uint4*>(ring + (q & ring_mask));
+        if (VAL == CSB_F32) {
+            const float2 w0 = make_float2(__uint_as_float(w.x), __uint_as_float(w.y)), w1 = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                const float4 x = xq[b];
+                lo[b] = ffma2(w0, make_float2(x.x, x.y), lo[b]);
+                hi[b] = ffma2(w1, make_float2(x.z, x.w), hi[b]);
+            }
+        } else {
+            const float2 w0 = h2f2(w.x), w1 = h2f2(w.y), w2 = h2f2(w.z), w3 = h2f2(w.w);
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                const float4 x = xq[b], y = xq[BT + b];
+                lo[b] = ffma2(w0, make_float2(x.x, x.y), lo[b]);
+                hi[b] = ffma2(w1, make_float2(x.z, x.w), hi[b]);
+                lo[b] = ffma2(w2, make_float2(y.x, y.y), lo[b]);
+                hi[b] = ffma2(w3, make_float2(y.z, y.w), hi[b]);
+            }
+        }
+        q += qstep;
+        xq += Q * S * BT;
+    }
+    if ((n & (U - 1)) && gl < m) {
+        // the columns left over, by halves (csb_panel_plan.cpp); two of them and the last one lie in one quad
+        uint32_t tb = off + ((uint32_t)(whole * m) << 4);
+        const float* xt = reinterpret_cast<const float*>(xq4 + (size_t)Q * whole * BT);
+        if (VAL != CSB_F32 && (n & 4)) {
+            const uint2 w = *reinterpret_cast<const uint2*>(ring + ((tb + 8u * gl) & ring_mask));
+#pragma unroll
+            for (int b = 0; b < BT; ++b) {
+                const float4 x = *reinterpret_cast<const float4*>(xt + 4 * b);
+                lo[b] = ffma2(h2f2(w.x), make_float2(x.x, x.y), lo[b]);
+                hi[b] = ffma2(h2f2(w.y), make_float2(x.z, x.w), hi[b]);
+            }
+            tb += 8u * m; xt += 4 * BT;
+        }
+        if (n & 2) {
+            float2 w;
+            if (VAL == CSB_F32) { w = *reinterpret_cast<const float2*>(ring + ((tb + 8u * gl) & ring_mask)); tb += 8u * m; }
+            else { w = h2f2(*reinterpret_cast<const uint32_t*>(ring + ((tb + 4u * gl) & ring_mask))); tb += 4u * m; }
+#pragma unroll
+            for (int b = 0; b < BT; ++b) lo[b] = ffma2(w, *reinterpret_cast<const float2*>(xt + 4 * b), lo[b]);
+        }
+        if (n & 1) {
+            const float w = VAL == CSB_F32 ? *reinterpret_cast<const float*>(ring + ((tb + 4u * gl) & ring_mask))
+                                           : __half2float(*reinterpret_cast<const __half*>(ring + ((tb + 2u * gl) & ring_mask)));
+#pragma unroll
+            for (int b = 0; b < BT; ++b) hi[b].x = fmaf(w, xt[4 * b + (n & 2)], hi[b].x);
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < BT; ++b) acc[b] = (lo[b].x + hi[b].x) + (lo[b].y + hi[b].y);
+}
+
+// VAL: type of the values; fp16 and fp32 with fp32 inputs and outputs, 16-bit fixed point with 64-bit
+// outputs.  BT: input vectors of a pass.
+template <int VAL, int BT>
 __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constant__ PanelArgs a) {
+    constexpr bool kQ = VAL == CSB_Q16;
+    constexpr uint32_t kXBytes = kQ ? 2u : 4u;
     extern __shared__ __align__(128) uint8_t smem[];
     const int W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const PanelSmem L(BT, W, a.log2_stage, a.log2_slots, a.cols, a.max_xg, a.max_rows, a.max_meta);
+    const PanelSmem L(kQ, a.staged != 0, BT, W, a.log2_stage, a.log2_slots, a.cols, a.max_xg, a.max_rows, a.max_meta);
     const uint4 ct = a.cta[blockIdx.x];
     const uint8_t* panel = a.panels + (size_t)ct.x * 16;
     const uint32_t meta_bytes = ct.y, value_bytes = ct.z;
@@ -237,8 +312,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
     volatile uint32_t* issued = reinterpret_cast<volatile uint32_t*>(smem + L.issued);
     volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(smem + L.dead);
 
-    const bool x_bulk = BT ? (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols & 7) == 0 && (a.nb == 1 || (a.ldx & 7) == 0)
-                           : (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols & 3) == 0;
+    const bool x_bulk = a.staged && (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols * kXBytes & 15) == 0 && (a.nb == 1 || (a.ldx * kXBytes & 15) == 0);
     // Launched with programmatic stream serialization, this grid may start while the kernel in
     // front of it on the stream is still draining: whatever comes next may be scheduled as early
     // as the hardware likes, and this grid touches x and y only behind grid_dependency_wait().
@@ -261,12 +335,11 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
         }
         if (s == slots + 1u && x_bulk) {
             grid_dependency_wait();
-            const uint32_t xb = (uint32_t)a.cols * (BT ? 2u : 4u);
-            const int nb = BT ? a.nb : 1;
-            mbar_expect_tx(xbar, xb * (uint32_t)nb);
-            for (int b = 0; b < nb; ++b)
+            const uint32_t xb = (uint32_t)a.cols * kXBytes;
+            mbar_expect_tx(xbar, xb * (uint32_t)a.nb);
+            for (int b = 0; b < a.nb; ++b)
                 for (uint32_t off = 0; off < xb; off += 16384u)
-                    bulk_g2s(smem + L.xs + b * L.xs_row + off, reinterpret_cast<const uint8_t*>(a.x) + (BT ? (size_t)b * a.ldx * 2 : 0) + off, min(16384u, xb - off), xbar);
+                    bulk_g2s(smem + L.xs + b * L.xs_row + off, reinterpret_cast<const uint8_t*>(a.x) + (size_t)b * a.ldx * kXBytes + off, min(16384u, xb - off), xbar);
         }
         __syncwarp(slots + 2u >= 32u ? 0xffffffffu : (1u << (slots + 2u)) - 1u);
         if (s < slots && s < n_stages) {
@@ -276,14 +349,14 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
             bulk_g2s(ring + ((size_t)s << a.log2_stage), values + ((size_t)s << a.log2_stage), bytes, &full[s]);
         }
     }
-    for (int i = threadIdx.x; i < (BT ? 2 * BT : W) * a.max_rows; i += blockDim.x) zs_all[i] = 0.f;
+    for (int i = threadIdx.x; i < (kQ ? 2 : W) * BT * a.max_rows; i += blockDim.x) zs_all[i] = 0.f;
     if (!x_bulk) {
         grid_dependency_wait();
-        if (BT == 0)
-            for (int i = threadIdx.x; i < a.cols; i += blockDim.x) xs[i] = __ldg(reinterpret_cast<const float*>(a.x) + i);
-        for (int b = 0; b < (BT ? a.nb : 0); ++b)
-            for (int i = threadIdx.x; i < a.cols; i += blockDim.x)
-                reinterpret_cast<int16_t*>(smem + L.xs + b * L.xs_row)[i] = __ldg(reinterpret_cast<const int16_t*>(a.x) + (long long)b * a.ldx + i);
+        for (int b = 0; b < (a.staged ? a.nb : 0); ++b)
+            for (int i = threadIdx.x; i < a.cols; i += blockDim.x) {
+                if (kQ) reinterpret_cast<int16_t*>(smem + L.xs + b * L.xs_row)[i] = __ldg(reinterpret_cast<const int16_t*>(a.x) + (long long)b * a.ldx + i);
+                else reinterpret_cast<float*>(smem + L.xs + b * L.xs_row)[i] = __ldg(reinterpret_cast<const float*>(a.x) + (long long)b * a.ldx + i);
+            }
     }
     __syncthreads();                                       // barriers initialised, counters and sums cleared
     PANEL_STAMP(1);
@@ -304,13 +377,15 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
             const uint2* gath = reinterpret_cast<const uint2*>(meta + H->gather_off);
             const uint8_t* cidx = meta + H->cidx_off;
             const int n_gather = (int)H->n_gather;
+            const float* xrow = a.staged ? xs : reinterpret_cast<const float*>(a.x);
+            const long long xpitch = a.staged ? (long long)(L.xs_row >> 2) : a.ldx;
             for (int g0 = warp * 4; g0 < n_gather; g0 += W * 4) {
                 const int g = g0 + (lane >> 3);
                 const uint2 gd = g < n_gather ? gath[g] : make_uint2(0u, 0u);
                 const uint32_t xbase = gd.x & 0xffffu, n = gd.x >> 16, xoff = gd.y;
                 for (uint32_t k = (uint32_t)(lane & 7) * 4u; k < n; k += 32u) {
                     const uint32_t c4 = *reinterpret_cast<const uint32_t*>(cidx + xoff + k);
-                    if (BT) {
+                    if (kQ) {
                         const int16_t* xr = reinterpret_cast<const int16_t*>(xs) + xbase;
                         uint2* dst = reinterpret_cast<uint2*>(xg) + (size_t)((xoff + k) >> 2) * BT;
 #pragma unroll
@@ -328,10 +403,16 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
                         }
                         continue;
                     }
-                    float4 v;
-                    v.x = xs[xbase + (c4 & 0xffu)]; v.y = xs[xbase + ((c4 >> 8) & 0xffu)];
-                    v.z = xs[xbase + ((c4 >> 16) & 0xffu)]; v.w = xs[xbase + (c4 >> 24)];
-                    *reinterpret_cast<float4*>(xg + xoff + k) = v;
+                    const float* xr = xrow + xbase;
+                    float4* dst = reinterpret_cast<float4*>(xg) + (size_t)((xoff + k) >> 2) * BT;
+#pragma unroll
+                    for (int b = 0; b < BT; ++b) {
+                        // (a column past nb stays 0)
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (b < a.nb) v = make_float4(xr[c4 & 0xffu], xr[(c4 >> 8) & 0xffu], xr[(c4 >> 16) & 0xffu], xr[c4 >> 24]);
+                        dst[b] = v;
+                        xr += xpitch;
+                    }
                 }
             }
         }
@@ -345,7 +426,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
         const uint16_t* expect = reinterpret_cast<const uint16_t*>(meta + H->expect_off);
         const uint8_t* ridx = meta + H->ridx_off;
         const float4* xg4 = reinterpret_cast<const float4*>(xg);
-        float* zs = zs_all + (size_t)warp * a.max_rows;
+        float* zs = zs_all + (size_t)warp * a.max_rows * BT;
         const uint32_t i_end = wb[warp + 1];
         uint32_t idx = wb[warp];
         uint32_t e = idx < i_end ? wlist[idx] : 0u;
@@ -362,9 +443,27 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
             const uint32_t st = off >> a.log2_stage;          // the same for every member of the bundle
             if (__any_sync(0xffffffffu, !panel_wait_stage(full, issued, st, a.log2_slots, s_dead))) { *s_dead = 1u; break; }
 
-            if (BT) {
-                panel_item_q16<BT ? BT : 1>(ring, ring_mask, off, reinterpret_cast<const uint2*>(xg) + (size_t)xoff4 * BT, n, m, gl, logp, logg, my_row, gl < m,
-                                            reinterpret_cast<unsigned long long*>(zs_all));
+            if (kQ) {
+                panel_item_q16<BT>(ring, ring_mask, off, reinterpret_cast<const uint2*>(xg) + (size_t)xoff4 * BT, n, m, gl, logp, logg, my_row, gl < m,
+                                   reinterpret_cast<unsigned long long*>(zs_all));
+            } else if (VAL == CSB_F32 || BT > 1) {
+                float acc[BT];
+                panel_item_float<VAL, BT>(ring, ring_mask, off, xg4 + (size_t)xoff4 * BT, n, m, gl, logp, logg, acc);
+                // join the lanes that split the columns of a row (fixed tree inside the lane group)
+                const int pmin = logg ? (int)__reduce_min_sync(0xffffffffu, 1u << logp) : 1 << logp;
+                for (int o = 16 >> logg; o >= pmin; o >>= 1)
+#pragma unroll
+                    for (int b = 0; b < BT; ++b) {
+                        const float t = __shfl_xor_sync(0xffffffffu, acc[b], o);
+                        if (o >= (1 << logp)) acc[b] += t;
+                    }
+                // members of a bundle may add into the same output: one lane group at a time
+                for (int g = 0; g < (1 << logg); ++g) {
+                    if (grp == g && gl < m)
+#pragma unroll
+                        for (int b = 0; b < BT; ++b) zs[my_row * BT + b] += acc[b];
+                    __syncwarp();
+                }
             } else {
             const int r = gl & ((1 << logp) - 1), sub = gl >> logp, S = 32 >> (logg + logp);
             const int noct = n >> 3;
@@ -479,17 +578,18 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
 
     // ---- add the warps' copies in warp order and store the CTA's rows
     const int n_rows = (int)H->n_rows, row0 = (int)H->row0;
-    if (BT) {
+    if (kQ) {
         for (int t = threadIdx.x; t < n_rows * a.nb; t += blockDim.x) {
             const int b = t / n_rows, r = t - b * n_rows;
             reinterpret_cast<long long*>(a.y)[(long long)b * a.ldy + row0 + r] = reinterpret_cast<const long long*>(zs_all)[r * BT + b];
         }
         return;
     }
-    for (int t = threadIdx.x; t < n_rows; t += blockDim.x) {
+    for (int t = threadIdx.x; t < n_rows * a.nb; t += blockDim.x) {
+        const int b = BT == 1 ? 0 : t / n_rows, r = t - b * n_rows;
         float v = 0.f;
-        for (int w = 0; w < W; ++w) v += zs_all[(size_t)w * a.max_rows + t];
-        reinterpret_cast<float*>(a.y)[row0 + t] = v;
+        for (int w = 0; w < W; ++w) v += zs_all[((size_t)w * a.max_rows + r) * BT + b];
+        reinterpret_cast<float*>(a.y)[(long long)b * a.ldy + row0 + r] = v;
     }
     PANEL_STAMP(5);
     PANEL_STAMP(7);
@@ -510,8 +610,15 @@ static int env_int(const char* name, int dflt) {
 }
 static int log2_floor(int v) { int l = 0; while ((2 << l) <= v) ++l; return l; }
 
+typedef void (*PanelKernel)(PanelArgs);
+template <int VAL>
+static PanelKernel pick_panel_kernel(int v) { return v == 0 ? csb_panel_kernel<VAL, 1> : v == 1 ? csb_panel_kernel<VAL, 2> : csb_panel_kernel<VAL, 4>; }
+static PanelKernel panel_kernel(int val_dtype, int v) {
+    return val_dtype == CSB_F16 ? pick_panel_kernel<CSB_F16>(v) : val_dtype == CSB_F32 ? pick_panel_kernel<CSB_F32>(v) : pick_panel_kernel<CSB_Q16>(v);
+}
+
 int plan_panels(csb_matrix* A) {
-    if ((A->val_dtype != CSB_F16 && A->val_dtype != CSB_Q16) || env_int("CSB_NO_PANEL", 0)) return CSB_OK;
+    if (env_int("CSB_NO_PANEL", 0)) return CSB_OK;
     const int warps = std::min(32, std::max(1, env_int("CSB_PANEL_WARPS", 32)));
     int stage = env_int("CSB_PANEL_STAGE", 16384);
     stage = 1 << std::min(15, std::max(13, log2_floor(stage)));
@@ -524,17 +631,20 @@ int plan_panels(csb_matrix* A) {
     P->ctas = (int)H.cta.size(); P->warps = warps; P->stage_bytes = stage;
     P->max_xg = (int)H.max_xg; P->max_meta = (int)H.max_meta; P->max_rows = (int)std::max<size_t>(H.max_rows, 1);
     const int want_ring = std::min(17, std::max(log2_floor(stage) + 1, env_int("CSB_PANEL_RING_LOG2", 17)));
-    // the deepest ring that leaves room for the rest, per variant of the kernel
-    for (int v = 0; v < PanelPlan::kVariants; ++v) {
-        P->log2_ring[v] = 0;
-        if ((PanelPlan::bt(v) != 0) != (A->val_dtype == CSB_Q16)) continue;
-        for (int lr = want_ring; lr > log2_floor(stage); --lr) {
-            const PanelSmem L(PanelPlan::bt(v), warps, log2_floor(stage), lr - log2_floor(stage), (int)A->cols, P->max_xg, P->max_rows, P->max_meta);
-            if (L.total <= A->smem_optin) { P->log2_ring[v] = lr; P->smem_bytes[v] = L.total; break; }
-        }
-    }
+    // The deepest ring that leaves room for the rest, per variant of the kernel.  Several float vectors: not
+    // below 64 KB (a pass of two over 8192 x 8192 fp32 values at 4x took 36 us on a ring of 32 KB, two passes of
+    // one 26); where the vectors themselves are in its way, they stay in global memory and the gather reads
+    // them there.
+    const bool q16 = A->val_dtype == CSB_Q16;
+    for (int v = 0; v < PanelPlan::kVariants; ++v)
+        for (int direct = 0; direct < (q16 || v == 0 ? 1 : 2) && !P->log2_ring[v]; ++direct)
+            for (int lr = want_ring; lr > log2_floor(stage); --lr) {
+                if (v > 0 && !q16 && lr < std::min(16, want_ring)) break;
+                const PanelSmem L(q16, !direct, PanelPlan::bt(v), warps, log2_floor(stage), lr - log2_floor(stage), (int)A->cols, P->max_xg, P->max_rows, P->max_meta);
+                if (L.total <= A->smem_optin) { P->log2_ring[v] = lr; P->smem_bytes[v] = L.total; P->staged[v] = !direct; break; }
+            }
     // the variant that takes one vector does not fit: the other path serves this matrix
-    if (!P->log2_ring[A->val_dtype == CSB_Q16 ? 1 : 0]) { delete P; return CSB_OK; }
+    if (!P->log2_ring[0]) { delete P; return CSB_OK; }
     int prev = 0;
     CSB_CUDA(cudaGetDevice(&prev));
     CSB_CUDA(cudaSetDevice(A->device));
@@ -544,8 +654,8 @@ int plan_panels(csb_matrix* A) {
     P->balance = H.balance; P->warp_balance = H.warp_balance;
     CSB_CUDA(cudaMalloc((void**)&P->d_panels, std::max<size_t>(H.bytes.size(), 16)));
     CSB_CUDA(cudaMemcpy(P->d_panels, H.bytes.data(), H.bytes.size(), cudaMemcpyHostToDevice));
-    for (const void* k : {(const void*)csb_panel_kernel<0>, (const void*)csb_panel_kernel<1>, (const void*)csb_panel_kernel<2>, (const void*)csb_panel_kernel<4>})
-        CSB_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
+    for (int v = 0; v < PanelPlan::kVariants; ++v)
+        CSB_CUDA(cudaFuncSetAttribute((const void*)panel_kernel(A->val_dtype, v), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
     CSB_CUDA(cudaDeviceSynchronize());
     CSB_CUDA(cudaSetDevice(prev));
     P->built = true;
@@ -582,7 +692,7 @@ static int launch_variant(const csb_matrix* A, int v, const void* x, int64_t ldx
     a.panels = P.d_panels; a.x = x; a.y = y; a.ldx = ldx; a.ldy = ldy; a.nb = nb; a.status = Q.d_status;
     a.rows = (int)A->rows; a.cols = (int)A->cols;
     a.log2_stage = log2_floor(P.stage_bytes); a.log2_slots = P.log2_ring[v] - a.log2_stage;
-    a.max_rows = P.max_rows; a.max_xg = P.max_xg; a.max_meta = P.max_meta;
+    a.staged = P.staged[v]; a.max_rows = P.max_rows; a.max_xg = P.max_xg; a.max_meta = P.max_meta;
     for (int c = 0; c < P.ctas; ++c) a.cta[c] = make_uint4(P.cta[c].off16, P.cta[c].meta_bytes, P.cta[c].value_bytes, P.cta[c].n_rows);
 #ifdef CSB_PANEL_CLOCKS
     static unsigned long long* d_clocks = nullptr;
@@ -601,29 +711,49 @@ static int launch_variant(const csb_matrix* A, int v, const void* x, int64_t ldx
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = use_pdl ? 1u : 0u;
-    cudaError_t e = v == 0 ? cudaLaunchKernelEx(&cfg, csb_panel_kernel<0>, a) : v == 1 ? cudaLaunchKernelEx(&cfg, csb_panel_kernel<1>, a)
-                  : v == 2 ? cudaLaunchKernelEx(&cfg, csb_panel_kernel<2>, a) : cudaLaunchKernelEx(&cfg, csb_panel_kernel<4>, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, panel_kernel(A->val_dtype, v), a);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (prev != A->device) cudaSetDevice(prev);
     if (e != cudaSuccess) { set_error("panel kernel launch failed: %s", cudaGetErrorString(e)); return CSB_ERR_CUDA; }
     return CSB_OK;
 }
 
-int launch_panels(const csb_matrix* A, const float* x, float* y, void* stream) {
-    return launch_variant(A, 0, x, A->cols, 1, y, A->rows, stream);
+// Passes of as many vectors as are left and as leave room for a ring.
+static int next_pass(const csb_matrix* A, int left) {
+    int v = left >= 3 ? 2 : left - 1;
+    while (v > 0 && !A->panel->log2_ring[v]) --v;
+    return v;
+}
+// The other kernel (csb_product.cu) takes vectors in passes of four, two and one.  A pass of this one takes about
+// half as long as one of its passes of four (3072 x 1536 fp32 values at 8x, four vectors: 5.0 against 14.9 us;
+// 2048 x 8192 fp16, two vectors: 9.4 against 16.5), so up to twice as many are allowed.
+bool panels_applicable(const csb_matrix* A, int batch) {
+    if (!A->panel || !A->panel->built || A->val_dtype == CSB_Q16) return false;
+    if (batch == 1) return true;
+    if (batch > 8) return false;
+    int passes = 0;
+    for (int b = 0; b < batch; ++passes) b += std::min(batch - b, PanelPlan::bt(next_pass(A, batch - b)));
+    return passes <= (batch <= 4 ? 1 : batch <= 6 ? 2 : 3);
 }
 
-int launch_panels_q16(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch, int64_t* acc, int64_t ldy, void* stream) {
+template <typename X, typename Y>
+static int launch_passes(const csb_matrix* A, const X* x, int64_t ldx, int batch, Y* y, int64_t ldy, void* stream) {
     for (int b0 = 0; b0 < batch;) {
-        // as many batch columns a pass as are left and as leave room for a ring
-        int v = batch - b0 >= 3 ? 3 : batch - b0;
-        while (v > 1 && !A->panel->log2_ring[v]) --v;
+        const int v = next_pass(A, batch - b0);
         const int nb = std::min(batch - b0, PanelPlan::bt(v));
-        const int rc = launch_variant(A, v, Xq + (int64_t)b0 * ldx, ldx, nb, acc + (int64_t)b0 * ldy, ldy, stream);
+        const int rc = launch_variant(A, v, x + (int64_t)b0 * ldx, ldx, nb, y + (int64_t)b0 * ldy, ldy, stream);
         if (rc != CSB_OK) return rc;
         b0 += nb;
     }
     return CSB_OK;
+}
+
+int launch_panels(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
+    return launch_passes(A, X, ldx, batch, Y, ldy, stream);
+}
+
+int launch_panels_q16(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch, int64_t* acc, int64_t ldy, void* stream) {
+    return launch_passes(A, Xq, ldx, batch, acc, ldy, stream);
 }
 
 }  // namespace csb

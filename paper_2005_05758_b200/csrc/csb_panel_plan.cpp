@@ -1,5 +1,5 @@
-// Host planner of the panel layout: the device form of a CSB matrix that the batch-1
-// product (SpMV) streams.
+// Host planner of the panel layout: the device form of a CSB matrix that the products with
+// one and with few vectors stream.
 //
 // The paper's CSB-Engine walks the blocks of a matrix in row-major order and hides their
 // uneven sizes with compile-time workload sharing (Sections 4.3.1, 5.2).  Here the output
@@ -16,8 +16,8 @@
 //
 // An item is at most 32 kept rows of one block with all its kept columns.  Its values are the
 // canonical row-major kernel-matrix rows re-tiled so that a lane reads 16 bytes = 8 consecutive
-// kept columns of one kept row: [octet o][row r][8], then the 4-, 2- and 1-column remainders
-// as [r][4], [r][2], [r][1].  No padding inside an item; items are padded to 16 bytes.
+// kept columns of one kept row (fp32 values: 4): [octet o][row r][8], then the 4-, 2- and 1-column
+// remainders as [r][4], [r][2], [r][1].  No padding inside an item; items are padded to 16 bytes.
 //
 // The gathered input of a block (its kept columns of x) is built once per CTA in shared
 // memory, so the multiply loop reads it with vector loads.  A panel's items are laid out
@@ -40,10 +40,10 @@ static inline int log2_ceil(int v) { int l = 0; while ((1 << l) < v) ++l; return
 // How many items of this height share a warp: one with more than 16 rows, two with 9..16, four
 // with 8 or fewer (log2 of that number).
 static inline int panel_item_logg(int mi) { return mi > 16 ? 0 : mi > 8 ? 1 : 2; }
-// Loop steps of an item: its column octets divided among the lane sub-groups of its lane group.
-static inline int panel_item_steps(int mi, int n) {
+// Loop steps of an item: its groups of `unit` columns (16 bytes of a row) divided among the lane sub-groups of its lane group.
+static inline int panel_item_steps(int mi, int n, int unit) {
     const int gw = 32 >> panel_item_logg(mi), S = gw >> log2_ceil(mi);
-    return ((n >> 3) + S - 1) / S;
+    return (n / unit + S - 1) / S;
 }
 // Modelled time of a bundle: a fixed part, and per member its loop steps, remainder columns and
 // joining shuffles.  The shape follows the kernel's instruction counts (110 fixed, 28 per step), but
@@ -53,13 +53,13 @@ static inline int panel_item_steps(int mi, int n) {
 // 8x: 8.3 -> 7.65, 25x: 6.0 -> 5.75 with the fitted ones).  CSB_PANEL_COST_FIXED / _STEP override them.
 static const double kPanelBundleFixed = getenv("CSB_PANEL_COST_FIXED") ? atof(getenv("CSB_PANEL_COST_FIXED")) : 55.0;
 static const double kPanelStep = getenv("CSB_PANEL_COST_STEP") ? atof(getenv("CSB_PANEL_COST_STEP")) : 4.0;
-static double panel_member_cost(int mi, int n) {
+static double panel_member_cost(int mi, int n, int unit) {
     const int gw = 32 >> panel_item_logg(mi), S = gw >> log2_ceil(mi);
-    return kPanelStep * panel_item_steps(mi, n) + ((n & 7) ? 34.0 : 0.0) + 8.0 * log2_ceil(S);
+    return kPanelStep * panel_item_steps(mi, n, unit) + (n % unit ? 34.0 : 0.0) + 8.0 * log2_ceil(S);
 }
 // Cost of an item as seen by the row cut: its share of a bundle.
-static double panel_item_cost(int mi, int n) {
-    return (kPanelBundleFixed + panel_member_cost(mi, n)) / (double)(1 << panel_item_logg(mi)) + 10.0;
+static double panel_item_cost(int mi, int n, int unit) {
+    return (kPanelBundleFixed + panel_member_cost(mi, n, unit)) / (double)(1 << panel_item_logg(mi)) + 10.0;
 }
 
 struct PanelItemSrc {
@@ -73,7 +73,7 @@ struct PanelItemSrc {
 int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, int max_xg_floats, int max_rows,
                      PanelHostPlan* out) {
     *out = PanelHostPlan{};
-    if (A->val_dtype != CSB_F16 && A->val_dtype != CSB_Q16) return 1;   // 16-bit values, moved as they are
+    const int vs = val_size(A->val_dtype), unit = 16 / vs; // columns in 16 bytes
     if (A->block_c > 128 || A->cols > 16384) return 1;
     if (stage_bytes < 8192 || (stage_bytes & (stage_bytes - 1))) return 1;
     const int BR = A->block_r, BC = A->block_c;
@@ -86,7 +86,7 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
         if (m == 0 || n == 0) continue;
         const uint8_t* ri = A->row_idx.data() + A->ridx_off[b];
         for (int r = 0; r < m; ++r) ++rb_begin[(b / A->nbc) * BR + ri[r] + 1];
-        total_bytes += (size_t)m * n * 2;
+        total_bytes += (size_t)m * n * vs;
     }
     for (int64_t r = 0; r < A->rows; ++r) rb_begin[r + 1] += rb_begin[r];
     std::vector<uint32_t> rb(rb_begin[A->rows]);
@@ -112,7 +112,7 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
     for (int n = 1; n <= BC; ++n)
         for (int m = 1; m <= BR; ++m) {
             double c = 0.0;
-            for (int r0 = 0; r0 < m; r0 += 32) c += panel_item_cost(std::min(32, m - r0), n);
+            for (int r0 = 0; r0 < m; r0 += 32) c += panel_item_cost(std::min(32, m - r0), n, unit);
             cost_table[(size_t)n * (BR + 1) + m] = c;
         }
     auto block_cost = [&](int m, int n) { return cost_table[(size_t)n * (BR + 1) + m]; };
@@ -188,8 +188,8 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
                 for (int r0 = ra; r0 < rb; r0 += 32) {
                     PanelItemSrc it{};
                     it.block = b; it.r0 = r0; it.mi = std::min(32, rb - r0);
-                    it.bytes = pad_to((size_t)it.mi * n * 2, 16);
-                    it.cost = panel_item_cost(it.mi, n);
+                    it.bytes = pad_to((size_t)it.mi * n * vs, 16);
+                    it.cost = panel_item_cost(it.mi, n, unit);
                     it.xoff = g.xoff;
                     items.push_back(it);
                 }
@@ -205,7 +205,7 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
             std::vector<uint32_t> cls;
             for (uint32_t i = 0; i < items.size(); ++i) if (panel_item_logg(items[i].mi) == logg) cls.push_back(i);
             std::stable_sort(cls.begin(), cls.end(), [&](uint32_t x, uint32_t y) {
-                return panel_item_steps(items[x].mi, A->n[items[x].block]) > panel_item_steps(items[y].mi, A->n[items[y].block]); });
+                return panel_item_steps(items[x].mi, A->n[items[x].block], unit) > panel_item_steps(items[y].mi, A->n[items[y].block], unit); });
             for (size_t k = 0; k < cls.size(); k += (size_t)1 << logg) {
                 Bundle bu{};
                 bu.logg = logg;
@@ -213,7 +213,7 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
                 for (size_t j = k; j < std::min(cls.size(), k + ((size_t)1 << logg)); ++j) {
                     bu.members.push_back(cls[j]);
                     bu.bytes += items[cls[j]].bytes;
-                    worst = std::max(worst, panel_member_cost(items[cls[j]].mi, A->n[items[cls[j]].block]));
+                    worst = std::max(worst, panel_member_cost(items[cls[j]].mi, A->n[items[cls[j]].block], unit));
                 }
                 bu.cost = kPanelBundleFixed + worst + 10.0 * (double)bu.members.size();
                 bundles.push_back(std::move(bu));
@@ -257,18 +257,19 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
                     d.m = (uint8_t)it.mi; d.logp = (uint8_t)log2_ceil(it.mi);
                     d.n = (uint16_t)n; d.pad = 0;
                     ridx.insert(ridx.end(), ri + it.r0, ri + it.r0 + it.mi);
-                    // values: [octet][row][8], then [row][4], [row][2], [row][1]
-                    const uint8_t* v = A->val.data() + (A->val_off[b] + (uint64_t)it.r0 * n) * 2;
+                    // values: [16 bytes of columns][row], then the remainder by halves: 16-bit [row][4], [row][2], [row][1],
+                    // 32-bit [row][2], [row][1]
+                    const uint8_t* v = A->val.data() + (A->val_off[b] + (uint64_t)it.r0 * n) * vs;
                     const size_t base = values.size();
                     values.resize(base + it.bytes, 0);
                     uint8_t* p = values.data() + base;
-                    const int noct = n >> 3;
-                    for (int o = 0; o < noct; ++o)
-                        for (int r = 0; r < it.mi; ++r, p += 16) std::memcpy(p, v + ((size_t)r * n + 8 * o) * 2, 16);
-                    int kk = noct * 8;
-                    for (int w2 = 4; w2 >= 1; w2 >>= 1)
+                    const int whole = n / unit;
+                    for (int o = 0; o < whole; ++o)
+                        for (int r = 0; r < it.mi; ++r, p += 16) std::memcpy(p, v + (size_t)r * n * vs + 16 * o, 16);
+                    int kk = whole * unit;
+                    for (int w2 = unit / 2; w2 >= 1; w2 >>= 1)
                         if (n & w2) {
-                            for (int r = 0; r < it.mi; ++r, p += 2 * w2) std::memcpy(p, v + ((size_t)r * n + kk) * 2, 2 * w2);
+                            for (int r = 0; r < it.mi; ++r, p += vs * w2) std::memcpy(p, v + ((size_t)r * n + kk) * vs, (size_t)vs * w2);
                             kk += w2;
                         }
                 }
