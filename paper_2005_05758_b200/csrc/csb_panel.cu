@@ -1,4 +1,5 @@
-// Batch-1 CSB product (SpMV) over the panel layout, fp16 values with fp32 accumulation.
+// CSB product with one and with few vectors over the panel layout, fp32 accumulation (and the
+// fixed-point product, csb_fixed.cu).
 //
 // The work of the paper's CSB-Engine (Section 4.3.1: read the kept inputs through ColIdx,
 // multiply by the kernel matrix, accumulate into the outputs through RowIdx, sum along the
@@ -19,9 +20,16 @@
 //     and reads 16 bytes = 8 kept columns per step; lanes left over in a group split the
 //     columns 2-, 4-, ... ways and a few shuffles join them.  Products are accumulated with
 //     packed fp32 multiply-adds;
+//   * with two or four vectors a pass the same walk holds a sum per vector: a weight is read and
+//     converted once, the gathered inputs of the vectors lie side by side;
 //   * every warp adds into its own copy of the CTA's output rows; at the end the CTA adds the
 //     copies in warp order and stores y.  The deal of items to warps is part of the plan, so
 //     the result does not depend on timing.
+//
+// What bounds it: a matrix of a few MB, start-up and the latency of copies, gather and walk one behind
+// the other (3072 x 1536 fp32 at 8x: one vector 3.6 us, four 5.2; the kernel of csb_product.cu 10.3 and 14.9,
+// which walks block by block and joins its CTAs through global memory); a large one, bundles per warp
+// (8192 x 8192 fp16 at 4x: 10.8 us for 33 MB).
 #include <algorithm>
 #include <cstdlib>
 
@@ -377,8 +385,6 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
             const uint2* gath = reinterpret_cast<const uint2*>(meta + H->gather_off);
             const uint8_t* cidx = meta + H->cidx_off;
             const int n_gather = (int)H->n_gather;
-            const float* xrow = a.staged ? xs : reinterpret_cast<const float*>(a.x);
-            const long long xpitch = a.staged ? (long long)(L.xs_row >> 2) : a.ldx;
             for (int g0 = warp * 4; g0 < n_gather; g0 += W * 4) {
                 const int g = g0 + (lane >> 3);
                 const uint2 gd = g < n_gather ? gath[g] : make_uint2(0u, 0u);
@@ -403,16 +409,19 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
                         }
                         continue;
                     }
-                    const float* xr = xrow + xbase;
                     float4* dst = reinterpret_cast<float4*>(xg) + (size_t)((xoff + k) >> 2) * BT;
+                    auto pick = [&](const float* xr, long long pitch) {
 #pragma unroll
-                    for (int b = 0; b < BT; ++b) {
-                        // (a column past nb stays 0)
-                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (b < a.nb) v = make_float4(xr[c4 & 0xffu], xr[(c4 >> 8) & 0xffu], xr[(c4 >> 16) & 0xffu], xr[c4 >> 24]);
-                        dst[b] = v;
-                        xr += xpitch;
-                    }
+                        for (int b = 0; b < BT; ++b) {
+                            // (a column past nb stays 0)
+                            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (BT == 1 || b < a.nb) v = make_float4(xr[c4 & 0xffu], xr[(c4 >> 8) & 0xffu], xr[(c4 >> 16) & 0xffu], xr[c4 >> 24]);
+                            dst[b] = v;
+                            xr += pitch;
+                        }
+                    };
+                    if (BT == 1 || a.staged) pick(xs + xbase, (long long)(L.xs_row >> 2));
+                    else pick(reinterpret_cast<const float*>(a.x) + xbase, a.ldx);
                 }
             }
         }
@@ -585,7 +594,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
         }
         return;
     }
-    for (int t = threadIdx.x; t < n_rows * a.nb; t += blockDim.x) {
+    for (int t = threadIdx.x; t < n_rows * (BT == 1 ? 1 : a.nb); t += blockDim.x) {
         const int b = BT == 1 ? 0 : t / n_rows, r = t - b * n_rows;
         float v = 0.f;
         for (int w = 0; w < W; ++w) v += zs_all[((size_t)w * a.max_rows + r) * BT + b];

@@ -99,7 +99,10 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
             for (int r = 0; r < m; ++r) rb[fill[(b / A->nbc) * BR + ri[r]]++] = (uint32_t)b;
         }
     }
-    int n_ctas = (int)std::min<int64_t>(ctas, std::max<int64_t>(1, (int64_t)total_bytes / 8192));
+    // 2 KB of values and more per CTA: a CTA's start-up and gather cost the same whatever it holds, so small matrices
+    // gain from CTAs until there is next to nothing in one (600 x 300 fp16 at 10x: 4.9 us on the 4 CTAs that 8 KB
+    // each gave, 3.2 here, with four vectors 8.5 and 4.7; 1 KB each differs by less than the runs do)
+    int n_ctas = (int)std::min<int64_t>(ctas, std::max<int64_t>(1, (int64_t)total_bytes / 2048));
     n_ctas = (int)std::min<int64_t>(std::min<int64_t>(n_ctas, (int64_t)kMaxPanelCtas), A->rows);
 
     // ---- one contiguous row range per CTA.  The cost of a range is the cost of its items, and an

@@ -98,7 +98,7 @@ void emit_warp(const Source& s, int cell, int op, int lu, int u0, int n, int BT,
                     const uint8_t* val = nullptr;
                     if (!v.empty()) {
                         size_t best = v.size() - 1;
-                        for (size_t q = v.size(); q-- > 0;) { const int u = used[v[q].col % banks]; if (u < 0 || u == v[q].col) { best = q; break; } }
+                        for (size_t q = v.size(), end = q > 24 ? q - 24 : 0; q-- > end;) { const int u = used[v[q].col % banks]; if (u < 0 || u == v[q].col) { best = q; break; } }
                         col = v[best].col; val = v[best].v;
                         v[best] = v.back();
                         v.pop_back();
@@ -192,7 +192,7 @@ int plan_unit_host(int cell, int L, const csb_matrix* const* W, const csb_matrix
     {
         const unsigned hw = std::thread::hardware_concurrency();
         std::vector<std::thread> pool;
-        try { for (unsigned t = 1; t < std::min<unsigned>(hw ? hw : 1, 8) && t < jobs.size() / 4; ++t) pool.emplace_back(work); } catch (const std::system_error&) {}
+        try { for (unsigned t = 1; t < std::min<unsigned>(hw ? hw : 1, 16) && t < jobs.size() / 4; ++t) pool.emplace_back(work); } catch (const std::system_error&) {}
         work();
         for (auto& t : pool) t.join();
     }

@@ -171,3 +171,15 @@ def test_cfg4_full_size_every_rate_and_batch(rate, spmv_path):
               % (rate, B, float(np.max(np.abs(outs[0] - want[:B])[big] / np.abs(want[:B])[big])), int(big.sum())))
     assert A.info()["balance"] > 0.5
     A.free()
+
+
+@pytest.mark.parametrize("vd", ["f16", "f32"])
+@pytest.mark.parametrize("shape", [(37, 23, 8, 8), (300, 1179, 32, 16), (130, 512, 64, 128), (96, 9000, 32, 64)])
+def test_few_vectors(shape, vd):
+    # every count of vectors that the panel kernel takes, in passes of four, two and one: column counts that leave each
+    # remainder of 16 bytes, inputs that are no multiple of 16 bytes, and more columns than four staged vectors fit
+    R, C, br, bc = shape
+    mat = workloads.make_matrix(41, R, C, br, bc, "uniform", lo=0.1, hi=1.0, w_std=0.1, val_dtype=vd)
+    X = np.random.default_rng(5).standard_normal((9, C)).astype(np.float32)
+    for B in range(1, 10):
+        run_case(mat, X[:B])
