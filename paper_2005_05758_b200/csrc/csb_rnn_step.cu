@@ -148,11 +148,46 @@ __global__ void csb_gru_gates_kernel(const float* __restrict__ Z, const float* _
 }
 
 // ---- the packed path (device functions in csb_gates.cuh) ----------------------------------------------
-// src [nb, ncols] (row stride ld) -> slots slot0 .. of the packed rows 0 .. ncols - 1 of xp; 32 columns per block.
-__global__ void csb_pack_rows_kernel(const float* __restrict__ src, long long ld, int nb, int ncols, uint8_t* __restrict__ xp, int pitch,
-                                     int cap, int slot0) {
+// Everything a sequence starts from, in one launch: the packed inputs of every layer, x_0 and h0 in
+// them and the rest zero, and the running states.  A block takes 32 columns of a layer, the input
+// columns first.  As separate clears, copies and packs it was half of the launches of a call of one
+// step (two layers with states: 15, with the copies of the final states; 7 now, 41 us for 16 sequences
+// on 2 x 900 units).
+struct BeginArgs {
+    const float* x; const float* h0; const float* c0;   // h0, c0: null = zeros; may be hs, c themselves
+    float* hs; float* c;                                 // [L, B, H]; c null: no cell state
+    uint8_t* xp[kMaxLayers];
+    int in_size[kMaxLayers], end[kMaxLayers];            // end: first block behind the layer
+    int pitch, cap, B, H, slot_h;                        // slot_h: first batch slot of the recurrent columns' inputs
+};
+__global__ void __launch_bounds__(256) csb_begin_kernel(const __grid_constant__ BeginArgs a) {
     __shared__ float tile[32][33];
-    pack_columns(tile, src, ld, nb, ncols, (int)blockIdx.x * 32, xp, pitch, cap, slot0);
+    pdl_launch_dependents();
+    int l = 0, first = 0;
+    while ((int)blockIdx.x >= a.end[l]) first = a.end[l++];
+    const int in_blocks = (a.in_size[l] + 31) / 32, blk = (int)blockIdx.x - first;
+    const bool rec = blk >= in_blocks;
+    const int n = rec ? a.H : a.in_size[l], c0 = (rec ? blk - in_blocks : blk) * 32;
+    uint8_t* xp = a.xp[l] + (rec ? (size_t)a.in_size[l] * a.pitch : 0);
+    uint4* rows = reinterpret_cast<uint4*>(xp + (size_t)c0 * a.pitch);
+    for (int i = threadIdx.x; i < min(32, n - c0) * a.pitch / 16; i += blockDim.x) rows[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    if (rec) {
+        const int tx = threadIdx.x & 31;
+        const size_t at = (size_t)l * a.B * a.H + c0 + tx;
+        for (int b = threadIdx.x >> 5; b < a.B; b += blockDim.x >> 5) {
+            const size_t e = at + (size_t)b * a.H;
+            const bool in = c0 + tx < n;
+            const float h = in && a.h0 ? a.h0[e] : 0.f;
+            tile[b][tx] = h;
+            if (in) a.hs[e] = h;
+            if (in && a.c) a.c[e] = a.c0 ? a.c0[e] : 0.f;
+        }
+        __syncthreads();
+        if (a.h0) pack_tile(tile, min(32, n - c0), a.B, reinterpret_cast<uint8_t*>(rows), a.pitch, a.cap, a.slot_h, nullptr, 0);
+    } else if (l == 0) {
+        pack_columns(tile, a.x, (long long)n, a.B, n, c0, xp, a.pitch, a.cap, 0);
+    }
 }
 
 // The gates of one tick: blocks [part, next part) take a layer's hidden units, 32 at a time and 8 batch
@@ -263,20 +298,29 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     if (P->pitch) {
         // ---- packed path: the gate kernels feed the products' packed inputs directly
         const int pitch = P->pitch, cap = P->cap;
-        if (h0) CSB_CUDA(cudaMemcpyAsync(P->d_h, h0, ns * 4, in_kind, st));
-        else CSB_CUDA(cudaMemsetAsync(P->d_h, 0, ns * 4, st));
+        // The states run in the caller's final-state arrays where nothing else lies there, else in the plan's
+        auto apart = [](const float* p, size_t n, const float* q, size_t m) { return !p || !q || p + n <= q || q + m <= p; };
+        const size_t nx1 = (size_t)T * B * I0;
+        const bool direct = !host_io && apart(hT, ns, cT, ns);
+        const bool own_h = !(direct && hT && apart(hT, ns, x, nx1) && apart(hT, ns, y, ny) && apart(hT, ns, c0, ns) && (h0 == hT || apart(hT, ns, h0, ns)));
+        const bool own_c = !(direct && cT && apart(cT, ns, x, nx1) && apart(cT, ns, y, ny) && apart(cT, ns, h0, ns) && (c0 == cT || apart(cT, ns, c0, ns)));
+        float* hs = own_h ? P->d_h : hT;
+        float* cs = gru ? nullptr : own_c ? P->d_c : cT;
+        BeginArgs ba{};
+        ba.x = dx; ba.h0 = h0; ba.c0 = c0; ba.hs = hs; ba.c = cs;
+        if (host_io) {
+            if (h0) { CSB_CUDA(cudaMemcpyAsync(hs, h0, ns * 4, in_kind, st)); ba.h0 = hs; }
+            if (c0 && cs) { CSB_CUDA(cudaMemcpyAsync(cs, c0, ns * 4, in_kind, st)); ba.c0 = cs; }
+        }
+        ba.pitch = pitch; ba.cap = cap; ba.B = B; ba.H = H; ba.slot_h = gru ? B : 0;
+        int begin_blocks = 0;
         for (int l = 0; l < L; ++l) {
-            CSB_CUDA(cudaMemsetAsync(P->d_xp[l], 0, (size_t)(in_size[l] + H) * pitch, st));
-            if (h0)
-                csb_pack_rows_kernel<<<(H + 31) / 32, 256, 0, st>>>(P->d_h + (size_t)l * B * H, (long long)H, B, H,
-                                                                   P->d_xp[l] + (size_t)in_size[l] * pitch, pitch, cap, gru ? B : 0);
+            ba.xp[l] = P->d_xp[l]; ba.in_size[l] = in_size[l];
+            begin_blocks += (in_size[l] + 31) / 32 + (H + 31) / 32;
+            ba.end[l] = begin_blocks;
         }
-        csb_pack_rows_kernel<<<(I0 + 31) / 32, 256, 0, st>>>(dx, (long long)I0, B, I0, P->d_xp[0], pitch, cap, 0);
+        csb_begin_kernel<<<begin_blocks, 256, 0, st>>>(ba);
         CSB_CUDA(cudaGetLastError());
-        if (!gru) {
-            if (c0) CSB_CUDA(cudaMemcpyAsync(P->d_c, c0, ns * 4, in_kind, st));
-            else CSB_CUDA(cudaMemsetAsync(P->d_c, 0, ns * 4, st));
-        }
         const int h_tiles = (H + 31) / 32, b_tiles = (B + 7) / 8, x_blocks = (I0 + 31) / 32;
         float* Z[kMaxLayers];
         for (int l = 0; l < L; ++l) Z[l] = P->d_z + (size_t)l * vrows * gates * H;
@@ -291,7 +335,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             for (int l = l0; l < l1; ++l) {
                 GatePart& g = a.part[l - l0];
                 const int64_t t = k - l;
-                g.Z = Z[l]; g.bias = bias ? bias[l] : nullptr; g.c = gru ? nullptr : P->d_c + (size_t)l * B * H; g.hs = P->d_h + (size_t)l * B * H;
+                g.Z = Z[l]; g.bias = bias ? bias[l] : nullptr; g.c = gru ? nullptr : cs + (size_t)l * B * H; g.hs = hs + (size_t)l * B * H;
                 g.xp_self = P->d_xp[l] + (size_t)in_size[l] * pitch; g.xp_next = l + 1 < L ? P->d_xp[l + 1] : nullptr;
                 g.y = (l == L - 1 && dy) ? dy + (size_t)t * B * H : nullptr;
                 blocks += h_tiles * b_tiles;
@@ -307,8 +351,8 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             CSB_CUDA(cudaLaunchKernelEx(&cfg, gru ? csb_gates_pack_kernel<3> : csb_gates_pack_kernel<4>, a));
             CSB_CUDA(cudaGetLastError());
         }
-        if (hT) CSB_CUDA(cudaMemcpyAsync(hT, P->d_h, ns * 4, out_kind, st));
-        if (cT && !gru) CSB_CUDA(cudaMemcpyAsync(cT, P->d_c, ns * 4, out_kind, st));
+        if (hT && own_h) CSB_CUDA(cudaMemcpyAsync(hT, hs, ns * 4, out_kind, st));
+        if (cT && !gru && own_c) CSB_CUDA(cudaMemcpyAsync(cT, cs, ns * 4, out_kind, st));
         if (host_io && y) CSB_CUDA(cudaMemcpyAsync(y, dy, ny * 4, cudaMemcpyDeviceToHost, st));
         if (host_io || !(flags & CSB_FLAG_ASYNC)) {
             CSB_CUDA(cudaStreamSynchronize(st));

@@ -282,3 +282,30 @@ def test_barrier_gives_up_and_context_survives():
     want, _, _ = R.lstm_forward(layers_of(w), w.bias, w.x)
     close(y.cpu().numpy(), want, "f16", "y after timeout")
     A.free()
+
+
+@pytest.mark.parametrize("cell,B,T", [("lstm", 16, 1), ("lstm", 11, 3), ("gru", 16, 1), ("gru", 9, 3)])
+@pytest.mark.parametrize("places", ["own", "in place", "crossed", "none"])
+def test_step_by_step_state_arrays(cell, B, T, places):
+    # the running states live in the caller's final-state arrays when those are apart from what is still read: given
+    # once more as initial states, exchanged with them, or missing, the outputs have to be the same bit for bit
+    L, H = 2, 512
+    w = workloads.make_rnn_workload(17, cell, 70, H, L, 32, 32, "uniform", lo=0.2, hi=0.9, T=T, B=B, w_std=0.05, bias_std=0.1, state_std=0.5)
+    want_y, want_h, want_c = check(w)
+    mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in w.layers]
+    bias = [torch.from_numpy(b).cuda() for b in w.bias]
+    x, y = torch.from_numpy(w.x).cuda(), torch.empty((T, B, H), device="cuda")
+    h = torch.from_numpy(w.h0).cuda()
+    c = torch.from_numpy(w.c0).cuda() if cell == "lstm" else None
+    hT, cT = {"own": (torch.empty_like(h), torch.empty_like(h)), "in place": (h, c), "crossed": (c, h), "none": (None, None)}[places]
+    if cell == "lstm":
+        binding.csb_lstm_forward(mats, bias, x, h, c, y, hT, cT, 0)
+    else:
+        hT = hT if places != "crossed" else h
+        binding.csb_gru_forward(mats, bias, x, h, y, hT, 0)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), want_y)
+    assert hT is None or np.array_equal(hT.cpu().numpy(), want_h)
+    assert cell == "gru" or cT is None or np.array_equal(cT.cpu().numpy(), want_c)
+    for m in mats:
+        m.free()
