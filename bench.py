@@ -349,7 +349,7 @@ def spmv_sweep(binding, torch, dev, rates, batch, l2, reps=10, with_cpu=False, c
         m = w.matrix
         A0 = binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, dev)
         info = A0.info()
-        panel = batch == 1 and info["panel_ctas"] > 0      # which kernel serves this batch size
+        panel = batch == 1 and info["panel_ctas"] > 0      # the batches of this sweep: 1, and 8 and more on tensor cores
         stream_bytes = info["panel_stream_bytes"] if panel else info["device_stream_bytes"]
         ncopy = max(2, int(160e6 // max(info["algorithmic_bytes"], 1)) + 1)
         As = [A0] + [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, dev)
@@ -453,6 +453,8 @@ def job_us_per_timestep(ms_slowest, seq_len, world):
 def stepwise(w, nnz):
     """Whether the library runs this workload step by step on tensor cores (its own rule, restated)."""
     rows = 2 * w.B if w.cell == "gru" else w.B
+    if w.B <= 8:                                               # the resident loops: every layer of these fits in shared memory
+        return False
     return (w.B >= 16 or (w.B >= 8 and nnz >= 100000)) and rows >= 8 and w.layers[0].val_dtype == "f16"
 
 
@@ -503,7 +505,10 @@ def config_entry(binding, torch, dev, flush, w, steps, hbm, l2, sm_mhz, with_cpu
          "GFLOPs": round(2 * nnz * w.B / us / 1e3, 1),
          "path": "per-step launches, products on tensor cores" if sw else "persistent time-loop kernel",
          "bound": "l2" if sw else "smem", "roofline": three_rooflines(alg, us, hbm, l2, sm_mhz)}
-    launches = (steps + 4) * (1 if not sw else w.T * len(w.layers) * 3)
+    # step by step: one to begin, then a product and a gate kernel per tick of the wavefront; beyond 32 product rows
+    # a pack, a product and a gate kernel per layer and step
+    wave = w.B * (2 if w.cell == "gru" else 1) <= 32
+    launches = (steps + 4) * (1 if not sw else 1 + 2 * (w.T + len(w.layers) - 1) if wave else w.T * len(w.layers) * 3)
     if with_cpu:
         ts, tl = t_sample
         o_us, err = oracle_sample(w, y, ts, tl)
@@ -551,10 +556,9 @@ def cells_bench(binding, torch, dev, flush, hbm, l2, sm_mhz, with_cpu):
         us = float(np.median(ms)) * 1e3 / w.T
         infos = [m.info() for m in mats + proj]
         alg = sum(i["algorithmic_bytes"] for i in infos) + sum((m.cols + m.rows) * 4 for m in w.layers + (w.proj or []))
-        per_step_launches = {"lstmp": 4, "ligru": 2, "gru_rb": 4}[cell] * kw["L"]
-        launches += 14 * w.T * per_step_launches
+        launches += 14                                     # one launch per call
         e = {"us_per_timestep": round(us, 3), "T": w.T, "B": 1, "layers": kw["L"], "nnz": sum(i["nnz"] for i in infos),
-             "algorithmic_bytes_per_step": alg, "launches_per_step": per_step_launches, "bound": "latency of %d dependent launches per step" % per_step_launches,
+             "algorithmic_bytes_per_step": alg, "launches_per_call": 1, "bound": "latency of the exchange between CTAs",
              "roofline": three_rooflines(alg, us, hbm, l2, sm_mhz), "paper_context": ctx}
         if with_cpu:
             lay = layer_tuples(w)
@@ -686,7 +690,7 @@ def main():
         line["l2_read_GBps_measured"] = round(l2, 1)
     alg_step = rnn_alg_bytes_per_step(w, infos)
     three = three_rooflines(alg_step, mean_ms * 1e3 / w.T, hbm, l2, sm_mhz)
-    line["roofline"] = {"kernel": "csb_rnn_kernel<half,1>", "bound": "smem", "achieved": three["GBps"],
+    line["roofline"] = {"kernel": "csb_rnn1_kernel<half,lstm,1>", "bound": "smem", "achieved": three["GBps"],
                         "peak": three["smem_peak_GBps_derived"], "peak_kind": "derived: 148 SMs x 128 B/clk x sampled SM clock",
                         "unit": "GB/s", "frac": three["frac_smem_derived"],
                         "frac_l2_measured": three["frac_l2_measured"], "frac_hbm_equivalent": three["frac_hbm_equivalent"],

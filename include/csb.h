@@ -92,7 +92,7 @@ typedef struct csb_info {
     int64_t device_stream_bytes; /* bytes of the private device layout actually streamed    */
     int32_t plan_ctas, plan_warps;
     double balance;              /* mean / max of the per-warp scheduled cost (1 = perfect) */
-    /* the panel layout that csb_spmv streams for fp16 matrices (all zero when it does not apply) */
+    /* the panel layout that csb_spmv streams (all zero when it does not apply) */
     int64_t panel_stream_bytes;  /* bytes of all panels (bookkeeping + values)              */
     int32_t panel_ctas, panel_warps;
     double panel_balance;        /* mean / max of the per-CTA modelled cost                 */
@@ -158,7 +158,7 @@ void csb_free(csb_matrix_t* A);
  *   become exactly 0).  fp32 accumulation, fixed summation order (bit-reproducible).
  * Asynchronous on `stream`.  Calls on the same handle must not overlap on the GPU: they share
  * the handle's scratch for partial block-row sums.
- * Matrices with fp16 values (block_c <= 128, cols <= 16384) run the panel kernel: every CTA owns
+ * Matrices with block_c <= 128 and cols <= 16384 run the panel kernel: every CTA owns
  * a range of output rows, so it needs no scratch.  That kernel is launched with programmatic
  * stream serialization: its start-up overlaps the end of the work in front of it on `stream`,
  * and it waits for that work before it reads x or writes y (CSB_PANEL_PDL=0 in the environment,
@@ -237,11 +237,13 @@ int csb_spmv_static_scratch(const csb_matrix_t* A, const float* x, float* y, voi
  * not overlap on the GPU.  Calls queued on one stream are safe; calls on different streams need an
  * event (or a synchronisation) between them, and then give identical bits.  The handles
  * themselves are immutable and may be used from any stream.
- * With B >= 16 (B >= 8 when the layers hold 100000 weights or more), fp16 values and block_r <= 64
- * the sequence is not run by the persistent kernel
- * but step by step: per layer and step the batched product on tensor cores (as csb_spmm, same
- * input-range rule) and one kernel with the gate arithmetic; same results within rounding, same
- * arguments and flags (CSB_RNN_NO_STEPWISE=1 in the environment keeps the persistent kernel).
+ * Up to B = 8 the weights stay in shared memory and one launch runs the sequence, where the layers fit
+ * there.  With B >= 16 (B >= 8 when they do not fit and hold 100000 weights or more, or B >= 9 then),
+ * fp16 values and block_r <= 64 the sequence runs step by step: per step of the stack one batched product
+ * on tensor cores (as csb_spmm, same input-range rule; the layers as a wavefront, each a step behind
+ * the one below) and one kernel with the gate arithmetic; same results within rounding, same
+ * arguments and flags (CSB_RNN_NO_STEPWISE=1 in the environment asks for the persistent kernel that
+ * serves the rest).  There the running states are kept in hT and cT when those are given.
  * Errors: SHAPE (rows != 4H, cols != I_l + H, layers disagree), LAUNCH (grid cannot be
  * co-resident; nothing was launched), TIMEOUT (the bounded grid barrier gave up; outputs are
  * undefined, the context stays usable), CUDA.
@@ -292,7 +294,8 @@ int csb_spmm_q16(const csb_matrix_t* A, const int16_t* Xq, int64_t ldx, int batc
 
 /*
  * Cell variants of the paper's benchmark models (Table 1) and of the GRU reference of Section 2.1.
- * They run one timestep at a time: per layer and step the CSB products go through the kernels of
+ * Up to B = 8, where the layers fit in shared memory, one launch runs the sequence as for the LSTM; else
+ * they run one timestep at a time: per layer and step the CSB products go through the kernels of
  * csb_spmv / csb_spmm (whichever serves the batch size) and small kernels do the element-wise
  * part.  Arguments, flags (CSB_FLAG_ASYNC, CSB_FLAG_HOST_IO), caching of per-(matrices, B) device
  * state on the first call and the no-overlap rule are those of csb_lstm_forward; T = 0 or B = 0

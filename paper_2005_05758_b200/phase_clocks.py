@@ -2,12 +2,11 @@
 
     python -m paper_2005_05758_b200.phase_clocks rnn   [cfg1 cfg2 cfg3 cfg5]
     python -m paper_2005_05758_b200.phase_clocks panel [4 8 16 25]
-    python -m paper_2005_05758_b200.phase_clocks loop  [cfgN:batch ...]      (default cfg5:32 cfg3:8: the one-launch time loop at batch)
     python -m paper_2005_05758_b200.phase_clocks spmm  [rate:batch | cfgN:batch ...]   (default 4:8 4:32 25:8; cfgN = first layer of that config)
 
 Builds libcsb_clocks.so beside the normal library with -DCSB_PHASE_CLOCKS -DCSB_PANEL_CLOCKS (see
 build.py), loads it instead of libcsb.so and prints
-  rnn:   cycles per timestep and phase of csb_rnn_kernel, summed by thread 0 of every CTA
+  rnn:   cycles per timestep and phase of the resident time loop, summed by thread 0 of every CTA
          (mean / min / max over the CTAs);
   panel: wall-clock stamps of csb_panel_kernel per CTA, in microseconds from the earliest CTA start;
   spmm:  cycles per phase of csb_spmm_tile_kernel, summed per warp (mean / max over the warps, and the
