@@ -736,7 +736,11 @@ int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch,
     CSB_CUDA(cudaGetDevice(&prev));
     if (prev != A->device) CSB_CUDA(cudaSetDevice(A->device));
     struct Restore { int prev, cur; ~Restore() { if (prev != cur) cudaSetDevice(prev); } } restore{prev, A->device};
-    int ci = spmm_class_index(batch);
+    // Eight columns run in tiles of 16: half as many warps with twice the columns meet at half as many hand-overs, and
+    // the columns of zeros cost less than that (8 x 32-warp tiles against these, us: 3072 x 1536 at 8x 13.0 / 10.5, 4096 x
+    // 4096 of 32 x 32 blocks at 5x 24.0 / 15.5, 8192 x 8192 at 4x 28.2 / 27.5; the one that lost, 4096 x 4096 of
+    // 64 x 64 blocks at 5x, 13.7 / 14.1).  The recurrent stacks keep tiles of 8, their plans share a grid.
+    int ci = std::max(1, spmm_class_index(batch));
     const int sms = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
     {
         std::lock_guard<std::mutex> lk(A->mma_mu);
@@ -744,7 +748,11 @@ int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch,
         // more than 32 columns: tiles of 64, so that row maps, weights and bookkeeping are paid once for all of
         // them (8192 x 8192 at 4x, batch 64: 74.9 -> 59.3 us); where that plan does not fit, passes of 32
         if (batch > 32 && make_spmm_plan(A, 3, sms, 0, true, &A->mma->cls[3]) == CSB_OK) ci = 3;
-        else if ((rc = make_spmm_plan(A, ci, sms, 0, true, &A->mma->cls[ci])) != CSB_OK) return rc;
+        else {
+            rc = make_spmm_plan(A, ci, sms, 0, true, &A->mma->cls[ci]);
+            if (rc == 1 && batch <= 8) rc = make_spmm_plan(A, ci = 0, sms, 0, true, &A->mma->cls[0]);   // takes less shared memory
+            if (rc != CSB_OK) return rc;
+        }
     }
     return pack_and_launch(A, &A->mma->cls[ci], 1 << ci, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
 }

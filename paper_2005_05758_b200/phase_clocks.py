@@ -129,7 +129,7 @@ def spmm(cases):
         ck = np.zeros((1 << 16, 16), np.int64)
         n = binding.lib.csb_debug_spmm_clocks(C.c_void_p(ck.ctypes.data), 1 << 16)
         ck = ck[:n].astype(np.float64)
-        wpc = 32 if int(B) <= 8 else 16 if int(B) <= 32 else 8
+        wpc = 16 if int(B) <= 32 else 8
         per_cta = ck.reshape(-1, wpc, 16)
         slow = per_cta[np.argmax(per_cta.sum(axis=2).max(axis=1))]
         last = ck[np.argmax(ck[:, :6].sum(axis=1))]      # the warp that reaches the end of its items last
