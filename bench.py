@@ -695,7 +695,7 @@ def main():
                         "unit": "GB/s", "frac": three["frac_smem_derived"],
                         "frac_l2_measured": three["frac_l2_measured"], "frac_hbm_equivalent": three["frac_hbm_equivalent"],
                         "hbm_peak": hbm, "hbm_peak_kind": peak_kind,
-                        "traffic": counters.get("csb_rnn_kernel cfg5 T=512 B=1") if (w.T == 512 and world == 1) else None,
+                        "traffic": counters.get("csb_rnn1_kernel cfg5 T=512 B=1") if (w.T == 512 and world == 1) else None,
                         "algorithmic_bytes_per_launch": alg_step * w.T,
                         "note": "the compressed weights are read from HBM once per call and then stay in shared memory, so the "
                                 "stream of a timestep is bounded by the shared-memory read rate (derived peak), not by DRAM (traffic "
