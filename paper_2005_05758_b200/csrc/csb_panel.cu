@@ -300,7 +300,9 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
     constexpr uint32_t kXBytes = kQ ? 2u : 4u;
     extern __shared__ __align__(128) uint8_t smem[];
     const int W = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const PanelSmem L(kQ, a.staged != 0, BT, W, a.log2_stage, a.log2_slots, a.cols, a.max_xg, a.max_rows, a.max_meta);
+    const bool staged = BT == 1 || a.staged != 0;          // one vector always is
+    const int nb = BT == 1 ? 1 : a.nb;
+    const PanelSmem L(kQ, staged, BT, W, a.log2_stage, a.log2_slots, a.cols, a.max_xg, a.max_rows, a.max_meta);
     const uint4 ct = a.cta[blockIdx.x];
     const uint8_t* panel = a.panels + (size_t)ct.x * 16;
     const uint32_t meta_bytes = ct.y, value_bytes = ct.z;
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
     volatile uint32_t* issued = reinterpret_cast<volatile uint32_t*>(smem + L.issued);
     volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(smem + L.dead);
 
-    const bool x_bulk = a.staged && (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols * kXBytes & 15) == 0 && (a.nb == 1 || (a.ldx * kXBytes & 15) == 0);
+    const bool x_bulk = staged && (reinterpret_cast<uintptr_t>(a.x) & 15) == 0 && (a.cols * kXBytes & 15) == 0 && (nb == 1 || (a.ldx * kXBytes & 15) == 0);
     // Launched with programmatic stream serialization, this grid may start while the kernel in
     // front of it on the stream is still draining: whatever comes next may be scheduled as early
     // as the hardware likes, and this grid touches x and y only behind grid_dependency_wait().
@@ -344,8 +346,8 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
         if (s == slots + 1u && x_bulk) {
             grid_dependency_wait();
             const uint32_t xb = (uint32_t)a.cols * kXBytes;
-            mbar_expect_tx(xbar, xb * (uint32_t)a.nb);
-            for (int b = 0; b < a.nb; ++b)
+            mbar_expect_tx(xbar, xb * (uint32_t)nb);
+            for (int b = 0; b < nb; ++b)
                 for (uint32_t off = 0; off < xb; off += 16384u)
                     bulk_g2s(smem + L.xs + b * L.xs_row + off, reinterpret_cast<const uint8_t*>(a.x) + (size_t)b * a.ldx * kXBytes + off, min(16384u, xb - off), xbar);
         }
@@ -360,7 +362,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
     for (int i = threadIdx.x; i < (kQ ? 2 : W) * BT * a.max_rows; i += blockDim.x) zs_all[i] = 0.f;
     if (!x_bulk) {
         grid_dependency_wait();
-        for (int b = 0; b < (a.staged ? a.nb : 0); ++b)
+        for (int b = 0; b < (staged ? nb : 0); ++b)
             for (int i = threadIdx.x; i < a.cols; i += blockDim.x) {
                 if (kQ) reinterpret_cast<int16_t*>(smem + L.xs + b * L.xs_row)[i] = __ldg(reinterpret_cast<const int16_t*>(a.x) + (long long)b * a.ldx + i);
                 else reinterpret_cast<float*>(smem + L.xs + b * L.xs_row)[i] = __ldg(reinterpret_cast<const float*>(a.x) + (long long)b * a.ldx + i);
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
                         for (int b = 0; b < BT; ++b) {
                             // two inputs to a word, then the bytes sorted into high and low ones; a column past nb stays 0
                             uint2 h = make_uint2(0u, 0u);
-                            if (b < a.nb) {
+                            if (b < nb) {
                                 const uint32_t v0 = (uint16_t)xr[c4 & 0xffu], v1 = (uint16_t)xr[(c4 >> 8) & 0xffu];
                                 const uint32_t v2 = (uint16_t)xr[(c4 >> 16) & 0xffu], v3 = (uint16_t)xr[c4 >> 24];
                                 const uint32_t p0 = v0 | (v1 << 16), p1 = v2 | (v3 << 16);
@@ -415,12 +417,12 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
                         for (int b = 0; b < BT; ++b) {
                             // (a column past nb stays 0)
                             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (BT == 1 || b < a.nb) v = make_float4(xr[c4 & 0xffu], xr[(c4 >> 8) & 0xffu], xr[(c4 >> 16) & 0xffu], xr[c4 >> 24]);
+                            if (b < nb) v = make_float4(xr[c4 & 0xffu], xr[(c4 >> 8) & 0xffu], xr[(c4 >> 16) & 0xffu], xr[c4 >> 24]);
                             dst[b] = v;
                             xr += pitch;
                         }
                     };
-                    if (BT == 1 || a.staged) pick(xs + xbase, (long long)(L.xs_row >> 2));
+                    if (staged) pick(xs + xbase, (long long)(L.xs_row >> 2));
                     else pick(reinterpret_cast<const float*>(a.x) + xbase, a.ldx);
                 }
             }
@@ -588,13 +590,13 @@ __global__ void __launch_bounds__(1024, 1) csb_panel_kernel(const __grid_constan
     // ---- add the warps' copies in warp order and store the CTA's rows
     const int n_rows = (int)H->n_rows, row0 = (int)H->row0;
     if (kQ) {
-        for (int t = threadIdx.x; t < n_rows * a.nb; t += blockDim.x) {
+        for (int t = threadIdx.x; t < n_rows * nb; t += blockDim.x) {
             const int b = t / n_rows, r = t - b * n_rows;
             reinterpret_cast<long long*>(a.y)[(long long)b * a.ldy + row0 + r] = reinterpret_cast<const long long*>(zs_all)[r * BT + b];
         }
         return;
     }
-    for (int t = threadIdx.x; t < n_rows * (BT == 1 ? 1 : a.nb); t += blockDim.x) {
+    for (int t = threadIdx.x; t < n_rows * nb; t += blockDim.x) {
         const int b = BT == 1 ? 0 : t / n_rows, r = t - b * n_rows;
         float v = 0.f;
         for (int w = 0; w < W; ++w) v += zs_all[((size_t)w * a.max_rows + r) * BT + b];
