@@ -230,6 +230,8 @@ int csb_spmv_static_scratch(const csb_matrix_t* A, const float* x, float* y, voi
  *   flags    CSB_FLAG_ASYNC: return without waiting (the status word is then not checked).
  *            CSB_FLAG_HOST_IO: x, h0, c0, y, hT, cT are HOST pointers; the call copies them
  *            through device staging buffers on `stream` and waits for the result.
+ * hT and cT may lie where h0, c0 or x lie (a state that is carried on in place), in y or in each other's place
+ * (hT then counts over y, cT over hT); y may lie where h0 and c0 lie.  y must not overlap x.
  * The first call for a given (W..., B) builds and caches the time-loop schedule and its
  * device state (allocates, synchronises); later calls reuse it.  T = 0 or B = 0 is a no-op.
  * That cached state (the ring of h slots, the barrier and status words, staging buffers) is one

@@ -40,7 +40,9 @@ struct Rnn1Plan {
     const void* kernel = nullptr;
     std::vector<void*> owned;                  // device memory
     uint32_t* h_status = nullptr;
-    float* d_stage = nullptr; size_t stage_cap = 0;      // host I/O
+    float* d_stage = nullptr; size_t stage_cap = 0;      // x and y of calls with host arrays
+    float* d_x = nullptr; size_t x_cap = 0;              // x of calls that write over it
+    float* d_states = nullptr;                 // [h0, c0, hT, cT] of calls with host arrays or with states in each other's places
     ~Rnn1Plan() {
         for (void* p : owned) cudaFree(p);
         cudaFree(d_stage);
@@ -86,6 +88,7 @@ static int put(Rnn1Plan* P, const V* h, size_t n, V** d) {
 static int put_common(Rnn1Plan* P, R1Common& c, int L, const int* in_size, const int* layer_ctas, int H, int S) {
     int rc;
     if ((rc = put(P, (const uint32_t*)nullptr, (size_t)P->n_ctas, &c.epoch)) != CSB_OK || (rc = put(P, (const uint32_t*)nullptr, (size_t)kMaxLayers, &c.progress)) != CSB_OK) return rc;
+    if ((rc = put(P, (const float*)nullptr, (size_t)2 * L * P->BT * (S + H), &P->d_states)) != CSB_OK) return rc;
     for (int l = 0; l < L; ++l) { c.in_size[l] = in_size[l]; c.layer_ctas[l] = layer_ctas[l]; }
     c.H = H; c.S = S; c.L = L;
     CSB_CUDA(cudaHostAlloc((void**)&P->h_status, 4, cudaHostAllocMapped));
@@ -243,26 +246,48 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     RuArgs au = P->u;
     R1Common& a = P->unit_loop ? (R1Common&)au : (R1Common&)a1;
     a.x = x; a.h0 = h0; a.c0 = has_c ? c0 : nullptr; a.y = y; a.hT = hT; a.cT = has_c ? cT : nullptr;
-    if (host_io) {
-        const size_t need = nx + ny + 2 * nh + 2 * nc;
-        if (need > P->stage_cap) {
-            CSB_CUDA(cudaStreamSynchronize(st));
-            cudaFree(P->d_stage); P->d_stage = nullptr; P->stage_cap = 0;
-            CSB_CUDA(cudaMalloc((void**)&P->d_stage, need * 4));
-            P->stage_cap = need;
+    // What lies elsewhere while the kernel runs: host arrays; an input that an output overlaps (a CTA stores its last
+    // states while another may still be reading the first ones; c0 given as cT is the exception, since a CTA reads
+    // and writes its own units only); final states that overlap another output (copied after it, hT before cT).
+    auto meets = [](const float* p, size_t n, const float* q, size_t m) { return p && q && n && m && p < q + m && q < p + n; };
+    auto read_and_written = [&](const float* p, size_t n) { return meets(p, n, a.y, ny) || meets(p, n, a.hT, nh) || meets(p, n, a.cT, nc); };
+    const bool move_x = host_io || read_and_written(a.x, nx), move_h0 = host_io || read_and_written(a.h0, nh);
+    const bool move_c0 = host_io || (a.c0 != a.cT ? read_and_written(a.c0, nc) : meets(a.c0, nc, a.y, ny) || meets(a.c0, nc, a.hT, nh));
+    const bool move_y = host_io, states_meet = meets(a.hT, nh, a.cT, nc);
+    const bool move_hT = host_io || states_meet || meets(a.hT, nh, a.y, ny), move_cT = host_io || states_meet || meets(a.cT, nc, a.y, ny);
+    {
+        // (the states' copies have a place of their own from the start, so that a captured call can have them; a place
+        // for x that was once used stays as long as the plan, for calls that were captured with it)
+        float* d = P->d_states;
+        float* dx = P->d_x;
+        if (host_io) {
+            const size_t need = nx + ny;
+            if (need > P->stage_cap) {
+                CSB_CUDA(cudaStreamSynchronize(st));
+                cudaFree(P->d_stage); P->d_stage = nullptr; P->stage_cap = 0;
+                CSB_CUDA(cudaMalloc((void**)&P->d_stage, need * 4));
+                P->stage_cap = need;
+            }
+            dx = P->d_stage;
+        } else if (move_x && nx > P->x_cap) {
+            const size_t cap = std::max(nx, 2 * P->x_cap);
+            CSB_CUDA(cudaMalloc((void**)&dx, cap * 4));
+            P->owned.push_back(dx);
+            P->d_x = dx; P->x_cap = cap;
         }
-        float* d = P->d_stage;
-        auto in = [&](const float*& p, size_t n) -> cudaError_t {
+        const cudaMemcpyKind kind = host_io ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+        auto in = [&](const float*& p, float* to, size_t n) -> cudaError_t {
             if (!p) return cudaSuccess;
-            const cudaError_t e = cudaMemcpyAsync(d, p, n * 4, cudaMemcpyHostToDevice, st);
-            p = d; d += n;
+            const cudaError_t e = cudaMemcpyAsync(to, p, n * 4, kind, st);
+            p = to;
             return e;
         };
-        auto out = [&](float*& p, size_t n) { if (p) { p = d; d += n; } };
-        CSB_CUDA(in(a.x, nx));
-        CSB_CUDA(in(a.h0, nh));
-        CSB_CUDA(in(a.c0, nc));
-        out(a.y, ny); out(a.hT, nh); out(a.cT, nc);
+        if (move_x) CSB_CUDA(in(a.x, dx, nx));
+        if (move_h0) CSB_CUDA(in(a.h0, d, nh));
+        if (move_c0) CSB_CUDA(in(a.c0, d + nh, nc));
+        if (move_y && a.y) a.y = dx + nx;
+        if (move_hT && a.hT) a.hT = d + nh + nc;
+        if (move_cT && a.cT) a.cT = d + 2 * nh + nc;
     }
     for (int l = 0; l < L; ++l) a.bias[l] = bias ? bias[l] : nullptr;
     a.T = (int)T; a.B = B;
@@ -284,11 +309,10 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     const cudaError_t e = cudaLaunchKernelExC(&cfg, P->kernel, params);
     if (e == cudaErrorCooperativeLaunchTooLarge) { set_error("cooperative launch too large"); return CSB_ERR_LAUNCH; }
     CSB_CUDA(e);
-    if (host_io) {
-        if (y) CSB_CUDA(cudaMemcpyAsync(y, a.y, ny * 4, cudaMemcpyDeviceToHost, st));
-        if (hT) CSB_CUDA(cudaMemcpyAsync(hT, a.hT, nh * 4, cudaMemcpyDeviceToHost, st));
-        if (has_c && cT) CSB_CUDA(cudaMemcpyAsync(cT, a.cT, nc * 4, cudaMemcpyDeviceToHost, st));
-    }
+    const cudaMemcpyKind out_kind = host_io ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    if (move_y && y) CSB_CUDA(cudaMemcpyAsync(y, a.y, ny * 4, out_kind, st));
+    if (move_hT && hT) CSB_CUDA(cudaMemcpyAsync(hT, a.hT, nh * 4, out_kind, st));
+    if (move_cT && has_c && cT) CSB_CUDA(cudaMemcpyAsync(cT, a.cT, nc * 4, out_kind, st));
     if (host_io || !(flags & CSB_FLAG_ASYNC)) {
         CSB_CUDA(cudaStreamSynchronize(st));
         if (*P->h_status != 0) {

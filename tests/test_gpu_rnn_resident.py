@@ -3,10 +3,12 @@ oracle: units that do not fill the last warp or CTA, odd vector lengths (values 
 time), batches below and at a tile of columns, two and four units per warp, fp32 values, stacked layers with more
 steps than a vector stays readable (32)."""
 import pytest
+import torch
 
 import test_gpu_cells as cells
 import test_gpu_rnn as rnn
 import workloads
+from paper_2005_05758_b200 import binding
 
 pytestmark = pytest.mark.gpu
 
@@ -33,3 +35,65 @@ def test_edges_of_units_columns_and_exchange(monkeypatch, cell, I, H, L, br, T, 
     w = workloads.make_rnn_workload(31, cell, I, H, L, br, br, "uniform", lo=keep[0], hi=keep[1], T=T, B=B,
                                     w_std=0.5 / max(1.0, (0.1 * (I + H)) ** 0.5), val_dtype=vd, bias_std=0.1, state_std=0.5, **extra)
     (rnn if cell in ("lstm", "gru") else cells).check(w)
+
+
+@pytest.mark.parametrize("other", [False, True])
+@pytest.mark.parametrize("cell", ["lstm", "gru", "lstmp", "ligru", "gru_rb"])
+@pytest.mark.parametrize("B,T", [(1, 1), (4, 1), (8, 1), (1, 3), (6, 3)])
+def test_arrays_in_each_others_places(monkeypatch, cell, B, T, other):
+    # final states in the place of the initial ones, of each other's, of x or inside y, and y in the place of x: the
+    # bits have to be those of arrays of their own.  (One step exchanges nothing before the states are stored, so
+    # there a CTA can be done while another has not begun to read.)
+    if other:
+        monkeypatch.setenv("CSB_RNN_NO_UNIT", "1")
+    L, H = 2, 512
+    extra = dict(proj_size=256) if cell == "lstmp" else {}
+    S = extra.get("proj_size", H)
+    w = workloads.make_rnn_workload(19, cell, S, H, L, 32, 32, "uniform", lo=0.2, hi=0.5, T=T, B=B, w_std=0.05, bias_std=0.1, state_std=0.5, **extra)
+    encode = lambda ms: [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in ms]   # noqa: E731
+    mats, proj = encode(w.layers), encode(w.proj) if cell == "lstmp" else []
+    bias = [torch.from_numpy(b).cuda() for b in w.bias]
+    has_c = cell in ("lstm", "lstmp")
+
+    def call(x, h0, c0, y, hT, cT):
+        if cell == "lstm":
+            binding.csb_lstm_forward(mats, bias, x, h0, c0, y, hT, cT)
+        elif cell == "lstmp":
+            binding.csb_lstmp_forward(mats, proj, bias, x, h0, c0, y, hT, cT)
+        else:
+            {"gru": binding.csb_gru_forward, "ligru": binding.csb_ligru_forward, "gru_rb": binding.csb_gru_reset_before_forward}[cell](
+                mats, bias, x, h0, y, hT)
+
+    def inputs():
+        # x with room behind it for what may be laid over it
+        x = torch.zeros(max(w.x.size, L * B * S), device="cuda")
+        x[:w.x.size] = torch.from_numpy(w.x.reshape(-1)).cuda()
+        return x, torch.from_numpy(w.h0).cuda(), torch.from_numpy(w.c0).cuda() if has_c else None
+    n = T * B * S
+    x, h, c = inputs()
+    want_y, want_h = torch.empty((T, B, S), device="cuda"), torch.empty_like(h)
+    want_c = torch.empty_like(c) if has_c else None
+    call(x[:n].view(T, B, S), h, c, want_y, want_h, want_c)
+    places = ["in place", "over x", "y over x"] + (["crossed"] if cell == "lstm" else []) + (["in y"] if T >= L else [])
+    for place in places:
+        for _ in range(10 if T == 1 else 2):
+            x, h, c = inputs()
+            y, hT, cT = torch.empty(n, device="cuda"), torch.empty_like(h), torch.empty_like(c) if has_c else None
+            if place == "in place":
+                hT, cT = h, c
+            elif place == "over x":
+                hT = x[:h.numel()].view_as(h)
+            elif place == "y over x":
+                y = x[:n]
+            elif place == "crossed":
+                hT, cT = c, h
+            elif place == "in y":
+                hT = y[:h.numel()].view_as(h)
+            call(x[:n].view(T, B, S), h, c, y.view(T, B, S), hT, cT)
+            torch.cuda.synchronize()
+            skip = h.numel() if place == "in y" else 0
+            assert torch.equal(hT, want_h), place
+            assert torch.equal(y[skip:], want_y.view(-1)[skip:]), place
+            assert not has_c or torch.equal(cT, want_c), place
+    for m in mats + proj:
+        m.free()
