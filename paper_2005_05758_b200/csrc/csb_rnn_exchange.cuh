@@ -40,7 +40,7 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
     return *reinterpret_cast<float2*>(&d);
 }
 __device__ __forceinline__ float2 half2_to_float2(uint32_t w) { return __half22float2(*reinterpret_cast<const __half2*>(&w)); }
-// 1 / d for 1 <= d <= 2: the hardware's approximation and one Newton step.
+// 1 / d for 1 <= d <= 2: the approximate reciprocal and one step of Newton's iteration r (2 - d r).
 __device__ __forceinline__ float reciprocal(float d) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
@@ -48,15 +48,19 @@ __device__ __forceinline__ float reciprocal(float d) {
 }
 // tanh (th) or the logistic function of x, without a branch: the gates of a unit sit on neighbouring lanes,
 // and a divergent choice would run one after the other.  Both from e = exp(-|x|) (tanh: exp(-2 |x|)):
-// 1 / (1 + e), e / (1 + e), (1 - e) / (1 + e); tanh near zero, where that cancels, as x + x^3 q(x^2) with
-// a least-squares polynomial q of degree 4 on |x| < 0.55 (error 1.4 half units in the last place there).
+// 1 / (1 + e), e / (1 + e), (1 - e) / (1 + e).  Near zero 1 - e is left with e's error while the result shrinks, so
+// there tanh is x + x^3 q(x^2), q the least-squares polynomial of degree 4 to (tanh(x) / x - 1) / x^2 at the Chebyshev
+// nodes of 0 <= x^2 <= 25/64 (tests/test_activation.py fits it again).  5/8 is as far as degree 4 goes: its own error
+// stays below 0.2 units in the last place there and is seven times that at 3/4.  Measured against float64, in units in the
+// last place: tanh 0.83 up to 5/8, 2.1 above (3.7 where the exponential form is used from 1/2 on), logistic 3.5;
+// tanhf has 1.8, 1 / (1 + expf(-x)) 3.1 where it does not flush to zero (x > -88).
 __device__ __forceinline__ float activation(float x, bool th) {
     const float ax = fabsf(x), e = expf(th ? -2.f * ax : -ax), d = reciprocal(1.f + e), s = x * x;
-    float q = fmaf(s, -0.006612742319703102f, 0.02130289375782013f);
-    q = fmaf(s, q, -0.05390606448054314f);
-    q = fmaf(s, q, 0.13333070278167725f);
-    q = fmaf(s, q, -0.3333333134651184f);
-    const float t = ax < 0.55f ? fmaf(x * s, q, x) : copysignf((1.f - e) * d, x);
+    float q = fmaf(s, -0.006104947999119759f, 0.021003641188144684f);
+    q = fmaf(s, q, -0.05385249853134155f);
+    q = fmaf(s, q, 0.13332782685756683f);
+    q = fmaf(s, q, -0.333333283662796f);
+    const float t = ax < 0.625f ? fmaf(x * s, q, x) : copysignf((1.f - e) * d, x);
     const float l = x >= 0.f ? d : e * d;
     return x != x ? x : th ? t : l;
 }
