@@ -276,8 +276,9 @@ int prepare_spmm_stack(int L, const csb_matrix* const* A, int batch, SpmmStack* 
 // Y[l] = A[l] . xp[l] for the layers l0 <= l < l1.
 int launch_spmm_stack(const SpmmStack& K, int l0, int l1, const csb_matrix* const* A, uint8_t* const* xp, float* const* Y, int nb, int64_t ldy, void* stream);
 bool spmm_mma_applicable(const csb_matrix* A, int batch);
-// Layer l alone, over fp32 inputs [batch, cols] (any batch).
-int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
+// Layer l alone, over fp32 inputs [batch, cols] (any batch), which are packed into xp (cols rows of spmm_pitch(K.NT) bytes).
+int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
+                           void* stream);
 void free_mma(csb_matrix* A);
 
 // ---- panel layout of the batch-1 product (csb_panel_plan.cpp, csb_panel.cu) ----

@@ -51,9 +51,9 @@ struct StepPlan {
     float* d_c = nullptr;              // [L, B, H] cell state
     float* d_stage = nullptr;          // host-I/O staging of x and y
     size_t stage_cap = 0;
-    // packed path (at most 32 product rows): per layer the packed inputs of its product, one row of
-    // `pitch` bytes per column of W_l, and the fp32 h of every layer
+    // per layer the packed inputs of its product, one row of `pitch` bytes per column of W_l
     uint8_t* d_xp[kMaxLayers] = {};
+    // packed path (at most 32 product rows): the fp32 h of every layer, and the layout of d_xp
     float* d_h = nullptr;              // [L, B, H]
     int pitch = 0, cap = 0;
     ~StepPlan() {
@@ -256,12 +256,14 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             np->L = L; np->B = B; np->H = H; np->gates = gates; np->device = W[0]->device;
             const int rows_v = (gates == 3 ? 2 : 1) * B;
             const bool packed_path = rows_v <= 32 && !env_flag("CSB_RNN_STEP_UNPACKED");
-            if (packed_path) { np->pitch = spmm_pitch(spmm_nt(rows_v)); np->cap = 8 * spmm_nt(rows_v); }
+            const int pitch = spmm_pitch(spmm_nt(std::min(rows_v, 32)));
+            if (packed_path) { np->pitch = pitch; np->cap = 8 * spmm_nt(rows_v); }
             for (int l = 0; l < L; ++l) {
                 np->uids.push_back(W[l]->uid);
                 np->in_size[l] = in_size[l];
-                if (packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], (size_t)(in_size[l] + H) * np->pitch));
-                else CSB_CUDA(cudaMalloc((void**)&np->d_v[l], (size_t)rows_v * (in_size[l] + H) * 4));
+                // (what is read of the packed inputs is written on the call's stream first, so they need no clearing here)
+                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], (size_t)(in_size[l] + H) * pitch));
+                if (!packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_v[l], (size_t)rows_v * (in_size[l] + H) * 4));
             }
             const int rc = prepare_spmm_stack(L, W, std::min(rows_v, 32), &np->stack);
             if (rc != CSB_OK) return rc;
@@ -384,7 +386,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     for (int64_t t = 0; t < T; ++t) {
         for (int l = 0; l < L; ++l) {
             const int ld = in_size[l] + H;
-            const int rc = launch_spmm_stack_fp32(P->stack, l, W[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
+            const int rc = launch_spmm_stack_fp32(P->stack, l, W[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
             if (rc != CSB_OK) return rc;
             const bool top = l == L - 1;
             const float* x_next = (l == 0 && t + 1 < T) ? dx + (size_t)(t + 1) * B * I0 : nullptr;

@@ -706,9 +706,9 @@ static int launch_parts(int n, const csb_matrix* const* A, const MmaPlan::PerCla
     return CSB_OK;
 }
 
-// Packs fp32 inputs and launches, 8 * NT batch columns at a time.
-static int pack_and_launch(const csb_matrix* A, const MmaPlan::PerClass* P, int NT, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
-                           cudaStream_t st) {
+// Packs fp32 inputs into `xp` and launches, 8 * NT batch columns at a time.
+static int pack_and_launch(const csb_matrix* A, const MmaPlan::PerClass* P, int NT, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y,
+                           int64_t ldy, cudaStream_t st) {
     const int cap = 8 * NT;
     for (int b0 = 0; b0 < batch; b0 += cap) {
         const int nb = std::min(cap, batch - b0);
@@ -718,11 +718,10 @@ static int pack_and_launch(const csb_matrix* A, const MmaPlan::PerClass* P, int 
         cudaLaunchConfig_t cfg{};
         cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
         cfg.gridDim = dim3((unsigned)((A->cols + 31) / 32)); cfg.blockDim = dim3(256); cfg.dynamicSmemBytes = 0;
-        CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_pack_x_kernel, X + (int64_t)b0 * ldx, (long long)ldx, nb, (int)A->cols, (uint8_t*)P->d_xp,
-                                    spmm_pitch(NT), NT));
-        const uint8_t* xp = (const uint8_t*)P->d_xp;
+        CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_pack_x_kernel, X + (int64_t)b0 * ldx, (long long)ldx, nb, (int)A->cols, xp, spmm_pitch(NT), NT));
+        const uint8_t* packed = xp;
         float* y = Y + (int64_t)b0 * ldy;
-        const int rc = launch_parts(1, &A, &P, &xp, &y, NT, nb, ldy, st);
+        const int rc = launch_parts(1, &A, &P, &packed, &y, NT, nb, ldy, st);
         if (rc != CSB_OK) return rc;
     }
     return CSB_OK;
@@ -754,7 +753,8 @@ int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch,
             if (rc != CSB_OK) return rc;
         }
     }
-    return pack_and_launch(A, &A->mma->cls[ci], 1 << ci, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
+    const MmaPlan::PerClass* P = &A->mma->cls[ci];
+    return pack_and_launch(A, P, 1 << ci, (uint8_t*)P->d_xp, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
 }
 
 // The products of a stack's layers over inputs packed by the caller (one row of spmm_pitch(NT) bytes per matrix
@@ -797,15 +797,11 @@ int prepare_spmm_stack(int L, const csb_matrix* const* A, int batch, SpmmStack* 
     return 1;
 }
 
-int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
-    int rc = gave_up(A);
+int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
+                           void* stream) {
+    const int rc = gave_up(A);
     if (rc != CSB_OK) return rc;
-    {
-        std::lock_guard<std::mutex> lk(A->mma_mu);
-        MmaPlan::PerClass* C = const_cast<MmaPlan::PerClass*>(K.plan[l]);
-        if (!C->d_xp && (rc = alloc_packed(A, K.NT, C)) != CSB_OK) return rc;
-    }
-    return pack_and_launch(A, K.plan[l], K.NT, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
+    return pack_and_launch(A, K.plan[l], K.NT, xp, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
 }
 
 int launch_spmm_stack(const SpmmStack& K, int l0, int l1, const csb_matrix* const* A, uint8_t* const* xp, float* const* Y, int nb, int64_t ldy, void* stream) {

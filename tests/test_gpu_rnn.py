@@ -309,3 +309,27 @@ def test_step_by_step_state_arrays(cell, B, T, places):
     assert cell == "gru" or cT is None or np.array_equal(cT.cpu().numpy(), want_c)
     for m in mats:
         m.free()
+
+
+def test_first_call_past_32_rows_beside_a_busy_default_stream():
+    # a batch of 32 has built the product's layout already, so the first call with 33 sequences waits for nothing: what it
+    # prepares must be ordered on its own stream, not behind what the default stream is doing
+    I, H, T = 40, 96, 4
+    w = workloads.make_rnn_workload(35, "lstm", I, H, 2, 32, 32, "uniform", lo=0.3, hi=0.7, T=T, B=33, w_std=0.1, bias_std=0.1, state_std=0.2)
+    mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in w.layers]
+    x, h0, c0 = (torch.from_numpy(a).cuda() for a in (w.x, w.h0, w.c0))
+    bias = [torch.from_numpy(b).cuda() for b in w.bias]
+    y32 = torch.zeros((T, 32, H), device="cuda")
+    binding.csb_lstm_forward(mats, bias, x[:, :32].contiguous(), h0[:, :32].contiguous(), c0[:, :32].contiguous(), y32, None, None)
+    side = torch.cuda.Stream()
+    y, hT, cT = torch.zeros((T, 33, H), device="cuda"), torch.empty_like(h0), torch.empty_like(c0)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)                       # some 50 ms on the default stream
+    binding.csb_lstm_forward(mats, bias, x, h0, c0, y, hT, cT, stream=side)
+    torch.cuda.synchronize()
+    want, wh, wc = R.lstm_forward(layers_of(w), w.bias, w.x, w.h0, w.c0)
+    close(y.cpu().numpy(), want, "f16", "y")
+    close(hT.cpu().numpy(), wh, "f16", "hT")
+    close(cT.cpu().numpy(), wc, "f16", "cT")
+    for m in mats:
+        m.free()
