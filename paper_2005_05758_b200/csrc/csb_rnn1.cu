@@ -27,10 +27,16 @@ extern "C" int csb_debug_rnn1_clocks(long long* host_out, int max_ctas) {
 }
 #endif
 
-// Everything one (cell, layer stack) needs on the device; built on first use and kept until one of
-// its matrices is freed.
+// Device memory that goes together.
+struct R1Memory {
+    std::vector<void*> p;
+    ~R1Memory() { for (void* q : p) cudaFree(q); }
+};
+// Everything one (cell, layer stack, batch size) needs on the device; built on first use and kept until one of
+// its matrices is freed.  The weights' layout is shared by the batch sizes of a tile; what a call writes is not, since calls
+// of different batch sizes may overlap.
 struct Rnn1Plan {
-    int cell = 0, L = 0, BT = 1, device = 0, n_ctas = 0, H = 0, S = 0, val_dtype = 0;
+    int cell = 0, L = 0, B = 0, BT = 1, device = 0, n_ctas = 0, H = 0, S = 0, val_dtype = 0;
     bool unusable = false;
     std::vector<uint64_t> uids;
     bool unit_loop = false;                    // csb_rnn_unit_kernel.cuh, else csb_rnn1_kernel.cuh
@@ -38,13 +44,13 @@ struct Rnn1Plan {
     RuArgs u{};
     size_t smem = 0;
     const void* kernel = nullptr;
-    std::vector<void*> owned;                  // device memory
+    std::shared_ptr<R1Memory> layout = std::make_shared<R1Memory>();
+    R1Memory own;
     uint32_t* h_status = nullptr;
     float* d_stage = nullptr; size_t stage_cap = 0;      // x and y of calls with host arrays
     float* d_x = nullptr; size_t x_cap = 0;              // x of calls that write over it
     float* d_states = nullptr;                 // [h0, c0, hT, cT] of calls with host arrays or with states in each other's places
     ~Rnn1Plan() {
-        for (void* p : owned) cudaFree(p);
         cudaFree(d_stage);
         if (h_status) cudaFreeHost(h_status);
     }
@@ -75,25 +81,40 @@ static int env_int(const char* name, int dflt) {
 }
 
 template <typename V>
-static int put(Rnn1Plan* P, const V* h, size_t n, V** d) {
-    const size_t bytes = std::max<size_t>(n, 1) * sizeof(V);
-    CSB_CUDA(cudaMalloc((void**)d, bytes));
-    P->owned.push_back(*d);
-    if (h) { if (n) CSB_CUDA(cudaMemcpy(*d, h, n * sizeof(V), cudaMemcpyHostToDevice)); }
-    else CSB_CUDA(cudaMemset(*d, 0, bytes));
+static int put(R1Memory* M, const std::vector<V>& h, V** d) {
+    CSB_CUDA(cudaMalloc((void**)d, std::max<size_t>(h.size(), 1) * sizeof(V)));
+    M->p.push_back(*d);
+    if (!h.empty()) CSB_CUDA(cudaMemcpy(*d, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice));
     return CSB_OK;
 }
 
-// What both loops need beside images and exchange buffers.
-static int put_common(Rnn1Plan* P, R1Common& c, int L, const int* in_size, const int* layer_ctas, int H, int S) {
-    int rc;
-    if ((rc = put(P, (const uint32_t*)nullptr, (size_t)P->n_ctas, &c.epoch)) != CSB_OK || (rc = put(P, (const uint32_t*)nullptr, (size_t)kMaxLayers, &c.progress)) != CSB_OK) return rc;
-    if ((rc = put(P, (const float*)nullptr, (size_t)2 * L * P->BT * (S + H), &P->d_states)) != CSB_OK) return rc;
-    for (int l = 0; l < L; ++l) { c.in_size[l] = in_size[l]; c.layer_ctas[l] = layer_ctas[l]; }
-    c.H = H; c.S = S; c.L = L;
+// What a call writes: exchange buffers, step numbers and progress (all from zero), states, the status word.
+static int build_state(Rnn1Plan* P) {
+    R1Common& c = P->unit_loop ? (R1Common&)P->u : (R1Common&)P->a;
+    size_t bytes = 0;
+    auto room = [&](size_t n) { const size_t at = bytes; bytes += (n + 255) & ~(size_t)255; return at; };
+    size_t ex[2][kMaxLayers] = {};
+    for (int e = 0; e < r1_ops(P->cell); ++e)
+        for (int l = 0; l < P->L; ++l) {
+            const size_t pairs = ((size_t)(e ? P->H : P->S) * P->BT + 1) & ~(size_t)1;
+            ex[e][l] = room(kR1Ring * (P->unit_loop ? pairs * sizeof(uint2) : (size_t)P->a.words[e][l] * sizeof(uint4)));
+        }
+    const size_t epoch = room((size_t)P->n_ctas * 4), progress = room((size_t)kMaxLayers * 4), states = room((size_t)2 * P->L * P->B * (P->S + P->H) * 4);
+    uint8_t* d = nullptr;
+    CSB_CUDA(cudaMalloc((void**)&d, bytes));
+    P->own.p.push_back(d);
+    CSB_CUDA(cudaMemset(d, 0, bytes));
+    for (int e = 0; e < r1_ops(P->cell); ++e)
+        for (int l = 0; l < P->L; ++l) {
+            if (P->unit_loop) P->u.ex[e][l] = reinterpret_cast<uint2*>(d + ex[e][l]);
+            else P->a.ex[e][l] = reinterpret_cast<uint4*>(d + ex[e][l]);
+        }
+    c.epoch = reinterpret_cast<uint32_t*>(d + epoch); c.progress = reinterpret_cast<uint32_t*>(d + progress);
+    P->d_states = reinterpret_cast<float*>(d + states);
     CSB_CUDA(cudaHostAlloc((void**)&P->h_status, 4, cudaHostAllocMapped));
     *P->h_status = 0;
     CSB_CUDA(cudaHostGetDevicePointer((void**)&c.status, P->h_status, 0));
+    CSB_CUDA(cudaDeviceSynchronize());
     return CSB_OK;
 }
 // Whether the grid can be resident at once.
@@ -105,6 +126,11 @@ static int fits(Rnn1Plan* P, const csb_matrix* A0, bool* yes) {
     CSB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, P->kernel, kR1Threads, P->smem));
     *yes = occ >= 1 && P->n_ctas <= occ * A0->sm_count;
     return CSB_OK;
+}
+
+static void fill_common(R1Common& c, int L, const int* in_size, const int* layer_ctas, int H, int S) {
+    for (int l = 0; l < L; ++l) { c.in_size[l] = in_size[l]; c.layer_ctas[l] = layer_ctas[l]; }
+    c.H = H; c.S = S; c.L = L;
 }
 
 // The unit loop's plan; 1 when it is not the one for these matrices.
@@ -144,19 +170,15 @@ static int build_unit_plan(int cell, int L, const csb_matrix* const* W, const cs
     if (rc != CSB_OK) return rc;
     if (!yes) return 1;
     uint8_t* d_img = nullptr; RuCta* d_ctas = nullptr;
-    if ((rc = put(P, Hp.bytes.data(), Hp.bytes.size(), &d_img)) != CSB_OK || (rc = put(P, Hp.ctas.data(), Hp.ctas.size(), &d_ctas)) != CSB_OK) return rc;
+    if ((rc = put(P->layout.get(), Hp.bytes, &d_img)) != CSB_OK || (rc = put(P->layout.get(), Hp.ctas, &d_ctas)) != CSB_OK) return rc;
     a.images = d_img; a.ctas = d_ctas;
-    for (int l = 0; l < L; ++l) {
-        if ((rc = put(P, (const uint2*)nullptr, (((size_t)S * BT + 1) & ~(size_t)1) * kR1Ring, &a.ex[0][l])) != CSB_OK) return rc;
-        if (ops == 2 && (rc = put(P, (const uint2*)nullptr, (((size_t)H * BT + 1) & ~(size_t)1) * kR1Ring, &a.ex[1][l])) != CSB_OK) return rc;
-    }
-    if ((rc = put_common(P, a, L, in_size, Hp.layer_ctas, H, S)) != CSB_OK) return rc;
+    fill_common(a, L, in_size, Hp.layer_ctas, H, S);
     P->unit_loop = true;
     return CSB_OK;
 }
 
-// Returns 1 (and marks the plan) when the kernel does not take these matrices.
-static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, Rnn1Plan* P) {
+// Layout of the weights, uploaded.  Returns 1 (and marks the plan) when neither kernel takes these matrices.
+static int build_layout(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, Rnn1Plan* P) {
     const csb_matrix* A0 = W[0];
     P->cell = cell; P->L = L; P->BT = BT; P->device = A0->device; P->H = H; P->S = S; P->val_dtype = A0->val_dtype;
     P->unusable = true;
@@ -169,7 +191,7 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
     }
     {
         const int rc = build_unit_plan(cell, L, W, Wp, in_size, H, S, BT, weights, P);
-        if (rc == CSB_OK) { CSB_CUDA(cudaDeviceSynchronize()); P->unusable = false; return CSB_OK; }
+        if (rc == CSB_OK) { P->unusable = false; return CSB_OK; }
         if (rc != 1) return rc;
     }
     if (BT == 8 && P->val_dtype != CSB_F16) return 1;      // not built for fp32 values
@@ -197,18 +219,16 @@ static int build_plan(int cell, int L, const csb_matrix* const* W, const csb_mat
     if (rc != CSB_OK) return rc;
     if (!yes) return 1;
     uint8_t* d_img = nullptr; R1Cta* d_ctas = nullptr;
-    if ((rc = put(P, Hp.bytes.data(), Hp.bytes.size(), &d_img)) != CSB_OK || (rc = put(P, Hp.ctas.data(), Hp.ctas.size(), &d_ctas)) != CSB_OK) return rc;
+    if ((rc = put(P->layout.get(), Hp.bytes, &d_img)) != CSB_OK || (rc = put(P->layout.get(), Hp.ctas, &d_ctas)) != CSB_OK) return rc;
     a.images = d_img; a.ctas = d_ctas;
     for (int e = 0; e < r1_ops(cell); ++e)
         for (int l = 0; l < L; ++l) {
             const std::vector<uint32_t>& m = Hp.wmap[e][l];
             uint32_t* d_map = nullptr;
-            if ((rc = put(P, m.data(), m.size(), &d_map)) != CSB_OK) return rc;
-            if ((rc = put(P, (const uint4*)nullptr, m.size() * kR1Ring, &a.ex[e][l])) != CSB_OK) return rc;
+            if ((rc = put(P->layout.get(), m, &d_map)) != CSB_OK) return rc;
             a.wmap[e][l] = d_map; a.words[e][l] = (int)m.size();
         }
-    if ((rc = put_common(P, a, L, in_size, Hp.layer_ctas, H, S)) != CSB_OK) return rc;
-    CSB_CUDA(cudaDeviceSynchronize());
+    fill_common(a, L, in_size, Hp.layer_ctas, H, S);
     P->unusable = false;
     return CSB_OK;
 }
@@ -222,17 +242,28 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     Rnn1Plan* P = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_r1_mu);
+        Rnn1Plan* like = nullptr;                          // a plan of the same tile: its layout serves
         for (auto& p : g_r1_plans) {
             if (p->cell != cell || p->L != L || p->BT != BT) continue;
             bool same = true;
             for (int l = 0; l < L; ++l) same = same && p->uids[l] == W[l]->uid && (!Wp || p->uids[L + l] == Wp[l]->uid);
-            if (same) { P = p.get(); break; }
+            if (!same) continue;
+            if (p->B == B) { P = p.get(); break; }
+            like = p.get();
         }
         if (!P) {
             std::unique_ptr<Rnn1Plan> np(new Rnn1Plan());
-            int rc;
-            try { rc = build_plan(cell, L, W, Wp, in_size, H, S, BT, np.get()); }
-            catch (const std::bad_alloc&) { set_error("out of host memory while planning the time loop"); rc = CSB_ERR_ALLOC; }
+            int rc = CSB_OK;
+            if (like) {
+                np->cell = like->cell; np->L = like->L; np->BT = like->BT; np->device = like->device; np->n_ctas = like->n_ctas; np->H = like->H; np->S = like->S;
+                np->val_dtype = like->val_dtype; np->unusable = like->unusable; np->uids = like->uids; np->unit_loop = like->unit_loop;
+                np->a = like->a; np->u = like->u; np->smem = like->smem; np->kernel = like->kernel; np->layout = like->layout;
+            } else {
+                try { rc = build_layout(cell, L, W, Wp, in_size, H, S, BT, np.get()); }
+                catch (const std::bad_alloc&) { set_error("out of host memory while planning the time loop"); rc = CSB_ERR_ALLOC; }
+            }
+            np->B = B;
+            if (rc == CSB_OK && !np->unusable) rc = build_state(np.get());
             if (rc != CSB_OK && rc != 1) return rc;
             P = np.get();
             g_r1_plans.push_back(std::move(np));
@@ -272,7 +303,7 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
         } else if (move_x && nx > P->x_cap) {
             const size_t cap = std::max(nx, 2 * P->x_cap);
             CSB_CUDA(cudaMalloc((void**)&dx, cap * 4));
-            P->owned.push_back(dx);
+            P->own.p.push_back(dx);
             P->d_x = dx; P->x_cap = cap;
         }
         const cudaMemcpyKind kind = host_io ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;

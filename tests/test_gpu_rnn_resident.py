@@ -97,3 +97,34 @@ def test_arrays_in_each_others_places(monkeypatch, cell, B, T, other):
             assert not has_c or torch.equal(cT, want_c), place
     for m in mats + proj:
         m.free()
+
+
+@pytest.mark.parametrize("other", [False, True])
+@pytest.mark.parametrize("B1,B2", [(3, 4), (5, 8)])
+def test_batch_sizes_of_one_tile_may_overlap(monkeypatch, B1, B2, other):
+    # calls on the same matrices with different batch sizes have exchange buffers and step numbers of their own, also
+    # where both sizes run on the same tile of columns: queued on two streams at once they give the bits of calls in turn
+    if other:
+        monkeypatch.setenv("CSB_RNN_NO_UNIT", "1")
+    L, I, H, T = 2, 40, 160, 150
+    ws = [workloads.make_rnn_workload(23, "lstm", I, H, L, 32, 32, "uniform", lo=0.3, hi=0.6, T=T, B=B, w_std=0.1, bias_std=0.1, state_std=0.5) for B in (B1, B2)]
+    mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in ws[0].layers]
+    bias = [torch.from_numpy(b).cuda() for b in ws[0].bias]
+    args = [[torch.from_numpy(a).cuda() for a in (w.x, w.h0, w.c0)] for w in ws]
+
+    def outputs():
+        return [[torch.zeros((T, w.B, H), device="cuda"), torch.zeros((L, w.B, H), device="cuda"), torch.zeros((L, w.B, H), device="cuda")] for w in ws]
+    want = outputs()
+    for a, o in zip(args, want):
+        binding.csb_lstm_forward(mats, bias, *a, *o)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for _ in range(5):
+        got = outputs()
+        torch.cuda.synchronize()
+        for a, o, st in zip(args, got, streams):
+            binding.csb_lstm_forward(mats, bias, *a, *o, binding.CSB_FLAG_ASYNC, stream=st)
+        torch.cuda.synchronize()
+        for g, v in zip(got, want):
+            assert all(torch.equal(p, q) for p, q in zip(g, v))
+    for m in mats:
+        m.free()
