@@ -4,7 +4,7 @@
 #include <cstdio>
 #include <new>
 
-#include "csb_internal.hpp"
+#include "csb_host.hpp"
 
 namespace csb {
 
@@ -112,14 +112,14 @@ static int encode_common(const float* dense, int64_t rows, int64_t cols, int64_t
     A->uid = g_uid.fetch_add(1);
     A->q_frac_bits = frac_bits;
     if (opts) A->opts = *opts;
-    int rc = encode_host(dense, rows, cols, ld, block_r, block_c, row_keep, col_keep, val_dtype, A);
-    if (rc == CSB_OK) rc = validate_host(A);
+    int rc = guarded([&] { return encode_host(dense, rows, cols, ld, block_r, block_c, row_keep, col_keep, val_dtype, A); });
+    if (rc == CSB_OK) rc = guarded([&] { return validate_host(A); });
     if (rc == CSB_OK && device >= 0) {
-        try {
-            if (val_dtype == CSB_Q16) rc = plan_fixed(A);
-            else { rc = plan_product(A); if (rc == CSB_OK) rc = plan_panels(A); }
-        }
-        catch (const std::bad_alloc&) { set_error("out of host memory while planning"); rc = CSB_ERR_ALLOC; }
+        rc = guarded([&] {
+            if (val_dtype == CSB_Q16) return plan_fixed(A);
+            const int planned = plan_product(A);
+            return planned == CSB_OK ? plan_panels(A) : planned;
+        });
     }
     if (rc != CSB_OK) { csb_free(A); return rc; }
     *out = A;
@@ -260,7 +260,7 @@ int csb_spmm(const csb_matrix_t* A, const float* X, int64_t ldx, int batch, floa
     if (ldx < A->cols || ldy < A->rows) { set_error("ldx=%lld < cols or ldy=%lld < rows", (long long)ldx, (long long)ldy); return CSB_ERR_SHAPE; }
     if (A->device < 0) { set_error("matrix was encoded host-only (device = -1)"); return CSB_ERR_UNSUPPORTED; }
     if (A->val_dtype == CSB_Q16) { set_error("fixed-point handles serve csb_spmm_q16 only"); return CSB_ERR_UNSUPPORTED; }
-    return product_any(A, X, ldx, batch, Y, ldy, stream);
+    return guarded([&] { return product_any(A, X, ldx, batch, Y, ldy, stream); });
 }
 
 int csb_spmv(const csb_matrix_t* A, const float* x, float* y, void* stream) {

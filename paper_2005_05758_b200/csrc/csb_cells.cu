@@ -17,6 +17,7 @@
 
 #include "csb_internal.hpp"
 #include "csb_device.cuh"
+#include "csb_host.hpp"
 #include "csb_rnn1.hpp"
 
 namespace csb {
@@ -349,17 +350,17 @@ extern "C" {
 
 int csb_lstmp_forward(int n_layers, const csb_matrix_t* const* W, const csb_matrix_t* const* Wp, const float* const* bias, const float* x, int64_t T,
                       int B, const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream) {
-    return csb::cell_forward(csb::kCellLstmp, n_layers, W, Wp, bias, x, T, B, h0, c0, y, hT, cT, flags, stream);
+    return csb::guarded([&] { return csb::cell_forward(csb::kCellLstmp, n_layers, W, Wp, bias, x, T, B, h0, c0, y, hT, cT, flags, stream); });
 }
 
 int csb_ligru_forward(int n_layers, const csb_matrix_t* const* W, const float* const* bias, const float* x, int64_t T, int B, const float* h0,
                       float* y, float* hT, unsigned flags, void* stream) {
-    return csb::cell_forward(csb::kCellLigru, n_layers, W, nullptr, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream);
+    return csb::guarded([&] { return csb::cell_forward(csb::kCellLigru, n_layers, W, nullptr, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream); });
 }
 
 int csb_gru_reset_before_forward(int n_layers, const csb_matrix_t* const* W, const float* const* bias, const float* x, int64_t T, int B,
                                  const float* h0, float* y, float* hT, unsigned flags, void* stream) {
-    return csb::cell_forward(csb::kCellGruRb, n_layers, W, nullptr, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream);
+    return csb::guarded([&] { return csb::cell_forward(csb::kCellGruRb, n_layers, W, nullptr, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream); });
 }
 
 }  // extern "C"

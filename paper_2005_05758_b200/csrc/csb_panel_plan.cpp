@@ -27,10 +27,8 @@
 #include <atomic>
 #include <cstdlib>
 #include <new>
-#include <system_error>
-#include <thread>
 
-#include "csb_internal.hpp"
+#include "csb_host.hpp"
 
 namespace csb {
 
@@ -333,8 +331,7 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
         return CSB_OK;
     };
     {
-        const unsigned hw = std::thread::hardware_concurrency();
-        const int n_threads = (int)std::min<int64_t>(std::min<int64_t>(hw ? hw : 1, 8), std::max<int64_t>(1, (int64_t)(total_bytes >> 18)));   // 256 KB of values and more per thread
+        const int n_threads = (int)std::min<int64_t>(8, std::max<int64_t>(1, (int64_t)(total_bytes >> 18)));   // 256 KB of values and more per thread
         std::atomic<int> next{0}, status{CSB_OK};
         auto work = [&]() {
             for (int c; status.load() == CSB_OK && (c = next.fetch_add(1)) < n_ctas;) {
@@ -343,10 +340,7 @@ int plan_panels_host(const csb_matrix* A, int ctas, int warps, int stage_bytes, 
                 if (rc != CSB_OK) status.store(rc);
             }
         };
-        std::vector<std::thread> pool;
-        try { for (int t = 1; t < n_threads; ++t) pool.emplace_back(work); } catch (const std::system_error&) {}   // fewer threads then
-        work();
-        for (auto& t : pool) t.join();
+        run_on_threads(n_threads, work);
         if (status.load() == CSB_ERR_ALLOC) throw std::bad_alloc();
         if (status.load() != CSB_OK) return status.load();
     }

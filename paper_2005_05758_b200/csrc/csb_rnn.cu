@@ -17,6 +17,7 @@
 
 #include "csb_internal.hpp"
 #include "csb_device.cuh"
+#include "csb_host.hpp"
 #include "csb_rnn1.hpp"
 
 namespace csb {
@@ -952,12 +953,12 @@ extern "C" {
 
 int csb_lstm_forward(int n_layers, const csb_matrix_t* const* W, const float* const* bias, const float* x, int64_t T, int B,
                      const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream) {
-    return csb::rnn_forward(4, n_layers, W, bias, x, T, B, h0, c0, y, hT, cT, flags, stream);
+    return csb::guarded([&] { return csb::rnn_forward(4, n_layers, W, bias, x, T, B, h0, c0, y, hT, cT, flags, stream); });
 }
 
 int csb_gru_forward(int n_layers, const csb_matrix_t* const* W, const float* const* bias, const float* x, int64_t T, int B,
                     const float* h0, float* y, float* hT, unsigned flags, void* stream) {
-    return csb::rnn_forward(3, n_layers, W, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream);
+    return csb::guarded([&] { return csb::rnn_forward(3, n_layers, W, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream); });
 }
 
 void csb_test_barrier_hook(unsigned int extra_arrivals, unsigned long long limit_ns) {

@@ -7,9 +7,8 @@
 #include <algorithm>
 #include <atomic>
 #include <new>
-#include <system_error>
-#include <thread>
 
+#include "csb_host.hpp"
 #include "csb_rnn1.hpp"
 
 namespace csb {
@@ -339,13 +338,7 @@ int plan_rnn1_host(int cell, int L, const csb_matrix* const* W, const csb_matrix
             if (rc != CSB_OK) status.store(rc);
         }
     };
-    {
-        const unsigned hw = std::thread::hardware_concurrency();
-        std::vector<std::thread> pool;
-        try { for (unsigned t = 1; t < std::min<unsigned>(hw ? hw : 1, 8) && t < jobs.size() / 8; ++t) pool.emplace_back(work); } catch (const std::system_error&) {}
-        work();
-        for (auto& t : pool) t.join();
-    }
+    run_on_threads((int)std::min<size_t>(8, std::max<size_t>(1, jobs.size() / 8)), work);
     if (status.load() == CSB_ERR_ALLOC) throw std::bad_alloc();
     if (status.load() != CSB_OK) return status.load();
     // ---- exchange words: three elements each (unit by unit, the batch columns of a unit side by side), CTA by CTA

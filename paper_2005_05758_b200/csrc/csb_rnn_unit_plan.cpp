@@ -2,9 +2,8 @@
 #include <algorithm>
 #include <atomic>
 #include <new>
-#include <system_error>
-#include <thread>
 
+#include "csb_host.hpp"
 #include "csb_rnn_unit.hpp"
 
 namespace csb {
@@ -189,13 +188,7 @@ int plan_unit_host(int cell, int L, const csb_matrix* const* W, const csb_matrix
             } catch (const std::bad_alloc&) { status.store(CSB_ERR_ALLOC); }
         }
     };
-    {
-        const unsigned hw = std::thread::hardware_concurrency();
-        std::vector<std::thread> pool;
-        try { for (unsigned t = 1; t < std::min<unsigned>(hw ? hw : 1, 16) && t < jobs.size() / 4; ++t) pool.emplace_back(work); } catch (const std::system_error&) {}
-        work();
-        for (auto& t : pool) t.join();
-    }
+    run_on_threads((int)std::min<size_t>(16, std::max<size_t>(1, jobs.size() / 4)), work);
     if (status.load() == CSB_ERR_ALLOC) throw std::bad_alloc();
     size_t base = 0;
     for (size_t c = 0; c < jobs.size(); ++c) {
