@@ -8,7 +8,7 @@
 
 enum { kMaxList = 64 };
 
-static PyObject *s_data_ptr, *s_shape, *s_stride, *s_handle, *s_zero;
+static PyObject *s_data_ptr, *s_shape, *s_stride, *s_handle, *s_value, *s_zero;
 
 /* Address of a torch tensor (data_ptr()) or of a numpy array (its buffer); None is NULL. */
 static int address(PyObject* o, void** out) {
@@ -27,10 +27,29 @@ static int address(PyObject* o, void** out) {
     Py_DECREF(p);
     return PyErr_Occurred() ? -1 : 0;
 }
-static int pointer(PyObject* o, void** out) {      /* an integer or None */
+/* A ctypes number or pointer counts as its value; everything else as itself.  A new reference. */
+static PyObject* plain(PyObject* o) {
+    if (o != Py_None && !PyLong_Check(o) && !PyIndex_Check(o)) {
+        PyObject* v = PyObject_GetAttr(o, s_value);
+        if (v) return v;
+        PyErr_Clear();
+    }
+    Py_INCREF(o);
+    return o;
+}
+static int pointer(PyObject* o, void** out) {      /* an integer, a ctypes pointer or None */
     *out = NULL;
-    if (o == Py_None) return 0;
-    *out = PyLong_AsVoidPtr(o);
+    PyObject* v = plain(o);
+    if (!v) return -1;
+    if (v != Py_None) *out = PyLong_AsVoidPtr(v);
+    Py_DECREF(v);
+    return PyErr_Occurred() ? -1 : 0;
+}
+static int flag_bits(PyObject* o, unsigned* out) {
+    PyObject* v = plain(o);
+    if (!v) return -1;
+    *out = (unsigned)PyLong_AsUnsignedLongMask(v);
+    Py_DECREF(v);
     return PyErr_Occurred() ? -1 : 0;
 }
 static int handle_of(PyObject* o, void** out) {
@@ -57,7 +76,7 @@ static int row_stride(PyObject* o, int64_t* out) {
     Py_DECREF(v);
     return PyErr_Occurred() ? -1 : 0;
 }
-/* The first n items of a sequence: handles of matrices, or addresses. */
+/* The first n items of a sequence: handles of matrices (None is NULL, which the library refuses), or addresses. */
 static int list_of(PyObject* o, Py_ssize_t n, int handles, void** out) {
     PyObject* s = PySequence_Fast(o, "a sequence is expected");
     if (!s) return -1;
@@ -65,7 +84,7 @@ static int list_of(PyObject* o, Py_ssize_t n, int handles, void** out) {
     if (PySequence_Fast_GET_SIZE(s) < n) { PyErr_SetString(PyExc_IndexError, "list index out of range"); rc = -1; }
     for (Py_ssize_t i = 0; i < n && !rc; ++i) {
         PyObject* v = PySequence_Fast_GET_ITEM(s, i);
-        rc = handles ? handle_of(v, &out[i]) : address(v, &out[i]);
+        rc = handles && v != Py_None ? handle_of(v, &out[i]) : address(v, &out[i]);
     }
     Py_DECREF(s);
     return rc;
@@ -107,9 +126,9 @@ static PyObject* py_recurrent(PyObject* self, PyObject* const* a, Py_ssize_t n) 
     int rc;
     if (arity(n, 13) || pointer(a[0], &f)) return NULL;
     const long kind = PyLong_AsLong(a[1]);
-    const unsigned flags = (unsigned)PyLong_AsUnsignedLongMask(a[11]);
     const Py_ssize_t L = PyObject_Length(a[2]);
-    if (PyErr_Occurred()) return NULL;
+    unsigned flags;
+    if (PyErr_Occurred() || flag_bits(a[11], &flags)) return NULL;
     const Py_ssize_t m = L < kMaxList ? L : kMaxList;      /* more layers than the library takes: it refuses by L */
     if (list_of(a[2], m, 1, W) || (kind == 2 && list_of(a[3], m, 1, Wp)) || (a[4] != Py_None && list_of(a[4], m, 0, bias))) return NULL;
     if (address(a[5], &x) || size_at(a[5], 0, &T) || size_at(a[5], 1, &B) || address(a[6], &h0) || address(a[7], &c0) || address(a[8], &y) ||
@@ -140,7 +159,8 @@ PyMODINIT_FUNC PyInit__csb_py(void) {
     s_shape = PyUnicode_InternFromString("shape");
     s_stride = PyUnicode_InternFromString("stride");
     s_handle = PyUnicode_InternFromString("handle");
+    s_value = PyUnicode_InternFromString("value");
     s_zero = PyLong_FromLong(0);
-    if (!s_data_ptr || !s_shape || !s_stride || !s_handle || !s_zero) return NULL;
+    if (!s_data_ptr || !s_shape || !s_stride || !s_handle || !s_value || !s_zero) return NULL;
     return PyModule_Create(&module);
 }
