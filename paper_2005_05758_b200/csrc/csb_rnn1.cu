@@ -238,7 +238,7 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
     if (env_int("CSB_RNN_NO_RNN1", 0)) return 1;
     if (B > 1 && env_int("CSB_RNN_NO_STEPWISE", 0)) return 1;   // asks for the persistent kernel of csb_rnn.cu
     const int BT = B == 1 ? 1 : B <= 4 ? 4 : 8;            // tiles of batch columns that the kernels are built for
-    if (B > 8) return 1;
+    if (B > 8 || T > 0x7fffffff) return 1;                 // (the kernels count steps in 32 bits)
     Rnn1Plan* P = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_r1_mu);
