@@ -174,13 +174,14 @@ int csb_spmv(const csb_matrix_t* A, const float* x, float* y, void* stream);
  *   Y  device, float32, batch rows of `rows` values, row stride ldy >= rows, overwritten.
  * batch = 0 is a no-op.  Same ordering / overlap rules as csb_spmv; results are bit-reproducible.
  * With batch >= 8, fp16 values and block_r <= 64 the product runs on tensor cores (the kernel
- * matrix times the gathered inputs is then a dense contraction), 32 batch columns per pass: the
+ * matrix times the gathered inputs is then a dense contraction), up to 64 batch columns per pass: the
  * inputs are split into two binary16 halves (x = hi + lo, so no input precision is lost as long
  * as |x| < 65504; larger or non-finite inputs give inf / NaN) and multiplied with
  * mma.sync.m16n8k16, fp32 accumulation, a block-row's outputs staying in registers across its
- * blocks.  The first such call on a handle for a batch size class (<= 8, <= 16, more)
+ * blocks.  The first such call on a handle for a batch size class (<= 16, <= 32, more)
  * builds a device layout for that class and a staging buffer for the packed inputs (allocates and
- * synchronises the device once; make it outside of any stream capture).  The two kernels of this path are launched
+ * synchronises the device once; make it outside of any stream capture, where more than 16 vectors are
+ * served by the layout of either of the larger classes).  The two kernels of this path are launched
  * with programmatic stream serialization and wait, first thing, for the work in front of them on
  * `stream`.  Other cases use the CUDA-core kernel in batch tiles of 8 / 4 / 1.
  */

@@ -620,14 +620,17 @@ static int build_spmm_plan(const csb_matrix* A, int ci, int sms, int force_S, bo
     return CSB_OK;
 }
 
+static void drop_plan(MmaPlan::PerClass& c) {
+    cudaFree(c.d_stream); cudaFree(c.d_warp_desc); cudaFree(c.d_ctas); cudaFree(c.d_xp);
+    c.d_stream = nullptr; c.d_warp_desc = nullptr; c.d_ctas = nullptr; c.d_xp = nullptr;
+}
 void free_mma(csb_matrix* A) {
     if (!A->mma) return;
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(A->device);
-    auto drop = [](MmaPlan::PerClass& c) { cudaFree(c.d_stream); cudaFree(c.d_warp_desc); cudaFree(c.d_ctas); cudaFree(c.d_xp); };
-    for (auto& c : A->mma->cls) drop(c);
-    for (auto& c : A->mma->shared) drop(c.plan);
+    for (auto& c : A->mma->cls) drop_plan(c);
+    for (auto& c : A->mma->shared) drop_plan(c.plan);
     cudaSetDevice(prev);
     delete A->mma;
     A->mma = nullptr;
@@ -647,7 +650,12 @@ static int make_spmm_plan(const csb_matrix* A, int ci, int sms, int force_S, boo
         int rc;
         try { rc = build_spmm_plan(A, ci, sms, force_S, with_x, C); }
         catch (const std::bad_alloc&) { set_error("out of host memory while planning the batched product"); rc = CSB_ERR_ALLOC; }
-        if (rc != CSB_OK) { C->unusable = true; return rc; }
+        if (rc != CSB_OK) {                                // (what it had allocated goes back, and no error is left behind for the next launch to find)
+            drop_plan(*C);
+            cudaGetLastError();
+            C->unusable = true;
+            return rc;
+        }
     }
     return (C->unusable || !C->built) ? 1 : CSB_OK;
 }
@@ -727,6 +735,12 @@ static int pack_and_launch(const csb_matrix* A, const MmaPlan::PerClass* P, int 
     return CSB_OK;
 }
 
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) { cudaGetLastError(); return false; }
+    return status != cudaStreamCaptureStatusNone;
+}
+
 // Returns CSB_OK after launching, or 1 when the caller should use the CUDA-core path.
 int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
     int rc = gave_up(A);
@@ -744,14 +758,16 @@ int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch,
     {
         std::lock_guard<std::mutex> lk(A->mma_mu);
         if ((rc = ensure_mma(A)) != CSB_OK) return rc;
+        MmaPlan::PerClass* cls = A->mma->cls;
         // more than 32 columns: tiles of 64, so that row maps, weights and bookkeeping are paid once for all of
         // them (8192 x 8192 at 4x, batch 64: 74.9 -> 59.3 us); where that plan does not fit, passes of 32
-        if (batch > 32 && make_spmm_plan(A, 3, sms, 0, true, &A->mma->cls[3]) == CSB_OK) ci = 3;
-        else {
-            rc = make_spmm_plan(A, ci, sms, 0, true, &A->mma->cls[ci]);
-            if (rc == 1 && batch <= 8) rc = make_spmm_plan(A, ci = 0, sms, 0, true, &A->mma->cls[0]);   // takes less shared memory
-            if (rc != CSB_OK) return rc;
-        }
+        if (batch > 32) ci = 3;
+        // either of the two wide layouts serves any batch: in a stream capture, where none can be built, the one there is
+        if (ci >= 2 && !cls[ci].built && cls[5 - ci].built && capturing((cudaStream_t)stream)) ci = 5 - ci;
+        if (ci == 3 && make_spmm_plan(A, 3, sms, 0, true, &cls[3]) != CSB_OK) { clear_error(); ci = 2; }
+        rc = make_spmm_plan(A, ci, sms, 0, true, &cls[ci]);
+        if (rc == 1 && batch <= 8) rc = make_spmm_plan(A, ci = 0, sms, 0, true, &cls[0]);   // takes less shared memory
+        if (rc != CSB_OK) return rc;
     }
     const MmaPlan::PerClass* P = &A->mma->cls[ci];
     return pack_and_launch(A, P, 1 << ci, (uint8_t*)P->d_xp, X, ldx, batch, Y, ldy, (cudaStream_t)stream);

@@ -183,3 +183,25 @@ def test_few_vectors(shape, vd):
     X = np.random.default_rng(5).standard_normal((9, C)).astype(np.float32)
     for B in range(1, 10):
         run_case(mat, X[:B])
+
+
+@pytest.mark.parametrize("first,captured", [(32, 64), (17, 40), (64, 20), (3, 1), (9, 16)])
+def test_a_class_that_one_call_has_set_up_serves_a_capture(first, captured):
+    # a call of more than 16 vectors outside sets up every batch of more than 16 for stream captures, in which
+    # nothing can be allocated
+    mat = workloads.make_matrix(43, 640, 500, 64, 32, "uniform", lo=0.3, hi=0.9, w_std=0.1, val_dtype="f16")
+    X = np.random.default_rng(6).standard_normal((64, 500)).astype(np.float32)
+    A = binding.csb_encode(mat.dense, 64, 32, mat.row_keep, mat.col_keep, "f16", 0)
+    Xd = torch.from_numpy(X).cuda()
+    binding.csb_spmm(A, Xd[:first], torch.empty((first, 640), device="cuda"))
+    Y = torch.full((captured, 640), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        binding.csb_spmm(A, Xd[:captured], Y)
+    graph.replay()
+    torch.cuda.synchronize()
+    args = (mat.dense, 64, 32, mat.row_keep, mat.col_keep, "f16")
+    check_product(Y.cpu().numpy(), O.spmm(*args, X[:captured]), O.abs_scale(*args, X[:captured]), "f16")
+    del graph
+    A.free()
