@@ -198,20 +198,15 @@ static int build_layout(int cell, int L, const csb_matrix* const* W, const csb_m
     int want = (int)std::min<int64_t>(A0->sm_count, std::max<int64_t>(L, weights / env_int("CSB_R1_MIN", 1024)));
     want = std::min(A0->sm_count, env_int("CSB_R1_CTAS", want));
     R1HostPlan Hp;
-    const int hrc = plan_rnn1_host(cell, L, W, Wp, in_size, H, S, BT, want, &Hp);
+    const int hrc = plan_rnn1_host(cell, L, W, Wp, in_size, H, S, BT, want, A0->smem_optin, &Hp);
     if (hrc != CSB_OK) return hrc;
     R1Args& a = P->a;
-    size_t at = Hp.max_bytes;
-    auto room = [&](size_t floats) { const size_t o = at; at = (at + floats * 4 + 15) & ~(size_t)15; return (uint32_t)o; };
     int max_in = 0;
     for (int l = 0; l < L; ++l) max_in = std::max(max_in, in_size[l]);
-    for (uint32_t& v : a.vu) v = room((size_t)(max_in + 1) * BT);
-    a.vr = room((size_t)(S + 1) * BT); a.vm = room(r1_ops(cell) == 2 ? (size_t)(H + 1) * BT : 0);
-    for (int op = 0; op < 2; ++op) a.part[op] = room(Hp.max_partials[op] * BT);
-    a.z[0] = room(4 * Hp.max_units * BT); a.z[1] = room(r1_ops(cell) == 2 ? Hp.max_units * BT : 0);
-    a.cs = room(Hp.max_units * BT); a.bias0 = room(4 * Hp.max_units); a.bias1 = room(Hp.max_units);
-    a.misc = room(4);
-    P->smem = at;
+    const R1Carve M(Hp, cell, max_in, H, S, BT);
+    for (int i = 0; i < 2; ++i) { a.vu[i] = M.vu[i]; a.part[i] = M.part[i]; a.z[i] = M.z[i]; }
+    a.vr = M.vr; a.vm = M.vm; a.cs = M.cs; a.bias0 = M.bias0; a.bias1 = M.bias1; a.misc = M.misc;
+    P->smem = M.total;
     P->n_ctas = (int)Hp.ctas.size();
     P->kernel = pick_kernel_bt(cell, BT, P->val_dtype);
     bool yes = false;

@@ -56,19 +56,24 @@ struct R1HostPlan {
     std::vector<uint8_t> bytes;                // the CTAs' images, each aligned to 128 bytes
     std::vector<R1Cta> ctas;
     std::vector<uint32_t> wmap[2][kMaxLayers]; // per exchange (0: state, 1: within the step) and layer: first element | elements << 24 of every word
-    size_t max_bytes = 0, max_partials[2] = {0, 0}, max_rows = 0, max_units = 0;
+    size_t max_bytes = 0, max_partials[2] = {0, 0}, max_units = 0;   // largest over the CTAs
     int layer_ctas[kMaxLayers] = {};
-    double balance = 1.0;
 };
 inline int r1_gates(int cell, int op) {
     return cell == kR1Lstm || (cell == kR1Lstmp && op == 0) ? 4 : cell == kR1Gru ? 3 : cell == kR1Ligru || (cell == kR1GruRb && op == 0) ? 2 : 1;
 }
 inline int r1_ops(int cell) { return cell == kR1Lstmp || cell == kR1GruRb ? 2 : 1; }
+// The kernel's shared memory behind a CTA's image: offsets in bytes, and all of it.
+struct R1Carve {
+    uint32_t vu[2], vr, vm, part[2], z[2], cs, bias0, bias1, misc;
+    size_t total;
+    R1Carve(const R1HostPlan& P, int cell, int max_in, int H, int S, int BT);
+};
 // W: per layer the gate matrix; Wp: LSTMP's projections.  in_size[l] + S columns (S the width of the
 // recurrent state); B batch columns, BT of them in shared memory side by side.  Returns CSB_OK, or 1
-// when the layout does not apply.
+// when the layout does not apply or a CTA needs more than smem_limit bytes of shared memory.
 int plan_rnn1_host(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, int n_ctas,
-                   R1HostPlan* out);
+                   size_t smem_limit, R1HostPlan* out);
 // One call of the time loop.  Returns 1 when the kernel does not take these matrices or this batch (nothing was done).
 int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const float* const* bias, const float* x, int64_t T, int B,
                  int H, int S, const int* in_size, const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream);

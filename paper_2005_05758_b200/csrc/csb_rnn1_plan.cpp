@@ -72,22 +72,27 @@ uint32_t append(std::vector<uint8_t>& b, const V* p, size_t n) {
     return at;
 }
 
-struct Image { std::vector<uint8_t> bytes; size_t partials[2] = {0, 0}, rows = 0; };
+// One product of a CTA before anything is emitted: its tasks and groups, where the partial sums lie, and how long it gets.
+struct GroupRef { int part, narrow, rows, warp; size_t from; };
+struct OpLayout {
+    std::vector<Task> tasks[2][2];             // [part][narrow], longest first
+    std::vector<uint32_t> count[2], first[2];  // partial sums of a row and part: how many, where
+    std::vector<R1Row> rows;
+    std::vector<GroupRef> groups;              // in the order in which they are emitted
+    size_t n_rows = 0, partials = 0, bytes = 0;
+};
+struct Image { std::vector<uint8_t> bytes; OpLayout op[2]; };
 
-// Lays one product out behind the image; returns 1 when it does not fit the layout.
-int emit_op(const OpSource& s, const int zero[2], int op, int BT, Image* img) {
+// Returns 1 when the product does not fit the layout.
+int lay_out_op(const OpSource& s, int BT, OpLayout* o) {
     const int wide = r1_wide(BT), vs = val_size(s.A->val_dtype);
-    const size_t n_rows = (size_t)s.gates * s.units;
-    // lanes that share a pass over the banks, and the banks (in units of BT floats) they must keep apart
-    const int pass = BT == 1 ? 32 : BT == 2 ? 16 : 8, banks = std::max(32 / BT, 4);
+    const size_t n_rows = o->n_rows = (size_t)s.gates * s.units;
     // ---- tasks: rows at most so many that there is about one group for every warp
-    std::vector<Task> tasks[2][2];             // [part][narrow]
-    std::vector<uint32_t> count[2];            // partial sums per row and part
     for (int p = 0; p < 2; ++p) {
         int limit = kR1MaxRows;
         for (;; limit = std::max(1, limit / 2)) {
-            for (auto& v : tasks[p]) v.clear();
-            count[p].assign(n_rows, 0);
+            for (auto& v : o->tasks[p]) v.clear();
+            o->count[p].assign(n_rows, 0);
             for_pieces(s, [&](int part, int64_t b, int ra, int rz, int k0, int k1, int row_base, int col_base) {
                 if (part != p) return;
                 const int splits = (rz - ra + limit - 1) / limit;
@@ -95,120 +100,132 @@ int emit_op(const OpSource& s, const int zero[2], int op, int BT, Image* img) {
                     const int ke = std::min(k1, k + wide);
                     for (int i = 0; i < splits; ++i) {
                         const int x = ra + (rz - ra) * i / splits, y = ra + (rz - ra) * (i + 1) / splits;
-                        tasks[p][ke - k <= wide / 2].push_back({s.A, b, k, ke, x, y, row_base, col_base});
+                        o->tasks[p][ke - k <= wide / 2].push_back({s.A, b, k, ke, x, y, row_base, col_base});
                     }
-                    for (int r = ra; r < rz; ++r) ++count[p][row_base + s.A->row_idx[s.A->ridx_off[b] + r]];
+                    for (int r = ra; r < rz; ++r) ++o->count[p][row_base + s.A->row_idx[s.A->ridx_off[b] + r]];
                 }
             });
             // halving the rows must not make more groups than there are warps
-            const size_t groups = (tasks[p][0].size() + 31) / 32 + (tasks[p][1].size() + 31) / 32;
+            const size_t groups = (o->tasks[p][0].size() + 31) / 32 + (o->tasks[p][1].size() + 31) / 32;
             if (limit == 1 || groups * 2 > (size_t)kR1Warps) break;
         }
     }
     // ---- places of the partial sums: row by row, input part then recurrent part, in quads; then one per lane for idle lanes
-    std::vector<R1Row> rows(std::max<size_t>(n_rows, 1));
-    std::vector<uint32_t> first[2] = {std::vector<uint32_t>(n_rows), std::vector<uint32_t>(n_rows)};
+    o->rows.assign(std::max<size_t>(n_rows, 1), R1Row{});
     size_t at = 0;
+    for (auto& f : o->first) f.assign(n_rows, 0);
     for (size_t r = 0; r < n_rows; ++r)
         for (int p = 0; p < 2; ++p) {
-            const size_t q = (count[p][r] + 3) / 4;
-            rows[r].base[p] = (uint16_t)(at / 4); rows[r].quads[p] = (uint16_t)q;
-            first[p][r] = (uint32_t)at;
+            const size_t q = (o->count[p][r] + 3) / 4;
+            o->rows[r].base[p] = (uint16_t)(at / 4); o->rows[r].quads[p] = (uint16_t)q;
+            o->first[p][r] = (uint32_t)at;
             at += 4 * q;
         }
-    const size_t idle = at;
     at += 32;
     if (at > 65535) return 1;
-    img->partials[op] = at;
-    img->rows = std::max(img->rows, n_rows);
-    std::vector<std::vector<uint16_t>> free_places[2];
-    for (int p = 0; p < 2; ++p) {
-        free_places[p].resize(n_rows);
-        for (size_t r = 0; r < n_rows; ++r) for (uint32_t i = 0; i < count[p][r]; ++i) free_places[p][r].push_back((uint16_t)(first[p][r] + i));
-    }
+    o->partials = at;
     // ---- groups: 32 tasks of about the same number of rows, longest first to the warp with the least work
-    std::vector<R1Group> groups[kR1Warps][2];
     double load[kR1Warps] = {};
     for (int p = 0; p < 2; ++p) {
-        struct G { size_t from; int narrow, rows; };
-        std::vector<G> order;
+        std::vector<GroupRef> order;
         for (int nw = 0; nw < 2; ++nw) {
-            std::vector<Task>& v = tasks[p][nw];
+            std::vector<Task>& v = o->tasks[p][nw];
             std::stable_sort(v.begin(), v.end(), [](const Task& a, const Task& b) { return a.r1 - a.r0 > b.r1 - b.r0; });
-            for (size_t i = 0; i < v.size(); i += 32) order.push_back({i, nw, v[i].r1 - v[i].r0});
+            for (size_t i = 0; i < v.size(); i += 32) order.push_back({p, nw, v[i].r1 - v[i].r0, 0, i});
         }
-        std::stable_sort(order.begin(), order.end(), [](const G& a, const G& b) { return a.rows > b.rows; });
+        std::stable_sort(order.begin(), order.end(), [](const GroupRef& a, const GroupRef& b) { return a.rows > b.rows; });
         double part_load[kR1Warps] = {};
-        for (const G& g : order) {
-            int w = 0;
-            for (int i = 1; i < kR1Warps; ++i) if (part_load[i] < part_load[w] || (part_load[i] == part_load[w] && load[i] < load[w])) w = i;
+        for (GroupRef& g : order) {
+            for (int i = 1; i < kR1Warps; ++i) if (part_load[i] < part_load[g.warp] || (part_load[i] == part_load[g.warp] && load[i] < load[g.warp])) g.warp = i;
             const double cost = kTaskCost + kRowCost * g.rows;
-            part_load[w] += cost; load[w] += cost;
-            const std::vector<Task>& v = tasks[p][g.narrow];
-            const size_t lanes = std::min<size_t>(32, v.size() - g.from);
-            const int width = g.narrow ? wide / 2 : wide;
-            // order of the columns inside each lane's chunk: in each step different banks within a pass
-            std::vector<uint16_t> cols((size_t)32 * width, (uint16_t)zero[p]);
-            std::vector<int> pick((size_t)32 * width, -1);
-            std::vector<uint32_t> left(32, 0);
-            for (size_t l = 0; l < lanes; ++l) left[l] = (1u << (v[g.from + l].k1 - v[g.from + l].k0)) - 1u;
-            for (int k = 0; k < width; ++k)
-                for (int l0 = 0; l0 < 32; l0 += pass) {
-                    std::vector<int> used((size_t)banks, -1);
-                    for (int l = l0; l < l0 + pass; ++l) {
-                        if (!left[l]) continue;
-                        const Task& t = v[g.from + l];
-                        const uint8_t* ci = t.A->col_idx.data() + t.A->cidx_off[t.block] + t.k0;
-                        int best = -1, col = 0;
-                        for (int i = 0; i < t.k1 - t.k0; ++i) {
-                            if (!(left[l] >> i & 1u)) continue;
-                            const int c = t.col_base + ci[i], u = used[c % banks];
-                            if (best < 0) { best = i; col = c; }
-                            if (u < 0 || u == c) { best = i; col = c; break; }
-                        }
-                        used[col % banks] = col;
-                        left[l] &= ~(1u << best);
-                        cols[(size_t)l * width + k] = (uint16_t)col;
-                        pick[(size_t)l * width + k] = best;
-                    }
-                }
-            std::vector<uint8_t> w_bytes((size_t)g.rows * 32 * width * vs, 0);
-            std::vector<uint16_t> pos((size_t)((g.rows + 1) / 2) * 64, 0);
-            for (int r = 0; r < (g.rows + 1) / 2 * 2; ++r)
-                for (int l0 = 0; l0 < 32; l0 += pass) {
-                    std::vector<uint8_t> used((size_t)banks, 0);
-                    for (int l = l0; l < l0 + pass; ++l) {
-                        uint16_t place = (uint16_t)(idle + l);
-                        if ((size_t)l < lanes && r < v[g.from + l].r1 - v[g.from + l].r0) {
-                            const Task& t = v[g.from + l];
-                            const int row = t.row_base + t.A->row_idx[t.A->ridx_off[t.block] + t.r0 + r];
-                            std::vector<uint16_t>& fp = free_places[p][row];
-                            size_t best = fp.size() - 1;
-                            for (size_t i = fp.size(); i-- > 0;) if (!used[fp[i] % banks]) { best = i; break; }
-                            place = fp[best];
-                            fp[best] = fp.back();
-                            fp.pop_back();
-                            const uint8_t* src = t.A->val.data() + (t.A->val_off[t.block] + (uint64_t)(t.r0 + r) * t.A->n[t.block] + t.k0) * vs;
-                            uint8_t* dst = w_bytes.data() + ((size_t)r * 32 + l) * width * vs;
-                            // fp32 values, eight columns: two halves of 16 bytes per lane, [half][lane]
-                            for (int k = 0; k < width; ++k) {
-                                const int i = pick[(size_t)l * width + k];
-                                if (i < 0) continue;
-                                uint8_t* d = width * vs == 32 ? w_bytes.data() + (((size_t)r * 2 + k / 4) * 32 + l) * 16 + (k % 4) * 4 : dst + (size_t)k * vs;
-                                std::memcpy(d, src + (size_t)i * vs, vs);
-                            }
-                        }
-                        used[place % banks] = 1;
-                        pos[((size_t)(r / 2) * 32 + l) * 2 + (r & 1)] = place;
-                    }
-                }
-            R1Group d{};
-            d.cols_off = append(img->bytes, cols.data(), cols.size());
-            d.w_off = append(img->bytes, w_bytes.data(), w_bytes.size());
-            d.pos_off = append(img->bytes, pos.data(), pos.size());
-            d.rows = (uint16_t)g.rows; d.narrow = (uint16_t)g.narrow;
-            groups[w][p].push_back(d);
+            part_load[g.warp] += cost; load[g.warp] += cost;
+            const size_t width = g.narrow ? wide / 2 : wide;
+            o->bytes += 64 * width + (size_t)g.rows * 32 * width * vs + (size_t)((g.rows + 1) / 2) * 128;
         }
+        o->groups.insert(o->groups.end(), order.begin(), order.end());
+    }
+    o->bytes += pad_to(n_rows * sizeof(R1Row), 16) + o->groups.size() * sizeof(R1Group) + (size_t)kR1Warps * 8;
+    return CSB_OK;
+}
+
+// Lays one product out behind the image.
+void emit_op(const OpSource& s, const OpLayout& o, const int zero[2], int op, int BT, std::vector<uint8_t>& out) {
+    const int wide = r1_wide(BT), vs = val_size(s.A->val_dtype);
+    // lanes that share a pass over the banks, and the banks (in units of BT floats) they must keep apart
+    const int pass = BT == 1 ? 32 : 8, banks = std::max(32 / BT, 4);
+    const size_t idle = o.partials - 32;
+    std::vector<std::vector<uint16_t>> free_places[2];
+    for (int p = 0; p < 2; ++p) {
+        free_places[p].resize(o.n_rows);
+        for (size_t r = 0; r < o.n_rows; ++r) for (uint32_t i = 0; i < o.count[p][r]; ++i) free_places[p][r].push_back((uint16_t)(o.first[p][r] + i));
+    }
+    std::vector<R1Group> groups[kR1Warps][2];
+    for (const GroupRef& g : o.groups) {
+        const int p = g.part;
+        const std::vector<Task>& v = o.tasks[p][g.narrow];
+        const size_t lanes = std::min<size_t>(32, v.size() - g.from);
+        const int width = g.narrow ? wide / 2 : wide;
+        // order of the columns inside each lane's chunk: in each step different banks within a pass
+        std::vector<uint16_t> cols((size_t)32 * width, (uint16_t)zero[p]);
+        std::vector<int> pick((size_t)32 * width, -1);
+        std::vector<uint32_t> left(32, 0);
+        for (size_t l = 0; l < lanes; ++l) left[l] = (1u << (v[g.from + l].k1 - v[g.from + l].k0)) - 1u;
+        for (int k = 0; k < width; ++k)
+            for (int l0 = 0; l0 < 32; l0 += pass) {
+                std::vector<int> used((size_t)banks, -1);
+                for (int l = l0; l < l0 + pass; ++l) {
+                    if (!left[l]) continue;
+                    const Task& t = v[g.from + l];
+                    const uint8_t* ci = t.A->col_idx.data() + t.A->cidx_off[t.block] + t.k0;
+                    int best = -1, col = 0;
+                    for (int i = 0; i < t.k1 - t.k0; ++i) {
+                        if (!(left[l] >> i & 1u)) continue;
+                        const int c = t.col_base + ci[i], u = used[c % banks];
+                        if (best < 0) { best = i; col = c; }
+                        if (u < 0 || u == c) { best = i; col = c; break; }
+                    }
+                    used[col % banks] = col;
+                    left[l] &= ~(1u << best);
+                    cols[(size_t)l * width + k] = (uint16_t)col;
+                    pick[(size_t)l * width + k] = best;
+                }
+            }
+        std::vector<uint8_t> w_bytes((size_t)g.rows * 32 * width * vs, 0);
+        std::vector<uint16_t> pos((size_t)((g.rows + 1) / 2) * 64, 0);
+        for (int r = 0; r < (g.rows + 1) / 2 * 2; ++r)
+            for (int l0 = 0; l0 < 32; l0 += pass) {
+                std::vector<uint8_t> used((size_t)banks, 0);
+                for (int l = l0; l < l0 + pass; ++l) {
+                    uint16_t place = (uint16_t)(idle + l);
+                    if ((size_t)l < lanes && r < v[g.from + l].r1 - v[g.from + l].r0) {
+                        const Task& t = v[g.from + l];
+                        const int row = t.row_base + t.A->row_idx[t.A->ridx_off[t.block] + t.r0 + r];
+                        std::vector<uint16_t>& fp = free_places[p][row];
+                        size_t best = fp.size() - 1;
+                        for (size_t i = fp.size(); i-- > 0;) if (!used[fp[i] % banks]) { best = i; break; }
+                        place = fp[best];
+                        fp[best] = fp.back();
+                        fp.pop_back();
+                        const uint8_t* src = t.A->val.data() + (t.A->val_off[t.block] + (uint64_t)(t.r0 + r) * t.A->n[t.block] + t.k0) * vs;
+                        uint8_t* dst = w_bytes.data() + ((size_t)r * 32 + l) * width * vs;
+                        // fp32 values, eight columns: two halves of 16 bytes per lane, [half][lane]
+                        for (int k = 0; k < width; ++k) {
+                            const int i = pick[(size_t)l * width + k];
+                            if (i < 0) continue;
+                            uint8_t* d = width * vs == 32 ? w_bytes.data() + (((size_t)r * 2 + k / 4) * 32 + l) * 16 + (k % 4) * 4 : dst + (size_t)k * vs;
+                            std::memcpy(d, src + (size_t)i * vs, vs);
+                        }
+                    }
+                    used[place % banks] = 1;
+                    pos[((size_t)(r / 2) * 32 + l) * 2 + (r & 1)] = place;
+                }
+            }
+        R1Group d{};
+        d.cols_off = append(out, cols.data(), cols.size());
+        d.w_off = append(out, w_bytes.data(), w_bytes.size());
+        d.pos_off = append(out, pos.data(), pos.size());
+        d.rows = (uint16_t)g.rows; d.narrow = (uint16_t)g.narrow;
+        groups[g.warp][p].push_back(d);
     }
     std::vector<R1Group> all;
     std::vector<uint16_t> warp_desc;
@@ -218,12 +235,11 @@ int emit_op(const OpSource& s, const int zero[2], int op, int BT, Image* img) {
         warp_desc.push_back(0);
     }
     R1Op d{};
-    d.n_rows = (uint16_t)n_rows; d.units = (uint16_t)s.units; d.unit0 = (uint32_t)s.unit0; d.partials = (uint32_t)at;
-    d.rows_off = append(img->bytes, rows.data(), n_rows);
-    d.groups_off = append(img->bytes, all.data(), all.size());
-    d.warp_off = append(img->bytes, warp_desc.data(), warp_desc.size());
-    std::memcpy(img->bytes.data() + op * sizeof(R1Op), &d, sizeof d);
-    return CSB_OK;
+    d.n_rows = (uint16_t)o.n_rows; d.units = (uint16_t)s.units; d.unit0 = (uint32_t)s.unit0; d.partials = (uint32_t)o.partials;
+    d.rows_off = append(out, o.rows.data(), o.n_rows);
+    d.groups_off = append(out, all.data(), all.size());
+    d.warp_off = append(out, warp_desc.data(), warp_desc.size());
+    std::memcpy(out.data() + op * sizeof(R1Op), &d, sizeof d);
 }
 
 // Contiguous ranges of units, at most `parts` of them, of about equal cost; cuts at multiples of `grain`.
@@ -263,9 +279,37 @@ std::vector<double> row_weights(const csb_matrix* A) {
 
 }  // namespace
 
+R1Carve::R1Carve(const R1HostPlan& P, int cell, int max_in, int H, int S, int BT) {
+    size_t at = P.max_bytes;
+    auto room = [&](size_t floats) { const size_t o = at; at = (at + floats * 4 + 15) & ~(size_t)15; return (uint32_t)o; };
+    for (uint32_t& v : vu) v = room((size_t)(max_in + 1) * BT);
+    vr = room((size_t)(S + 1) * BT); vm = room(r1_ops(cell) == 2 ? (size_t)(H + 1) * BT : 0);
+    for (int op = 0; op < 2; ++op) part[op] = room(P.max_partials[op] * BT);
+    z[0] = room(4 * P.max_units * BT); z[1] = room(r1_ops(cell) == 2 ? P.max_units * BT : 0);
+    cs = room(P.max_units * BT); bias0 = room(4 * P.max_units); bias1 = room(P.max_units);
+    misc = room(4);
+    total = at;
+}
+
 int plan_rnn1_host(int cell, int L, const csb_matrix* const* W, const csb_matrix* const* Wp, const int* in_size, int H, int S, int BT, int n_ctas,
-                   R1HostPlan* out) {
+                   size_t smem_limit, R1HostPlan* out) {
     *out = R1HostPlan{};
+    // ---- What the weights take at least, whichever way they are dealt: their chunks' rows (values and a position) and
+    // partial sums.  If the CTAs' mean is past the limit already, nothing need be planned (two 2048-unit LSTM layers at
+    // 4x: 0.15 ms instead of 67; at 8x, where only the layouts below show it, 4.6 instead of 38).
+    {
+        const size_t wide = (size_t)r1_wide(BT);
+        double least = 0;
+        auto add = [&](const csb_matrix* A) {
+            for (int64_t b = 0; b < A->nblk; ++b) {
+                const size_t n = A->n[b], tail = n % wide, width = n / wide * wide + (tail == 0 ? 0 : tail <= wide / 2 ? wide / 2 : wide);
+                least += (double)A->m[b] * (double)(width * val_size(A->val_dtype) + (n + wide - 1) / wide * (2 + 4 * (size_t)BT));
+            }
+        };
+        int max_in = 0;
+        for (int l = 0; l < L; ++l) { add(W[l]); if (cell == kR1Lstmp) add(Wp[l]); max_in = std::max(max_in, in_size[l]); }
+        if (least / std::max(n_ctas, 1) + (double)R1Carve(*out, cell, max_in, H, S, BT).total > (double)smem_limit) return 1;
+    }
     const int G = r1_gates(cell, 0) + (cell == kR1GruRb ? 1 : 0);
     for (int l = 0; l < L; ++l) if (in_size[l] >= 65535 || S >= 65535 || H >= 65535) return 1;
     // ---- CTAs per layer in proportion to the weights
@@ -288,25 +332,49 @@ int plan_rnn1_host(int cell, int L, const csb_matrix* const* W, const csb_matrix
     }
     // ---- unit ranges: the granularity with the shortest longest CTA
     const int wide = r1_wide(BT);
-    auto best_cut = [&](const csb_matrix* A, const std::vector<double>& cost, int parts, int gates, int64_t stride, int split) {
-        std::vector<int> best;
-        double best_cost = 0;
-        for (int grain = 1; grain <= A->block_r; grain = grain == 1 ? std::max(2, A->block_r / 8) : grain * 2) {
-            if (grain > 1 && A->block_r % grain) continue;
-            const std::vector<int> cut = cut_units(cost, parts, grain, kR1MaxUnits);
-            if ((int)cut.size() - 1 > parts) continue;
-            double worst = 0;
-            for (size_t i = 0; i + 1 < cut.size(); ++i) worst = std::max(worst, range_cost({A, 0, stride, gates, cut[i], cut[i + 1] - cut[i], split}, wide));
-            if (best.empty() || worst < best_cost) { best = cut; best_cost = worst; }
-        }
-        return best;
+    struct Cut { const csb_matrix* A; const std::vector<double>* cost; int parts, gates; int64_t stride; int split, grain; std::vector<int> cut; double worst; };
+    std::vector<Cut> cuts;                                   // of every matrix, the granularities ascending
+    auto add_cuts = [&](const csb_matrix* A, const std::vector<double>& cost, int parts, int gates, int64_t stride, int split) {
+        for (int grain = 1; grain <= A->block_r; grain = grain == 1 ? std::max(2, A->block_r / 8) : grain * 2)
+            if (grain == 1 || A->block_r % grain == 0) cuts.push_back({A, &cost, parts, gates, stride, split, grain, {}, 0.0});
+    };
+    for (int l = 0; l < L; ++l) {
+        add_cuts(W[l], unit_cost[l], per[l], G, H, in_size[l]);
+        if (cell == kR1Lstmp) add_cuts(Wp[l], proj_cost[l], per[l], 1, S, 0);
+    }
+    std::atomic<int> next{0}, status{CSB_OK};
+    // items of work taken from a counter by a few host threads
+    auto in_parallel = [&](int n, auto&& item) {
+        next.store(0);
+        run_on_threads(std::max(1, std::min(8, n / 2)), [&]() {
+            for (int c; status.load() == CSB_OK && (c = next.fetch_add(1)) < n;) {
+                int rc;
+                try { rc = item(c); } catch (const std::bad_alloc&) { rc = CSB_ERR_ALLOC; }
+                if (rc != CSB_OK) status.store(rc);
+            }
+        });
+        if (status.load() == CSB_ERR_ALLOC) throw std::bad_alloc();
+        return status.load();
+    };
+    in_parallel((int)cuts.size(), [&](int i) {
+        Cut& c = cuts[i];
+        c.cut = cut_units(*c.cost, c.parts, c.grain, kR1MaxUnits);
+        if ((int)c.cut.size() - 1 > c.parts) { c.cut.clear(); return (int)CSB_OK; }
+        for (size_t k = 0; k + 1 < c.cut.size(); ++k)
+            c.worst = std::max(c.worst, range_cost({c.A, 0, c.stride, c.gates, c.cut[k], c.cut[k + 1] - c.cut[k], c.split}, wide));
+        return (int)CSB_OK;
+    });
+    auto best_cut = [&](const csb_matrix* A, const std::vector<double>& cost) {
+        const Cut* best = nullptr;
+        for (const Cut& c : cuts) if (c.A == A && c.cost == &cost && !c.cut.empty() && (!best || c.worst < best->worst)) best = &c;
+        return best ? best->cut : std::vector<int>();
     };
     struct Job { int layer, u0, units, p0, punits; };
     std::vector<Job> jobs;
     for (int l = 0; l < L; ++l) {
-        const std::vector<int> cu = best_cut(W[l], unit_cost[l], per[l], G, H, in_size[l]);
+        const std::vector<int> cu = best_cut(W[l], unit_cost[l]);
         std::vector<int> cp;
-        if (cell == kR1Lstmp) cp = best_cut(Wp[l], proj_cost[l], per[l], 1, S, 0);
+        if (cell == kR1Lstmp) cp = best_cut(Wp[l], proj_cost[l]);
         if (cu.empty() || (cell == kR1Lstmp && cp.empty())) return 1;
         const int n = std::max((int)cu.size(), (int)cp.size()) - 1;
         for (int i = 0; i < n; ++i) {
@@ -317,32 +385,42 @@ int plan_rnn1_host(int cell, int L, const csb_matrix* const* W, const csb_matrix
         }
         out->layer_ctas[l] = n;
     }
-    // ---- the CTAs' images, on a few host threads
+    // ---- the CTAs' layouts; what they take of shared memory; only then their images
     std::vector<Image> img(jobs.size());
-    std::atomic<int> next{0}, status{CSB_OK};
-    auto work = [&]() {
-        for (int c; status.load() == CSB_OK && (c = next.fetch_add(1)) < (int)jobs.size();) {
-            int rc = CSB_OK;
-            try {
-                const Job& j = jobs[c];
-                Image& I = img[c];
-                I.bytes.assign(sizeof(R1Header), 0);
-                const int zero[2] = {in_size[j.layer], S};
-                rc = emit_op({W[j.layer], 0, H, r1_gates(cell, 0), j.u0, j.units, in_size[j.layer]}, zero, 0, BT, &I);
-                if (rc == CSB_OK && cell == kR1GruRb) rc = emit_op({W[j.layer], 2 * (int64_t)H, H, 1, j.u0, j.units, in_size[j.layer]}, zero, 1, BT, &I);
-                if (rc == CSB_OK && cell == kR1Lstmp) {
-                    const int zero_m[2] = {0, H};
-                    rc = emit_op({Wp[j.layer], 0, S, 1, j.p0, j.punits, 0}, zero_m, 1, BT, &I);
-                }
-            } catch (const std::bad_alloc&) { rc = CSB_ERR_ALLOC; }
-            if (rc != CSB_OK) status.store(rc);
-        }
+    auto source = [&](const Job& j, int op) -> OpSource {
+        if (op == 0) return {W[j.layer], 0, H, r1_gates(cell, 0), j.u0, j.units, in_size[j.layer]};
+        if (cell == kR1GruRb) return {W[j.layer], 2 * (int64_t)H, H, 1, j.u0, j.units, in_size[j.layer]};
+        return {Wp[j.layer], 0, S, 1, j.p0, j.punits, 0};
     };
-    run_on_threads((int)std::min<size_t>(8, std::max<size_t>(1, jobs.size() / 8)), work);
-    if (status.load() == CSB_ERR_ALLOC) throw std::bad_alloc();
-    if (status.load() != CSB_OK) return status.load();
+    const int ops = r1_ops(cell);
+    if (in_parallel((int)jobs.size(), [&](int c) {
+            int rc = CSB_OK;
+            for (int op = 0; op < ops && rc == CSB_OK; ++op) rc = lay_out_op(source(jobs[c], op), BT, &img[c].op[op]);
+            return rc;
+        }) != CSB_OK) return status.load();
+    for (size_t c = 0; c < jobs.size(); ++c) {
+        size_t bytes = sizeof(R1Header);
+        for (int op = 0; op < ops; ++op) {
+            bytes += img[c].op[op].bytes;
+            out->max_partials[op] = std::max(out->max_partials[op], img[c].op[op].partials);
+        }
+        out->max_bytes = std::max(out->max_bytes, pad_to(bytes, 128));
+        out->max_units = std::max(out->max_units, (size_t)std::max(jobs[c].units, cell == kR1Lstmp ? jobs[c].punits : 0));
+    }
+    int max_in = 0;
+    for (int l = 0; l < L; ++l) max_in = std::max(max_in, in_size[l]);
+    if (R1Carve(*out, cell, max_in, H, S, BT).total > smem_limit) return 1;
+    if (in_parallel((int)jobs.size(), [&](int c) {
+            const Job& j = jobs[c];
+            std::vector<uint8_t>& bytes = img[c].bytes;
+            bytes.reserve(out->max_bytes);
+            bytes.assign(sizeof(R1Header), 0);
+            const int zero[2] = {in_size[j.layer], S}, zero_m[2] = {0, H};
+            for (int op = 0; op < ops; ++op) emit_op(source(j, op), img[c].op[op], cell == kR1Lstmp && op == 1 ? zero_m : zero, op, BT, bytes);
+            return (int)CSB_OK;
+        }) != CSB_OK) return status.load();
     // ---- exchange words: three elements each (unit by unit, the batch columns of a unit side by side), CTA by CTA
-    size_t base = 0, sum = 0;
+    size_t base = 0;
     const int last = r1_ops(cell) - 1;
     if ((size_t)std::max(H, S) * BT >= (1u << 24)) return 1;
     for (size_t c = 0; c < jobs.size(); ++c) {
@@ -354,20 +432,13 @@ int plan_rnn1_host(int cell, int L, const csb_matrix* const* W, const csb_matrix
             const bool proj = cell == kR1Lstmp && op == 1;
             const int e0 = (proj ? j.p0 : j.u0) * BT, n = (proj ? j.punits : j.units) * BT;
             for (int e = 0; e < n; e += 3) map.push_back((uint32_t)(e0 + e) | ((uint32_t)std::min(3, n - e) << 24));
-            out->max_units = std::max(out->max_units, (size_t)(proj ? j.punits : j.units));
-            out->max_partials[op] = std::max(out->max_partials[op], img[c].partials[op]);
         }
         img[c].bytes.resize(pad_to(img[c].bytes.size(), 128), 0);
         out->ctas.push_back({(uint32_t)(base / 16), (uint32_t)img[c].bytes.size(), j.layer, 0});
         base += img[c].bytes.size();
-        sum += img[c].bytes.size();
-        out->max_bytes = std::max(out->max_bytes, img[c].bytes.size());
-        out->max_rows = std::max(out->max_rows, img[c].rows);
     }
-    out->balance = out->max_bytes ? (double)sum / jobs.size() / out->max_bytes : 1.0;
-    out->bytes.resize(base);
-    base = 0;
-    for (Image& i : img) { std::memcpy(out->bytes.data() + base, i.bytes.data(), i.bytes.size()); base += i.bytes.size(); std::vector<uint8_t>().swap(i.bytes); }
+    out->bytes.reserve(base);
+    for (Image& i : img) { out->bytes.insert(out->bytes.end(), i.bytes.begin(), i.bytes.end()); std::vector<uint8_t>().swap(i.bytes); }
     return CSB_OK;
 }
 

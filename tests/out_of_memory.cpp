@@ -48,7 +48,7 @@ int main(int argc, char** argv) {
         case 2: rc = csb_panel_dump(A, 148, 32, 16384, info, nullptr, 0, nullptr, 0); break;
         case 3: rc = csb_spmm_plan_dump(A, 32, 148, info, nullptr, 0, nullptr, 0, nullptr, 0, nullptr, 0); break;
         case 4: { RuHostPlan P; try { rc = plan_unit_host(kR1Lstm, 1, M, nullptr, &I, R / 4, R / 4, 1, 64, &P); } catch (const std::bad_alloc&) { rc = CSB_ERR_ALLOC; } break; }
-        default: { R1HostPlan P; try { rc = plan_rnn1_host(kR1Lstm, 1, M, nullptr, &I, R / 4, R / 4, 1, 64, &P); } catch (const std::bad_alloc&) { rc = CSB_ERR_ALLOC; } break; }
+        default: { R1HostPlan P; try { rc = plan_rnn1_host(kR1Lstm, 1, M, nullptr, &I, R / 4, R / 4, 1, 64, (size_t)1 << 40, &P); } catch (const std::bad_alloc&) { rc = CSB_ERR_ALLOC; } break; }
     }
     g_left = -1;
     return rc == CSB_OK || rc == CSB_ERR_ALLOC ? 0 : 4;
