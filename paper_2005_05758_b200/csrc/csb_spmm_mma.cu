@@ -278,11 +278,11 @@ __global__ void __launch_bounds__(kWarpsOf<NT> * 32, 1) csb_spmm_tile_kernel(con
     auto release_x = [&]() {
         __syncwarp();
         uint32_t last = 0u;
-        // A plain (relaxed) add: the loads this warp made from the slot have all returned (the tensor
-        // instructions that used them have been issued), and a fence here would also wait for the
-        // weight copies this lane has in flight from HBM.
+        // The add releases this warp's reads of the slot and, for the last warp, acquires the others' before its
+        // copy overwrites the slot (a relaxed add would lean on the order in which the hardware happens to do a
+        // warp's accesses to shared memory; 60.2 against 60.1 us, 8192 x 8192 at 4x, batch 64).
         if (lane == 0) {
-            last = atomicAdd(&xcnt[xs], 1u) == (uint32_t)kSpmmWarps - 1u;
+            last = atom_add_acq_rel_shared(&xcnt[xs], 1u) == (uint32_t)kSpmmWarps - 1u;
             if (last) *reinterpret_cast<volatile uint32_t*>(&xcnt[xs]) = 0u;
         }
         last = __shfl_sync(0xffffffffu, last, 0);
