@@ -128,11 +128,8 @@ int plan_fixed(csb_matrix* A) {
     CSB_CUDA(cudaGetDevice(&prev));
     CSB_CUDA(cudaSetDevice(A->device));
     struct Restore { int prev; ~Restore() { cudaSetDevice(prev); } } restore{prev};
-    cudaDeviceProp prop{};
-    CSB_CUDA(cudaGetDeviceProperties(&prop, A->device));
-    if (prop.major < 10) { set_error("device %d is sm_%d%d; this library is built for sm_100a", A->device, prop.major, prop.minor); return CSB_ERR_UNSUPPORTED; }
-    A->sm_count = prop.multiProcessorCount;
-    A->smem_optin = prop.sharedMemPerBlockOptin;
+    const int found = query_device(A);
+    if (found != CSB_OK) return found;
     FixedPlan* P = new (std::nothrow) FixedPlan();
     if (!P) { set_error("out of host memory"); return CSB_ERR_ALLOC; }
     A->fixed = P;
@@ -140,8 +137,10 @@ int plan_fixed(csb_matrix* A) {
     CSB_CUDA(cudaHostAlloc((void**)&Q.h_status, 4, cudaHostAllocMapped));
     *Q.h_status = 0;
     CSB_CUDA(cudaHostGetDevicePointer((void**)&Q.d_status, Q.h_status, 0));
-    int rc;
-    if ((rc = plan_panels(A)) != CSB_OK) return rc;
+    PanelHostPlan H;
+    int rc = plan_panels(A, &H);
+    if (rc == CSB_OK && (rc = upload_panels(A, H)) != CSB_OK) return rc;
+    if (rc != CSB_OK && rc != 1) return rc;
     if (A->panel) return CSB_OK;
     if ((rc = upload_arr(A->m.data(), A->m.size(), &P->d_m)) != CSB_OK) return rc;
     if ((rc = upload_arr(A->n.data(), A->n.size(), &P->d_n)) != CSB_OK) return rc;

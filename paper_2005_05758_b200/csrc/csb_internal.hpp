@@ -332,14 +332,16 @@ struct PanelPlan {                         // device side
     int64_t stream_bytes = 0;
     double balance = 1.0, warp_balance = 1.0;
 };
-int plan_panels(csb_matrix* A);            // after plan_product; leaves A->panel NULL when the path does not apply
+int plan_panels(const csb_matrix* A, PanelHostPlan* out);   // on the host, after query_device; 1: the path does not apply
+int upload_panels(csb_matrix* A, const PanelHostPlan& H);   // leaves A->panel NULL when the kernel does not hold the plan
 void free_panels(csb_matrix* A);
 bool panels_applicable(const csb_matrix* A, int batch);    // and faster than launch_product
 int launch_panels(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
 int launch_panels_q16(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch, int64_t* acc, int64_t ldy, void* stream);
 
 // csb_product.cu
-int plan_product(csb_matrix* A);           // plans, uploads, fills A->product
+int query_device(csb_matrix* A);           // SMs and shared memory of A's device
+int plan_product(csb_matrix* A);           // after query_device; plans, uploads, fills A->product
 void free_product(csb_matrix* A);
 int launch_product(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
                    void* stream);

@@ -628,16 +628,17 @@ static PanelKernel panel_kernel(int val_dtype, int v) {
     return val_dtype == CSB_F16 ? pick_panel_kernel<CSB_F16>(v) : val_dtype == CSB_F32 ? pick_panel_kernel<CSB_F32>(v) : pick_panel_kernel<CSB_Q16>(v);
 }
 
-int plan_panels(csb_matrix* A) {
-    if (env_int("CSB_NO_PANEL", 0)) return CSB_OK;
+static int panel_stage() { return 1 << std::min(15, std::max(13, log2_floor(env_int("CSB_PANEL_STAGE", 16384)))); }
+
+int plan_panels(const csb_matrix* A, PanelHostPlan* out) {
+    if (env_int("CSB_NO_PANEL", 0)) return 1;
     const int warps = std::min(32, std::max(1, env_int("CSB_PANEL_WARPS", 32)));
-    int stage = env_int("CSB_PANEL_STAGE", 16384);
-    stage = 1 << std::min(15, std::max(13, log2_floor(stage)));
     const int ctas = std::min<int>(kMaxPanelCtas, A->opts.ctas > 0 ? A->opts.ctas : A->sm_count);
-    PanelHostPlan H;
-    const int hrc = plan_panels_host(A, ctas, warps, stage, 16384, 8192 / warps, &H);
-    if (hrc == 1) return CSB_OK;
-    if (hrc != CSB_OK) return hrc;
+    return plan_panels_host(A, ctas, warps, panel_stage(), 16384, 8192 / warps, out);
+}
+
+int upload_panels(csb_matrix* A, const PanelHostPlan& H) {
+    const int warps = H.warps, stage = H.stage_bytes;
     PanelPlan* P = new PanelPlan();
     P->ctas = (int)H.cta.size(); P->warps = warps; P->stage_bytes = stage;
     P->max_xg = (int)H.max_xg; P->max_meta = (int)H.max_meta; P->max_rows = (int)std::max<size_t>(H.max_rows, 1);

@@ -332,16 +332,23 @@ static int fit_warps(const csb_matrix* A, int want, int BT, int cols_in_smem, si
     return 0;
 }
 
+int query_device(csb_matrix* A) {
+    int major = 0, minor = 0, sms = 0, smem = 0;
+    CSB_CUDA(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, A->device));
+    CSB_CUDA(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, A->device));
+    if (major < 10) { set_error("device %d is sm_%d%d; this library is built for sm_100a", A->device, major, minor); return CSB_ERR_UNSUPPORTED; }
+    CSB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A->device));
+    CSB_CUDA(cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, A->device));
+    A->sm_count = sms;
+    A->smem_optin = (size_t)smem;
+    return CSB_OK;
+}
+
 int plan_product(csb_matrix* A) {
     ProductPlan& P = A->product;
     int dev_prev = 0;
     CSB_CUDA(cudaGetDevice(&dev_prev));
     CSB_CUDA(cudaSetDevice(A->device));
-    cudaDeviceProp prop{};
-    CSB_CUDA(cudaGetDeviceProperties(&prop, A->device));
-    if (prop.major < 10) { set_error("device %d is sm_%d%d; this library is built for sm_100a", A->device, prop.major, prop.minor); return CSB_ERR_UNSUPPORTED; }
-    A->sm_count = prop.multiProcessorCount;
-    A->smem_optin = prop.sharedMemPerBlockOptin;
     const int ctas = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
     const int wpc = std::min(16, A->opts.warps_per_cta > 0 ? A->opts.warps_per_cta : 16);
     P.stage_bytes = ((A->opts.stage_bytes > 0 ? A->opts.stage_bytes : 4096) + 15) & ~15;
