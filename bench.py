@@ -606,7 +606,7 @@ def fixed_bench(binding, torch, dev, hbm, with_cpu, reps=10):
         alg = v["nnz"] * 2 + len(v["row_idx"]) + len(v["col_idx"]) + 6 * len(v["m"]) + m.cols * 2 * batch + m.rows * 8 * batch
         out.append({"rate": rate, "batch": batch, "nnz": int(v["nnz"]), "us": round(us, 3), "algorithmic_bytes": int(alg), "GBps": round(alg / us / 1e3, 1),
                     "frac_hbm_measured": round(alg / us / 1e3 / hbm, 4), "GMACs": round(v["nnz"] * batch / us / 1e3, 1), "equals_oracle": exact,
-                    "kernel": "csb_q16_kernel", "copies": ncopy})
+                    "kernel": "csb_panel_kernel" if As[0].info()["panel_ctas"] else "csb_q16_kernel", "copies": ncopy})
         for a in As:
             a.free()
     return out, launches

@@ -344,6 +344,13 @@ int csb_gru_reset_before_forward(int n_layers, const csb_matrix_t* const* W, con
 void csb_test_barrier_hook(unsigned int extra_arrivals, unsigned long long limit_ns);
 
 /*
+ * csb_last_recurrent_path -- testing aid (the paper has no counterpart): which kernels served the calling thread's most
+ * recent recurrent call: 1 the unit loop, 2 the block loop (both resident), 3 batched steps over packed inputs, 4 batched
+ * steps over fp32 inputs, 5 the persistent kernel, 6 steps of a cell variant; 0 before the first call.
+ */
+int csb_last_recurrent_path(void);
+
+/*
  * csb_plan_dump -- inspection / testing aid (the paper has no counterpart): plan the bare product
  * for a persistent grid of `ctas` x `warps_per_cta` warps and ring stages of `stage_bytes` bytes,
  * on the host only (works for handles encoded with device = -1), and copy the planned device
@@ -363,18 +370,18 @@ int csb_plan_dump(const csb_matrix_t* A, int ctas, int warps_per_cta, int stage_
 
 /*
  * csb_panel_dump -- inspection / testing aid (the paper has no counterpart): plan the panel layout
- * that csb_spmv streams for fp16 matrices (one panel per CTA, which owns a contiguous range of
- * output rows: bookkeeping, then the re-tiled kernel-matrix rows), on the host only, and copy it
- * out so that layout and schedule can be checked without a GPU.
+ * that csb_spmv, csb_spmm with few vectors and csb_spmm_q16 stream (one panel per CTA, which owns a
+ * contiguous range of output rows: bookkeeping, then the re-tiled kernel-matrix rows), on the host
+ * only, and copy it out so that layout and schedule can be checked without a GPU.
  *   info_out    host, int64[8]: CTAs, bytes of all panels, 0, largest bookkeeping part, largest
  *               gathered-input count, most output rows per CTA, and the CTA-level and warp-level
  *               balance (mean / max of the modelled cost) times 1e6.
  *   panels_out  host, `panels_cap` bytes, or NULL;  cta_out  host, four uint32 per CTA (offset of
  *               the panel in 16-byte units, bytes of bookkeeping, bytes of values, output rows),
  *               `cta_cap` entries, or NULL.
- * Errors: UNSUPPORTED when the layout does not apply (fp32 values, block_c > 128, cols > 16384,
- * stage_bytes not a power of two >= 8192, or a panel beyond the kernel's limits), INVALID_ARG for
- * a buffer that is too small; call once with NULL buffers to learn the sizes.
+ * Errors: UNSUPPORTED when the layout does not apply (block_c > 128, cols > 16384, stage_bytes not
+ * a power of two >= 8192, or a panel beyond the kernel's limits), INVALID_ARG for a buffer that is
+ * too small; call once with NULL buffers to learn the sizes.
  */
 int csb_panel_dump(const csb_matrix_t* A, int ctas, int warps_per_cta, int stage_bytes, int64_t* info_out,
                    uint8_t* panels_out, int64_t panels_cap, uint32_t* cta_out, int64_t cta_cap);
@@ -382,10 +389,10 @@ int csb_panel_dump(const csb_matrix_t* A, int ctas, int warps_per_cta, int stage
 /*
  * csb_spmm_plan_dump -- inspection / testing aid (the paper has no counterpart): plan the
  * tensor-core layout of the batched product for a pass of `batch` columns (the class of batch sizes
- * <= 8, <= 16 or more) and `sm_count` SMs on the host only and copy it out, so that the layout and
- * the block -> CTA -> warp schedule can be checked without a GPU.  A CTA covers RG consecutive
- * block-rows times a range of block-columns and has W warps (32 for up to 8 batch columns, else
- * 16), each working for one block-row of the group; S CTAs share a row group.  Weight stream
+ * <= 8, <= 16, <= 32 or more; csb_spmm uses the last three, recurrent stacks the first three) and
+ * `sm_count` SMs on the host only and copy it out, so that the layout and the block -> CTA -> warp
+ * schedule can be checked without a GPU.  A CTA covers RG consecutive block-rows times a range of
+ * block-columns and has W warps (32, 16, 16 and 8 in these classes), each working for one block-row of the group; S CTAs share a row group.  Weight stream
  * cta * W + w belongs to warp w.
  *   info_out          host, int64[8]: CTAs, chunks, stream bytes, RG, 8-column batch tiles per warp
  *                     + 256 * W + 65536 * G (an input tile spans G block-columns), S, and the

@@ -236,9 +236,9 @@ int csb_panel_dump(const csb_matrix_t* A, int ctas, int warps_per_cta, int stage
     if (!A || !info_out || ctas < 1 || warps_per_cta < 1 || warps_per_cta > 32) { set_error("csb_panel_dump: bad argument"); return CSB_ERR_INVALID_ARG; }
     PanelHostPlan H;
     int rc;
-    try { rc = A->val_dtype == CSB_F16 ? plan_panels_host(A, ctas, warps_per_cta, stage_bytes, 16384, 8192 / warps_per_cta, &H) : 1; }
+    try { rc = plan_panels_host(A, ctas, warps_per_cta, stage_bytes, 16384, 8192 / warps_per_cta, &H); }
     catch (const std::bad_alloc&) { set_error("out of host memory while planning"); return CSB_ERR_ALLOC; }
-    if (rc == 1) { set_error("the panel layout does not apply to this matrix (fp16 values, block_c <= 128, cols <= 16384, power-of-two stage >= 8192)"); return CSB_ERR_UNSUPPORTED; }
+    if (rc == 1) { set_error("the panel layout does not apply to this matrix (block_c <= 128, cols <= 16384, power-of-two stage >= 8192)"); return CSB_ERR_UNSUPPORTED; }
     if (rc != CSB_OK) return rc;
     info_out[0] = (int64_t)H.cta.size(); info_out[1] = (int64_t)H.bytes.size(); info_out[2] = 0;
     info_out[3] = (int64_t)H.max_meta; info_out[4] = (int64_t)H.max_xg; info_out[5] = (int64_t)H.max_rows;

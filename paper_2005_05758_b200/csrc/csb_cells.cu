@@ -262,6 +262,7 @@ static int cell_forward(int kind, int L, const csb_matrix_t* const* W, const csb
             g_cell_plans.push_back(std::move(np));
         }
     }
+    note_recurrent_path(kPathCellSteps);
     cudaStream_t st = (cudaStream_t)stream;
     const bool host_io = (flags & CSB_FLAG_HOST_IO) != 0;
     const int I0 = in_size[0];

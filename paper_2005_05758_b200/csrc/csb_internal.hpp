@@ -203,7 +203,7 @@ int plan_rnn_host(int gates, int n_layers, const csb_matrix* const* Wm, const in
 
 // ---- tensor-core SpMM path (csb_spmm_plan.cpp, csb_spmm_mma.cu) ----
 // The matrix is cut into CTA tiles: a group of RG consecutive block-rows times a contiguous range of
-// block-columns.  The warps of a CTA (16, or 32 for batches of up to 8) are dealt to the block-rows of its group in proportion to
+// block-columns.  The warps of a CTA (spmm_warps()) are dealt to the block-rows of its group in proportion to
 // their work; a warp keeps the block_r x batch outputs of its block-row in registers for the whole
 // range, and the blocks of a block-row go, in block-column order, to whichever of its warps has the
 // least work so far.  A warp's weights come through its own ring of bulk copies as items; the batch
@@ -230,9 +230,11 @@ struct SpmmCta {
 };
 static_assert(sizeof(SpmmCta) == 48, "three 16-byte words");
 // Warps per CTA: the 16 accumulator registers of one 8-column batch tile leave room for 32 warps per
-// SM, which halves the chain of dependent work a warp has to get through; wider tiles allow 16.
+// SM, which halves the chain of dependent work a warp has to get through; wider tiles allow 16, the widest 8.
 inline int spmm_warps(int NT) { return NT == 1 ? 32 : NT == 8 ? 8 : 16; }   // (a tile of 64 columns: 128 accumulators a thread)
-// Batch classes: how many 8-column batch tiles a warp carries.  A pass covers 8 * NT <= 32 batch columns.
+// Batch classes: how many 8-column batch tiles a warp carries.  A pass covers 8 * NT <= 64 batch columns: products of
+// up to 16, 32 and more vectors run with NT = 2, 4 and 8 (8 where that plan fits, else 4), recurrent stacks of up to 8, 16
+// and 32 rows with NT = 1, 2 and 4.
 inline int spmm_nt(int batch) { return batch <= 8 ? 1 : batch <= 16 ? 2 : 4; }
 inline int spmm_class_index(int batch) { return batch <= 8 ? 0 : batch <= 16 ? 1 : 2; }
 inline int spmm_pitch(int NT) { return NT * 32 + 16; }   // bytes of one packed input column: hi parts, lo parts, 16 spare
@@ -361,6 +363,8 @@ int launch_fixed(const csb_matrix* A, const int16_t* Xq, int64_t ldx, int batch,
 void drop_cell_plans(const csb_matrix* A); // forget cached plans of the cell variants that use A
 
 // csb_rnn.cu
+enum RecurrentPath { kPathUnitLoop = 1, kPathBlockLoop, kPathStepsPacked, kPathSteps, kPathPersistent, kPathCellSteps };
+void note_recurrent_path(RecurrentPath path);   // for csb_last_recurrent_path
 void drop_rnn_plans(const csb_matrix* A);  // forget cached time-loop plans that use A
 
 // csb_rnn_step.cu -- batch >= 16 (>= 8 for big layers): one timestep at a time, products on tensor cores

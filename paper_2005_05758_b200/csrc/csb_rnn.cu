@@ -919,6 +919,7 @@ static int rnn_forward(int gates, int L, const csb_matrix_t* const* W, const flo
     g_rnn_clocks = d_rclocks;
     g_rnn_clock_ctas = P->n_ctas;
 #endif
+    note_recurrent_path(kPathPersistent);
     int rc;
     const bool half = P->val_dtype == CSB_F16;
     if (P->BT == 1) rc = half ? dispatch_rnn_gw<__half, 1>(P, a, st) : dispatch_rnn_gw<float, 1>(P, a, st);
@@ -940,6 +941,10 @@ static int rnn_forward(int gates, int L, const csb_matrix_t* const* W, const flo
     return CSB_OK;
 }
 
+static thread_local int g_path = 0;
+void note_recurrent_path(RecurrentPath path) { g_path = path; }
+int recurrent_path() { return g_path; }
+
 void barrier_test_hook(unsigned int* extra, unsigned long long* ns) { *extra = g_barrier_extra; *ns = g_barrier_ns; }
 
 void set_barrier_test_hook(unsigned int extra, unsigned long long ns) {
@@ -960,6 +965,8 @@ int csb_gru_forward(int n_layers, const csb_matrix_t* const* W, const float* con
                     const float* h0, float* y, float* hT, unsigned flags, void* stream) {
     return csb::guarded([&] { return csb::rnn_forward(3, n_layers, W, bias, x, T, B, h0, nullptr, y, hT, nullptr, flags, stream); });
 }
+
+int csb_last_recurrent_path(void) { return csb::recurrent_path(); }
 
 void csb_test_barrier_hook(unsigned int extra_arrivals, unsigned long long limit_ns) {
     csb::set_barrier_test_hook(extra_arrivals, limit_ns);

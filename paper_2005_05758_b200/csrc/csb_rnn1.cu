@@ -265,6 +265,7 @@ int rnn1_forward(int cell, int L, const csb_matrix* const* W, const csb_matrix* 
         }
     }
     if (P->unusable) return 1;
+    note_recurrent_path(P->unit_loop ? kPathUnitLoop : kPathBlockLoop);
     cudaStream_t st = (cudaStream_t)stream;
     const bool host_io = (flags & CSB_FLAG_HOST_IO) != 0, has_c = cell == kR1Lstm || cell == kR1Lstmp;
     const size_t nx = (size_t)T * B * in_size[0], ny = y ? (size_t)T * B * S : 0, nh = (size_t)L * B * S, nc = has_c ? (size_t)L * B * H : 0;

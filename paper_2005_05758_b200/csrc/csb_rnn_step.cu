@@ -274,6 +274,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             g_step_plans.push_back(std::move(np));
         }
     }
+    note_recurrent_path(P->pitch ? kPathStepsPacked : kPathSteps);
     cudaStream_t st = (cudaStream_t)stream;
     const bool host_io = (flags & CSB_FLAG_HOST_IO) != 0;
     const int I0 = in_size[0];

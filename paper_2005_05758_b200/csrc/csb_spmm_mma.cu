@@ -5,7 +5,7 @@
 // on this path where tensor cores apply.  How it is laid out here:
 //
 //   * A warp works for one block-row over a range of block-columns and keeps that block-row's
-//     outputs, all block_r rows x up to 32 batch columns, in the accumulator registers of
+//     outputs, all block_r rows x up to 64 batch columns, in the accumulator registers of
 //     mma.sync.m16n8k16 for the whole range (several warps share a block-row's blocks; their sums
 //     meet once, at the end).  The kernel matrix is the A operand with its kept rows put back at their
 //     RowIdx positions: a lane finds the stored row behind an output row with a population count
@@ -26,8 +26,8 @@
 //     is divided between S CTAs these are launched as one thread-block cluster and add their sums
 //     through distributed shared memory, every CTA for a share of the rows and in the order of the
 //     ranges, so results are bit-reproducible and no scratch in global memory is needed.
-//   * More than 32 batch columns are served in passes of 32 (the weights of the later passes come
-//     from L2).
+//   * More than 32 batch columns go through in tiles of 64 on 8 warps a CTA, or, where that plan does
+//     not fit, in passes of 32; more than 64 in passes (the weights of the later ones come from L2).
 #include <algorithm>
 #include <cstdio>
 #include <mutex>
@@ -844,14 +844,15 @@ extern "C" int csb_spmm_plan_dump(const csb_matrix_t* A, int batch, int sm_count
     using namespace csb;
     clear_error();
     if (!A || !info_out || batch < 1 || sm_count < 1) { set_error("csb_spmm_plan_dump: bad argument"); return CSB_ERR_INVALID_ARG; }
+    const int NT = batch > 32 ? 8 : spmm_nt(batch);
     SpmmHostPlan H;
     int rc;
-    try { rc = plan_spmm_host(A, spmm_nt(batch), sm_count, 0, &H); }
+    try { rc = plan_spmm_host(A, NT, sm_count, 0, &H); }
     catch (const std::bad_alloc&) { set_error("out of host memory while planning"); return CSB_ERR_ALLOC; }
     if (rc == 1) { set_error("the tensor-core layout does not apply to this matrix (fp16 values, block_r <= 64)"); return CSB_ERR_UNSUPPORTED; }
     if (rc != CSB_OK) return rc;
     info_out[0] = (int64_t)H.ctas.size(); info_out[1] = (int64_t)H.chunks.size(); info_out[2] = (int64_t)H.bytes.size();
-    info_out[3] = H.RG; info_out[4] = spmm_nt(batch) | (spmm_warps(spmm_nt(batch)) << 8) | (spmm_tile_blocks(A->block_c) << 16); info_out[5] = H.S; info_out[6] = (int64_t)(H.warp_balance * 1e6);
+    info_out[3] = H.RG; info_out[4] = NT | (spmm_warps(NT) << 8) | (spmm_tile_blocks(A->block_c) << 16); info_out[5] = H.S; info_out[6] = (int64_t)(H.warp_balance * 1e6);
     info_out[7] = (int64_t)(H.balance * 1e6);
     if (stream_out) {
         if (stream_cap < (int64_t)H.bytes.size()) { set_error("stream buffer too small"); return CSB_ERR_INVALID_ARG; }

@@ -73,11 +73,11 @@ def test_cfg4_shape_sampled_block_columns():
 
 
 @pytest.mark.parametrize("R,C,br,bc,pr,law", [
-    (9000, 2100, 64, 64, 0.75, "normal"),      # three chunks of block-columns; more row segments than a selection keeps in registers
+    (9000, 2100, 64, 64, 0.75, "normal"),      # more row segments than a selection keeps in registers
     (8192, 1090, 32, 64, 0.9, "coarse"),       # exact ties by the hundred: the radix selection
     (8193, 1030, 64, 256, 0.6, "normal"), (130, 300, 16, 5, 0.75, "normal"), (70, 515, 33, 16, 0.8, "normal"), (515, 70, 200, 8, 0.5, "coarse"),
     (300, 200, 40, 17, 0.7, "huge")])
-def test_chunks_widths_and_selections(R, C, br, bc, pr, law):
+def test_widths_edges_and_selections(R, C, br, bc, pr, law):
     W = np.random.default_rng(R * C).standard_normal((R, C)).astype(np.float32)
     if law == "coarse":
         W = np.round(W).astype(np.float32)

@@ -134,12 +134,16 @@ def test_resume_equals_one_call_bitwise_and_host_io():
 
 
 @pytest.mark.parametrize("B,I,H,L,br,bc", [(16, 40, 48, 2, 16, 16), (32, 153, 160, 1, 32, 32), (40, 70, 192, 2, 64, 32), (8, 200, 512, 1, 32, 32)])
-def test_lstm_large_batch_runs_step_by_step_on_tensor_cores(B, I, H, L, br, bc):
+def test_lstm_large_batch_runs_step_by_step_on_tensor_cores(monkeypatch, B, I, H, L, br, bc):
     # batches of 16 and more take the path of one product (tensor cores) + one gate kernel per layer
-    # and step; bias, initial states, resumption and host I/O as for the persistent kernel
+    # and step (8 where no resident loop holds the layers); bias, initial states, resumption and host I/O
+    # as for the persistent kernel
+    if B <= 8:
+        monkeypatch.setenv("CSB_RNN_NO_RNN1", "1")
     w = workloads.make_rnn_workload(31, "lstm", I, H, L, br, bc, "lognormal", rate=4.0, T=6, B=B, w_std=0.15,
                                     bias_std=0.2, state_std=0.4)
     y1, h1, c1 = check(w)
+    assert binding.lib.csb_last_recurrent_path() == (3 if B <= 32 else 4)
     y2, h2, c2 = run(w, chunks=[(0, 2), (2, 6)])
     assert np.array_equal(y1, y2) and np.array_equal(h1, h2) and np.array_equal(c1, c2)
     y3, h3, c3 = run(w, host_io=True)
@@ -171,27 +175,30 @@ def test_step_by_step_packed_inputs_equal_the_fp32_buffers(monkeypatch, cell, B,
 
 @pytest.mark.parametrize("cell,B,I,H,L,br", [("lstm", 32, 153, 512, 2, 32), ("lstm", 16, 40, 48, 2, 16), ("gru", 16, 70, 512, 2, 32),
                                              ("gru", 8, 300, 512, 1, 32), ("lstm", 24, 64, 256, 3, 64)])
-def test_one_launch_time_loop_equals_the_launches(monkeypatch, cell, B, I, H, L, br):
-    # CSB_RNN_STEP_LOOP=1: all steps of all layers in one cooperative launch of the product kernel
-    # (product pass, grid barrier, gates, grid barrier); the same arithmetic in the same order
+def test_wavefront_of_layers_resumes_bitwise(monkeypatch, cell, B, I, H, L, br):
+    # the layers run a step behind one another: a sequence cut anywhere, down to single steps, gives the bits of one call
+    monkeypatch.setenv("CSB_RNN_NO_RNN1", "1")
     w = workloads.make_rnn_workload(34, cell, I, H, L, br, br, "lognormal", rate=4.0, T=9, B=B, w_std=0.15,
                                     bias_std=0.2, state_std=0.4)
     ya, ha, ca = check(w)
-    monkeypatch.setenv("CSB_RNN_STEP_LOOP", "1")
-    yb, hb, cb = check(w)
-    assert np.array_equal(ya, yb) and np.array_equal(ha, hb)
-    if cell == "lstm":
-        assert np.array_equal(ca, cb)
-    yc, hc, cc = run(w, chunks=[(0, 4), (4, 9)])
-    assert np.array_equal(ya, yc) and np.array_equal(ha, hc)
+    assert binding.lib.csb_last_recurrent_path() == 3
+    for cuts in ([(0, 4), (4, 9)], [(t, t + 1) for t in range(9)]):
+        yb, hb, cb = run(w, chunks=cuts)
+        assert np.array_equal(ya, yb) and np.array_equal(ha, hb)
+        if cell == "lstm":
+            assert np.array_equal(ca, cb)
 
 
 @pytest.mark.parametrize("B,I,H,L,br,bc", [(16, 40, 48, 2, 16, 16), (20, 39, 100, 1, 32, 32), (33, 70, 192, 2, 64, 32), (8, 300, 512, 1, 32, 32)])
-def test_gru_batch_runs_step_by_step_on_tensor_cores(B, I, H, L, br, bc):
-    # GRU from batch 16 (from batch 8 for layers of 100 k weights and more): one product over 2B rows ([u ; 0] and [0 ; h]) keeps the candidate's two parts apart
+def test_gru_batch_runs_step_by_step_on_tensor_cores(monkeypatch, B, I, H, L, br, bc):
+    # GRU from batch 16 (from batch 8 for layers of 100 k weights and more, where no resident loop holds them): one
+    # product over 2B rows ([u ; 0] and [0 ; h]) keeps the candidate's two parts apart
+    if B <= 8:
+        monkeypatch.setenv("CSB_RNN_NO_RNN1", "1")
     w = workloads.make_rnn_workload(41, "gru", I, H, L, br, bc, "lognormal", rate=4.0, T=6, B=B, w_std=0.15,
                                     bias_std=0.2, state_std=0.4)
     y1, h1, _ = check(w)
+    assert binding.lib.csb_last_recurrent_path() == (3 if B <= 16 else 4)
     y2, h2, _ = run(w, chunks=[(0, 2), (2, 6)])
     assert np.array_equal(y1, y2) and np.array_equal(h1, h2)
     y3, h3, _ = run(w, host_io=True)

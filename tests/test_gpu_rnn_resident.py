@@ -12,6 +12,8 @@ from paper_2005_05758_b200 import binding
 
 pytestmark = pytest.mark.gpu
 
+UNIT_LOOP, BLOCK_LOOP, STEPS_PACKED, STEPS, PERSISTENT, CELL_STEPS = range(1, 7)      # csb_last_recurrent_path
+
 SIZES = [   # input, hidden, layers, block, steps, batch, values, per-block keep range
     (1, 1, 1, 8, 3, 1, "f16", (1.0, 1.0)),
     (39, 17, 2, 16, 45, 1, "f16", (0.3, 0.9)),
@@ -35,6 +37,29 @@ def test_edges_of_units_columns_and_exchange(monkeypatch, cell, I, H, L, br, T, 
     w = workloads.make_rnn_workload(31, cell, I, H, L, br, br, "uniform", lo=keep[0], hi=keep[1], T=T, B=B,
                                     w_std=0.5 / max(1.0, (0.1 * (I + H)) ** 0.5), val_dtype=vd, bias_std=0.1, state_std=0.5, **extra)
     (rnn if cell in ("lstm", "gru") else cells).check(w)
+    # (the block loop is not built for eight columns of fp32 values: the persistent kernel or the cells' steps take those)
+    want = UNIT_LOOP if not other else BLOCK_LOOP if (B, vd) != (8, "f32") else PERSISTENT if cell in ("lstm", "gru") else CELL_STEPS
+    assert binding.lib.csb_last_recurrent_path() == want
+
+
+@pytest.mark.parametrize("cell", ["lstm", "gru"])
+@pytest.mark.parametrize("I,H,L,B,T,vd", [(40, 48, 2, 1, 11, "f16"), (39, 161, 3, 1, 9, "f32"), (70, 200, 1, 1, 1, "f16"), (33, 64, 2, 3, 9, "f16"), (25, 60, 2, 8, 5, "f32")])
+def test_persistent_kernel_behind_the_resident_loops(monkeypatch, cell, I, H, L, B, T, vd):
+    # what serves layers that do not fit in shared memory: at batch 1 with h exchanged as flagged values, else with grid barriers
+    monkeypatch.setenv("CSB_RNN_NO_RNN1", "1")
+    w = workloads.make_rnn_workload(37, cell, I, H, L, 16, 16, "uniform", lo=0.3, hi=0.9, T=T, B=B, w_std=0.1, val_dtype=vd, bias_std=0.1, state_std=0.5)
+    y, h, c = rnn.check(w)
+    assert binding.lib.csb_last_recurrent_path() == PERSISTENT
+    if T > 4:                                              # resumed: the bits of one call
+        y2, h2, c2 = rnn.run(w, chunks=[(0, 4), (4, T)])
+        assert (y == y2).all() and (h == h2).all() and (c is None or (c == c2).all())
+
+
+def test_layers_that_do_not_fit_take_the_persistent_kernel():
+    # two layers of 1024 units with nothing pruned: 34 MB of fp16 values, past what the SMs' shared memory holds
+    w = workloads.make_rnn_workload(38, "lstm", 1024, 1024, 2, 64, 64, "uniform", lo=1.0, hi=1.0, T=3, B=1, w_std=0.03, bias_std=0.1, state_std=0.5)
+    rnn.check(w)
+    assert binding.lib.csb_last_recurrent_path() == PERSISTENT
 
 
 @pytest.mark.parametrize("other", [False, True])
@@ -91,6 +116,7 @@ def test_arrays_in_each_others_places(monkeypatch, cell, B, T, other):
                 hT = y[:h.numel()].view_as(h)
             call(x[:n].view(T, B, S), h, c, y.view(T, B, S), hT, cT)
             torch.cuda.synchronize()
+            assert binding.lib.csb_last_recurrent_path() == (BLOCK_LOOP if other else UNIT_LOOP)
             skip = h.numel() if place == "in y" else 0
             assert torch.equal(hT, want_h), place
             assert torch.equal(y[skip:], want_y.view(-1)[skip:]), place

@@ -1,4 +1,4 @@
-"""Host logic without a GPU: the panel layout that the batch-1 product streams is decoded in
+"""Host logic without a GPU: the panel layout that the products with one and few vectors stream is decoded in
 Python with the addressing rules of the kernel (lane -> row and column octet, remainder columns,
 gather descriptors, stages) and must (a) give back the masked dense matrix, every stored weight
 exactly once, (b) keep every size and alignment rule the kernel and its bulk copies rely on, and
@@ -8,13 +8,20 @@ import pytest
 
 import workloads
 from oracle import csb_oracle as O
+from oracle import fixed_oracle as F
 from paper_2005_05758_b200 import binding
 
 HDR = ("n_items", "n_gather", "n_xg", "n_stages", "value_bytes", "ridx_bytes", "row0", "n_rows",
        "warp_off", "items_off", "gather_off", "expect_off", "cidx_off", "ridx_off", "list_off", "n_bundles")
 
 
-def decode(plan, rows, cols, block_r, warps, stage):
+VALUES = {"f16": np.float16, "f32": np.float32, "q16": np.int16}
+
+
+def decode(plan, rows, cols, block_r, warps, stage, vd="f16"):
+    dt = VALUES[vd]
+    vs = np.dtype(dt).itemsize
+    unit = 16 // vs                                       # columns in 16 bytes
     dense = np.zeros((rows, cols), np.float64)
     count = np.zeros((rows, cols), np.int32)
     ranges = []
@@ -79,7 +86,7 @@ def decode(plan, rows, cols, block_r, warps, stage):
                     real += 1
                     assert 1 <= m <= GW and 1 <= n and P >= m and P < 2 * m
                     assert (m > 16) == (logg == 0) and (m <= 8) == (logg == 2), "items are bundled by height"
-                    nbytes = m * n * 2
+                    nbytes = m * n * vs
                     assert off + nbytes <= value_bytes
                     assert off // stage == (off + nbytes - 1) // stage, "no item straddles a stage"
                     spans.append((off, off + ((nbytes + 15) & ~15)))
@@ -88,9 +95,9 @@ def decode(plan, rows, cols, block_r, warps, stage):
                     assert (np.diff(rr) > 0).all() and rr.min() >= 0 and rr.max() < n_rows
                     cc = xg_col[4 * xoff4:4 * xoff4 + n]
                     assert (cc >= 0).all() and (np.diff(cc) > 0).all(), "kept columns of a block are ascending"
-                    v = vals[off:off + nbytes].view(np.float16).astype(np.float64)
-                    noct = n >> 3
-                    # what the lanes of the group read: lane (sub, r) takes octets sub, sub + S, ... of row r
+                    v = vals[off:off + nbytes].view(dt).astype(np.float64)
+                    noct = n // unit
+                    # what the lanes of the group read: lane (sub, r) takes groups of columns sub, sub + S, ... of row r
                     S = GW // P
                     got = np.zeros((m, n))
                     for gl in range(GW):
@@ -98,10 +105,10 @@ def decode(plan, rows, cols, block_r, warps, stage):
                         if r >= m:
                             continue
                         for o in range(sub, noct, S):
-                            q = (o * m + r) * 8
-                            got[r, 8 * o:8 * o + 8] = v[q:q + 8]
-                    tb, k = noct * m * 8, noct * 8
-                    for wdt in (4, 2, 1):
+                            q = (o * m + r) * unit
+                            got[r, unit * o:unit * o + unit] = v[q:q + unit]
+                    tb, k = noct * m * unit, noct * unit
+                    for wdt in (4, 2, 1) if unit == 8 else (2, 1):
                         if n & wdt:
                             for r in range(m):
                                 got[r, k:k + wdt] = v[tb + r * wdt:tb + r * wdt + wdt]
@@ -138,16 +145,24 @@ CASES = [
 ]
 
 
+@pytest.mark.parametrize("vd", ["f16", "f32", "q16"])
 @pytest.mark.parametrize("case", CASES)
-def test_panels_decode_to_the_masked_matrix(case):
+def test_panels_decode_to_the_masked_matrix(case, vd):
     rows, cols, br, bc, law, kw, ctas, warps, stage = case
-    w = workloads.make_spmv_workload(5, rows, cols, br, bc, law, batch=1, w_std=0.1, val_dtype="f16", **kw)
+    if vd == "f32":
+        stage = 16384                                      # (32 rows of 128 columns are one stage)
+    w = workloads.make_spmv_workload(5, rows, cols, br, bc, law, batch=1, w_std=0.1, val_dtype="f32" if vd == "q16" else vd, **kw)
     m = w.matrix
-    A = binding.csb_encode(m.dense, br, bc, m.row_keep, m.col_keep, "f16", device=-1)
+    if vd == "q16":
+        A = binding.csb_encode_q16(m.dense, br, bc, m.row_keep, m.col_keep, 12, device=-1)
+    else:
+        A = binding.csb_encode(m.dense, br, bc, m.row_keep, m.col_keep, vd, device=-1)
     plan = binding.csb_panel_dump(A, ctas, warps, stage)
     assert 1 <= plan["ctas"] <= ctas
-    dense, count, ranges = decode(plan, rows, cols, br, warps, stage)
-    want = O.masked_dense(m.dense, br, bc, m.row_keep, m.col_keep, "f16")
+    dense, count, ranges = decode(plan, rows, cols, br, warps, stage, vd)
+    want = O.masked_dense(m.dense, br, bc, m.row_keep, m.col_keep, "f32" if vd == "q16" else vd)
+    if vd == "q16":
+        want = F.quantize(want, 12)
     mask = O.block_mask(rows, cols, br, bc, m.row_keep, m.col_keep)
     assert np.array_equal(count, mask.astype(np.int32)), "every stored weight exactly once, nothing else"
     assert np.array_equal(dense, want)
@@ -173,7 +188,11 @@ def test_panels_empty_block_rows_and_refusals():
     assert binding.lib.csb_panel_dump(A.handle, 2, 2, 5000, info.ctypes.data, None, 0, None, 0) == -8   # stage not a power of two
     A.free()
     B = binding.csb_encode(W, 32, 64, rk, np.ones(4 * 64, np.uint8), "f32", device=-1)
-    assert binding.lib.csb_panel_dump(B.handle, 2, 2, 8192, info.ctypes.data, None, 0, None, 0) == -8      # fp32 values
+    assert binding.lib.csb_panel_dump(B.handle, 2, 2, 8192, info.ctypes.data, None, 0, None, 0) == 0       # fp32 values have panels too
+    B.free()
+    W2 = np.ones((8, 400), np.float32)
+    B = binding.csb_encode(W2, 8, 200, np.ones(16, np.uint8), np.ones(400, np.uint8), "f16", device=-1)
+    assert binding.lib.csb_panel_dump(B.handle, 2, 2, 8192, info.ctypes.data, None, 0, None, 0) == -8      # blocks wider than 128 columns
     B.free()
     # a matrix that keeps nothing at all still plans: one CTA that writes zeros
     Z = binding.csb_encode(W, 32, 64, np.zeros(4 * 32, np.uint8), np.ones(4 * 64, np.uint8), "f16", device=-1)

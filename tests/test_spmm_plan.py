@@ -57,7 +57,8 @@ def decode(plan, rows, cols, br, bc):
 
 
 @pytest.mark.parametrize("shape,batch,sms", [((300, 1177, 32, 32), 8, 148), ((512, 192, 16, 16), 32, 148), ((1024, 1536, 64, 64), 64, 148),
-                                              ((1024, 768, 64, 64), 16, 20), ((96, 4096, 32, 128), 33, 148), ((200, 130, 64, 8), 8, 7)])
+                                              ((1024, 768, 64, 64), 16, 20), ((96, 4096, 32, 128), 33, 148), ((200, 130, 64, 8), 8, 7),
+                                              ((300, 1177, 32, 32), 9, 148), ((96, 4096, 32, 128), 32, 148)])
 def test_every_weight_once_in_the_right_stream(shape, batch, sms):
     R, C, br, bc = shape
     w = workloads.make_spmv_workload(R + C, R, C, br, bc, "lognormal", rate=5.0, batch=1, w_std=0.05)
@@ -65,8 +66,8 @@ def test_every_weight_once_in_the_right_stream(shape, batch, sms):
     A = binding.csb_encode(m.dense, br, bc, m.row_keep, m.col_keep, "f16", -1)
     plan = binding.csb_spmm_plan_dump(A, batch, sms)
     A.free()
-    assert plan["RG"] in (1, 2, 4) and plan["NT"] == (1 if batch <= 8 else 2 if batch <= 16 else 4)
-    assert plan["warps"] == (32 if batch <= 8 else 16)
+    assert plan["RG"] in (1, 2, 4) and plan["NT"] == (1 if batch <= 8 else 2 if batch <= 16 else 4 if batch <= 32 else 8)
+    assert plan["warps"] == (32 if batch <= 8 else 16 if batch <= 32 else 8)
     nbr, nbc = -(-R // br), -(-C // bc)
     groups = -(-nbr // plan["RG"])
     assert plan["ctas"] == groups * plan["S"]
