@@ -65,7 +65,6 @@ __device__ __forceinline__ void walk_group(const uint8_t* img, const R1Group& g,
     for (int k = 0; k < K; ++k) {
         const float* p = v + (size_t)((c.v[k / 2] >> (16 * (k & 1))) & 0xffffu) * BT;
         if (BT == 1) x[k][0] = *p;
-        if (BT == 2) { const float2 t = *reinterpret_cast<const float2*>(p); x[k][0] = t.x; x[k][BT > 1 ? 1 : 0] = t.y; }
 #pragma unroll
         for (int b = 0; b + 4 <= BT; b += 4) {
             const float4 t = *reinterpret_cast<const float4*>(p + b);
@@ -95,7 +94,6 @@ __device__ __forceinline__ void walk_group(const uint8_t* img, const R1Group& g,
             for (int k = 0; k < K; ++k)
 #pragma unroll
                 for (int b = 0; b < BT / 2; ++b) a[b] = fma2(make_float2(wf[k], wf[k]), make_float2(x[k][2 * b], x[k][(2 * b + 1) % BT]), a[b]);
-            if (BT == 2) *reinterpret_cast<float2*>(out) = a[0];
 #pragma unroll
             for (int b = 0; b + 1 < BT / 2; b += 2)
                 *reinterpret_cast<float4*>(out + 2 * b) = make_float4(a[b].x, a[b].y, a[(b + 1) % (BT / 2 > 0 ? BT / 2 : 1)].x, a[(b + 1) % (BT / 2 > 0 ? BT / 2 : 1)].y);
