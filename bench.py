@@ -743,7 +743,7 @@ def main():
         for bsz in [int(b) for b in args.spmm_batches.split(",")]:
             res, n_l = spmv_sweep(binding, torch, local, rates, bsz, l2, reps=args.spmv_reps, with_cpu=with_cpu)
             line["spmm"] += res
-            launches += 2 * -(-bsz // 32) * n_l          # per pass of 32 batch columns: the pack kernel and the product kernel
+            launches += 2 * -(-bsz // 64) * n_l          # per pass of up to 64 batch columns: the pack kernel and the product kernel
         best = max(line["spmm"], key=lambda r: r["frac_hbm_measured"])
         line["roofline_spmm"] = {"kernel": "csb_spmm_tile_kernel", "bound": "hbm", "achieved": best["GBps"], "peak": hbm, "peak_kind": peak_kind,
                                  "unit": "GB/s", "frac": best["frac_hbm_measured"],

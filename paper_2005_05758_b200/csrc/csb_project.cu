@@ -13,7 +13,7 @@
 //
 // Bound by memory, 0.40 GB for 8192 x 8192 at 0.75.  Measured there: 88.5 us a call (166.4 with a thread
 // per row segment, 16 bytes of every 256 per load, and radix selections); the row pass reads at 5.4
-// TB/s, the column pass at 4.3 TB/s (profiler, cold caches).  Chunks of block-columns, so that the column
+// TB/s, the column pass at 4.2 TB/s (profiler, cold caches).  Chunks of block-columns, so that the column
 // pass finds its rows in L2, were slower: eleven short launches, 207 us.
 #include <algorithm>
 
