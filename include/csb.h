@@ -176,12 +176,13 @@ int csb_spmv(const csb_matrix_t* A, const float* x, float* y, void* stream);
  * With batch >= 8, fp16 values and block_r <= 64 the product runs on tensor cores (the kernel
  * matrix times the gathered inputs is then a dense contraction), up to 64 batch columns per pass: the
  * inputs are split into two binary16 halves (x = hi + lo, so no input precision is lost as long
- * as |x| < 65504; larger or non-finite inputs give inf / NaN) and multiplied with
- * mma.sync.m16n8k16, fp32 accumulation, a block-row's outputs staying in registers across its
- * blocks.  The first such call on a handle for a batch size class (<= 16, <= 32, more)
- * builds a device layout for that class and a staging buffer for the packed inputs (allocates and
- * synchronises the device once; make it outside of any stream capture, where more than 16 vectors are
- * served by the layout of either of the larger classes).  The two kernels of this path are launched
+ * as |x| < 65504; larger or non-finite inputs give inf / NaN in the outputs of their batch column), fp32
+ * accumulation.  Blocks of 16, 32 or a multiple of 64 columns are expanded into dense tiles for tcgen05.mma,
+ * with one device layout for all batch sizes; the others go through mma.sync.m16n8k16, with a layout per class
+ * of batch sizes (<= 16, <= 32, more).  The first such call on a handle builds the layout and a
+ * staging buffer for the packed inputs (allocates and synchronises once; make it outside of any stream
+ * capture, where the second form serves more than 16 vectors by the layout of either of the larger classes).
+ * The two kernels of this path are launched
  * with programmatic stream serialization and wait, first thing, for the work in front of them on
  * `stream`.  Other cases use the CUDA-core kernel in batch tiles of 8 / 4 / 1.
  */
@@ -242,11 +243,12 @@ int csb_spmv_static_scratch(const csb_matrix_t* A, const float* x, float* y, voi
  * themselves are immutable and may be used from any stream.
  * Up to B = 8 the weights stay in shared memory and one launch runs the sequence, where the layers fit
  * there.  With B >= 16 (B >= 8 when they do not fit and hold 100000 weights or more, or B >= 9 then),
- * fp16 values and block_r <= 64 the sequence runs step by step: per step of the stack one batched product
- * on tensor cores (as csb_spmm, same input-range rule; the layers as a wavefront, each a step behind
- * the one below) and one kernel with the gate arithmetic; same results within rounding, same
+ * fp16 values and block_r <= 64 the products run on tensor cores (as csb_spmm, same input-range rule; the
+ * layers as a wavefront, each a step behind the one below): up to B = 32, for blocks of 16, 32 or a
+ * multiple of 64 columns and stacks whose tiles one grid holds, in one launch for the sequence, else step
+ * by step, a batched product and a kernel with the gate arithmetic; same results within rounding, same
  * arguments and flags (CSB_RNN_NO_STEPWISE=1 in the environment asks for the persistent kernel that
- * serves the rest).  There the running states are kept in hT and cT when those are given.
+ * serves the rest).
  * Errors: SHAPE (rows != 4H, cols != I_l + H, layers disagree), LAUNCH (grid cannot be
  * co-resident; nothing was launched), TIMEOUT (the bounded grid barrier gave up; outputs are
  * undefined, the context stays usable), CUDA.
@@ -263,9 +265,9 @@ int csb_lstm_forward(int n_layers, const csb_matrix_t* const* W, const float* co
  *   r = s(zx_r + zh_r + b_r);  z = s(zx_z + zh_z + b_z);
  *   n = tanh(zx_n + b_in + r * (zh_n + b_hn));  h_t = (1 - z) * n + z * h_{t-1},
  * where zx / zh are the parts of the product over the input / hidden columns.
- * At the same batch sizes as for the LSTM (fp16 values, block_r <= 64) the sequence runs step by
- * step: one tensor-core product per layer and step over 2B rows (row b holds [u_t ; 0], row
- * B + b holds [0 ; h_{t-1}], which keeps zx and zh apart) and one gate kernel.
+ * At the same batch sizes as for the LSTM (fp16 values, block_r <= 64) the products run on tensor cores
+ * in the same two ways; zx and zh of the candidate stay apart as output rows of their own, or, step by step with
+ * the blocks that mma.sync takes, as the product's 2B rows (row b holds [u_t ; 0], row B + b [0 ; h_{t-1}]).
  */
 int csb_gru_forward(int n_layers, const csb_matrix_t* const* W, const float* const* bias,
                     const float* x, int64_t T, int B, const float* h0, float* y, float* hT,
@@ -345,8 +347,8 @@ void csb_test_barrier_hook(unsigned int extra_arrivals, unsigned long long limit
 
 /*
  * csb_last_recurrent_path -- testing aid (the paper has no counterpart): which kernels served the calling thread's most
- * recent recurrent call: 1 the unit loop, 2 the block loop (both resident), 3 batched steps over packed inputs, 4 batched
- * steps over fp32 inputs, 5 the persistent kernel, 6 steps of a cell variant; 0 before the first call.
+ * recent recurrent call: 1 the unit loop, 2 the block loop (both resident), 3 and 4 batched steps on tensor cores (up to 32 and more
+ * rows of the step-by-step product, which has B rows, for the GRU 2B), 5 the persistent kernel, 6 steps of a cell variant; 0 before the first call.
  */
 int csb_last_recurrent_path(void);
 

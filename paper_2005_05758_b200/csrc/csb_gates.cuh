@@ -14,6 +14,17 @@ namespace csb {
 
 __device__ __forceinline__ float gate_logistic(float a) { return 1.f / (1.f + expf(-a)); }
 
+// The same arithmetic with every rounding spelled out, for kernels that have to give the same bits.
+__device__ __forceinline__ float cell_logistic(float a) { return __fdiv_rn(1.f, __fadd_rn(1.f, expf(-a))); }
+__device__ __forceinline__ float lstm_cell(float zi, float zf, float zg, float zo, float& c) {
+    c = __fmaf_rn(cell_logistic(zf), c, __fmul_rn(cell_logistic(zi), tanhf(zg)));
+    return __fmul_rn(cell_logistic(zo), tanhf(c));
+}
+__device__ __forceinline__ float gru_cell(float zr, float zz, float n_in, float n_hid, float h) {
+    const float z = cell_logistic(zz);
+    return __fmaf_rn(z, h, __fmul_rn(__fadd_rn(1.f, -z), tanhf(__fmaf_rn(cell_logistic(zr), n_hid, n_in))));
+}
+
 // tile[b][c], 32 columns x nb batch values, into slots slot0 .. slot0 + nb - 1 of the packed rows of
 // those columns (and of a second set of rows, when given).  Consecutive threads take consecutive batch
 // values of a column, so that a row's stores are contiguous.  All threads of the CTA call this.

@@ -254,6 +254,19 @@ struct SpmmHostPlan {
 // Plans for `sm_count` SMs; returns CSB_OK, or 1 when the path does not suit the matrix.
 // force_S > 0: this many column ranges per row group.
 int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, int force_S, SpmmHostPlan* out);
+// The same product on tcgen05 (csb_umma.hpp, csb_umma_plan.cpp, csb_umma.cu): blocks of 16, 32 or a multiple of 64 columns.
+struct UmmaCta;
+struct UmmaQuad;
+struct UmmaPlan {                          // device side
+    bool built = false, unusable = false;
+    int MT = 1, S = 1, flush = 1, n_ctas = 0, windows = 0, seg_words = 32;
+    uint8_t* d_stream = nullptr; UmmaCta* d_ctas = nullptr; UmmaQuad* d_quads = nullptr;
+    uint8_t* d_xp = nullptr;               // packed inputs of a bare product
+};
+bool umma_applicable(const csb_matrix* A);
+int launch_umma(const csb_matrix* A, UmmaPlan* P, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
+void drop_umma_plan(UmmaPlan& P);
+
 struct MmaPlan {                           // device side, one per batch class, built on first use
     struct PerClass {
         bool built = false, unusable = false;
@@ -267,6 +280,7 @@ struct MmaPlan {                           // device side, one per batch class, 
     // plans without inputs of their own, for a share of the SMs (the layers of a recurrent stack); S = 0: free choice
     struct Shared { int ci, sms, S; PerClass plan; };
     std::list<Shared> shared;
+    UmmaPlan umma;
 };
 int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream);
 struct SpmmStack {                         // the products of a recurrent stack's layers (plans belong to the matrices)
@@ -368,6 +382,10 @@ void note_recurrent_path(RecurrentPath path);   // for csb_last_recurrent_path
 void drop_rnn_plans(const csb_matrix* A);  // forget cached time-loop plans that use A
 
 // csb_rnn_step.cu -- batch >= 16 (>= 8 for big layers): one timestep at a time, products on tensor cores
+// csb_umma_rnn.cu -- the same batches as one launch per sequence, where one grid holds the stack; else 1, nothing written
+int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* const* bias, const float* x, int64_t T, int B, int H, const int* in_size,
+                     const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream);
+void drop_umma_rnn_plans(const csb_matrix* A);
 bool rnn_stepwise_wanted(int gates, int L, const csb_matrix* const* W, int B);
 int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const float* const* bias, const float* x, int64_t T, int B, int H,
                          const int* in_size, const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags,

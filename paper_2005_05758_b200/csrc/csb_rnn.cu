@@ -665,6 +665,7 @@ static unsigned int g_barrier_extra = 0;
 
 void drop_rnn_plans(const csb_matrix* A) {
     drop_step_plans(A);
+    drop_umma_rnn_plans(A);
     drop_rnn1_plans(A);
     std::lock_guard<std::mutex> lk(g_rnn_mu);
     int prev = 0;
@@ -836,6 +837,9 @@ static int rnn_forward(int gates, int L, const csb_matrix_t* const* W, const flo
 
     // larger batches with fp16 values: step by step, the products on tensor cores
     if (rnn_stepwise_wanted(gates, L, W, B)) {
+        const int urc = rnn_forward_umma(gates, L, W, bias, x, T, B, H, in_size, h0, c0, y, hT, cT, flags, stream);
+        if (urc != 1) return urc;
+        clear_error();
         const int rc = rnn_forward_stepwise(gates, L, W, bias, x, T, B, H, in_size, h0, c0, y, hT, cT, flags, stream);
         if (rc != 1) return rc;
     }

@@ -29,6 +29,7 @@
 #include "csb_internal.hpp"
 #include "csb_device.cuh"
 #include "csb_gates.cuh"
+#include "csb_umma_rnn.hpp"
 
 namespace csb {
 
@@ -48,6 +49,7 @@ struct StepPlan {
     float* d_v[kMaxLayers] = {};       // [B, in_size[l] + H] per layer (GRU: [2B, ...], input rows then recurrent rows)
     float* d_z = nullptr;              // [B, 4H] (GRU: [2B, 3H]) pre-activations; packed path: one such per layer
     SpmmStack stack;                   // packed path
+    std::shared_ptr<UmmaStack> umma;   // the products run on these layouts (fp32 buffers only), one row per sequence for the GRU too
     float* d_c = nullptr;              // [L, B, H] cell state
     float* d_stage = nullptr;          // host-I/O staging of x and y
     size_t stage_cap = 0;
@@ -78,8 +80,6 @@ void drop_step_plans(const csb_matrix* A) {
     cudaSetDevice(prev);
 }
 
-__device__ __forceinline__ float logistic(float a) { return 1.f / (1.f + expf(-a)); }
-
 // Gate arithmetic of one LSTM layer and step for the whole batch (Section 2.1):
 //   c_t = s(z_f) c_{t-1} + s(z_i) tanh(z_g),  h_t = s(z_o) tanh(c_t),  rows of z stacked i, f, g, o.
 // h_t goes to v_self[b, off_self + j] (this layer's next product), to v_next[b, j] (the layer
@@ -97,8 +97,8 @@ __global__ void csb_lstm_gates_kernel(const float* __restrict__ Z, const float* 
         const float* z = Z + (size_t)b * 4 * H;
         float zi = z[j], zf = z[H + j], zg = z[2 * H + j], zo = z[3 * H + j];
         if (bias) { zi += bias[j]; zf += bias[H + j]; zg += bias[2 * H + j]; zo += bias[3 * H + j]; }
-        const float cn = logistic(zf) * c[e] + logistic(zi) * tanhf(zg);
-        const float h = logistic(zo) * tanhf(cn);
+        float cn = c[e];
+        const float h = lstm_cell(zi, zf, zg, zo, cn);
         c[e] = cn;
         v_self[(size_t)b * ld_self + off_self + j] = h;
         if (v_next) v_next[(size_t)b * ld_next + j] = h;
@@ -118,6 +118,9 @@ __global__ void csb_lstm_gates_kernel(const float* __restrict__ Z, const float* 
 //   h_t = (1 - u) n + u h_{t-1};  zx = row b, zh = row B + b of Z [2B, 3H]; bias = b_r, b_z, b_in, b_hn.
 // h_t goes to the recurrent rows of v_self (row B + b, columns off_self ..), to the input rows of
 // v_next (row b) when there is a layer above, and to y_t; x_next as for the LSTM kernel.
+// APART: the product itself has kept the candidate's parts apart, row b of Z [B, 4H] is r, z and the two parts, and v_self has
+// one row per sequence.
+template <bool APART>
 __global__ void csb_gru_gates_kernel(const float* __restrict__ Z, const float* __restrict__ bias, float* __restrict__ v_self,
                                      int ld_self, int off_self, float* __restrict__ v_next, int ld_next, float* __restrict__ y_t,
                                      const float* __restrict__ x_next, int I, float* __restrict__ v0, int ld0, int B, int H) {
@@ -126,14 +129,13 @@ __global__ void csb_gru_gates_kernel(const float* __restrict__ Z, const float* _
     const int n = B * H;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
         const int b = e / H, j = e - b * H;
-        const float* zx = Z + (size_t)b * 3 * H;
+        const float* zx = Z + (size_t)b * (APART ? 4 : 3) * H;
         const float* zh = Z + (size_t)(B + b) * 3 * H;
-        float ar = zx[j] + zh[j], au = zx[H + j] + zh[H + j], nx = zx[2 * H + j], nh = zh[2 * H + j];
+        float ar = zx[j], au = zx[H + j], nx = zx[2 * H + j], nh = APART ? zx[3 * H + j] : zh[2 * H + j];
+        if (!APART) { ar += zh[j]; au += zh[H + j]; }
         if (bias) { ar += bias[j]; au += bias[H + j]; nx += bias[2 * H + j]; nh += bias[3 * H + j]; }
-        const float r = logistic(ar), u = logistic(au);
-        const float cand = tanhf(nx + r * nh);
-        float* hp = v_self + (size_t)(B + b) * ld_self + off_self + j;
-        const float h = (1.f - u) * cand + u * *hp;
+        float* hp = v_self + (size_t)(APART ? b : B + b) * ld_self + off_self + j;
+        const float h = gru_cell(ar, au, nx, nh, *hp);
         *hp = h;
         if (v_next) v_next[(size_t)b * ld_next + j] = h;
         if (y_t) y_t[e] = h;
@@ -254,21 +256,28 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
         if (!P) {
             std::unique_ptr<StepPlan> np(new StepPlan());
             np->L = L; np->B = B; np->H = H; np->gates = gates; np->device = W[0]->device;
-            const int rows_v = (gates == 3 ? 2 : 1) * B;
-            const bool packed_path = rows_v <= 32 && !env_flag("CSB_RNN_STEP_UNPACKED");
+            // The layouts of the time loop serve the fp32 buffers as well: its numbers bit for bit, and batches past 32 at the
+            // speed of the bare product.
+            const bool small = (gates == 3 ? 2 : 1) * B <= 32, unpacked = env_flag("CSB_RNN_STEP_UNPACKED");
+            if (!small || unpacked) {
+                const int urc = umma_stack(gates, L, W, in_size, H, &np->umma);
+                if (urc != CSB_OK) return urc;
+            }
+            const int rows_v = (gates == 3 && !np->umma ? 2 : 1) * B;
+            const bool packed_path = small && !unpacked;
             const int pitch = spmm_pitch(spmm_nt(std::min(rows_v, 32)));
             if (packed_path) { np->pitch = pitch; np->cap = 8 * spmm_nt(rows_v); }
             for (int l = 0; l < L; ++l) {
                 np->uids.push_back(W[l]->uid);
                 np->in_size[l] = in_size[l];
                 // (what is read of the packed inputs is written on the call's stream first, so they need no clearing here)
-                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], (size_t)(in_size[l] + H) * pitch));
+                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], np->umma ? (size_t)np->umma->plan[l].windows * kUmmaStage : (size_t)(in_size[l] + H) * pitch));
                 if (!packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_v[l], (size_t)rows_v * (in_size[l] + H) * 4));
             }
-            const int rc = prepare_spmm_stack(L, W, std::min(rows_v, 32), &np->stack);
+            const int rc = np->umma ? (int)CSB_OK : prepare_spmm_stack(L, W, std::min(rows_v, 32), &np->stack);
             if (rc != CSB_OK) return rc;
             if (packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_h, (size_t)L * B * H * 4));
-            CSB_CUDA(cudaMalloc((void**)&np->d_z, (size_t)(packed_path ? L : 1) * (gates == 3 ? 2 : 1) * B * gates * H * 4));
+            CSB_CUDA(cudaMalloc((void**)&np->d_z, (size_t)(packed_path ? L : 1) * rows_v * (np->umma ? 4 : gates) * H * 4));
             if (gates == 4) CSB_CUDA(cudaMalloc((void**)&np->d_c, (size_t)L * B * H * 4));
             P = np.get();
             g_step_plans.push_back(std::move(np));
@@ -297,7 +306,8 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     const cudaMemcpyKind out_kind = host_io ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     const size_t hrow = (size_t)H * 4;
     const bool gru = gates == 3;
-    const int vrows = gru ? 2 * B : B;                  // rows of V_l and of the product
+    const bool apart_rows = gru && !P->umma;            // input and recurrent rows of their own
+    const int vrows = apart_rows ? 2 * B : B;           // rows of V_l and of the product
     if (P->pitch) {
         // ---- packed path: the gate kernels feed the products' packed inputs directly
         const int pitch = P->pitch, cap = P->cap;
@@ -371,10 +381,10 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     // recurrent rows (B ..) carry h and zeros on the left, the input rows zeros on the right.
     for (int l = 0; l < L; ++l) {
         const int ld = in_size[l] + H;
-        float* hpart = P->d_v[l] + (gru ? (size_t)B * ld : 0) + in_size[l];
-        if (gru) CSB_CUDA(cudaMemsetAsync(P->d_v[l], 0, (size_t)vrows * ld * 4, st));
+        float* hpart = P->d_v[l] + (apart_rows ? (size_t)B * ld : 0) + in_size[l];
+        if (apart_rows) CSB_CUDA(cudaMemsetAsync(P->d_v[l], 0, (size_t)vrows * ld * 4, st));
         if (h0) CSB_CUDA(cudaMemcpy2DAsync(hpart, (size_t)ld * 4, h0 + (size_t)l * B * H, hrow, hrow, B, in_kind, st));
-        else if (!gru) CSB_CUDA(cudaMemset2DAsync(hpart, (size_t)ld * 4, 0, hrow, B, st));
+        else if (!apart_rows) CSB_CUDA(cudaMemset2DAsync(hpart, (size_t)ld * 4, 0, hrow, B, st));
     }
     CSB_CUDA(cudaMemcpy2DAsync(P->d_v[0], (size_t)(I0 + H) * 4, dx, (size_t)I0 * 4, (size_t)I0 * 4, B, cudaMemcpyDeviceToDevice, st));
     if (!gru) {
@@ -387,7 +397,8 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     for (int64_t t = 0; t < T; ++t) {
         for (int l = 0; l < L; ++l) {
             const int ld = in_size[l] + H;
-            const int rc = launch_spmm_stack_fp32(P->stack, l, W[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
+            const int rc = P->umma ? launch_umma_fp32(W[l], &P->umma->plan[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)4 * H, st)
+                                   : launch_spmm_stack_fp32(P->stack, l, W[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
             if (rc != CSB_OK) return rc;
             const bool top = l == L - 1;
             const float* x_next = (l == 0 && t + 1 < T) ? dx + (size_t)(t + 1) * B * I0 : nullptr;
@@ -402,7 +413,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             const int ldn = top ? 0 : in_size[l + 1] + H;
             float* yt = (top && dy) ? dy + (size_t)t * B * H : nullptr;
             if (gru)
-                CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_gru_gates_kernel, (const float*)P->d_z, bl, P->d_v[l], ld, in_size[l], vn, ldn, yt,
+                CSB_CUDA(cudaLaunchKernelEx(&cfg, P->umma ? csb_gru_gates_kernel<true> : csb_gru_gates_kernel<false>, (const float*)P->d_z, bl, P->d_v[l], ld, in_size[l], vn, ldn, yt,
                                             x_next, I0, P->d_v[0], I0 + H, B, H));
             else
                 CSB_CUDA(cudaLaunchKernelEx(&cfg, csb_lstm_gates_kernel, (const float*)P->d_z, bl, P->d_c + (size_t)l * B * H, P->d_v[l], ld,
@@ -412,7 +423,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     }
     if (hT)
         for (int l = 0; l < L; ++l)
-            CSB_CUDA(cudaMemcpy2DAsync(hT + (size_t)l * B * H, hrow, P->d_v[l] + (gru ? (size_t)B * (in_size[l] + H) : 0) + in_size[l],
+            CSB_CUDA(cudaMemcpy2DAsync(hT + (size_t)l * B * H, hrow, P->d_v[l] + (apart_rows ? (size_t)B * (in_size[l] + H) : 0) + in_size[l],
                                        (size_t)(in_size[l] + H) * 4, hrow, B, out_kind, st));
     if (cT && !gru) CSB_CUDA(cudaMemcpyAsync(cT, P->d_c, ns * 4, out_kind, st));
     if (host_io && y) CSB_CUDA(cudaMemcpyAsync(y, dy, ny * 4, cudaMemcpyDeviceToHost, st));

@@ -631,6 +631,7 @@ void free_mma(csb_matrix* A) {
     cudaSetDevice(A->device);
     for (auto& c : A->mma->cls) drop_plan(c);
     for (auto& c : A->mma->shared) drop_plan(c.plan);
+    drop_umma_plan(A->mma->umma);
     cudaSetDevice(prev);
     delete A->mma;
     A->mma = nullptr;
@@ -749,6 +750,12 @@ int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch,
     CSB_CUDA(cudaGetDevice(&prev));
     if (prev != A->device) CSB_CUDA(cudaSetDevice(A->device));
     struct Restore { int prev, cur; ~Restore() { if (prev != cur) cudaSetDevice(prev); } } restore{prev, A->device};
+    if (umma_applicable(A)) {
+        std::lock_guard<std::mutex> lk(A->mma_mu);
+        if ((rc = ensure_mma(A)) != CSB_OK) return rc;
+        if ((rc = launch_umma(A, &A->mma->umma, X, ldx, batch, Y, ldy, stream)) != 1) return rc;
+        clear_error();
+    }
     // Eight columns run in tiles of 16: half as many warps with twice the columns meet at half as many hand-overs, and
     // the columns of zeros cost less than that (8 x 32-warp tiles against these, us: 3072 x 1536 at 8x 13.0 / 10.5, 4096 x
     // 4096 of 32 x 32 blocks at 5x 24.0 / 15.5, 8192 x 8192 at 4x 28.2 / 27.5; the one that lost, 4096 x 4096 of

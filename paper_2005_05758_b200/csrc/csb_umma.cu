@@ -1,0 +1,183 @@
+// Host side of the batched product on tcgen05 tensor cores (csb_umma_kernel.cuh): plans, packing, launches.
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <mutex>
+
+#include "csb_umma_rnn.hpp"
+#include "csb_umma_kernel.cuh"
+
+namespace csb {
+
+// Packs fp32 inputs [nb][cols] into the operand images: one CTA per window, a thread per batch column and 8 matrix columns.
+template <int NB>
+__global__ void __launch_bounds__(NB * 8) csb_umma_pack_kernel(const float* __restrict__ X, long long ldx, int nb, int cols, int vec, uint8_t* __restrict__ xp) {
+    pdl_launch_dependents();
+    pdl_wait();                                           // X may come from the kernel in front; xp may still be read by it
+    const int b = threadIdx.x >> 3, c = (int)blockIdx.x * kUmmaWindow + (threadIdx.x & 7) * 8;
+    if (b < nb && c + 8 <= cols) { put_eight<NB>(xp, b, c, cols, X + (long long)b * ldx + c, vec != 0); return; }
+    float x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = b < nb && c + i < cols ? X[(long long)b * ldx + c + i] : 0.f;
+    uint4 hi, lo;
+    hi.x = split_pair(x[0], x[1], lo.x); hi.y = split_pair(x[2], x[3], lo.y);
+    hi.z = split_pair(x[4], x[5], lo.z); hi.w = split_pair(x[6], x[7], lo.w);
+    uint8_t* at = xp + image_at<NB>(b, c);
+    *reinterpret_cast<uint4*>(at) = hi;
+    *reinterpret_cast<uint4*>(at + NB * 128) = lo;
+}
+
+#define CSB_CUDA(call)                                                                     \
+    do {                                                                                   \
+        cudaError_t e_ = (call);                                                           \
+        if (e_ != cudaSuccess) {                                                           \
+            set_error("%s failed: %s", #call, cudaGetErrorString(e_));                     \
+            return e_ == cudaErrorMemoryAllocation ? CSB_ERR_ALLOC : CSB_ERR_CUDA;         \
+        }                                                                                  \
+    } while (0)
+
+template <int MODE>
+static const void* pick_mode(int NB, int MT) {
+    if (MT == 1) return NB == 16 ? (const void*)csb_umma_kernel<16, 1, MODE> : (const void*)csb_umma_kernel<32, 1, MODE>;
+    return NB == 16 ? (const void*)csb_umma_kernel<16, 2, MODE> : (const void*)csb_umma_kernel<32, 2, MODE>;
+}
+// mode: 0 a product, 1 and 2 the time loops of LSTM and GRU (up to 32 batch columns)
+const void* pick_umma(int mode, int NB, int MT) {
+    if (mode == 1) return pick_mode<1>(NB, MT);
+    if (mode == 2) return pick_mode<2>(NB, MT);
+    if (NB < 64) return pick_mode<0>(NB, MT);
+    return MT == 1 ? (const void*)csb_umma_kernel<64, 1, 0> : (const void*)csb_umma_kernel<64, 2, 0>;
+}
+size_t umma_smem(int mode, int NB, int MT) { return UmmaSmem(mode, NB, MT).total; }
+
+static cudaLaunchConfig_t umma_config(int ctas, int S, size_t smem, cudaStream_t st, cudaLaunchAttribute (&attr)[2]) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3(kUmmaThreads); cfg.dynamicSmemBytes = smem;
+    cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = S > 1 ? 2 : 1;
+    return cfg;
+}
+
+// Clusters of S CTAs that the device holds at a time, S = 1 .. kUmmaMaxS (SMs that a processing cluster's size leaves over
+// are lost: 4 x 37 SMs do not make 37 clusters of four).
+int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]) {
+    const int sms = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
+    n[0] = 0; n[1] = sms;
+    const void* kernel = pick_umma(0, 64, 2);
+    const size_t smem = umma_smem(1, 32, 2);               // the largest
+    if (smem > A->smem_optin) { for (int S = 1; S <= kUmmaMaxS; ++S) n[S] = 0; return CSB_OK; }
+    CSB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
+    for (int S = 2; S <= kUmmaMaxS; ++S) {
+        cudaLaunchAttribute attr[2];
+        cudaLaunchConfig_t cfg = umma_config(S * sms, S, smem, 0, attr);
+        CSB_CUDA(cudaOccupancyMaxActiveClusters(&n[S], kernel, &cfg));
+        n[S] = std::min(n[S], sms / S);
+    }
+    return CSB_OK;
+}
+
+void drop_umma_plan(UmmaPlan& P) {
+    cudaFree(P.d_stream); cudaFree(P.d_ctas); cudaFree(P.d_quads); cudaFree(P.d_xp);
+    P.d_stream = nullptr; P.d_ctas = nullptr; P.d_quads = nullptr; P.d_xp = nullptr;
+}
+
+// Uploads a host plan.
+int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P) {
+    P->MT = H.MT; P->S = H.S; P->n_ctas = (int)H.ctas.size(); P->windows = H.windows; P->seg_words = H.seg_words; P->flush = H.flush;
+    CSB_CUDA(cudaMalloc((void**)&P->d_stream, std::max<size_t>(H.total128, 1) * 128));
+    for (size_t i = 0; i < H.ctas.size(); ++i)
+        if (!H.streams[i].empty())
+            CSB_CUDA(cudaMemcpyAsync(P->d_stream + (size_t)H.ctas[i].off128 * 128, H.streams[i].data(), H.streams[i].size(), cudaMemcpyHostToDevice, cudaStreamPerThread));
+    CSB_CUDA(cudaMalloc((void**)&P->d_ctas, H.ctas.size() * sizeof(UmmaCta)));
+    CSB_CUDA(cudaMemcpyAsync(P->d_ctas, H.ctas.data(), H.ctas.size() * sizeof(UmmaCta), cudaMemcpyHostToDevice, cudaStreamPerThread));
+    CSB_CUDA(cudaMalloc((void**)&P->d_quads, H.quads.size() * sizeof(UmmaQuad)));
+    CSB_CUDA(cudaMemcpyAsync(P->d_quads, H.quads.data(), H.quads.size() * sizeof(UmmaQuad), cudaMemcpyHostToDevice, cudaStreamPerThread));
+    CSB_CUDA(cudaStreamSynchronize(cudaStreamPerThread));
+    for (int NB = 16; NB <= 64; NB *= 2)
+        CSB_CUDA(cudaFuncSetAttribute(pick_umma(0, NB, H.MT), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
+    P->built = true;
+    return CSB_OK;
+}
+
+static int make_umma_plan(const csb_matrix* A, UmmaPlan* P) {
+    if (P->built || P->unusable) return P->built ? CSB_OK : 1;
+    int rc;
+    try {
+        UmmaHostPlan H;
+        H.windows = (int)((A->cols + kUmmaWindow - 1) / kUmmaWindow);
+        H.seg_words = umma_seg_words(A->block_c);
+        int clusters[kUmmaMaxS + 1];
+        if ((rc = umma_clusters(A, clusters)) != CSB_OK) { P->unusable = true; return rc; }
+        if (clusters[1] < 1) { P->unusable = true; return 1; }
+        umma_shape((int)((A->rows + 127) / 128), H.windows, clusters, &H.MT, &H.S);
+        H.flush = umma_flush(H.windows);
+        H.quads = umma_row_quads(A, H.MT);
+        H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
+        if (!plan_umma_host(A, &H)) { P->unusable = true; return 1; }
+        rc = upload_umma(A, H, P);
+        if (rc == CSB_OK && P->built) CSB_CUDA(cudaMalloc((void**)&P->d_xp, (size_t)H.windows * 64 * 256));
+    } catch (const std::bad_alloc&) { set_error("out of host memory while planning the batched product"); rc = CSB_ERR_ALLOC; }
+    if (rc != CSB_OK) {
+        drop_umma_plan(*P);
+        cudaGetLastError();
+        P->built = false; P->unusable = true;
+        return rc;
+    }
+    return P->built ? CSB_OK : 1;
+}
+
+bool umma_applicable(const csb_matrix* A) {
+    if (getenv("CSB_NO_UMMA") && atoi(getenv("CSB_NO_UMMA"))) return false;
+    return A->val_dtype == CSB_F16 && A->device >= 0 && umma_seg_words(A->block_c) > 0;
+}
+
+int umma_nb(int batch) { return batch <= 16 ? 16 : batch <= 32 ? 32 : 64; }
+
+// Y = A . (packed inputs) with the plan's output rows.
+int launch_umma_packed(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, float* Y, int NB, int nb, int64_t ldy, cudaStream_t st) {
+    UmmaArgs a{};
+    a.n_parts = 1; a.nb = nb; a.ldy = ldy; a.status = A->product.d_status; a.S = P->S; a.flush = P->flush;
+    UmmaPart& p = a.part[0];
+    p.stream = P->d_stream; p.ctas = P->d_ctas; p.quads = P->d_quads; p.xp = xp; p.Y = Y;
+    p.block_r = A->block_r; p.seg_words = P->seg_words; p.windows = P->windows; p.cta_end = P->n_ctas;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = umma_config(P->n_ctas, P->S, umma_smem(0, NB, P->MT), st, attr);
+    void* args[] = {&a};
+    CSB_CUDA(cudaLaunchKernelExC(&cfg, pick_umma(0, NB, P->MT), args));
+    return CSB_OK;
+}
+
+int launch_umma_pack(const float* X, int64_t ldx, int nb, int cols, int NB, uint8_t* xp, cudaStream_t st) {
+    const int vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0 && ldx % 4 == 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.gridDim = dim3((unsigned)((cols + kUmmaWindow - 1) / kUmmaWindow)); cfg.blockDim = dim3((unsigned)NB * 8);
+    CSB_CUDA(cudaLaunchKernelEx(&cfg, NB == 16 ? csb_umma_pack_kernel<16> : NB == 32 ? csb_umma_pack_kernel<32> : csb_umma_pack_kernel<64>, X, (long long)ldx, nb,
+                                cols, vec, xp));
+    return CSB_OK;
+}
+
+// Packs fp32 inputs into xp (windows * 16 KB) and launches, 64 batch columns at a time.
+int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st) {
+    for (int b0 = 0; b0 < batch; b0 += 64) {
+        const int nb = std::min(64, batch - b0), NB = umma_nb(nb);
+        int rc = launch_umma_pack(X + (int64_t)b0 * ldx, ldx, nb, (int)A->cols, NB, xp, st);
+        if (rc == CSB_OK) rc = launch_umma_packed(A, P, xp, Y + (int64_t)b0 * ldy, NB, nb, ldy, st);
+        if (rc != CSB_OK) return rc;
+    }
+    return CSB_OK;
+}
+
+// Returns CSB_OK after launching, or 1 when the path does not take the matrix.
+int launch_umma(const csb_matrix* A, UmmaPlan* P, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
+    const int rc = make_umma_plan(A, P);
+    return rc != CSB_OK ? rc : launch_umma_fp32(A, P, P->d_xp, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
+}
+
+}  // namespace csb

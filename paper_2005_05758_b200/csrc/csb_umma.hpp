@@ -1,0 +1,75 @@
+// The batched product on tcgen05 tensor cores: layout shared by the planner (csb_umma_plan.cpp) and the
+// kernel (csb_umma.cu).
+//
+// The matrix is cut into tiles of 128 output rows (four quadrants of 32, one per TMEM lane quarter) and
+// windows of 64 columns.  A CTA takes MT tiles (a row group) over a range of windows; the S ranges of a row
+// group are one thread-block cluster.  A tile-window is kept as four items, one per quadrant, each expanded by
+// one warp, whose lanes are the rows, into the dense 32 x 64 operand:
+//
+//   header  uint4 per (row segment, column segment), row segments first:
+//             x  bit l: lane l's row is kept (zero outside of the segment's rows, and where no column is kept)
+//             y  where the segment's values start, bytes from the item
+//             w  first header only: where the warp's next item starts (16-byte units of the CTA's stream; ~0: none)
+//   values  16 bytes per eight columns and kept row, [eight columns][row], binary16, zero where a column is not kept
+//
+// A row segment is the part of one block-row that lies in the quadrant, a column segment 16, 32 or 64 columns, the
+// part of one block that lies in the window.  Rows are compact and columns are not: a lane then has its row of a window in
+// eight 16-byte loads.  With the columns compact by pairs (1.5 instead of 2 times the compact size at 4x, 1.8 instead of
+// 5 at 25x) it took a predicated load and add for every pair, and the expanding warps' instructions set the time.
+//
+// The items of a CTA lie back to back in the order (group of `flush` windows, tile, window, quadrant): the sums of a tile
+// over such a group come out of the tensor cores' accumulators before they grow further.  No item straddles a multiple of
+// kUmmaStage bytes of the CTA's stream, which travels in stages of that size.
+#pragma once
+
+#include "csb_internal.hpp"
+
+namespace csb {
+
+enum { kUmmaStage = 16384, kUmmaStages = 6, kUmmaWindow = 64, kUmmaExpandWarps = 16, kUmmaMaxMT = 2, kUmmaMaxS = 8 };
+
+struct UmmaQuad {             // 32 lanes of a tile
+    int32_t row0, nrows;      // their rows of the matrix (none: nrows = 0)
+    int32_t c0, c1;           // and the columns that count
+    int32_t out0, pad[3];     // the first one's place in a product's output
+};
+static_assert(sizeof(UmmaQuad) == 32, "two 16-byte words");
+struct UmmaCta {
+    uint32_t off128;          // where its stream starts, 128-byte units
+    uint32_t bytes;
+    int32_t group, split;     // row group and which column range of it
+    int32_t w0, nw;           // windows
+    int32_t pad[2];
+    uint32_t first[kUmmaExpandWarps];   // per expanding warp: its first item, 16-byte units of the CTA's stream (~0: none)
+};
+static_assert(sizeof(UmmaCta) == 96, "six 16-byte words");
+
+struct UmmaHostPlan {
+    int MT = 1, S = 1, flush = 1, n_groups = 0, windows = 0, seg_words = 32;   // seg_words: 32-bit words of a row of a column segment
+    std::vector<UmmaQuad> quads;          // [n_groups][MT][4]
+    std::vector<UmmaCta> ctas;            // [n_groups][S]
+    std::vector<std::vector<uint8_t>> streams;   // per CTA
+    uint64_t total128 = 0;                // all streams, 128-byte units
+};
+
+// 32-bit words of a row of a column segment for blocks of this width; 0: the layout does not take them.
+inline int umma_seg_words(int block_c) { return block_c == 16 ? 8 : block_c == 32 ? 16 : block_c % 64 == 0 ? 32 : 0; }
+// Rows of the matrix in order, in groups of MT tiles.
+std::vector<UmmaQuad> umma_row_quads(const csb_matrix* A, int MT);
+// A layer of a recurrent stack: a tile is 32 hidden units, its quadrants the gates i, f, g, o or r, z and the input and the
+// recurrent part of the candidate, whose sums stay apart (output rows 2H .. and 3H ..).
+std::vector<UmmaQuad> umma_gate_quads(int gates, int in_size, int H, int MT);
+// Tiles per CTA and column ranges per group for `tiles` tiles of `windows` windows on a device that holds clusters[S] clusters of S.
+double umma_cost(int MT, int S, int windows);          // a CTA's modelled time, in tile-windows
+void umma_shape(int tiles, int windows, const int* clusters, int* MT, int* S);
+// Windows per flush group.  The tensor cores truncate each sum, so the error follows the number of steps between two flushes;
+// the bounds are those at which it stays below what mma.sync gave, whose chains grow with the number of columns
+// (2-norm of the error against 64 bits, mma.sync / 1 / 2 windows: 1024 x 1536 at 4x 1.40e-7 / 1.30e-7 / 1.52e-7, 700 x
+// 2050 at 6x 1.75 / 1.08 / 1.27, 8192 x 8192 at 4x 8.37 / 1.45 / 1.73, 25x 2.07 / 1.23 / 1.32).
+inline int umma_flush(int windows) { return windows < 32 ? 1 : 2; }
+// Fills streams, ctas (the other members are set); throws std::bad_alloc.  False: the layout does not take the matrix (a warp's
+// last item lies more than the ring's stages in front of the end of its CTA's stream, which nobody would then free: blocks
+// of a few rows with next to nothing pruned).
+bool plan_umma_host(const csb_matrix* A, UmmaHostPlan* P);
+
+}  // namespace csb

@@ -1,0 +1,652 @@
+// Batched CSB product on tcgen05 tensor cores, alone and as the time loop of a recurrent stack (fp16 values, fp32
+// accumulation).
+//
+// The kernel matrices of the blocks (Section 4.3.1) are small and all different, and with rows and columns put back in their
+// places a block is mostly zeros.  Tensor instructions for those zeros are cheap on this chip (8192 x 8192 dense, 64 columns as
+// hi and lo halves: 7.5 us of all SMs), so a warp expands the kept values into the dense tile and the contraction is a dense one:
+//
+//   * sixteen warps expand: lane = output row, eight 16-byte loads of its row's 64 columns, zeros where the row is not
+//     kept, and one tcgen05.st puts the 32 words into TMEM as the A operand (128 rows x 64 columns per tile-window).  A never
+//     passes through shared memory in its dense form, whose bandwidth the B operand needs;
+//   * the inputs are packed into binary16 pairs x = hi + lo (no input precision is lost as long as |x| < 65504) as 128-byte
+//     swizzled, K-major operand images, 64 columns each, the hi rows of all batch columns, then the lo rows; a
+//     bulk copy brings an image as it is;
+//   * one thread issues the tcgen05.mma, one the copies of the inputs, one those of the values;
+//   * the tensor cores add into TMEM with truncation, so the sums of a unit (a tile over `flush` windows) start from zero
+//     and are taken out by the same sixteen warps, which add them in registers with rounding.  The units' buffers go
+//     round, so that the next ones run meanwhile;
+//   * a row group's column ranges are one thread-block cluster and are added in range order through distributed
+//     shared memory: results are bit-reproducible, no scratch, no atomics.
+//
+// As a time loop (MODE 1 LSTM, 2 GRU) the grid stays for the whole sequence, each CTA with its tiles of one layer, whose
+// quadrants are the gates of the same 32 hidden units.  In tick k layer l does step k - l.  After the cluster's sums every CTA does the
+// gate arithmetic of its share of (units, batch column) and writes h_t into the other one of two buffers of operand
+// images; a counter in global memory says when all CTAs have.  Only the thread that copies the inputs waits for it: the
+// values of the next step are on their way and the first tiles expanded by then.
+#pragma once
+
+#include "csb_umma.hpp"
+#include "csb_device.cuh"
+#include "csb_gates.cuh"
+
+namespace csb {
+
+constexpr int kXStage = 16384;                 // bytes of a stage of inputs: one window of 64 batch columns, two of 32, four of 16
+constexpr int kWDepth = kUmmaStages;           // stages of values in shared memory
+constexpr int kASlots = 8;                     // tile-windows of the A operand in TMEM, 32 columns each
+constexpr int kDCols = 256;                    // columns of TMEM for sums
+constexpr int kExpandThreads = kUmmaExpandWarps * 32, kUmmaThreads = kExpandThreads + 3 * 32;
+__host__ __device__ constexpr int x_depth(int mode) { return mode ? 4 : 5; }
+
+struct UmmaPart {
+    const uint8_t* stream;
+    const UmmaCta* ctas;
+    const UmmaQuad* quads;
+    uint8_t* xp;               // packed inputs: per window an image of 2 * NB rows of 128 bytes (time loop: two such buffers)
+    float* Y;
+    int cta_end;               // the part's CTAs end here in the grid
+    int block_r, seg_words, windows;
+};
+struct UmmaArgs {
+    UmmaPart part[kMaxLayers];
+    long long ldy;
+    uint32_t* status;
+    int n_parts, nb, S, flush;
+    // time loop: a part is a layer
+    const float* x; float* y; const float* state0;        // [T, nb, in_size[0]]; [T, nb, H] or null; [L, nb, H]: c (LSTM) or h (GRU) at the start
+    float *hT, *cT;                                        // [L, nb, H] or null
+    const float* bias[kMaxLayers];
+    int in_size[kMaxLayers];
+    uint32_t* count;                                       // CTAs that have finished a tick, summed over ticks
+    unsigned long long limit_ns;
+    uint32_t never;                                        // test hook: arrivals that never come
+    int T, H, x_vec;                                       // x_vec: rows of x start at multiples of 16 bytes
+};
+
+// ---- tcgen05 -----------------------------------------------------------------------------------------
+__device__ __forceinline__ void tc_alloc(uint32_t smem_out, uint32_t cols) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_out), "r"(cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tc_dealloc(uint32_t taddr, uint32_t cols) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(cols));
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// D (TMEM) (+)= A (TMEM, 128 x 16 binary16) . B (shared memory, K-major)
+__device__ __forceinline__ void tc_mma_f16(uint32_t d, uint32_t a, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d), "r"(a), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t (&r)[32]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
+        "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]),
+        "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]),
+        "r"(r[30]), "r"(r[31]) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+// N columns of this lane; the values are there after tc_wait_ld.
+template <int N> __device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t* r) {
+    if constexpr (N > 16) {
+        tc_ld<16>(taddr, r);
+        tc_ld<N - 16>(taddr + 16, r + 16);
+    } else if constexpr (N == 16) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+                       "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]) : "r"(taddr) : "memory");
+    } else if constexpr (N == 8) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+    } else {
+        static_assert(N == 4, "columns of a load");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr) : "memory");
+    }
+}
+__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// K-major operand image, 128-byte swizzle, groups of eight rows 1024 bytes apart.
+__device__ __forceinline__ uint64_t b_descriptor(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3fffu) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+// binary16 x binary16 -> fp32, both K-major, 128 x N
+__host__ __device__ constexpr uint32_t mma_idesc(int N) { return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24); }
+
+// One lane of a converged warp, the same one every time.
+__device__ __forceinline__ bool elect_lane() {
+    uint32_t yes;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(yes));
+    return yes != 0;
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+__device__ __forceinline__ void umma_cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t umma_cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ float ld_peer(uint32_t addr, uint32_t rank) {
+    float v;
+    uint32_t at;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void arrive_peer(uint64_t* bar, uint32_t rank) {
+    uint32_t at;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"(smem_u32(bar)), "r"(rank));
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(at) : "memory");
+}
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return ok != 0;
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return ok != 0;
+}
+// Barrier of the expanding warps; true when `ok` was true for all of them.
+__device__ __forceinline__ bool expand_barrier(bool ok) {
+    uint32_t all;
+    asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\tbarrier.cta.red.and.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(all) : "r"((uint32_t)ok), "n"(kExpandThreads) : "memory");
+    return all != 0;
+}
+__device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void add_release_gpu(uint32_t* p, uint32_t v) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// a += b + c, two floats at a time
+__device__ __forceinline__ void add_pair(float2& a, uint32_t b0, uint32_t b1, uint32_t c0, uint32_t c1) {
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%0, %1};\n\t"
+        "add.rn.f32x2 x, x, y;\n\tadd.rn.f32x2 z, z, x;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "+f"(a.x), "+f"(a.y) : "r"(b0), "r"(b1), "r"(c0), "r"(c1));
+}
+
+// Byte of (row n, column c of the matrix) in the operand images of 2 * NB rows.
+template <int NB> __device__ __forceinline__ size_t image_at(int n, int c) {
+    return (size_t)(c >> 6) * (NB * 256) + (size_t)(n * 128 + ((((c >> 3) & 7) ^ (n & 7)) << 4) + (c & 7) * 2);
+}
+__device__ __forceinline__ uint32_t split_pair(float a, float b, uint32_t& lo) {
+    const __half h0 = __float2half_rn(a), h1 = __float2half_rn(b);
+    const __half l0 = __float2half_rn(a - __half2float(h0)), l1 = __float2half_rn(b - __half2float(h1));
+    lo = (uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16);
+    return (uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16);
+}
+template <int NB> __device__ __forceinline__ void put_value(uint8_t* images, int b, int c, float x) {
+    const __half hi = __float2half_rn(x);
+    uint8_t* at = images + image_at<NB>(b, c);
+    *reinterpret_cast<__half*>(at) = hi;
+    *reinterpret_cast<__half*>(at + NB * 128) = __float2half_rn(x - __half2float(hi));
+}
+// Columns c .. c + 7 (those below n) of batch column b; src points at column c.
+template <int NB> __device__ __forceinline__ void put_eight(uint8_t* images, int b, int c, int n, const float* src, bool vec) {
+    if (c + 8 <= n) {
+        float x[8];
+        if (vec) {
+            const float4 u = __ldg(reinterpret_cast<const float4*>(src)), v = __ldg(reinterpret_cast<const float4*>(src) + 1);
+            x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w; x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = src[i];
+        }
+        uint4 hi, lo;
+        hi.x = split_pair(x[0], x[1], lo.x); hi.y = split_pair(x[2], x[3], lo.y);
+        hi.z = split_pair(x[4], x[5], lo.z); hi.w = split_pair(x[6], x[7], lo.w);
+        uint8_t* at = images + image_at<NB>(b, c);
+        *reinterpret_cast<uint4*>(at) = hi;
+        *reinterpret_cast<uint4*>(at + NB * 128) = lo;
+    } else {
+        for (int i = 0; c + i < n; ++i) put_value<NB>(images, b, c + i, src[i]);
+    }
+}
+
+// One column segment of W words: the lane's row of it, zeros where the row is not kept.
+template <int W>
+__device__ __forceinline__ void expand_segment(uint32_t item, uint32_t header, int lane, uint32_t* r) {
+    const uint4 h = lds128(header);
+    const uint32_t kept = (h.x >> lane) & 1u, step = (uint32_t)__popc(h.x) * 16u;
+    uint32_t p = item + h.y + (uint32_t)__popc(h.x & ((1u << lane) - 1u)) * 16u;
+#pragma unroll
+    for (int j = 0; j < W; j += 4, p += step)
+        asm volatile(
+            "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\tmov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+            "@q ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+            : "=&r"(r[j]), "=&r"(r[j + 1]), "=&r"(r[j + 2]), "=&r"(r[j + 3]) : "r"(p), "r"(kept));
+}
+
+// Shared memory: the two rings (a bare product reuses them for the CTA's sums when the loop is over), then the time loop's
+// sums and cell states, then barriers.
+struct UmmaSmem {
+    size_t x, w, part, cs, bars, total;
+    __host__ __device__ constexpr UmmaSmem(int mode, int NB, int MT)
+        : x(0), w((size_t)x_depth(mode) * kXStage), part(mode ? w + (size_t)kWDepth * kUmmaStage : 0),
+          cs(mode ? part + (size_t)NB * MT * 512 : 0), bars(mode ? cs + (size_t)NB * MT * 128 : w + (size_t)kWDepth * kUmmaStage), total(bars + 512 + 1024) {}
+};
+static_assert(UmmaSmem(0, 64, 2).w + (size_t)kWDepth * kUmmaStage >= 64 * 2 * 512, "the rings hold the sums");
+
+template <int NB, int MT, int MODE>
+__global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_constant__ UmmaArgs a) {
+    constexpr int N = 2 * NB;                             // hi and lo rows of the operand
+    constexpr int kWin = N * 128;                         // bytes of a window's image
+    constexpr int XW = kXStage / kWin;                    // windows per stage of inputs
+    constexpr int DB = kDCols / N;                        // buffers of sums in TMEM (even)
+    constexpr int CN = NB * MT / 4;                       // batch columns whose sums a warp keeps
+    constexpr int XD = x_depth(MODE), kRows = 128 * MT;
+    static_assert(kDCols + kASlots * 32 <= 512 && DB % 2 == 0, "TMEM");
+    constexpr UmmaSmem L(MODE, NB, MT);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
+    uint64_t *xfull = bars, *xempty = xfull + XD, *wfull = xempty + XD, *wempty = wfull + kWDepth;
+    uint64_t *afull = wempty + kWDepth, *aempty = afull + kASlots, *dfull = aempty + kASlots, *dempty = dfull + DB, *pfull = dempty + DB;
+    volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(pfull + 1);
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(pfull + 1) + 1;
+    float* part = reinterpret_cast<float*>(smem + L.part);        // the CTA's sums: [batch column][row of the group]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+    pdl_launch_dependents();
+    int p_idx = 0, cta0 = 0;                              // which product (layer) this CTA works for, and its first CTA
+    while (p_idx + 1 < a.n_parts && (int)blockIdx.x >= a.part[p_idx].cta_end) { cta0 = a.part[p_idx].cta_end; ++p_idx; }
+    const UmmaPart& pt = a.part[p_idx];
+    const UmmaCta* me = pt.ctas + ((int)blockIdx.x - cta0);
+    const int nw = me->nw, w0 = me->w0, F = a.flush, T_ = MODE ? a.T : 1;
+    const int ntw = nw * MT, ntw4 = MODE ? (ntw + 3) & ~3 : ntw;      // (a step's tile-windows are filled up: a warp's slots stay its own)
+    const int groups = (nw + F - 1) / F, units = groups * MT;
+    const int xstages = (nw + XW - 1) / XW, wstages = (int)((me->bytes + kUmmaStage - 1) / kUmmaStage);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < XD; ++i) { mbar_init(xfull + i, 1); mbar_init(xempty + i, 1); }
+        for (int i = 0; i < kWDepth; ++i) { mbar_init(wfull + i, 1); mbar_init(wempty + i, kUmmaExpandWarps); }
+        for (int i = 0; i < kASlots; ++i) { mbar_init(afull + i, 4); mbar_init(aempty + i, 1); }
+        for (int i = 0; i < DB; ++i) { mbar_init(dfull + i, 1); mbar_init(dempty + i, kUmmaExpandWarps / MT); }
+        mbar_init(pfull, (uint32_t)a.S);
+        *s_dead = 0u;
+        mbar_fence_init();
+    }
+    if (warp == kUmmaExpandWarps) tc_alloc(smem_u32(s_tmem), 512);
+    tc_fence_before();
+    __syncthreads();
+    if (MODE && a.S > 1) umma_cluster_barrier();          // the peers' barriers are there before anybody arrives on them
+    tc_fence_after();
+    // (all of TMEM is this CTA's, so it starts at column 0: as a constant the addresses stay in uniform registers)
+    constexpr uint32_t tmem = 0u, a_base = kDCols;
+    if (threadIdx.x == 0 && *s_tmem != 0u) { *s_dead = 1u; *(volatile uint32_t*)a.status = (uint32_t)kDevCopyTimeout; }
+
+    // A wait gives up after a second, or as soon as another one of the CTA has given up.
+    auto gave_up = [&](unsigned int& spins, unsigned long long& t0, unsigned long long limit, uint32_t code) -> bool {
+        if ((++spins & 255u) != 0) return false;
+        if (*s_dead) return true;
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        else if (now - t0 > limit) { *s_dead = 1u; *(volatile uint32_t*)a.status = code; return true; }
+        return false;
+    };
+    // (in the time loop a wait may last as long as the one for other CTAs)
+    const unsigned long long limit = MODE ? kCopyWaitNs + a.limit_ns : kCopyWaitNs;
+    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+        if (mbar_try_wait(bar, parity)) return true;
+        unsigned long long t0 = 0;
+        unsigned int spins = 0;
+        while (!mbar_try_wait_parked(bar, parity, 4000u)) if (gave_up(spins, t0, limit, kDevCopyTimeout)) return false;
+        return true;
+    };
+    float2 acc[CN / 2];
+#pragma unroll
+    for (int i = 0; i < CN / 2; ++i) acc[i] = make_float2(0.f, 0.f);
+    const int quad = warp & 3, slot = warp >> 2;          // expanding warps: lanes of the tile, tile-windows slot, slot + 4, ..
+    const int my_mt = MT == 2 ? slot >> 1 : 0, my_b0 = MT == 2 ? (slot & 1) * CN : slot * CN;      // and whose sums the warp keeps
+    const UmmaQuad* quads = pt.quads + (size_t)me->group * MT * 4;
+
+    if (warp < kUmmaExpandWarps) {
+        const int seg_words = pt.seg_words, segs = 32 / seg_words;
+        uint32_t seg_off[MT];                             // the lane's row segment: where its headers start in an item
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+            const UmmaQuad q = quads[mt * 4 + quad];
+            seg_off[mt] = lane < q.nrows ? (uint32_t)((q.row0 + lane) / pt.block_r - q.row0 / pt.block_r) * (uint32_t)(segs * 16) : 0u;
+        }
+        const uint32_t rank = a.S > 1 ? umma_cluster_rank() : 0u;
+        float* cs = reinterpret_cast<float*>(smem + L.cs);
+        // the time loop's share of this warp: (tile of 32 units, batch column) pairs
+        const int tasks = MODE ? (MT * a.nb - (int)rank + a.S - 1) / a.S : 0;
+        if (MODE)
+            for (int j = warp; j < tasks; j += kUmmaExpandWarps) {
+                const int k = (int)rank + a.S * j, ut = k / a.nb, b = k - ut * a.nb;
+                const UmmaQuad q = quads[ut * 4];
+                cs[j * 32 + lane] = lane < q.nrows ? __ldg(a.state0 + ((size_t)p_idx * a.nb + b) * a.H + q.row0 + lane) : 0.f;
+            }
+        int stage = -1;                                   // of the values: running number, its slot, its parity
+        uint32_t w_slot = kWDepth - 1, w_par = 1u, taken = 0; // taken: items expanded so far
+        bool ok = true;
+        const int unit_shift = (F == 2) + (MT == 2);      // log2 of a full flush group's tile-windows
+        // Tile-windows come unit by unit; a unit is one tile over the windows of a flush group.
+        auto first_of = [&](int u) -> int {
+            const int g = u / MT;
+            return u >= units ? 0x40000000 : g * F * MT + (u % MT) * min(F, nw - g * F);
+        };
+        // Sums of a unit (by the running number) out of TMEM, hi and lo parts added.
+        auto drain = [&](int run) {
+            const int buf = run % DB;
+            tc_fence_after();
+            const uint32_t d = tmem + ((uint32_t)quad << 21) + (uint32_t)(buf * N + my_b0);
+            uint32_t hi[CN], lo[CN];
+            tc_ld<CN>(d, hi);
+            tc_ld<CN>(d + NB, lo);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < CN / 2; ++i) add_pair(acc[i], hi[2 * i], hi[2 * i + 1], lo[2 * i], lo[2 * i + 1]);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(dempty + buf);
+        };
+        auto pass_stages = [&](int want) {                // in order, whether this warp has an item in them or not
+            while (stage < want && ok) {
+                if (stage >= 0) { __syncwarp(); if (lane == 0) mbar_arrive(wempty + w_slot); }
+                ++stage;
+                if (++w_slot == kWDepth) { w_slot = 0; w_par ^= 1u; }
+                ok = __all_sync(0xffffffffu, wait(wfull + w_slot, w_par));
+            }
+        };
+        int unit0 = 0, stage0 = 0;                        // running numbers of the step's first unit and stage of values
+        for (int t = 0; t < T_ && ok; ++t) {
+            uint32_t off = me->first[warp];
+            int unit = my_mt;                             // the next one whose sums this warp takes
+            for (int i = slot; i < ntw4 && ok; i += 4) {
+                // Sums are taken as soon as they are there, and waited for when the operand slots behind them are full
+                // of units that need their buffer.
+                while (unit < units) {
+                    const int run = unit0 + unit;
+                    uint64_t* bar = dfull + run % DB;
+                    const uint32_t par = (uint32_t)(run / DB) & 1u;
+                    if (!__all_sync(0xffffffffu, mbar_test(bar, par))) {
+                        if (i < first_of(unit + DB) + kASlots) break;
+                        ok = __all_sync(0xffffffffu, wait(bar, par));
+                        if (!ok) break;
+                    }
+                    drain(run);
+                    unit += MT;
+                }
+                if (!ok) break;
+                uint32_t r[32];
+                if (i < ntw) {
+                    pass_stages(stage0 + (int)(off / (kUmmaStage / 16)));
+                    if (!ok) break;
+                    const uint32_t item = smem_u32(smem + L.w) + w_slot * kUmmaStage + (off % (kUmmaStage / 16)) * 16u;
+                    const int g = i >> unit_shift, mt = MT == 1 ? 0 : i - (g << unit_shift) >= min(F, nw - g * F);
+                    const uint32_t header = item + (mt ? seg_off[MT - 1] : seg_off[0]);
+                    off = lds32(item + 12);
+                    if (seg_words == 32) expand_segment<32>(item, header, lane, r);
+                    else if (seg_words == 16) { expand_segment<16>(item, header, lane, r); expand_segment<16>(item, header + 16, lane, r + 16); }
+                    else
+#pragma unroll
+                        for (int s = 0; s < 4; ++s) expand_segment<8>(item, header + 16 * s, lane, r + 8 * s);
+                }
+                // (a warp's items go to two of the eight operand slots in turn; a fresh slot's wait ends at once)
+                static_assert(kASlots == 8, "four slots of tile-windows, two of them a warp");
+                const uint32_t as = (uint32_t)slot + ((taken & 1u) << 2);
+                ok = __all_sync(0xffffffffu, wait(aempty + as, ((taken >> 1) & 1u) ^ 1u));
+                if (!ok) break;
+                ++taken;
+                tc_fence_after();
+                if (i < ntw) tc_st32(a_base + ((uint32_t)quad << 21) + as * 32u, r);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(afull + as);
+            }
+            while (ok && unit < units) {
+                const int run = unit0 + unit;
+                ok = __all_sync(0xffffffffu, wait(dfull + run % DB, (uint32_t)(run / DB) & 1u));
+                if (ok) drain(run);
+                unit += MT;
+            }
+            if (!MODE) break;
+            // ---- the step's sums are complete: cluster, gates, h_t
+            if (ok) pass_stages(stage0 + wstages - 1);    // the next step's values can come
+#pragma unroll
+            for (int i = 0; i < CN / 2; ++i) {
+                float* at = part + (my_b0 + 2 * i) * kRows + my_mt * 128 + quad * 32 + lane;
+                at[0] = acc[i].x; at[kRows] = acc[i].y;
+                acc[i] = make_float2(0.f, 0.f);
+            }
+            ok = expand_barrier(ok);
+            if (!ok) break;
+            if (a.S > 1 && (int)threadIdx.x < a.S) arrive_peer(pfull, threadIdx.x);
+            const bool more = t + 1 < T_;
+            const int next = (t + p_idx + 1) & 1;         // the buffer of images that the next tick reads
+            if (p_idx == 0 && more) {                     // x_{t+1}, shared between the CTAs of the first layer
+                const int I = a.in_size[0], chunks = (I + 7) / 8;
+                uint8_t* images = pt.xp + (size_t)next * pt.windows * kWin;
+                for (int i = (int)blockIdx.x * kExpandThreads + (int)threadIdx.x; i < chunks * a.nb; i += pt.cta_end * kExpandThreads) {
+                    const int b = i / chunks, c = (i - b * chunks) * 8;
+                    put_eight<NB>(images, b, c, I, a.x + ((size_t)(t + 1) * a.nb + b) * I + c, a.x_vec != 0);
+                }
+            }
+            if (a.S > 1) {
+                unsigned long long t0 = 0;
+                unsigned int spins = 0;
+                while (!mbar_try_wait_cluster(pfull, (uint32_t)t & 1u)) if (gave_up(spins, t0, limit, kDevBarrierTimeout)) { ok = false; break; }
+                ok = __all_sync(0xffffffffu, ok);
+            }
+            for (int j = warp; j < tasks && ok; j += kUmmaExpandWarps) {
+                const int k = (int)rank + a.S * j, ut = k / a.nb, b = k - ut * a.nb;
+                const UmmaQuad q = quads[ut * 4];
+                const int u = q.row0 + lane;
+                const bool live = lane < q.nrows;
+                const uint32_t at = smem_u32(part) + (uint32_t)(b * kRows + ut * 128 + lane) * 4u;
+                float z[4];
+#pragma unroll
+                for (int gt = 0; gt < 4; ++gt) {
+                    float v[kUmmaMaxS];
+#pragma unroll
+                    for (int s = 0; s < kUmmaMaxS; ++s) v[s] = s < a.S ? (a.S > 1 ? ld_peer(at + gt * 128u, (uint32_t)s) : __uint_as_float(lds32(at + gt * 128u))) : 0.f;
+                    z[gt] = v[0];
+#pragma unroll
+                    for (int s = 1; s < kUmmaMaxS; ++s) z[gt] += v[s];
+                }
+                if (!live) continue;
+                const float* bl = a.bias[p_idx];
+                if (bl) {
+#pragma unroll
+                    for (int gt = 0; gt < 4; ++gt) z[gt] += __ldg(bl + (size_t)gt * a.H + u);
+                }
+                float st = cs[j * 32 + lane], h;
+                if (MODE == 1) h = lstm_cell(z[0], z[1], z[2], z[3], st);
+                else st = h = gru_cell(z[0], z[1], z[2], z[3], st);
+                cs[j * 32 + lane] = st;
+                if (more) put_value<NB>(pt.xp + (size_t)next * pt.windows * kWin, b, a.in_size[p_idx] + u, h);
+                if (p_idx + 1 < a.n_parts) {
+                    const UmmaPart& above = a.part[p_idx + 1];
+                    put_value<NB>(above.xp + (size_t)next * above.windows * kWin, b, u, h);
+                } else if (a.y) a.y[((size_t)t * a.nb + b) * a.H + u] = h;
+                if (!more) {
+                    const size_t e = ((size_t)p_idx * a.nb + b) * a.H + u;
+                    if (a.hT) a.hT[e] = h;
+                    if (MODE == 1 && a.cT) a.cT[e] = st;
+                }
+            }
+            ok = expand_barrier(ok);
+            if (!ok) break;
+            if (threadIdx.x == 0) { __threadfence(); add_release_gpu(a.count, 1u); }
+            unit0 += units; stage0 += wstages;
+        }
+    } else if (warp == kUmmaExpandWarps) {
+        // The whole warp runs along, so that addresses and descriptors live in uniform registers, and one lane issues (with a
+        // single lane running, a tile-window took this warp 1100 cycles: it was what the others waited for).
+        const bool leader = elect_lane();
+        bool ok = true;
+        uint32_t as = 0, a_par = 0, xs = 0, x_par = 0, xin = 0, buf = 0, d_par = 1;
+        const uint64_t x_desc = b_descriptor(smem_u32(smem + L.x));
+        for (int t = 0; t < T_ && ok; ++t) {
+            for (int w_lo = 0; w_lo < nw && ok; w_lo += F) {
+                const int len = min(F, nw - w_lo);
+                const uint32_t xs_lo = xs, x_par_lo = x_par, xin_lo = xin;
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) {
+                    xs = xs_lo; x_par = x_par_lo; xin = xin_lo;
+                    ok = ok && __all_sync(0xffffffffu, wait(dempty + buf, d_par));
+                    for (int w = 0; w < len && ok; ++w) {
+                        if (mt == 0 && xin == 0) ok = wait(xfull + xs, x_par);
+                        ok = __all_sync(0xffffffffu, ok && wait(afull + as, a_par));
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint64_t b = x_desc + (uint64_t)((xs * kXStage + xin * kWin) >> 4);
+                        const bool last = mt == MT - 1 && (xin == XW - 1 || w_lo + w == nw - 1);
+                        if (leader) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                tc_mma_f16(tmem + buf * N, a_base + as * 32u + k * 8, b + (uint64_t)(2 * k), mma_idesc(N), w != 0 || k != 0);
+                            tc_commit(aempty + as);
+                            if (last) tc_commit(xempty + xs);
+                            if (w == len - 1) tc_commit(dfull + buf);
+                        }
+                        __syncwarp();
+                        if (++as == kASlots) { as = 0; a_par ^= 1u; }
+                        if (++xin == XW) { xin = 0; if (++xs == XD) { xs = 0; x_par ^= 1u; } }
+                    }
+                    if (++buf == DB) { buf = 0; d_par ^= 1u; }
+                }
+            }
+            if (xin != 0) { xin = 0; if (++xs == XD) { xs = 0; x_par ^= 1u; } }
+            for (int i = ntw; i < ntw4 && ok; ++i) {
+                ok = __all_sync(0xffffffffu, wait(afull + as, a_par));
+                if (ok && leader) tc_commit(aempty + as);
+                if (++as == kASlots) { as = 0; a_par ^= 1u; }
+            }
+        }
+    } else if (warp == kUmmaExpandWarps + 1) {
+        if (lane == 0) {
+            if (!MODE) pdl_wait();                        // the packed inputs belong to the work in front on the stream
+            bool ok = true;
+            for (int t = 0, run = 0; t < T_ && ok; ++t) {
+                const uint8_t* src = pt.xp + (size_t)w0 * kWin;
+                if (MODE) {
+                    const int tick = t + p_idx;
+                    src += (size_t)(tick & 1) * pt.windows * kWin;
+                    // every CTA with a step in an earlier tick has finished it
+                    uint32_t need = a.never;
+                    for (int l = 0; l < a.n_parts; ++l)
+                        need += (uint32_t)(a.part[l].cta_end - (l ? a.part[l - 1].cta_end : 0)) * (uint32_t)min(max(tick - l, 0), T_);
+                    unsigned long long t0 = 0;
+                    unsigned int spins = 0;
+                    while ((int32_t)(ld_acquire_gpu(a.count) - need) < 0) if (gave_up(spins, t0, a.limit_ns, kDevBarrierTimeout)) { ok = false; break; }
+                    fence_proxy_async_all();              // what others have stored is read by copies
+                }
+                for (int i = 0; i < xstages && ok; ++i, ++run) {
+                    const int at = run % XD;
+                    if (run >= XD) ok = wait(xempty + at, (uint32_t)(run / XD - 1) & 1u);
+                    if (!ok) break;
+                    const uint32_t bytes = (uint32_t)min(XW, nw - i * XW) * kWin;
+                    mbar_expect_tx(xfull + at, bytes);
+                    bulk_g2s(smem + L.x + (size_t)at * kXStage, src + (size_t)i * kXStage, bytes, xfull + at);
+                }
+            }
+        }
+    } else {
+        if (lane == 0) {                                  // (written at plan time: the copies need not wait for the work in front)
+            const uint8_t* src = pt.stream + (size_t)me->off128 * 128;
+            const uint32_t total = me->bytes;
+            bool ok = true;
+            for (int t = 0, run = 0; t < T_ && ok; ++t)
+                for (int i = 0; i < wstages; ++i, ++run) {
+                    const int at = run % kWDepth;
+                    if (run >= kWDepth && !wait(wempty + at, (uint32_t)(run / kWDepth - 1) & 1u)) { ok = false; break; }
+                    const uint32_t bytes = min((uint32_t)kUmmaStage, total - (uint32_t)i * kUmmaStage);
+                    mbar_expect_tx(wfull + at, bytes);
+                    bulk_g2s(smem + L.w + (size_t)at * kUmmaStage, src + (size_t)i * kUmmaStage, bytes, wfull + at);
+                }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const bool dead = *s_dead != 0u;
+    if (dead) {
+        // a wait gave up (the status word says so): copies and tensor instructions that may still be in flight get a bounded
+        // time to end before the CTA's memories go away, and nothing is written
+        const unsigned long long t0 = global_ns();
+        while (global_ns() - t0 < 200000ull) __nanosleep(1000);
+    }
+    if (warp == kUmmaExpandWarps) tc_dealloc(tmem, 512);
+    if (MODE) {
+        if (a.S > 1) umma_cluster_barrier();              // nobody leaves before everybody has read
+        return;
+    }
+    pdl_wait();                                           // Y belongs to the work in front
+    if (a.S == 1) {
+        if (!dead && warp < kUmmaExpandWarps) {
+            const UmmaQuad q = quads[my_mt * 4 + quad];
+            if (lane < q.nrows)
+#pragma unroll
+                for (int i = 0; i < CN; ++i)
+                    if (my_b0 + i < a.nb) pt.Y[(long long)(my_b0 + i) * a.ldy + q.out0 + lane] = i & 1 ? acc[i / 2].y : acc[i / 2].x;
+        }
+        return;
+    }
+    if (warp < kUmmaExpandWarps)
+#pragma unroll
+        for (int i = 0; i < CN / 2; ++i) {
+            float* at = part + (my_b0 + 2 * i) * kRows + my_mt * 128 + quad * 32 + lane;
+            at[0] = acc[i].x; at[kRows] = acc[i].y;
+        }
+    __syncthreads();
+    umma_cluster_barrier();
+    // every CTA adds the ranges, in range order, for its share of the quadrants
+    const uint32_t rank = umma_cluster_rank(), base = smem_u32(part);
+    if (!dead && warp < kUmmaExpandWarps) {
+        const int mine = (4 * MT - (int)rank + a.S - 1) / a.S;         // quadrants rank, rank + S, ..
+        for (int i0 = warp; i0 < mine * a.nb; i0 += 2 * kUmmaExpandWarps) {
+            float v[2][kUmmaMaxS];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int i = min(i0 + j * kUmmaExpandWarps, mine * a.nb - 1), qi = (int)rank + (i / a.nb) * a.S, b = i % a.nb;
+                const uint32_t at = base + (uint32_t)(b * kRows + qi * 32 + lane) * 4u;
+#pragma unroll
+                for (int s = 0; s < kUmmaMaxS; ++s) v[j][s] = s < a.S ? ld_peer(at, (uint32_t)s) : 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int i = i0 + j * kUmmaExpandWarps, qi = (int)rank + (i / a.nb) * a.S, b = i % a.nb;
+                if (i >= mine * a.nb) break;
+                float sum = v[j][0];
+#pragma unroll
+                for (int s = 1; s < kUmmaMaxS; ++s) sum += v[j][s];
+                const UmmaQuad q = quads[qi];
+                if (lane < q.nrows) pt.Y[(long long)b * a.ldy + q.out0 + lane] = sum;
+            }
+        }
+    }
+    __syncthreads();
+    umma_cluster_barrier();                               // nobody leaves before everybody has read
+}
+
+}  // namespace csb

@@ -1,0 +1,31 @@
+// The batched recurrent stacks on tcgen05: what csb_umma.cu, csb_umma_rnn.cu and csb_rnn_step.cu share.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <memory>
+
+#include "csb_umma.hpp"
+
+namespace csb {
+
+// csb_umma.cu
+int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]);
+int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P);
+const void* pick_umma(int mode, int NB, int MT);
+size_t umma_smem(int mode, int NB, int MT);
+int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st);
+
+// The layouts of a stack's layers, for every batch size.
+struct UmmaStack {
+    std::vector<uint64_t> uids;
+    int gates = 0, L = 0, H = 0, device = -1;
+    int in_size[kMaxLayers] = {};
+    bool taken = false;                // false: a layer does not suit the layout
+    bool resident = false;             // one grid holds all layers: the time loop serves it
+    UmmaPlan plan[kMaxLayers];
+    ~UmmaStack();
+};
+int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size, int H, std::shared_ptr<UmmaStack>* out);   // csb_umma_rnn.cu; null: not taken
+
+}  // namespace csb

@@ -1,0 +1,70 @@
+"""The batched product and time loop on tcgen05 at the sizes where their tiles, windows and batch tiles end."""
+import numpy as np
+import pytest
+import torch
+
+import workloads
+from oracle import csb_oracle as O
+from oracle import rnn_oracle as R
+from paper_2005_05758_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+# Error of an output in units of sum |w| |x|: the split x = hi + lo (2^-22), a chain of at most 8 truncated sums in the
+# tensor cores (2^-23 each), then one rounded sum per flush group and column range, at most 64 here (2^-24 each).
+TOL = 2.0 ** -22 + 8 * 2.0 ** -23 + 64 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("rows,cols,br,bc,batch", [(1, 1, 16, 16, 8), (127, 63, 32, 32, 9), (129, 65, 16, 16, 17), (300, 1177, 32, 32, 33),
+                                                   (513, 2049, 64, 64, 64), (200, 130, 64, 128, 65), (70, 4200, 24, 64, 16), (1000, 192, 50, 32, 32)])
+def test_product_against_the_oracle(rows, cols, br, bc, batch):
+    w = workloads.make_spmv_workload(rows + cols, rows, cols, br, bc, "uniform", lo=0.3, hi=0.9, batch=batch, w_std=0.05)
+    m = w.matrix
+    A = binding.csb_encode(m.dense, br, bc, m.row_keep, m.col_keep, "f16", 0)
+    args = (m.dense, br, bc, m.row_keep, m.col_keep, "f16")
+    want, scale = O.spmm(*args, w.X), O.abs_scale(*args, w.X)
+    for pad in (0, 3):                                   # rows of x and y with and without 16-byte alignment
+        x = torch.full((batch, cols + pad), float("nan"), device="cuda")
+        x[:, :cols] = torch.from_numpy(w.X).cuda()
+        y = torch.full((batch, rows + pad), float("nan"), device="cuda")
+        binding.csb_spmm(A, x[:, :cols], y[:, :rows])
+        torch.cuda.synchronize()
+        got = y.cpu().numpy()
+        assert np.all(np.abs(got[:, :rows] - want) <= TOL * scale)
+        assert np.isnan(got[:, rows:]).all()
+    A.free()
+
+
+@pytest.mark.parametrize("cell,B,I,H,L,T", [("lstm", 16, 39, 100, 3, 5), ("lstm", 31, 1, 33, 1, 4), ("gru", 32, 70, 96, 2, 5), ("gru", 17, 153, 160, 1, 1)])
+def test_time_loop_against_the_oracle(cell, B, I, H, L, T):
+    w = workloads.make_rnn_workload(61, cell, I, H, L, 32, 32, "uniform", lo=0.3, hi=0.8, T=T, B=B, w_std=0.15, bias_std=0.2, state_std=0.4)
+    mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in w.layers]
+    lay = [(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype) for m in w.layers]
+    x, h0, bias = torch.from_numpy(w.x).cuda(), torch.from_numpy(w.h0).cuda(), [torch.from_numpy(b).cuda() for b in w.bias]
+    y, hT = torch.full((T, B, H), float("nan"), device="cuda"), torch.full((L, B, H), float("nan"), device="cuda")
+
+    def run():
+        if cell == "gru":
+            binding.csb_gru_forward(mats, bias, x, h0, y, hT, 0)
+        else:
+            binding.csb_lstm_forward(mats, bias, x, h0, torch.from_numpy(w.c0).cuda(), y, hT, None, 0)
+    run()
+    want = R.gru_forward(lay, w.bias, w.x, w.h0) if cell == "gru" else R.lstm_forward(lay, w.bias, w.x, w.h0, w.c0)
+    # fp32 sums of fp16 weights: an absolute error of 1e-6 of a pre-activation of size 1 a step (TOL and the activations'), which
+    # the recurrence carries on; 5 steps of up to 3 layers
+    for got, ref in ((y, want[0]), (hT, want[1])):
+        assert np.max(np.abs(got.cpu().numpy() - np.asarray(ref))) < 15 * 2e-6
+    if T > 1:
+        # a wait that runs out is a status, and the next call is as good as the first
+        binding.lib.csb_test_barrier_hook(1, 200_000)
+        try:
+            with pytest.raises(binding.CsbError) as e:
+                run()
+            assert e.value.status == -7
+        finally:
+            binding.lib.csb_test_barrier_hook(0, 0)
+        y.fill_(float("nan"))
+        run()
+        assert np.max(np.abs(y.cpu().numpy() - np.asarray(want[0]))) < 15 * 2e-6
+    for m in mats:
+        m.free()
