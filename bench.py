@@ -390,7 +390,7 @@ def spmv_sweep(binding, torch, dev, rates, batch, l2, reps=10, with_cpu=False, c
              "us_warm_l2": round(us_warm, 3), "GBps_warm_l2": round(alg / us_warm / 1e3, 1),
              "frac_l2_warm": round(alg / us_warm / 1e3 / l2, 4) if l2 else None,
              "balance": round(info["panel_balance"] if panel else info["balance"], 3), "copies": ncopy, "launches_per_graph": n,
-             "kernel": "csb_panel_kernel" if panel else ("csb_product_kernel" if batch < 8 else "csb_pack_x_kernel + csb_spmm_tile_kernel"),
+             "kernel": "csb_panel_kernel" if panel else ("csb_product_kernel" if batch < 8 else "csb_umma_pack_kernel + csb_umma_kernel"),
              "streamed_bytes": stream_bytes if batch < 8 else None, "max_rel_err": err}
         if us_serial is not None:
             e["launch"] = "programmatic stream serialization (start-up overlaps the launch in front)"
@@ -503,12 +503,10 @@ def config_entry(binding, torch, dev, flush, w, steps, hbm, l2, sm_mhz, with_cpu
     sw = stepwise(w, nnz)
     e = {"us_per_timestep": round(us, 3), "T": w.T, "B": w.B, "algorithmic_bytes_per_step": alg,
          "GFLOPs": round(2 * nnz * w.B / us / 1e3, 1),
-         "path": "per-step launches, products on tensor cores" if sw else "persistent time-loop kernel",
+         "path": "time loop on tensor cores" if sw else "persistent time-loop kernel",
          "bound": "l2" if sw else "smem", "roofline": three_rooflines(alg, us, hbm, l2, sm_mhz)}
-    # step by step: one to begin, then a product and a gate kernel per tick of the wavefront; beyond 32 product rows
-    # a pack, a product and a gate kernel per layer and step
-    wave = w.B * (2 if w.cell == "gru" else 1) <= 32
-    launches = (steps + 4) * (1 if not sw else 1 + 2 * (w.T + len(w.layers) - 1) if wave else w.T * len(w.layers) * 3)
+    # one to begin and one for the sequence; beyond 32 sequences a pack, a product and a gate kernel per layer and step
+    launches = (steps + 4) * (1 if not sw else 2 if w.B <= 32 else w.T * len(w.layers) * 3)
     if with_cpu:
         ts, tl = t_sample
         o_us, err = oracle_sample(w, y, ts, tl)
@@ -745,10 +743,10 @@ def main():
             line["spmm"] += res
             launches += 2 * -(-bsz // 64) * n_l          # per pass of up to 64 batch columns: the pack kernel and the product kernel
         best = max(line["spmm"], key=lambda r: r["frac_hbm_measured"])
-        line["roofline_spmm"] = {"kernel": "csb_spmm_tile_kernel", "bound": "hbm", "achieved": best["GBps"], "peak": hbm, "peak_kind": peak_kind,
+        line["roofline_spmm"] = {"kernel": "csb_umma_kernel", "bound": "hbm", "achieved": best["GBps"], "peak": hbm, "peak_kind": peak_kind,
                                  "unit": "GB/s", "frac": best["frac_hbm_measured"],
-                                 "traffic": counters.get("csb_spmm_tile_kernel cfg4 4x B=64") if (best["rate"] == 4.0 and best["batch"] == 64) else None,
-                                 "traffic_per_pass_4x_batch64": counters.get("csb_spmm_tile_kernel cfg4 4x B=64"),
+                                 "traffic": counters.get("csb_umma_kernel cfg4 4x B=64") if (best["rate"] == 4.0 and best["batch"] == 64) else None,
+                                 "traffic_per_pass_4x_batch64": counters.get("csb_umma_kernel cfg4 4x B=64"),
                                  "workload": "cfg4 8192x8192, 64x64 blocks, rate %gx, batch %d, cold" % (best["rate"], best["batch"])}
     if rank == 0 and "project" in sections:
         line["project"] = project_bench(binding, torch)

@@ -257,10 +257,12 @@ int plan_spmm_host(const csb_matrix* A, int NT, int sm_count, int force_S, SpmmH
 // The same product on tcgen05 (csb_umma.hpp, csb_umma_plan.cpp, csb_umma.cu): blocks of 16, 32 or a multiple of 64 columns.
 struct UmmaCta;
 struct UmmaQuad;
+struct UmmaRound;
 struct UmmaPlan {                          // device side
     bool built = false, unusable = false;
     int MT = 1, S = 1, flush = 1, n_ctas = 0, windows = 0, seg_words = 32;
-    uint8_t* d_stream = nullptr; UmmaCta* d_ctas = nullptr; UmmaQuad* d_quads = nullptr;
+    int max_round = 0;                     // bytes of the largest round of values
+    uint8_t* d_stream = nullptr; UmmaCta* d_ctas = nullptr; UmmaQuad* d_quads = nullptr; UmmaRound* d_rounds = nullptr;
     uint8_t* d_xp = nullptr;               // packed inputs of a bare product
 };
 bool umma_applicable(const csb_matrix* A);

@@ -1,4 +1,5 @@
-// LSTM and GRU layers at larger batch, one timestep at a time on tensor cores.
+// LSTM and GRU layers at larger batch, one timestep at a time on tensor cores: what the time loop of csb_umma_rnn.cu does not
+// take (more than 32 sequences, stacks that one grid does not hold, blocks whose width is not 16, 32 or a multiple of 64).
 //
 // With a batch of 16 or more the per-step product of Section 2.1, W . [u_t ; h_{t-1}] for all
 // batch columns at once, is a dense contraction per block (kernel matrix times gathered inputs),
@@ -21,6 +22,7 @@
 // GRU (reset gate applied after the recurrent product) needs the input part and the recurrent part
 // of the candidate's pre-activation apart.  One product still does: V_l has 2B rows, row b holds
 // [u_t ; 0] and row B + b holds [0 ; h_{t-1}], so row b of the product is W_x u and row B + b is W_h h.
+// On the layouts of csb_umma.hpp the two parts are output rows of their own, and V_l has B rows.
 #include <algorithm>
 #include <list>
 #include <memory>
@@ -271,7 +273,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
                 np->uids.push_back(W[l]->uid);
                 np->in_size[l] = in_size[l];
                 // (what is read of the packed inputs is written on the call's stream first, so they need no clearing here)
-                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], np->umma ? (size_t)np->umma->plan[l].windows * kUmmaStage : (size_t)(in_size[l] + H) * pitch));
+                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], np->umma ? (size_t)np->umma->plan[l].windows * kUmmaImage : (size_t)(in_size[l] + H) * pitch));
                 if (!packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_v[l], (size_t)rows_v * (in_size[l] + H) * 4));
             }
             const int rc = np->umma ? (int)CSB_OK : prepare_spmm_stack(L, W, std::min(rows_v, 32), &np->stack);

@@ -1,4 +1,6 @@
-// Tensor-core CSB-SpMM (batch >= 8, fp16 values, fp32 accumulation).
+// Tensor-core CSB-SpMM (batch >= 8, fp16 values, fp32 accumulation) for blocks whose width is not 16, 32 or a multiple of 64;
+// those go through csb_umma_kernel.cuh, whose column segments need such widths (at 20 sizes from 512 x 256 to 8192 x 8192, 8 to
+// 64 columns, 4x to 25x, that kernel was the faster one at each).
 //
 // With a batch of vectors the product of a block's kernel matrix (m kept rows x n kept columns)
 // with the gathered inputs (n x batch) of Section 4.3.1 is a small dense contraction, the one place

@@ -48,7 +48,20 @@ const void* pick_umma(int mode, int NB, int MT) {
     if (NB < 64) return pick_mode<0>(NB, MT);
     return MT == 1 ? (const void*)csb_umma_kernel<64, 1, 0> : (const void*)csb_umma_kernel<64, 2, 0>;
 }
-size_t umma_smem(int mode, int NB, int MT) { return UmmaSmem(mode, NB, MT).total; }
+// Stages of inputs, and what is left of `room` bytes of shared memory for values, in rounds of up to max_round bytes; false: too
+// little.  (All of the room: a CTA takes all of TMEM, so two must not meet on an SM.)
+bool umma_stages(int mode, int NB, int MT, int max_round, size_t room, UmmaStages* out) {
+    for (int xd = x_windows(NB, MT) * NB * 256 >= 32768 ? 3 : kMaxXDepth; xd >= 2; --xd) {
+        const UmmaSmem none(mode, NB, MT, xd, 0);
+        const size_t fixed = (size_t)none.total - none.bars + none.w + (mode ? none.bars - none.part : 0);
+        if (fixed >= room) continue;
+        const int bytes = (int)((room - fixed) & ~(size_t)1023);
+        if (bytes < (xd > 2 ? 2 : 1) * max_round || UmmaSmem(mode, NB, MT, xd, bytes).total > room) continue;
+        *out = UmmaStages{xd, bytes, room};
+        return true;
+    }
+    return false;
+}
 
 static cudaLaunchConfig_t umma_config(int ctas, int S, size_t smem, cudaStream_t st, cudaLaunchAttribute (&attr)[2]) {
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -67,8 +80,7 @@ int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]) {
     const int sms = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
     n[0] = 0; n[1] = sms;
     const void* kernel = pick_umma(0, 64, 2);
-    const size_t smem = umma_smem(1, 32, 2);               // the largest
-    if (smem > A->smem_optin) { for (int S = 1; S <= kUmmaMaxS; ++S) n[S] = 0; return CSB_OK; }
+    const size_t smem = A->smem_optin;                     // (one CTA an SM in any case)
     CSB_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
     for (int S = 2; S <= kUmmaMaxS; ++S) {
         cudaLaunchAttribute attr[2];
@@ -80,13 +92,14 @@ int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]) {
 }
 
 void drop_umma_plan(UmmaPlan& P) {
-    cudaFree(P.d_stream); cudaFree(P.d_ctas); cudaFree(P.d_quads); cudaFree(P.d_xp);
-    P.d_stream = nullptr; P.d_ctas = nullptr; P.d_quads = nullptr; P.d_xp = nullptr;
+    cudaFree(P.d_stream); cudaFree(P.d_ctas); cudaFree(P.d_quads); cudaFree(P.d_rounds); cudaFree(P.d_xp);
+    P.d_stream = nullptr; P.d_ctas = nullptr; P.d_quads = nullptr; P.d_rounds = nullptr; P.d_xp = nullptr;
 }
 
 // Uploads a host plan.
 int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P) {
     P->MT = H.MT; P->S = H.S; P->n_ctas = (int)H.ctas.size(); P->windows = H.windows; P->seg_words = H.seg_words; P->flush = H.flush;
+    P->max_round = (int)H.max_round;
     CSB_CUDA(cudaMalloc((void**)&P->d_stream, std::max<size_t>(H.total128, 1) * 128));
     for (size_t i = 0; i < H.ctas.size(); ++i)
         if (!H.streams[i].empty())
@@ -95,9 +108,14 @@ int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P) {
     CSB_CUDA(cudaMemcpyAsync(P->d_ctas, H.ctas.data(), H.ctas.size() * sizeof(UmmaCta), cudaMemcpyHostToDevice, cudaStreamPerThread));
     CSB_CUDA(cudaMalloc((void**)&P->d_quads, H.quads.size() * sizeof(UmmaQuad)));
     CSB_CUDA(cudaMemcpyAsync(P->d_quads, H.quads.data(), H.quads.size() * sizeof(UmmaQuad), cudaMemcpyHostToDevice, cudaStreamPerThread));
+    CSB_CUDA(cudaMalloc((void**)&P->d_rounds, H.rounds.size() * sizeof(UmmaRound)));
+    CSB_CUDA(cudaMemcpyAsync(P->d_rounds, H.rounds.data(), H.rounds.size() * sizeof(UmmaRound), cudaMemcpyHostToDevice, cudaStreamPerThread));
     CSB_CUDA(cudaStreamSynchronize(cudaStreamPerThread));
-    for (int NB = 16; NB <= 64; NB *= 2)
+    UmmaStages st;
+    for (int NB = 16; NB <= 64; NB *= 2) {
+        if (!umma_stages(0, NB, H.MT, P->max_round, A->smem_optin, &st)) { P->unusable = true; return CSB_OK; }
         CSB_CUDA(cudaFuncSetAttribute(pick_umma(0, NB, H.MT), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)A->smem_optin));
+    }
     P->built = true;
     return CSB_OK;
 }
@@ -116,9 +134,9 @@ static int make_umma_plan(const csb_matrix* A, UmmaPlan* P) {
         H.flush = umma_flush(H.windows);
         H.quads = umma_row_quads(A, H.MT);
         H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
-        if (!plan_umma_host(A, &H)) { P->unusable = true; return 1; }
+        plan_umma_host(A, &H);
         rc = upload_umma(A, H, P);
-        if (rc == CSB_OK && P->built) CSB_CUDA(cudaMalloc((void**)&P->d_xp, (size_t)H.windows * 64 * 256));
+        if (rc == CSB_OK && P->built) CSB_CUDA(cudaMalloc((void**)&P->d_xp, (size_t)H.windows * kUmmaImage));
     } catch (const std::bad_alloc&) { set_error("out of host memory while planning the batched product"); rc = CSB_ERR_ALLOC; }
     if (rc != CSB_OK) {
         drop_umma_plan(*P);
@@ -141,10 +159,13 @@ int launch_umma_packed(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, floa
     UmmaArgs a{};
     a.n_parts = 1; a.nb = nb; a.ldy = ldy; a.status = A->product.d_status; a.S = P->S; a.flush = P->flush;
     UmmaPart& p = a.part[0];
-    p.stream = P->d_stream; p.ctas = P->d_ctas; p.quads = P->d_quads; p.xp = xp; p.Y = Y;
+    UmmaStages g;
+    if (!umma_stages(0, NB, P->MT, P->max_round, A->smem_optin, &g)) { set_error("the batched product's stages do not fit"); return CSB_ERR_LAUNCH; }
+    a.x_depth = g.x_depth; a.w_bytes = g.w_bytes;
+    p.stream = P->d_stream; p.ctas = P->d_ctas; p.rounds = P->d_rounds; p.quads = P->d_quads; p.xp = xp; p.Y = Y;
     p.block_r = A->block_r; p.seg_words = P->seg_words; p.windows = P->windows; p.cta_end = P->n_ctas;
     cudaLaunchAttribute attr[2];
-    const cudaLaunchConfig_t cfg = umma_config(P->n_ctas, P->S, umma_smem(0, NB, P->MT), st, attr);
+    const cudaLaunchConfig_t cfg = umma_config(P->n_ctas, P->S, g.smem, st, attr);
     void* args[] = {&a};
     CSB_CUDA(cudaLaunchKernelExC(&cfg, pick_umma(0, NB, P->MT), args));
     return CSB_OK;
@@ -163,7 +184,7 @@ int launch_umma_pack(const float* X, int64_t ldx, int nb, int cols, int NB, uint
     return CSB_OK;
 }
 
-// Packs fp32 inputs into xp (windows * 16 KB) and launches, 64 batch columns at a time.
+// Packs fp32 inputs into xp (windows * kUmmaImage bytes) and launches, 64 batch columns at a time.
 int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st) {
     for (int b0 = 0; b0 < batch; b0 += 64) {
         const int nb = std::min(64, batch - b0), NB = umma_nb(nb);

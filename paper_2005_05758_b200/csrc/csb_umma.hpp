@@ -9,7 +9,6 @@
 //   header  uint4 per (row segment, column segment), row segments first:
 //             x  bit l: lane l's row is kept (zero outside of the segment's rows, and where no column is kept)
 //             y  where the segment's values start, bytes from the item
-//             w  first header only: where the warp's next item starts (16-byte units of the CTA's stream; ~0: none)
 //   values  16 bytes per eight columns and kept row, [eight columns][row], binary16, zero where a column is not kept
 //
 // A row segment is the part of one block-row that lies in the quadrant, a column segment 16, 32 or 64 columns, the
@@ -17,16 +16,18 @@
 // eight 16-byte loads.  With the columns compact by pairs (1.5 instead of 2 times the compact size at 4x, 1.8 instead of
 // 5 at 25x) it took a predicated load and add for every pair, and the expanding warps' instructions set the time.
 //
-// The items of a CTA lie back to back in the order (group of `flush` windows, tile, window, quadrant): the sums of a tile
-// over such a group come out of the tensor cores' accumulators before they grow further.  No item straddles a multiple of
-// kUmmaStage bytes of the CTA's stream, which travels in stages of that size.
+// The tile-windows of a CTA go in rounds of four, one for each four of the sixteen expanding warps, in the order (group of
+// `flush` windows, tile, window): the sums of a tile over such a group, a unit, come out of the tensor cores' accumulators
+// before they grow further.  A round's items travel together, behind a table of where each warp's item starts.
+// (Rounds, and not single tile-windows with a barrier each: the warp that issues the tensor instructions spent 530
+// cycles on each with its waits and commits, 8192 x 8192 at batch 8 22 us.)
 #pragma once
 
 #include "csb_internal.hpp"
 
 namespace csb {
 
-enum { kUmmaStage = 16384, kUmmaStages = 6, kUmmaWindow = 64, kUmmaExpandWarps = 16, kUmmaMaxMT = 2, kUmmaMaxS = 8 };
+enum { kUmmaWindow = 64, kUmmaImage = 64 * 256 /* bytes of a window of packed inputs, 64 batch columns */, kUmmaExpandWarps = 16, kUmmaMaxMT = 2, kUmmaMaxS = 8 };
 
 struct UmmaQuad {             // 32 lanes of a tile
     int32_t row0, nrows;      // their rows of the matrix (none: nrows = 0)
@@ -35,20 +36,22 @@ struct UmmaQuad {             // 32 lanes of a tile
 };
 static_assert(sizeof(UmmaQuad) == 32, "two 16-byte words");
 struct UmmaCta {
-    uint32_t off128;          // where its stream starts, 128-byte units
-    uint32_t bytes;
+    uint32_t off128;          // where its rounds start, 128-byte units
+    int32_t table;            // its first entry in the table of rounds
     int32_t group, split;     // row group and which column range of it
     int32_t w0, nw;           // windows
     int32_t pad[2];
-    uint32_t first[kUmmaExpandWarps];   // per expanding warp: its first item, 16-byte units of the CTA's stream (~0: none)
 };
-static_assert(sizeof(UmmaCta) == 96, "six 16-byte words");
+static_assert(sizeof(UmmaCta) == 32, "two 16-byte words");
+struct UmmaRound { uint32_t off16, bytes; };   // a round of a CTA, from its start
 
 struct UmmaHostPlan {
     int MT = 1, S = 1, flush = 1, n_groups = 0, windows = 0, seg_words = 32;   // seg_words: 32-bit words of a row of a column segment
     std::vector<UmmaQuad> quads;          // [n_groups][MT][4]
     std::vector<UmmaCta> ctas;            // [n_groups][S]
+    std::vector<UmmaRound> rounds;        // CTA after CTA
     std::vector<std::vector<uint8_t>> streams;   // per CTA
+    uint32_t max_round = 0;               // bytes
     uint64_t total128 = 0;                // all streams, 128-byte units
 };
 
@@ -62,14 +65,25 @@ std::vector<UmmaQuad> umma_gate_quads(int gates, int in_size, int H, int MT);
 // Tiles per CTA and column ranges per group for `tiles` tiles of `windows` windows on a device that holds clusters[S] clusters of S.
 double umma_cost(int MT, int S, int windows);          // a CTA's modelled time, in tile-windows
 void umma_shape(int tiles, int windows, const int* clusters, int* MT, int* S);
+// Tile-window j of a round that has nj of them: which of the MT tiles, and which of the round's windows.  `len` is the
+// number of windows of a unit.
+struct UmmaPlace { int mt, window; };
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int umma_unit_len(int MT, int flush, int nj) { return MT == 2 && 2 * flush > nj ? nj / 2 : flush; }
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline UmmaPlace umma_place(int MT, int len, int j) {
+    return MT == 1 ? UmmaPlace{0, j} : len == 2 ? UmmaPlace{j >> 1, j & 1} : UmmaPlace{j & 1, j >> 1};
+}
 // Windows per flush group.  The tensor cores truncate each sum, so the error follows the number of steps between two flushes;
 // the bounds are those at which it stays below what mma.sync gave, whose chains grow with the number of columns
 // (2-norm of the error against 64 bits, mma.sync / 1 / 2 windows: 1024 x 1536 at 4x 1.40e-7 / 1.30e-7 / 1.52e-7, 700 x
 // 2050 at 6x 1.75 / 1.08 / 1.27, 8192 x 8192 at 4x 8.37 / 1.45 / 1.73, 25x 2.07 / 1.23 / 1.32).
 inline int umma_flush(int windows) { return windows < 32 ? 1 : 2; }
-// Fills streams, ctas (the other members are set); throws std::bad_alloc.  False: the layout does not take the matrix (a warp's
-// last item lies more than the ring's stages in front of the end of its CTA's stream, which nobody would then free: blocks
-// of a few rows with next to nothing pruned).
-bool plan_umma_host(const csb_matrix* A, UmmaHostPlan* P);
+// Fills streams, rounds, ctas (the other members are set); throws std::bad_alloc.
+void plan_umma_host(const csb_matrix* A, UmmaHostPlan* P);
 
 }  // namespace csb

@@ -11,10 +11,10 @@
 //   * the inputs are packed into binary16 pairs x = hi + lo (no input precision is lost as long as |x| < 65504) as 128-byte
 //     swizzled, K-major operand images, 64 columns each, the hi rows of all batch columns, then the lo rows; a
 //     bulk copy brings an image as it is;
-//   * one thread issues the tcgen05.mma, one the copies of the inputs, one those of the values;
-//   * the tensor cores add into TMEM with truncation, so the sums of a unit (a tile over `flush` windows) start from zero
-//     and are taken out by the same sixteen warps, which add them in registers with rounding.  The units' buffers go
-//     round, so that the next ones run meanwhile;
+//   * one warp issues the tcgen05.mma, one thread the copies of the inputs, one those of the values;
+//   * the tensor cores add into TMEM with truncation, so the hi rows' sums of a unit (a tile over `flush` windows) start
+//     from zero and are taken out by the same sixteen warps, which add them in registers with rounding.  The units' buffers
+//     go round, so that the next ones run meanwhile.  The lo rows' sums are 2^-11 of the others and may stay until the end;
 //   * a row group's column ranges are one thread-block cluster and are added in range order through distributed
 //     shared memory: results are bit-reproducible, no scratch, no atomics.
 //
@@ -31,16 +31,17 @@
 
 namespace csb {
 
-constexpr int kXStage = 16384;                 // bytes of a stage of inputs: one window of 64 batch columns, two of 32, four of 16
-constexpr int kWDepth = kUmmaStages;           // stages of values in shared memory
-constexpr int kASlots = 8;                     // tile-windows of the A operand in TMEM, 32 columns each
+constexpr int kASlots = 8;                     // tile-windows of the A operand in TMEM, 32 columns each: two rounds
 constexpr int kDCols = 256;                    // columns of TMEM for sums
-constexpr int kExpandThreads = kUmmaExpandWarps * 32, kUmmaThreads = kExpandThreads + 3 * 32;
-__host__ __device__ constexpr int x_depth(int mode) { return mode ? 4 : 5; }
+constexpr int kMaxXDepth = 4, kWRounds = 6;    // stages of inputs, rounds of values in shared memory
+constexpr int kExpandThreads = kUmmaExpandWarps * 32, kUmmaThreads = kExpandThreads + 4 * 32;
+// Windows of a stage of inputs: a round's, or half of it for 64 batch columns on one tile (32 KB).
+__host__ __device__ constexpr int x_windows(int NB, int MT) { return MT == 2 || NB == 64 ? 2 : 4; }
 
 struct UmmaPart {
     const uint8_t* stream;
     const UmmaCta* ctas;
+    const UmmaRound* rounds;
     const UmmaQuad* quads;
     uint8_t* xp;               // packed inputs: per window an image of 2 * NB rows of 128 bytes (time loop: two such buffers)
     float* Y;
@@ -52,6 +53,7 @@ struct UmmaArgs {
     long long ldy;
     uint32_t* status;
     int n_parts, nb, S, flush;
+    int x_depth, w_bytes;                                  // stages of inputs, bytes for rounds of values (UmmaSmem)
     // time loop: a part is a layer
     const float* x; float* y; const float* state0;        // [T, nb, in_size[0]]; [T, nb, H] or null; [L, nb, H]: c (LSTM) or h (GRU) at the start
     float *hT, *cT;                                        // [L, nb, H] or null
@@ -185,11 +187,10 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
 __device__ __forceinline__ void add_release_gpu(uint32_t* p, uint32_t v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-// a += b + c, two floats at a time
-__device__ __forceinline__ void add_pair(float2& a, uint32_t b0, uint32_t b1, uint32_t c0, uint32_t c1) {
-    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%0, %1};\n\t"
-        "add.rn.f32x2 x, x, y;\n\tadd.rn.f32x2 z, z, x;\n\tmov.b64 {%0, %1}, z;\n\t}"
-        : "+f"(a.x), "+f"(a.y) : "r"(b0), "r"(b1), "r"(c0), "r"(c1));
+// a += b, two floats at a time
+__device__ __forceinline__ void add_pair(float2& a, uint32_t b0, uint32_t b1) {
+    asm("{\n\t.reg .b64 x, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 z, {%0, %1};\n\tadd.rn.f32x2 z, z, x;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "+f"(a.x), "+f"(a.y) : "r"(b0), "r"(b1));
 }
 
 // Byte of (row n, column c of the matrix) in the operand images of 2 * NB rows.
@@ -247,30 +248,43 @@ __device__ __forceinline__ void expand_segment(uint32_t item, uint32_t header, i
 // Shared memory: the two rings (a bare product reuses them for the CTA's sums when the loop is over), then the time loop's
 // sums and cell states, then barriers.
 struct UmmaSmem {
-    size_t x, w, part, cs, bars, total;
-    __host__ __device__ constexpr UmmaSmem(int mode, int NB, int MT)
-        : x(0), w((size_t)x_depth(mode) * kXStage), part(mode ? w + (size_t)kWDepth * kUmmaStage : 0),
-          cs(mode ? part + (size_t)NB * MT * 512 : 0), bars(mode ? cs + (size_t)NB * MT * 128 : w + (size_t)kWDepth * kUmmaStage), total(bars + 512 + 1024) {}
+    uint32_t w, part, cs, bars, total;         // (the inputs start at 0)
+    __host__ __device__ UmmaSmem(int mode, int NB, int MT, int x_depth, int w_bytes) {
+        const uint32_t sums = (uint32_t)(NB * MT * 512);
+        w = (uint32_t)(x_depth * x_windows(NB, MT) * NB * 256);
+        const uint32_t end = w + (uint32_t)w_bytes;
+        part = mode ? end : 0u;
+        cs = part + sums;
+        bars = mode ? cs + sums / 4u : end > sums ? end : sums;
+        total = bars + 512u + 1024u;
+    }
 };
-static_assert(UmmaSmem(0, 64, 2).w + (size_t)kWDepth * kUmmaStage >= 64 * 2 * 512, "the rings hold the sums");
 
 template <int NB, int MT, int MODE>
 __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_constant__ UmmaArgs a) {
     constexpr int N = 2 * NB;                             // hi and lo rows of the operand
     constexpr int kWin = N * 128;                         // bytes of a window's image
-    constexpr int XW = kXStage / kWin;                    // windows per stage of inputs
-    constexpr int DB = kDCols / N;                        // buffers of sums in TMEM (even)
+    constexpr int XW = x_windows(NB, MT), kXStage = XW * kWin;
+    // lo rows with an instruction and sums of their own, which stay in TMEM until the end; else the two kinds side by side.  Twice the
+    // instructions for half the loads from TMEM (some 57 bytes a cycle): 8192 x 8192 at 4x, batch 64, 44.4 -> 29.6 us,
+    // two 2048-unit LSTM layers with 32 sequences 23.8 -> 20.9 us a step; batch 8 19.1 -> 19.8.
+    constexpr bool kSplit = NB >= 32;
+    constexpr int DW = kSplit ? NB : N;                   // columns of a unit's sums
+    constexpr int kLoCol = 128;                           // where the lo rows' own begin
+    constexpr int DB = (kSplit ? kLoCol : kDCols) / DW;   // buffers of sums, one per unit (a power of two)
     constexpr int CN = NB * MT / 4;                       // batch columns whose sums a warp keeps
-    constexpr int XD = x_depth(MODE), kRows = 128 * MT;
-    static_assert(kDCols + kASlots * 32 <= 512 && DB % 2 == 0, "TMEM");
-    constexpr UmmaSmem L(MODE, NB, MT);
+    constexpr int kRows = 128 * MT;
+    static_assert((!kSplit || kLoCol + MT * NB <= kDCols) && kDCols + kASlots * 32 <= 512 && DB >= 2, "TMEM");
+    const int XD = a.x_depth;
+    const UmmaSmem L(MODE, NB, MT, XD, a.w_bytes);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
-    uint64_t *xfull = bars, *xempty = xfull + XD, *wfull = xempty + XD, *wempty = wfull + kWDepth;
-    uint64_t *afull = wempty + kWDepth, *aempty = afull + kASlots, *dfull = aempty + kASlots, *dempty = dfull + DB, *pfull = dempty + DB;
-    volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(pfull + 1);
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(pfull + 1) + 1;
+    uint64_t *xfull = bars, *xempty = xfull + kMaxXDepth, *wfull = xempty + kMaxXDepth, *wempty = wfull + kWRounds;
+    uint64_t *afull = wempty + kWRounds, *aempty = afull + 2, *dfull = aempty + 2, *dempty = dfull + DB, *pfull = dempty + DB, *xdone = pfull + 1;
+    volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(xdone + 1);
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(xdone + 1) + 1;
+    volatile uint32_t* w_at = reinterpret_cast<volatile uint32_t*>(xdone + 2);       // where a round of values lies in its ring
     float* part = reinterpret_cast<float*>(smem + L.part);        // the CTA's sums: [batch column][row of the group]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -280,15 +294,14 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     const UmmaPart& pt = a.part[p_idx];
     const UmmaCta* me = pt.ctas + ((int)blockIdx.x - cta0);
     const int nw = me->nw, w0 = me->w0, F = a.flush, T_ = MODE ? a.T : 1;
-    const int ntw = nw * MT, ntw4 = MODE ? (ntw + 3) & ~3 : ntw;      // (a step's tile-windows are filled up: a warp's slots stay its own)
-    const int groups = (nw + F - 1) / F, units = groups * MT;
-    const int xstages = (nw + XW - 1) / XW, wstages = (int)((me->bytes + kUmmaStage - 1) / kUmmaStage);
+    const int ntw = nw * MT, rounds = (ntw + 3) / 4;
     if (threadIdx.x == 0) {
         for (int i = 0; i < XD; ++i) { mbar_init(xfull + i, 1); mbar_init(xempty + i, 1); }
-        for (int i = 0; i < kWDepth; ++i) { mbar_init(wfull + i, 1); mbar_init(wempty + i, kUmmaExpandWarps); }
-        for (int i = 0; i < kASlots; ++i) { mbar_init(afull + i, 4); mbar_init(aempty + i, 1); }
+        for (int i = 0; i < kWRounds; ++i) { mbar_init(wfull + i, 1); mbar_init(wempty + i, kUmmaExpandWarps); }
+        for (int i = 0; i < 2; ++i) { mbar_init(afull + i, kUmmaExpandWarps); mbar_init(aempty + i, 1); }
         for (int i = 0; i < DB; ++i) { mbar_init(dfull + i, 1); mbar_init(dempty + i, kUmmaExpandWarps / MT); }
         mbar_init(pfull, (uint32_t)a.S);
+        mbar_init(xdone, 1);
         *s_dead = 0u;
         mbar_fence_init();
     }
@@ -319,10 +332,20 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         while (!mbar_try_wait_parked(bar, parity, 4000u)) if (gave_up(spins, t0, limit, kDevCopyTimeout)) return false;
         return true;
     };
+    // Time loop: every CTA with a step in an earlier tick than this layer's step t has finished it.
+    auto wait_tick = [&](int t) -> bool {
+        uint32_t need = a.never;
+        for (int l = 0; l < a.n_parts; ++l)
+            need += (uint32_t)(a.part[l].cta_end - (l ? a.part[l - 1].cta_end : 0)) * (uint32_t)min(max(t + p_idx - l, 0), T_);
+        unsigned long long t0 = 0;
+        unsigned int spins = 0;
+        while ((int32_t)(ld_acquire_gpu(a.count) - need) < 0) if (gave_up(spins, t0, a.limit_ns, kDevBarrierTimeout)) return false;
+        return true;
+    };
     float2 acc[CN / 2];
 #pragma unroll
     for (int i = 0; i < CN / 2; ++i) acc[i] = make_float2(0.f, 0.f);
-    const int quad = warp & 3, slot = warp >> 2;          // expanding warps: lanes of the tile, tile-windows slot, slot + 4, ..
+    const int quad = warp & 3, slot = warp >> 2;          // expanding warps: lanes of the tile, which tile-window of a round
     const int my_mt = MT == 2 ? slot >> 1 : 0, my_b0 = MT == 2 ? (slot & 1) * CN : slot * CN;      // and whose sums the warp keeps
     const UmmaQuad* quads = pt.quads + (size_t)me->group * MT * 4;
 
@@ -344,93 +367,76 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 const UmmaQuad q = quads[ut * 4];
                 cs[j * 32 + lane] = lane < q.nrows ? __ldg(a.state0 + ((size_t)p_idx * a.nb + b) * a.H + q.row0 + lane) : 0.f;
             }
-        int stage = -1;                                   // of the values: running number, its slot, its parity
-        uint32_t w_slot = kWDepth - 1, w_par = 1u, taken = 0; // taken: items expanded so far
         bool ok = true;
-        const int unit_shift = (F == 2) + (MT == 2);      // log2 of a full flush group's tile-windows
-        // Tile-windows come unit by unit; a unit is one tile over the windows of a flush group.
-        auto first_of = [&](int u) -> int {
-            const int g = u / MT;
-            return u >= units ? 0x40000000 : g * F * MT + (u % MT) * min(F, nw - g * F);
-        };
-        // Sums of a unit (by the running number) out of TMEM, hi and lo parts added.
-        auto drain = [&](int run) {
-            const int buf = run % DB;
-            tc_fence_after();
-            const uint32_t d = tmem + ((uint32_t)quad << 21) + (uint32_t)(buf * N + my_b0);
-            uint32_t hi[CN], lo[CN];
-            tc_ld<CN>(d, hi);
-            tc_ld<CN>(d + NB, lo);
-            tc_wait_ld();
+        // The warp's share of sums in TMEM from this column on, added to its own; both: hi rows' and, NB columns on, lo rows'.
+        auto take = [&](uint32_t column, bool both) {
+            constexpr int CP = CN < 16 ? CN : 16;         // columns at a time: what the registers hold beside the sums
+            const uint32_t d = tmem + ((uint32_t)quad << 21) + column + (uint32_t)my_b0;
 #pragma unroll
-            for (int i = 0; i < CN / 2; ++i) add_pair(acc[i], hi[2 * i], hi[2 * i + 1], lo[2 * i], lo[2 * i + 1]);
+            for (int c = 0; c < CN; c += CP) {
+                uint32_t v[CP], lo[CP];
+                tc_ld<CP>(d + c, v);
+                if (both) tc_ld<CP>(d + NB + c, lo);
+                tc_wait_ld();
+#pragma unroll
+                for (int i = 0; i < CP / 2; ++i) {
+                    if (both) {
+                        float2 h = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                        add_pair(h, lo[2 * i], lo[2 * i + 1]);
+                        add_pair(acc[c / 2 + i], __float_as_uint(h.x), __float_as_uint(h.y));
+                    } else add_pair(acc[c / 2 + i], v[2 * i], v[2 * i + 1]);
+                }
+            }
+        };
+        // Sums of a unit (by the running number).
+        auto drain = [&](uint32_t run) {
+            const uint32_t buf = run % DB;
+            ok = __all_sync(0xffffffffu, wait(dfull + buf, (run / DB) & 1u));
+            if (!ok) return;
+            tc_fence_after();
+            take(buf * DW, !kSplit);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(dempty + buf);
         };
-        auto pass_stages = [&](int want) {                // in order, whether this warp has an item in them or not
-            while (stage < want && ok) {
-                if (stage >= 0) { __syncwarp(); if (lane == 0) mbar_arrive(wempty + w_slot); }
-                ++stage;
-                if (++w_slot == kWDepth) { w_slot = 0; w_par ^= 1u; }
-                ok = __all_sync(0xffffffffu, wait(wfull + w_slot, w_par));
-            }
-        };
-        int unit0 = 0, stage0 = 0;                        // running numbers of the step's first unit and stage of values
+        uint32_t ws = 0, w_par = 0, half = 0, a_par = 1, run = 0;     // slot and parity of the values and of the operand; running number of units
         for (int t = 0; t < T_ && ok; ++t) {
-            uint32_t off = me->first[warp];
-            int unit = my_mt;                             // the next one whose sums this warp takes
-            for (int i = slot; i < ntw4 && ok; i += 4) {
-                // Sums are taken as soon as they are there, and waited for when the operand slots behind them are full
-                // of units that need their buffer.
-                while (unit < units) {
-                    const int run = unit0 + unit;
-                    uint64_t* bar = dfull + run % DB;
-                    const uint32_t par = (uint32_t)(run / DB) & 1u;
-                    if (!__all_sync(0xffffffffu, mbar_test(bar, par))) {
-                        if (i < first_of(unit + DB) + kASlots) break;
-                        ok = __all_sync(0xffffffffu, wait(bar, par));
-                        if (!ok) break;
-                    }
-                    drain(run);
-                    unit += MT;
-                }
+            int before = 0;                               // units of the round in front, whose sums are still in TMEM
+            for (int rd = 0; rd < rounds && ok; ++rd) {
+                const int nj = min(4, ntw - 4 * rd), len = umma_unit_len(MT, F, nj);
+                ok = __all_sync(0xffffffffu, wait(wfull + ws, w_par));
                 if (!ok) break;
                 uint32_t r[32];
-                if (i < ntw) {
-                    pass_stages(stage0 + (int)(off / (kUmmaStage / 16)));
-                    if (!ok) break;
-                    const uint32_t item = smem_u32(smem + L.w) + w_slot * kUmmaStage + (off % (kUmmaStage / 16)) * 16u;
-                    const int g = i >> unit_shift, mt = MT == 1 ? 0 : i - (g << unit_shift) >= min(F, nw - g * F);
-                    const uint32_t header = item + (mt ? seg_off[MT - 1] : seg_off[0]);
-                    off = lds32(item + 12);
+                if (slot < nj) {
+                    const uint32_t blob = smem_u32(smem) + L.w + w_at[ws], item = blob + lds32(blob + 4u * warp);
+                    const uint32_t header = item + (umma_place(MT, len, slot).mt ? seg_off[MT - 1] : seg_off[0]);
                     if (seg_words == 32) expand_segment<32>(item, header, lane, r);
                     else if (seg_words == 16) { expand_segment<16>(item, header, lane, r); expand_segment<16>(item, header + 16, lane, r + 16); }
                     else
 #pragma unroll
                         for (int s = 0; s < 4; ++s) expand_segment<8>(item, header + 16 * s, lane, r + 8 * s);
                 }
-                // (a warp's items go to two of the eight operand slots in turn; a fresh slot's wait ends at once)
-                static_assert(kASlots == 8, "four slots of tile-windows, two of them a warp");
-                const uint32_t as = (uint32_t)slot + ((taken & 1u) << 2);
-                ok = __all_sync(0xffffffffu, wait(aempty + as, ((taken >> 1) & 1u) ^ 1u));
+                ok = __all_sync(0xffffffffu, wait(aempty + half, a_par));      // (fresh: ends at once)
                 if (!ok) break;
-                ++taken;
                 tc_fence_after();
-                if (i < ntw) tc_st32(a_base + ((uint32_t)quad << 21) + as * 32u, r);
+                if (slot < nj) tc_st32(a_base + ((uint32_t)quad << 21) + (half * 4u + (uint32_t)slot) * 32u, r);
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(afull + as);
+                if (lane == 0) { mbar_arrive(afull + half); mbar_arrive(wempty + ws); }
+                if (++ws == kWRounds) { ws = 0; w_par ^= 1u; }
+                half ^= 1u;
+                a_par ^= half ^ 1u;
+                // The sums of the round in front, while this one's products run.  (Half of the warps before they expand and half
+                // after it: a quarter slower.)
+                for (int u = my_mt; u < before && ok; u += MT) drain(run + u);
+                run += (uint32_t)before;
+                before = MT == 2 ? nj / len : (nj + len - 1) / len;
             }
-            while (ok && unit < units) {
-                const int run = unit0 + unit;
-                ok = __all_sync(0xffffffffu, wait(dfull + run % DB, (uint32_t)(run / DB) & 1u));
-                if (ok) drain(run);
-                unit += MT;
-            }
-            if (!MODE) break;
+            for (int u = my_mt; u < before && ok; u += MT) drain(run + u);
+            run += (uint32_t)before;
+            if (kSplit && ok) { take(kLoCol + (uint32_t)(my_mt * NB), false); tc_fence_before(); }   // the lo rows' sums, complete with the tile's last unit
+            if constexpr (MODE != 0) {
             // ---- the step's sums are complete: cluster, gates, h_t
-            if (ok) pass_stages(stage0 + wstages - 1);    // the next step's values can come
 #pragma unroll
             for (int i = 0; i < CN / 2; ++i) {
                 float* at = part + (my_b0 + 2 * i) * kRows + my_mt * 128 + quad * 32 + lane;
@@ -442,147 +448,197 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
             if (a.S > 1 && (int)threadIdx.x < a.S) arrive_peer(pfull, threadIdx.x);
             const bool more = t + 1 < T_;
             const int next = (t + p_idx + 1) & 1;         // the buffer of images that the next tick reads
-            if (p_idx == 0 && more) {                     // x_{t+1}, shared between the CTAs of the first layer
-                const int I = a.in_size[0], chunks = (I + 7) / 8;
-                uint8_t* images = pt.xp + (size_t)next * pt.windows * kWin;
-                for (int i = (int)blockIdx.x * kExpandThreads + (int)threadIdx.x; i < chunks * a.nb; i += pt.cta_end * kExpandThreads) {
-                    const int b = i / chunks, c = (i - b * chunks) * 8;
-                    put_eight<NB>(images, b, c, I, a.x + ((size_t)(t + 1) * a.nb + b) * I + c, a.x_vec != 0);
-                }
-            }
             if (a.S > 1) {
                 unsigned long long t0 = 0;
                 unsigned int spins = 0;
                 while (!mbar_try_wait_cluster(pfull, (uint32_t)t & 1u)) if (gave_up(spins, t0, limit, kDevBarrierTimeout)) { ok = false; break; }
                 ok = __all_sync(0xffffffffu, ok);
             }
-            for (int j = warp; j < tasks && ok; j += kUmmaExpandWarps) {
-                const int k = (int)rank + a.S * j, ut = k / a.nb, b = k - ut * a.nb;
-                const UmmaQuad q = quads[ut * 4];
-                const int u = q.row0 + lane;
-                const bool live = lane < q.nrows;
-                const uint32_t at = smem_u32(part) + (uint32_t)(b * kRows + ut * 128 + lane) * 4u;
-                float z[4];
-#pragma unroll
-                for (int gt = 0; gt < 4; ++gt) {
-                    float v[kUmmaMaxS];
-#pragma unroll
-                    for (int s = 0; s < kUmmaMaxS; ++s) v[s] = s < a.S ? (a.S > 1 ? ld_peer(at + gt * 128u, (uint32_t)s) : __uint_as_float(lds32(at + gt * 128u))) : 0.f;
-                    z[gt] = v[0];
-#pragma unroll
-                    for (int s = 1; s < kUmmaMaxS; ++s) z[gt] += v[s];
-                }
-                if (!live) continue;
+            // two of the warp's tasks at a time, so that their loads are in flight together (one after the other 4 us a step)
+            for (int j0 = warp; j0 < tasks && ok; j0 += 2 * kUmmaExpandWarps) {
+                float z[2][4], zb[2][4];
+                uint32_t at[2];
+                int u[2], b[2];
+                bool live[2];
                 const float* bl = a.bias[p_idx];
-                if (bl) {
 #pragma unroll
-                    for (int gt = 0; gt < 4; ++gt) z[gt] += __ldg(bl + (size_t)gt * a.H + u);
+                for (int p = 0; p < 2; ++p) {
+                    const int j = min(j0 + p * kUmmaExpandWarps, tasks - 1), k = (int)rank + a.S * j, ut = k / a.nb;
+                    b[p] = k - ut * a.nb;
+                    const UmmaQuad q = quads[ut * 4];
+                    u[p] = q.row0 + lane;
+                    live[p] = lane < q.nrows && j0 + p * kUmmaExpandWarps < tasks;
+                    at[p] = smem_u32(part) + (uint32_t)(b[p] * kRows + ut * 128 + lane) * 4u;
+#pragma unroll
+                    for (int gt = 0; gt < 4; ++gt) zb[p][gt] = bl && live[p] ? __ldg(bl + (size_t)gt * a.H + u[p]) : 0.f;
                 }
-                float st = cs[j * 32 + lane], h;
-                if (MODE == 1) h = lstm_cell(z[0], z[1], z[2], z[3], st);
-                else st = h = gru_cell(z[0], z[1], z[2], z[3], st);
-                cs[j * 32 + lane] = st;
-                if (more) put_value<NB>(pt.xp + (size_t)next * pt.windows * kWin, b, a.in_size[p_idx] + u, h);
-                if (p_idx + 1 < a.n_parts) {
-                    const UmmaPart& above = a.part[p_idx + 1];
-                    put_value<NB>(above.xp + (size_t)next * above.windows * kWin, b, u, h);
-                } else if (a.y) a.y[((size_t)t * a.nb + b) * a.H + u] = h;
-                if (!more) {
-                    const size_t e = ((size_t)p_idx * a.nb + b) * a.H + u;
-                    if (a.hT) a.hT[e] = h;
-                    if (MODE == 1 && a.cT) a.cT[e] = st;
+                auto range = [&](int s, float (&v)[2][4]) {
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+#pragma unroll
+                        for (int gt = 0; gt < 4; ++gt) v[p][gt] = a.S > 1 ? ld_peer(at[p] + gt * 128u, (uint32_t)s) : __uint_as_float(lds32(at[p] + gt * 128u));
+                };
+                range(0, z);
+                for (int s = 1; s < a.S; ++s) {
+                    float v[2][4];
+                    range(s, v);
+#pragma unroll
+                    for (int p = 0; p < 2; ++p)
+#pragma unroll
+                        for (int gt = 0; gt < 4; ++gt) z[p][gt] += v[p][gt];
+                }
+#pragma unroll
+                for (int p = 0; p < 2; ++p) {
+                    if (!live[p]) continue;
+                    if (bl) {
+#pragma unroll
+                        for (int gt = 0; gt < 4; ++gt) z[p][gt] += zb[p][gt];
+                    }
+                    float* state = cs + (j0 + p * kUmmaExpandWarps) * 32 + lane;
+                    float st = *state, h;
+                    if (MODE == 1) h = lstm_cell(z[p][0], z[p][1], z[p][2], z[p][3], st);
+                    else st = h = gru_cell(z[p][0], z[p][1], z[p][2], z[p][3], st);
+                    *state = st;
+                    if (more) put_value<NB>(pt.xp + (size_t)next * pt.windows * kWin, b[p], a.in_size[p_idx] + u[p], h);
+                    if (p_idx + 1 < a.n_parts) {
+                        const UmmaPart& above = a.part[p_idx + 1];
+                        put_value<NB>(above.xp + (size_t)next * above.windows * kWin, b[p], u[p], h);
+                    } else if (a.y) a.y[((size_t)t * a.nb + b[p]) * a.H + u[p]] = h;
+                    if (!more) {
+                        const size_t e = ((size_t)p_idx * a.nb + b[p]) * a.H + u[p];
+                        if (a.hT) a.hT[e] = h;
+                        if (MODE == 1 && a.cT) a.cT[e] = st;
+                    }
                 }
             }
             ok = expand_barrier(ok);
             if (!ok) break;
-            if (threadIdx.x == 0) { __threadfence(); add_release_gpu(a.count, 1u); }
-            unit0 += units; stage0 += wstages;
+            if (warp == 0) {
+                if (p_idx == 0 && more) ok = __all_sync(0xffffffffu, wait(xdone, (uint32_t)t & 1u));
+                if (ok && lane == 0) { __threadfence(); add_release_gpu(a.count, 1u); }
+            }
+            }
         }
     } else if (warp == kUmmaExpandWarps) {
         // The whole warp runs along, so that addresses and descriptors live in uniform registers, and one lane issues (with a
         // single lane running, a tile-window took this warp 1100 cycles: it was what the others waited for).
         const bool leader = elect_lane();
         bool ok = true;
-        uint32_t as = 0, a_par = 0, xs = 0, x_par = 0, xin = 0, buf = 0, d_par = 1;
-        const uint64_t x_desc = b_descriptor(smem_u32(smem + L.x));
-        for (int t = 0; t < T_ && ok; ++t) {
-            for (int w_lo = 0; w_lo < nw && ok; w_lo += F) {
-                const int len = min(F, nw - w_lo);
-                const uint32_t xs_lo = xs, x_par_lo = x_par, xin_lo = xin;
-#pragma unroll
-                for (int mt = 0; mt < MT; ++mt) {
-                    xs = xs_lo; x_par = x_par_lo; xin = xin_lo;
-                    ok = ok && __all_sync(0xffffffffu, wait(dempty + buf, d_par));
-                    for (int w = 0; w < len && ok; ++w) {
-                        if (mt == 0 && xin == 0) ok = wait(xfull + xs, x_par);
-                        ok = __all_sync(0xffffffffu, ok && wait(afull + as, a_par));
-                        if (!ok) break;
-                        tc_fence_after();
-                        const uint64_t b = x_desc + (uint64_t)((xs * kXStage + xin * kWin) >> 4);
-                        const bool last = mt == MT - 1 && (xin == XW - 1 || w_lo + w == nw - 1);
-                        if (leader) {
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                tc_mma_f16(tmem + buf * N, a_base + as * 32u + k * 8, b + (uint64_t)(2 * k), mma_idesc(N), w != 0 || k != 0);
-                            tc_commit(aempty + as);
-                            if (last) tc_commit(xempty + xs);
-                            if (w == len - 1) tc_commit(dfull + buf);
-                        }
-                        __syncwarp();
-                        if (++as == kASlots) { as = 0; a_par ^= 1u; }
-                        if (++xin == XW) { xin = 0; if (++xs == XD) { xs = 0; x_par ^= 1u; } }
+        uint32_t half = 0, a_par = 0, xs = 0, x_par = 0, buf = 0, d_par = 1;
+        const uint64_t x_desc = b_descriptor(smem_u32(smem));
+        for (int t = 0; t < T_ && ok; ++t)
+            for (int rd = 0; rd < rounds && ok; ++rd) {
+                const int nj = min(4, ntw - 4 * rd), len = umma_unit_len(MT, F, nj);
+                ok = wait(xfull + xs, x_par) && wait(afull + half, a_par);
+                uint64_t x = x_desc + (uint64_t)((xs * kXStage) >> 4);
+                for (int j0 = 0; j0 < nj && ok; j0 += len) {
+                    if (XW < 4 / MT && j0 == XW) {        // the second stage of the round
+                        if (leader) tc_commit(xempty + xs);
+                        if (++xs == (uint32_t)XD) { xs = 0; x_par ^= 1u; }
+                        ok = wait(xfull + xs, x_par);
+                        x = x_desc + (uint64_t)((xs * kXStage) >> 4);
                     }
+                    ok = __all_sync(0xffffffffu, ok && wait(dempty + buf, d_par));
+                    if (!ok) break;
+                    tc_fence_after();
+                    if (leader) {
+#pragma unroll 2
+                        for (int j = j0; j < min(j0 + len, nj); ++j) {
+                            const UmmaPlace at = umma_place(MT, len, j);
+                            const uint64_t b = x + (uint64_t)((at.window % XW * kWin) >> 4);
+                            const uint32_t lo = tmem + kLoCol + at.mt * NB;
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const uint32_t op = a_base + (half * 4u + (uint32_t)j) * 32u + k * 8;
+                                tc_mma_f16(tmem + buf * DW, op, b + (uint64_t)(2 * k), mma_idesc(DW), j != j0 || k != 0);
+                                if (kSplit) tc_mma_f16(lo, op, b + (uint64_t)(NB * 8 + 2 * k), mma_idesc(NB), rd != 0 || at.window != 0 || k != 0);
+                            }
+                        }
+                        tc_commit(dfull + buf);
+                    }
+                    __syncwarp();
                     if (++buf == DB) { buf = 0; d_par ^= 1u; }
                 }
+                if (!ok) break;
+                if (leader) { tc_commit(aempty + half); tc_commit(xempty + xs); }
+                __syncwarp();
+                if (++xs == (uint32_t)XD) { xs = 0; x_par ^= 1u; }
+                half ^= 1u;
+                a_par ^= half ^ 1u;
             }
-            if (xin != 0) { xin = 0; if (++xs == XD) { xs = 0; x_par ^= 1u; } }
-            for (int i = ntw; i < ntw4 && ok; ++i) {
-                ok = __all_sync(0xffffffffu, wait(afull + as, a_par));
-                if (ok && leader) tc_commit(aempty + as);
-                if (++as == kASlots) { as = 0; a_par ^= 1u; }
-            }
-        }
     } else if (warp == kUmmaExpandWarps + 1) {
         if (lane == 0) {
             if (!MODE) pdl_wait();                        // the packed inputs belong to the work in front on the stream
             bool ok = true;
-            for (int t = 0, run = 0; t < T_ && ok; ++t) {
+            uint32_t at = 0, par = 1;
+            for (int t = 0; t < T_ && ok; ++t) {
                 const uint8_t* src = pt.xp + (size_t)w0 * kWin;
                 if (MODE) {
-                    const int tick = t + p_idx;
-                    src += (size_t)(tick & 1) * pt.windows * kWin;
-                    // every CTA with a step in an earlier tick has finished it
-                    uint32_t need = a.never;
-                    for (int l = 0; l < a.n_parts; ++l)
-                        need += (uint32_t)(a.part[l].cta_end - (l ? a.part[l - 1].cta_end : 0)) * (uint32_t)min(max(tick - l, 0), T_);
-                    unsigned long long t0 = 0;
-                    unsigned int spins = 0;
-                    while ((int32_t)(ld_acquire_gpu(a.count) - need) < 0) if (gave_up(spins, t0, a.limit_ns, kDevBarrierTimeout)) { ok = false; break; }
+                    src += (size_t)((t + p_idx) & 1) * pt.windows * kWin;
+                    ok = wait_tick(t);
                     fence_proxy_async_all();              // what others have stored is read by copies
                 }
-                for (int i = 0; i < xstages && ok; ++i, ++run) {
-                    const int at = run % XD;
-                    if (run >= XD) ok = wait(xempty + at, (uint32_t)(run / XD - 1) & 1u);
+                for (int w = 0; w < nw && ok; w += XW) {
+                    ok = wait(xempty + at, par);
                     if (!ok) break;
-                    const uint32_t bytes = (uint32_t)min(XW, nw - i * XW) * kWin;
+                    const uint32_t bytes = (uint32_t)min(XW, nw - w) * kWin;
                     mbar_expect_tx(xfull + at, bytes);
-                    bulk_g2s(smem + L.x + (size_t)at * kXStage, src + (size_t)i * kXStage, bytes, xfull + at);
+                    bulk_g2s(smem + at * kXStage, src + (size_t)w * kWin, bytes, xfull + at);
+                    if (++at == (uint32_t)XD) { at = 0; par ^= 1u; }
                 }
             }
         }
-    } else {
+    } else if (warp == kUmmaExpandWarps + 2) {
         if (lane == 0) {                                  // (written at plan time: the copies need not wait for the work in front)
             const uint8_t* src = pt.stream + (size_t)me->off128 * 128;
-            const uint32_t total = me->bytes;
+            const uint2* table = reinterpret_cast<const uint2*>(pt.rounds) + me->table;
+            // Rounds lie one behind the other in the ring, each in one piece; the next one goes where the oldest have left room.
+            const uint32_t cap = (uint32_t)a.w_bytes;
             bool ok = true;
-            for (int t = 0, run = 0; t < T_ && ok; ++t)
-                for (int i = 0; i < wstages; ++i, ++run) {
-                    const int at = run % kWDepth;
-                    if (run >= kWDepth && !wait(wempty + at, (uint32_t)(run / kWDepth - 1) & 1u)) { ok = false; break; }
-                    const uint32_t bytes = min((uint32_t)kUmmaStage, total - (uint32_t)i * kUmmaStage);
-                    mbar_expect_tx(wfull + at, bytes);
-                    bulk_g2s(smem + L.w + (size_t)at * kUmmaStage, src + (size_t)i * kUmmaStage, bytes, wfull + at);
+            uint32_t head = 0, tail = 0, there = 0, at = 0, old = 0, old_par = 0;      // there: rounds in the ring, from slot `old` on
+            uint2 next = __ldg(table);
+            for (int t = 0; t < T_ && ok; ++t)
+                for (int rd = 0; rd < rounds && ok; ++rd) {
+                    const uint2 now = next;
+                    next = __ldg(table + (rd + 1 < rounds ? rd + 1 : 0));
+                    for (;;) {
+                        if (there == 0) { head = tail = 0; break; }
+                        if (there < kWRounds) {
+                            if (head > tail) {
+                                if (cap - head >= now.y) break;
+                                if (tail > now.y) { head = 0; break; }
+                            } else if (tail > head && tail - head > now.y) break;
+                        }
+                        ok = wait(wempty + old, old_par);
+                        if (!ok) break;
+                        if (++old == kWRounds) { old = 0; old_par ^= 1u; }
+                        --there;
+                        tail = w_at[old];
+                    }
+                    if (!ok) break;
+                    w_at[at] = head;
+                    mbar_expect_tx(wfull + at, now.y);
+                    bulk_g2s(smem + L.w + head, src + (size_t)now.x * 16, now.y, wfull + at);
+                    head += now.y;
+                    ++there;
+                    if (++at == kWRounds) at = 0;
                 }
+        }
+    }
+    if (MODE != 0 && warp == kUmmaExpandWarps + 3 && p_idx == 0) {
+        // x_{t+1}, shared between the CTAs of the first layer, while step t runs
+        const int I = a.in_size[0], chunks = (I + 7) / 8;
+        bool ok = true;
+        for (int t = 0; t + 1 < T_ && ok; ++t) {
+            ok = __all_sync(0xffffffffu, lane != 0 || wait_tick(t));
+            if (!ok) break;
+            uint8_t* images = pt.xp + (size_t)((t + 1) & 1) * pt.windows * kWin;
+            for (int i = (int)blockIdx.x * 32 + lane; i < chunks * a.nb; i += pt.cta_end * 32) {
+                const int b = i / chunks, c = (i - b * chunks) * 8;
+                put_eight<NB>(images, b, c, I, a.x + ((size_t)(t + 1) * a.nb + b) * I + c, a.x_vec != 0);
+            }
+            __syncwarp();
+            if (lane == 0) { __threadfence(); mbar_arrive(xdone); }
         }
     }
     __syncwarp();

@@ -93,61 +93,55 @@ struct ItemWriter {
         out.resize(start + (size_t)ng * ns * 16, 0);
         for (int g = 0; g < ng; ++g)
             for (int s = 0; s < ns; ++s) {
-                uint32_t h[4] = {0u, (uint32_t)(out.size() - start), 0u, 0xffffffffu};
+                uint32_t h[4] = {0u, (uint32_t)(out.size() - start), 0u, 0u};
                 h[0] = segment(q, g, w0 + (int64_t)s * 2 * seg_words, out);
                 std::memcpy(out.data() + start + (size_t)(g * ns + s) * 16, h, 16);
             }
     }
 };
 
-bool plan_cta(const csb_matrix* A, const UmmaHostPlan& P, UmmaCta* cta, std::vector<uint8_t>* out) {
+void plan_cta(const csb_matrix* A, const UmmaHostPlan& P, const UmmaCta& cta, UmmaRound* rounds, std::vector<uint8_t>* out) {
     const ItemWriter w{A, P.seg_words};
-    std::fill(cta->first, cta->first + kUmmaExpandWarps, 0xffffffffu);
-    size_t last[kUmmaExpandWarps];
-    std::fill(last, last + kUmmaExpandWarps, SIZE_MAX);
-    std::vector<uint8_t> item;
-    int n = 0;                                             // tile-windows so far
-    for (int g = 0; g < cta->nw; g += P.flush)
-        for (int mt = 0; mt < P.MT; ++mt)
-            for (int wi = g; wi < std::min(cta->nw, g + P.flush); ++wi, ++n)
-                for (int q = 0; q < 4; ++q) {
-                    item.clear();
-                    w.write(P.quads[((size_t)cta->group * P.MT + mt) * 4 + q], (int64_t)(cta->w0 + wi) * kUmmaWindow, item);
-                    size_t at = out->size();
-                    if (at / kUmmaStage != (at + item.size() - 1) / kUmmaStage) at = (at / kUmmaStage + 1) * kUmmaStage;
-                    out->resize(at, 0);
-                    out->insert(out->end(), item.begin(), item.end());
-                    const int warp = (n & 3) * 4 + q;
-                    const uint32_t off16 = (uint32_t)(at / 16);
-                    if (last[warp] == SIZE_MAX) cta->first[warp] = off16;
-                    else std::memcpy(out->data() + last[warp] + 12, &off16, 4);
-                    last[warp] = at;
-                }
-    cta->bytes = (uint32_t)out->size();
-    const size_t stages = (out->size() + kUmmaStage - 1) / kUmmaStage;
-    for (size_t l : last) if ((l == SIZE_MAX ? 0 : l / kUmmaStage + 1) + kUmmaStages < stages + (l == SIZE_MAX ? 0 : 1)) return false;
-    return true;
+    const int ntw = cta.nw * P.MT, per = 4 / P.MT;         // windows of a round
+    for (int r = 0; 4 * r < ntw; ++r) {
+        const int nj = std::min(4, ntw - 4 * r), len = umma_unit_len(P.MT, P.flush, nj);
+        const size_t start = out->size();
+        uint32_t table[kUmmaExpandWarps] = {};
+        out->resize(start + sizeof table);
+        for (int j = 0; j < nj; ++j) {
+            const UmmaPlace at = umma_place(P.MT, len, j);
+            for (int q = 0; q < 4; ++q) {
+                table[j * 4 + q] = (uint32_t)(out->size() - start);
+                w.write(P.quads[((size_t)cta.group * P.MT + at.mt) * 4 + q], (int64_t)(cta.w0 + r * per + at.window) * kUmmaWindow, *out);
+            }
+        }
+        std::memcpy(out->data() + start, table, sizeof table);
+        rounds[r] = UmmaRound{(uint32_t)(start / 16), (uint32_t)(out->size() - start)};
+    }
 }
 
 }  // namespace
 
-bool plan_umma_host(const csb_matrix* A, UmmaHostPlan* P) {
+void plan_umma_host(const csb_matrix* A, UmmaHostPlan* P) {
     P->ctas.assign((size_t)P->n_groups * P->S, UmmaCta{});
     P->streams.assign(P->ctas.size(), {});
+    P->rounds.clear();
     for (int g = 0; g < P->n_groups; ++g)
         for (int s = 0; s < P->S; ++s) {
             UmmaCta& c = P->ctas[(size_t)g * P->S + s];
             c.group = g; c.split = s;
             c.w0 = (int)((int64_t)P->windows * s / P->S);
             c.nw = (int)((int64_t)P->windows * (s + 1) / P->S) - c.w0;
+            c.table = (int)P->rounds.size();
+            P->rounds.resize(P->rounds.size() + (size_t)(c.nw * P->MT + 3) / 4);
         }
     // the CTAs' streams are independent of one another
     std::atomic<size_t> next{0};
-    std::atomic<bool> failed{false}, taken{true};
+    std::atomic<bool> failed{false};
     run_on_threads(A->nnz < 100000 ? 1 : (int)std::min<size_t>(16, P->ctas.size()), [&]() {
         try {
             for (size_t i; (i = next.fetch_add(1)) < P->ctas.size() && !failed;)
-                if (!plan_cta(A, *P, &P->ctas[i], &P->streams[i])) taken = false;
+                plan_cta(A, *P, P->ctas[i], P->rounds.data() + P->ctas[i].table, &P->streams[i]);
         } catch (const std::bad_alloc&) { failed = true; }
     });
     if (failed) throw std::bad_alloc();
@@ -156,7 +150,8 @@ bool plan_umma_host(const csb_matrix* A, UmmaHostPlan* P) {
         P->ctas[i].off128 = (uint32_t)P->total128;
         P->total128 += (P->streams[i].size() + 127) / 128;
     }
-    return taken;
+    P->max_round = 0;
+    for (const UmmaRound& r : P->rounds) P->max_round = std::max(P->max_round, r.bytes);
 }
 
 }  // namespace csb

@@ -93,12 +93,15 @@ static int build_stack(const csb_matrix* const* W, UmmaStack* K) {
         else umma_shape(tiles, windows[l], clusters, &H.MT, &H.S);
         H.quads = umma_gate_quads(K->gates, K->in_size[l], K->H, H.MT);
         H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
-        if (!plan_umma_host(W[l], &H)) return 1;
+        plan_umma_host(W[l], &H);
         if ((rc = upload_umma(W[l], H, &K->plan[l])) != CSB_OK) return rc;
+        if (!K->plan[l].built) return 1;
+        K->max_round = std::max(K->max_round, K->plan[l].max_round);
     }
+    UmmaStages g;
     if (K->resident)
         for (int NB = 16; NB <= 32; NB *= 2) {
-            if (umma_smem(1, NB, MT) > W[0]->smem_optin) { K->resident = false; break; }
+            if (!umma_stages(1, NB, MT, K->max_round, W[0]->smem_optin, &g)) { K->resident = false; break; }
             CSB_CUDA(cudaFuncSetAttribute(pick_umma(K->gates == 4 ? 1 : 2, NB, MT), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W[0]->smem_optin));
         }
     return CSB_OK;
@@ -192,6 +195,8 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
             g_umma_plans.push_back(std::move(np));
         }
     }
+    UmmaStages g;
+    if (!umma_stages(1, P->NB, K->plan[0].MT, K->max_round, W[0]->smem_optin, &g)) return 1;
     // (as the step-by-step forms count: rows of their product, two per sequence for the GRU)
     note_recurrent_path((gates == 3 ? 2 : 1) * B <= 32 ? kPathStepsPacked : kPathSteps);
     cudaStream_t st = (cudaStream_t)stream;
@@ -225,11 +230,12 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
     ba.x_vec = (reinterpret_cast<uintptr_t>(dx) & 15) == 0 && in_size[0] % 4 == 0;
     UmmaArgs a{};
     a.n_parts = L; a.nb = B; a.status = P->d_status; a.S = K->plan[0].S; a.flush = K->plan[0].flush;
+    a.x_depth = g.x_depth; a.w_bytes = g.w_bytes;
     int ctas = 0;
     for (int l = 0; l < L; ++l) {
         const UmmaPlan& Q = K->plan[l];
         UmmaPart& p = a.part[l];
-        p.stream = Q.d_stream; p.ctas = Q.d_ctas; p.quads = Q.d_quads; p.xp = P->d_xp[l];
+        p.stream = Q.d_stream; p.ctas = Q.d_ctas; p.rounds = Q.d_rounds; p.quads = Q.d_quads; p.xp = P->d_xp[l];
         p.block_r = W[l]->block_r; p.seg_words = Q.seg_words; p.windows = Q.windows;
         ctas += Q.n_ctas;
         p.cta_end = ctas;
@@ -255,7 +261,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)a.S; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3(kUmmaThreads); cfg.dynamicSmemBytes = umma_smem(1, NB, K->plan[0].MT);
+    cfg.gridDim = dim3((unsigned)ctas); cfg.blockDim = dim3(kUmmaThreads); cfg.dynamicSmemBytes = g.smem;
     cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = a.S > 1 ? 2 : 1;
     void* params[] = {&a};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, pick_umma(lstm ? 1 : 2, NB, K->plan[0].MT), params);

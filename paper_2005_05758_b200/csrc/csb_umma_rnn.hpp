@@ -13,7 +13,8 @@ namespace csb {
 int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]);
 int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P);
 const void* pick_umma(int mode, int NB, int MT);
-size_t umma_smem(int mode, int NB, int MT);
+struct UmmaStages { int x_depth, w_bytes; size_t smem; };
+bool umma_stages(int mode, int NB, int MT, int max_round, size_t room, UmmaStages* out);
 int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st);
 
 // The layouts of a stack's layers, for every batch size.
@@ -23,6 +24,7 @@ struct UmmaStack {
     int in_size[kMaxLayers] = {};
     bool taken = false;                // false: a layer does not suit the layout
     bool resident = false;             // one grid holds all layers: the time loop serves it
+    int max_round = 0;
     UmmaPlan plan[kMaxLayers];
     ~UmmaStack();
 };

@@ -111,6 +111,7 @@ SPMM_PHASES = ["set-up, first copies, wait for the work in front", "waiting for 
 
 def spmm(cases):
     import workloads
+    os.environ["CSB_NO_UMMA"] = "1"                # (blocks of these sizes take the kernel without such counters)
     torch, binding = _load()
     for case in cases:
         rate, B = case.split(":")

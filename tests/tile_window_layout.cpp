@@ -1,6 +1,6 @@
-// The tile-window layout of the batched product, walked with the kernel's addressing rules: per expanding warp its chain
-// of items, per lane its segment headers and words.  Every stored value must come back at its place, no item may straddle
-// a stage, and a warp's chain must end within the ring's stages of the stream's end.  Prints the failures; exit code 1 on any.
+// The tile-window layout of the batched product, walked with the kernel's addressing rules: round by round, per expanding
+// warp its item, per lane its segment headers and words.  Every stored value must come back once, at its place.
+// Prints the failures; exit code 1 on any.
 #include <cstdarg>
 #include <cstdio>
 #include <random>
@@ -20,20 +20,20 @@ static int decode(const csb_matrix& A, const UmmaHostPlan& P, std::vector<uint16
     for (size_t c = 0; c < P.ctas.size(); ++c) {
         const UmmaCta& me = P.ctas[c];
         const std::vector<uint8_t>& S = P.streams[c];
-        const int stages = (int)((S.size() + kUmmaStage - 1) / kUmmaStage), segs = 32 / P.seg_words;
-        bad += S.size() != me.bytes;
-        for (int warp = 0; warp < kUmmaExpandWarps; ++warp) {
-            const int quad = warp & 3;
-            uint32_t off = me.first[warp];
-            int stage = -1;
-            for (int i = warp >> 2; i < me.nw * P.MT; i += 4) {
-                const int per = P.flush * P.MT, g = i / per, len = std::min(P.flush, me.nw - g * P.flush), mt = (i - g * per) / len;
-                const int window = me.w0 + g * P.flush + (i - g * per) % len;
-                const size_t item = (size_t)off * 16;
-                if (item + 16 > S.size() || (int)(item / kUmmaStage) < stage) return bad + 1;
-                stage = (int)(item / kUmmaStage);
-                const UmmaQuad q = P.quads[((size_t)me.group * P.MT + mt) * 4 + quad];
-                size_t end = item + 16;
+        const int segs = 32 / P.seg_words, ntw = me.nw * P.MT;
+        for (int r = 0; 4 * r < ntw; ++r) {
+            const UmmaRound round = P.rounds[(size_t)me.table + r];
+            const size_t start = (size_t)round.off16 * 16;
+            if (start + round.bytes > S.size() || round.bytes % 16 || round.bytes > P.max_round) return bad + 1;
+            const int nj = std::min(4, ntw - 4 * r), len = umma_unit_len(P.MT, P.flush, nj);
+            for (int warp = 0; warp < 4 * nj; ++warp) {
+                uint32_t at;
+                std::memcpy(&at, &S[start + 4 * (size_t)warp], 4);
+                const size_t item = start + at;
+                const UmmaPlace place = umma_place(P.MT, len, warp >> 2);
+                const int window = me.w0 + r * 4 / P.MT + place.window;
+                bad += item % 16 != 0 || window >= me.w0 + me.nw;
+                const UmmaQuad q = P.quads[((size_t)me.group * P.MT + place.mt) * 4 + (warp & 3)];
                 for (int lane = 0; lane < 32; ++lane) {
                     const int seg = lane < q.nrows ? (q.row0 + lane) / A.block_r - q.row0 / A.block_r : 0;
                     for (int s = 0; s < segs; ++s) {
@@ -42,22 +42,18 @@ static int decode(const csb_matrix& A, const UmmaHostPlan& P, std::vector<uint16
                         if (!((h[0] >> lane) & 1)) continue;
                         size_t p = item + h[1] + 16 * (size_t)__builtin_popcount(h[0] & ((1u << lane) - 1));
                         for (int j = 0; j < P.seg_words; j += 4, p += 16 * (size_t)__builtin_popcount(h[0])) {
-                            if (p + 16 > S.size()) return bad + 1;
+                            if (p + 16 > start + round.bytes) return bad + 1;
                             uint16_t w[8];
                             std::memcpy(w, &S[p], 16);
-                            end = std::max(end, p + 16);
                             for (int o = 0; o < 8; ++o) {
                                 const int64_t col = (int64_t)window * kUmmaWindow + s * 2 * P.seg_words + 2 * j + o;
                                 if (col >= A.cols || lane >= q.nrows) bad += w[o] != 0;
-                                else if (w[o]) got[(size_t)(q.out0 + lane) * A.cols + col] = w[o];
+                                else if (w[o]) { bad += got[(size_t)(q.out0 + lane) * A.cols + col] != 0; got[(size_t)(q.out0 + lane) * A.cols + col] = w[o]; }
                             }
                         }
                     }
                 }
-                bad += (end - 1) / kUmmaStage != item / kUmmaStage;
-                std::memcpy(&off, &S[item + 12], 4);
             }
-            bad += off != 0xffffffffu || stage + kUmmaStages < stages;
         }
     }
     return bad;
@@ -86,7 +82,7 @@ static int check(int R, int C, int br, int bc, double keep, int MT, int S, int g
     const int H = gates ? R / gates : 0, I = gates ? C - H : 0;
     P.quads = gates ? umma_gate_quads(gates, I, H, MT) : umma_row_quads(&A, MT);
     P.n_groups = (int)(P.quads.size() / (4 * MT));
-    const bool taken = plan_umma_host(&A, &P);
+    plan_umma_host(&A, &P);
     const int out_rows = gates ? 4 * H : R;
     std::vector<uint16_t> want((size_t)out_rows * C, 0), got((size_t)out_rows * C, 0);
     const uint16_t* v = reinterpret_cast<const uint16_t*>(A.val.data());
@@ -98,9 +94,9 @@ static int check(int R, int C, int br, int bc, double keep, int MT, int S, int g
                 if (gates == 3 && row >= 2 * H && col >= I) row += H;      // the candidate's recurrent part
                 want[(size_t)row * C + col] = v[A.val_off[b] + (size_t)i * A.n[b] + k] & 0x7fff ? v[A.val_off[b] + (size_t)i * A.n[b] + k] : 0;
             }
-    int bad = taken ? decode(A, P, got) : 1, diff = 0;
+    int bad = decode(A, P, got), diff = 0;
     for (size_t i = 0; i < want.size(); ++i) diff += want[i] != got[i];
-    if (bad || diff) printf("%dx%d blocks %dx%d keep %.2f MT %d S %d gates %d: taken %d, %d rules broken, %d values wrong\n", R, C, br, bc, keep, MT, S, gates, taken, bad, diff);
+    if (bad || diff) printf("%dx%d blocks %dx%d keep %.2f MT %d S %d gates %d: %d rules broken, %d values wrong\n", R, C, br, bc, keep, MT, S, gates, bad, diff);
     return bad || diff;
 }
 
