@@ -79,11 +79,10 @@ struct ItemWriter {
         out.resize(at + (size_t)kr * seg_words * 4, 0);
         uint16_t* v = reinterpret_cast<uint16_t*>(out.data() + at);
         const uint16_t* src = reinterpret_cast<const uint16_t*>(A->val.data()) + A->val_off[b] + (size_t)first * n;
-        for (int i = 0; i < kr; ++i, src += n)
-            for (int k = k0; k < k1; ++k) {
-                const int c = ci[k] - base;
-                v[((size_t)(c >> 3) * kr + i) * 8 + (c & 7)] = src[k];
-            }
+        uint16_t place[64];                                    // of the kept columns, in the first row
+        for (int k = k0; k < k1; ++k) { const int c = ci[k] - base; place[k - k0] = (uint16_t)((c >> 3) * kr * 8 + (c & 7)); }
+        for (int i = 0; i < kr; ++i, src += n, v += 8)
+            for (int k = k0; k < k1; ++k) v[place[k - k0]] = src[k];
         return rows;
     }
 
@@ -103,6 +102,7 @@ struct ItemWriter {
 void plan_cta(const csb_matrix* A, const UmmaHostPlan& P, const UmmaCta& cta, UmmaRound* rounds, std::vector<uint8_t>* out) {
     const ItemWriter w{A, P.seg_words};
     const int ntw = cta.nw * P.MT, per = 4 / P.MT;         // windows of a round
+    out->reserve((size_t)ntw * 128 * 128 + (size_t)ntw * 1024);     // every row kept: pages that are not written cost nothing
     for (int r = 0; 4 * r < ntw; ++r) {
         const int nj = std::min(4, ntw - 4 * r), len = umma_unit_len(P.MT, P.flush, nj);
         const size_t start = out->size();

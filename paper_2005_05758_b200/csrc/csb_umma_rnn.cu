@@ -1,11 +1,13 @@
 // LSTM and GRU stacks at larger batch as one launch per sequence on tcgen05 tensor cores: host side of the time loop of
 // csb_umma_kernel.cuh, and the layouts of the layers, which the step-by-step form (csb_rnn_step.cu) shares.
 #include <algorithm>
+#include <atomic>
 #include <cstdlib>
 #include <list>
 #include <memory>
 #include <mutex>
 
+#include "csb_host.hpp"
 #include "csb_rnn1.hpp"
 #include "csb_umma_rnn.hpp"
 #include "csb_umma_kernel.cuh"
@@ -84,17 +86,30 @@ static int build_stack(const csb_matrix* const* W, UmmaStack* K) {
             if (cost < best) { best = cost; MT = mt; S = s; }
         }
     K->resident = best < 1e300;
+    // the layers side by side: planning one and uploading it take about as long as each other
+    std::atomic<int> next{0};
+    int layer_rc[kMaxLayers] = {};
+    run_on_threads(K->L, [&]() {
+        for (int l; (l = next.fetch_add(1)) < K->L;) {
+            layer_rc[l] = guarded([&]() -> int {
+                CSB_CUDA(cudaSetDevice(K->device));
+                UmmaHostPlan H;
+                H.windows = windows[l];
+                H.seg_words = umma_seg_words(W[l]->block_c);
+                H.flush = umma_flush(most);
+                if (K->resident) { H.MT = MT; H.S = S; }
+                else umma_shape(tiles, windows[l], clusters, &H.MT, &H.S);
+                H.quads = umma_gate_quads(K->gates, K->in_size[l], K->H, H.MT);
+                H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
+                plan_umma_host(W[l], &H);
+                return upload_umma(W[l], H, &K->plan[l]);
+            });
+        }
+    });
     for (int l = 0; l < K->L; ++l) {
-        UmmaHostPlan H;
-        H.windows = windows[l];
-        H.seg_words = umma_seg_words(W[l]->block_c);
-        H.flush = umma_flush(most);
-        if (K->resident) { H.MT = MT; H.S = S; }
-        else umma_shape(tiles, windows[l], clusters, &H.MT, &H.S);
-        H.quads = umma_gate_quads(K->gates, K->in_size[l], K->H, H.MT);
-        H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
-        plan_umma_host(W[l], &H);
-        if ((rc = upload_umma(W[l], H, &K->plan[l])) != CSB_OK) return rc;
+        if (layer_rc[l] == CSB_ERR_ALLOC) set_error("out of memory");            // (another thread's error text is its own)
+        else if (layer_rc[l] != CSB_OK) set_error("uploading layer %d of the batched time loop failed", l);
+        if (layer_rc[l] != CSB_OK) { cudaGetLastError(); return layer_rc[l]; }
         if (!K->plan[l].built) return 1;
         K->max_round = std::max(K->max_round, K->plan[l].max_round);
     }
