@@ -71,7 +71,7 @@ struct UmmaPlace { int mt, window; };
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-inline int umma_unit_len(int MT, int flush, int nj) { return MT == 2 && 2 * flush > nj ? nj / 2 : flush; }
+inline int umma_unit_len(int MT, int flush, int nj) { return MT == 2 && 2 * flush > nj ? nj >> 1 : flush; }
 #ifdef __CUDACC__
 __host__ __device__
 #endif

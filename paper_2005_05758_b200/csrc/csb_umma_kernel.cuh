@@ -266,8 +266,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     constexpr int kWin = N * 128;                         // bytes of a window's image
     constexpr int XW = x_windows(NB, MT), kXStage = XW * kWin;
     // lo rows with an instruction and sums of their own, which stay in TMEM until the end; else the two kinds side by side.  Twice the
-    // instructions for half the loads from TMEM (some 57 bytes a cycle): 8192 x 8192 at 4x, batch 64, 44.4 -> 29.6 us,
-    // two 2048-unit LSTM layers with 32 sequences 23.8 -> 20.9 us a step; batch 8 19.1 -> 19.8.
+    // instructions for half the loads from TMEM (those of 64 columns took 17 of 44 us): 8192 x 8192 at 4x, batch 64, 44.4 ->
+    // 29.6 us, two 2048-unit LSTM layers with 32 sequences 23.8 -> 20.9 us a step; batch 8 19.1 -> 19.8.
     constexpr bool kSplit = NB >= 32;
     constexpr int DW = kSplit ? NB : N;                   // columns of a unit's sums
     constexpr int kLoCol = 128;                           // where the lo rows' own begin
@@ -430,7 +430,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 // after it: a quarter slower.)
                 for (int u = my_mt; u < before && ok; u += MT) drain(run + u);
                 run += (uint32_t)before;
-                before = MT == 2 ? nj / len : (nj + len - 1) / len;
+                before = (nj + (MT == 2 ? 0 : len - 1)) >> (len - 1);       // nj / len, rounded up for one tile; len is 1 or 2
             }
             for (int u = my_mt; u < before && ok; u += MT) drain(run + u);
             run += (uint32_t)before;
