@@ -15,7 +15,7 @@ namespace csb {
 __device__ __forceinline__ float gate_logistic(float a) { return 1.f / (1.f + expf(-a)); }
 
 // The same arithmetic with every rounding spelled out, for kernels that have to give the same bits.
-__device__ __forceinline__ float cell_logistic(float a) { return __fdiv_rn(1.f, __fadd_rn(1.f, expf(-a))); }
+__device__ __forceinline__ float cell_logistic(float a) { return __frcp_rn(__fadd_rn(1.f, expf(-a))); }
 __device__ __forceinline__ float lstm_cell(float zi, float zf, float zg, float zo, float& c) {
     c = __fmaf_rn(cell_logistic(zf), c, __fmul_rn(cell_logistic(zi), tanhf(zg)));
     return __fmul_rn(cell_logistic(zo), tanhf(c));
