@@ -11,7 +11,7 @@ import tempfile
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libcsb.so")
-SOURCES = ["csb_api.cpp", "csb_encode.cpp", "csb_plan.cpp", "csb_schedule.cpp", "csb_spmm_plan.cpp", "csb_panel_plan.cpp", "csb_product.cu", "csb_panel.cu", "csb_spmm_mma.cu", "csb_umma_plan.cpp", "csb_umma.cu", "csb_umma_rnn.cu", "csb_rnn.cu", "csb_rnn_step.cu", "csb_rnn1_plan.cpp", "csb_rnn1.cu", "csb_rnn1_b1.cu", "csb_rnn1_b4.cu", "csb_rnn1_b8.cu", "csb_rnn_unit_plan.cpp", "csb_rnn_unit_b1.cu", "csb_rnn_unit_b4.cu", "csb_rnn_unit_b8.cu", "csb_cells.cu", "csb_fixed.cu", "csb_project.cu"]
+SOURCES = ["csb_api.cpp", "csb_encode.cpp", "csb_plan.cpp", "csb_schedule.cpp", "csb_spmm_plan.cpp", "csb_panel_plan.cpp", "csb_product.cu", "csb_panel.cu", "csb_spmm_mma.cu", "csb_umma_plan.cpp", "csb_umma_upload.cpp", "csb_umma.cu", "csb_umma_rnn.cu", "csb_rnn.cu", "csb_rnn_step.cu", "csb_rnn1_plan.cpp", "csb_rnn1.cu", "csb_rnn1_b1.cu", "csb_rnn1_b4.cu", "csb_rnn1_b8.cu", "csb_rnn_unit_plan.cpp", "csb_rnn_unit_b1.cu", "csb_rnn_unit_b4.cu", "csb_rnn_unit_b8.cu", "csb_cells.cu", "csb_fixed.cu", "csb_project.cu"]
 HEADERS = ["csb_internal.hpp", "csb_umma.hpp", "csb_umma_kernel.cuh", "csb_umma_rnn.hpp", "csb_host.hpp", "csb_device.cuh", "csb_rnn1.hpp", "csb_rnn1_args.hpp", "csb_rnn1_kernel.cuh", "csb_rnn_unit.hpp", "csb_rnn_unit_kernel.cuh", "csb_rnn_exchange.cuh", "csb_gates.cuh", os.path.join("..", "..", "include", "csb.h")]
 
 

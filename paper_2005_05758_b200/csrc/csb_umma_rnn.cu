@@ -107,10 +107,10 @@ static int build_stack(const csb_matrix* const* W, UmmaStack* K) {
         }
     });
     for (int l = 0; l < K->L; ++l) {
+        if (layer_rc[l] == 1) return 1;
         if (layer_rc[l] == CSB_ERR_ALLOC) set_error("out of memory");            // (another thread's error text is its own)
         else if (layer_rc[l] != CSB_OK) set_error("uploading layer %d of the batched time loop failed", l);
         if (layer_rc[l] != CSB_OK) { cudaGetLastError(); return layer_rc[l]; }
-        if (!K->plan[l].built) return 1;
         K->max_round = std::max(K->max_round, K->plan[l].max_round);
     }
     UmmaStages g;

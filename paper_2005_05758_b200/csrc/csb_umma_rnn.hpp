@@ -1,4 +1,4 @@
-// The batched recurrent stacks on tcgen05: what csb_umma.cu, csb_umma_rnn.cu and csb_rnn_step.cu share.
+// The batched recurrent stacks on tcgen05: what csb_umma.cu, csb_umma_upload.cpp, csb_umma_rnn.cu and csb_rnn_step.cu share.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -11,11 +11,14 @@ namespace csb {
 
 // csb_umma.cu
 int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]);
-int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P);
 const void* pick_umma(int mode, int NB, int MT);
 struct UmmaStages { int x_depth, w_bytes; size_t smem; };
 bool umma_stages(int mode, int NB, int MT, int max_round, size_t room, UmmaStages* out);
 int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st);
+
+// csb_umma_upload.cpp
+int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P);
+int make_umma_plan(const csb_matrix* A, UmmaPlan* P);   // 1: the path does not take the matrix
 
 // The layouts of a stack's layers, for every batch size.
 struct UmmaStack {
