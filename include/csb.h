@@ -183,8 +183,8 @@ int csb_spmv(const csb_matrix_t* A, const float* x, float* y, void* stream);
  * staging buffer for the packed inputs (allocates and synchronises once; make it outside of any stream
  * capture, where the second form serves more than 16 vectors by the layout of either of the larger classes).
  * The two kernels of this path are launched
- * with programmatic stream serialization and wait, first thing, for the work in front of them on
- * `stream`.  Other cases use the CUDA-core kernel in batch tiles of 8 / 4 / 1.
+ * with programmatic stream serialization: they may start while the work in front of them on `stream` runs, and wait
+ * for it before they read X or write Y (the limit of a wait, a second, counts from there).  Other cases use the CUDA-core kernel in batch tiles of 8 / 4 / 1.
  */
 int csb_spmm(const csb_matrix_t* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
              void* stream);

@@ -288,7 +288,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     float* part = reinterpret_cast<float*>(smem + L.part);        // the CTA's sums: [batch column][row of the group]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    pdl_launch_dependents();
+    if (MODE == 0) pdl_launch_dependents();               // (a time loop may run for long: nothing need wait on its SMs so long)
     int p_idx = 0, cta0 = 0;                              // which product (layer) this CTA works for, and its first CTA
     while (p_idx + 1 < a.n_parts && (int)blockIdx.x >= a.part[p_idx].cta_end) { cta0 = a.part[p_idx].cta_end; ++p_idx; }
     const UmmaPart& pt = a.part[p_idx];
@@ -314,7 +314,9 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     constexpr uint32_t tmem = 0u, a_base = kDCols;
     if (threadIdx.x == 0 && *s_tmem != 0u) { *s_dead = 1u; *(volatile uint32_t*)a.status = (uint32_t)kDevCopyTimeout; }
 
-    // A wait gives up after a second, or as soon as another one of the CTA has given up.
+    // A wait gives up after a second, or as soon as another one of the CTA has given up.  What a product's wait stands behind
+    // must be this kernel's own work: each role passes pdl_wait before its first wait that needs the inputs, so that the
+    // time of the work in front does not count.
     auto gave_up = [&](unsigned int& spins, unsigned long long& t0, unsigned long long limit, uint32_t code) -> bool {
         if ((++spins & 255u) != 0) return false;
         if (*s_dead) return true;
@@ -426,12 +428,14 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 if (++ws == kWRounds) { ws = 0; w_par ^= 1u; }
                 half ^= 1u;
                 a_par ^= half ^ 1u;
+                if (MODE == 0 && rd == 1) pdl_wait();     // (two rounds of operands fit in TMEM without the inputs)
                 // The sums of the round in front, while this one's products run.  (Half of the warps before they expand and half
                 // after it: a quarter slower.)
                 for (int u = my_mt; u < before && ok; u += MT) drain(run + u);
                 run += (uint32_t)before;
                 before = (nj + (MT == 2 ? 0 : len - 1)) >> (len - 1);       // nj / len, rounded up for one tile; len is 1 or 2
             }
+            if (MODE == 0 && rounds == 1) pdl_wait();
             for (int u = my_mt; u < before && ok; u += MT) drain(run + u);
             run += (uint32_t)before;
             if (kSplit && ok) { take(kLoCol + (uint32_t)(my_mt * NB), false); tc_fence_before(); }   // the lo rows' sums, complete with the tile's last unit
@@ -523,6 +527,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         // The whole warp runs along, so that addresses and descriptors live in uniform registers, and one lane issues (with a
         // single lane running, a tile-window took this warp 1100 cycles: it was what the others waited for).
         const bool leader = elect_lane();
+        if (MODE == 0) pdl_wait();
         bool ok = true;
         uint32_t half = 0, a_par = 0, xs = 0, x_par = 0, buf = 0, d_par = 1;
         const uint64_t x_desc = b_descriptor(smem_u32(smem));
@@ -596,6 +601,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
             const uint32_t cap = (uint32_t)a.w_bytes;
             bool ok = true;
             uint32_t head = 0, tail = 0, there = 0, at = 0, old = 0, old_par = 0;      // there: rounds in the ring, from slot `old` on
+            int freed = 0;                                // (the expanding warps are done with two rounds before they need the inputs)
             uint2 next = __ldg(table);
             for (int t = 0; t < T_ && ok; ++t)
                 for (int rd = 0; rd < rounds && ok; ++rd) {
@@ -609,6 +615,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                                 if (tail > now.y) { head = 0; break; }
                             } else if (tail > head && tail - head > now.y) break;
                         }
+                        if (MODE == 0 && freed++ == 2) pdl_wait();
                         ok = wait(wempty + old, old_par);
                         if (!ok) break;
                         if (++old == kWRounds) { old = 0; old_par ^= 1u; }

@@ -1,4 +1,8 @@
 """The batched product and time loop on tcgen05 at the sizes where their tiles, windows and batch tiles end."""
+import ctypes
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -68,3 +72,26 @@ def test_time_loop_against_the_oracle(cell, B, I, H, L, T):
         assert np.max(np.abs(y.cpu().numpy() - np.asarray(want[0]))) < 15 * 2e-6
     for m in mats:
         m.free()
+
+
+@pytest.mark.parametrize("rows,cols,batch", [(200, 100, 9), (1024, 512, 16), (4096, 8192, 64)])
+def test_time_in_front_of_a_product_does_not_count(tmp_path, rows, cols, batch):
+    # the product's CTAs may start while the kernel in front runs (here past the limit of the product's own waits, a
+    # second): with one round a CTA, with two, and with more than its rings hold
+    here = os.path.dirname(os.path.abspath(__file__))
+    out = str(tmp_path / "slow_front.so")
+    subprocess.run([os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"), "-gencode", "arch=compute_100a,code=sm_100a", "-O2", "-shared", "-Xcompiler", "-fPIC", "-o", out,
+                    os.path.join(here, "slow_front.cu")], check=True)
+    w = workloads.make_spmv_workload(3, rows, cols, 32, 64, "uniform", lo=0.3, hi=0.9, batch=batch, w_std=0.05)
+    m = w.matrix
+    A = binding.csb_encode(m.dense, 32, 64, m.row_keep, m.col_keep, "f16", 0)
+    x = torch.from_numpy(w.X).cuda()
+    want, y = torch.empty((batch, rows), device="cuda"), torch.full((batch, rows), float("nan"), device="cuda")
+    binding.csb_spmm(A, x, want)
+    torch.cuda.synchronize()
+    assert ctypes.CDLL(out).slow_front(ctypes.c_ulonglong(1_300_000_000), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)) == 0
+    binding.csb_spmm(A, x, y)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    binding.csb_spmm(A, x, y)                            # (reports a wait that an earlier product gave up)
+    A.free()
