@@ -33,6 +33,7 @@ namespace csb {
 
 constexpr int kASlots = 8;                     // tile-windows of the A operand in TMEM, 32 columns each: two rounds
 constexpr int kDCols = 256;                    // columns of TMEM for sums
+constexpr uint32_t kNever = 0x40000000u;       // more arrivals than a sequence has
 constexpr int kMaxXDepth = 4, kWRounds = 6;    // stages of inputs, rounds of values in shared memory
 constexpr int kExpandThreads = kUmmaExpandWarps * 32, kUmmaThreads = kExpandThreads + 4 * 32;
 // Windows of a stage of inputs: a round's, or half of it for 64 batch columns on one tile (32 KB).
@@ -61,7 +62,8 @@ struct UmmaArgs {
     int in_size[kMaxLayers];
     uint32_t* count;                                       // CTAs that have finished a tick, summed over ticks
     unsigned long long limit_ns;
-    uint32_t never;                                        // test hook: arrivals that never come
+    uint32_t never;                                        // test hook: arrivals that never come,
+    int never_step;                                        // and the step at which they are missing for the warps that pack x alone
     int T, H, x_vec;                                       // x_vec: rows of x start at multiples of 16 bytes
 };
 
@@ -335,8 +337,8 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         return true;
     };
     // Time loop: every CTA with a step in an earlier tick than this layer's step t has finished it.
-    auto wait_tick = [&](int t) -> bool {
-        uint32_t need = a.never;
+    auto wait_tick = [&](int t, uint32_t never) -> bool {
+        uint32_t need = never;
         for (int l = 0; l < a.n_parts; ++l)
             need += (uint32_t)(a.part[l].cta_end - (l ? a.part[l - 1].cta_end : 0)) * (uint32_t)min(max(t + p_idx - l, 0), T_);
         unsigned long long t0 = 0;
@@ -515,12 +517,11 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                     }
                 }
             }
+            // (in front of the barrier: a warp that gives up takes the others along, which would wait for it at the next one)
+            if (warp == 0 && p_idx == 0 && more && ok) ok = __all_sync(0xffffffffu, wait(xdone, (uint32_t)t & 1u));
             ok = expand_barrier(ok);
             if (!ok) break;
-            if (warp == 0) {
-                if (p_idx == 0 && more) ok = __all_sync(0xffffffffu, wait(xdone, (uint32_t)t & 1u));
-                if (ok && lane == 0) { __threadfence(); add_release_gpu(a.count, 1u); }
-            }
+            if (threadIdx.x == 0) { __threadfence(); add_release_gpu(a.count, 1u); }
             }
         }
     } else if (warp == kUmmaExpandWarps) {
@@ -534,7 +535,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         for (int t = 0; t < T_ && ok; ++t)
             for (int rd = 0; rd < rounds && ok; ++rd) {
                 const int nj = min(4, ntw - 4 * rd), len = umma_unit_len(MT, F, nj);
-                ok = wait(xfull + xs, x_par) && wait(afull + half, a_par);
+                ok = __all_sync(0xffffffffu, wait(xfull + xs, x_par) && wait(afull + half, a_par));
                 uint64_t x = x_desc + (uint64_t)((xs * kXStage) >> 4);
                 for (int j0 = 0; j0 < nj && ok; j0 += len) {
                     if (XW < 4 / MT && j0 == XW) {        // the second stage of the round
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 const uint8_t* src = pt.xp + (size_t)w0 * kWin;
                 if (MODE) {
                     src += (size_t)((t + p_idx) & 1) * pt.windows * kWin;
-                    ok = wait_tick(t);
+                    ok = wait_tick(t, a.never);
                     fence_proxy_async_all();              // what others have stored is read by copies
                 }
                 for (int w = 0; w < nw && ok; w += XW) {
@@ -637,7 +638,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         const int I = a.in_size[0], chunks = (I + 7) / 8;
         bool ok = true;
         for (int t = 0; t + 1 < T_ && ok; ++t) {
-            ok = __all_sync(0xffffffffu, lane != 0 || wait_tick(t));
+            ok = __all_sync(0xffffffffu, lane != 0 || wait_tick(t, t == a.never_step ? kNever : a.never));
             if (!ok) break;
             uint8_t* images = pt.xp + (size_t)((t + 1) & 1) * pt.windows * kWin;
             for (int i = (int)blockIdx.x * 32 + lane; i < chunks * a.nb; i += pt.cta_end * 32) {

@@ -264,7 +264,8 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
     a.count = P->d_count; a.T = (int)T; a.H = H; a.x_vec = ba.x_vec;
     uint32_t extra = 0;
     barrier_test_hook(&extra, &a.limit_ns);
-    a.never = extra ? 0x40000000u : 0u;
+    a.never = extra == 1 ? kNever : 0u;
+    a.never_step = (int)extra - 2;
     *P->h_status = 0;
     const size_t all = ns + (size_t)B * ((in_size[0] + 7) / 8);
     const unsigned blocks = (unsigned)std::min<size_t>((all + 255) / 256, 4096);

@@ -95,3 +95,29 @@ def test_time_in_front_of_a_product_does_not_count(tmp_path, rows, cols, batch):
     assert torch.equal(y, want)
     binding.csb_spmm(A, x, y)                            # (reports a wait that an earlier product gave up)
     A.free()
+
+
+@pytest.mark.parametrize("I,H,L", [(153, 160, 1), (39, 100, 3), (512, 1024, 2)])
+@pytest.mark.parametrize("step", [0, 1, 3])
+def test_one_warp_that_gives_up_takes_the_sequence_along(I, H, L, step):
+    # the warps that pack x_{t+1} give up at one step, everybody else has what that step needs: the call ends with the status,
+    # and the next one is as good as the first
+    T, B = 6, 20
+    w = workloads.make_rnn_workload(7, "lstm", I, H, L, 32, 32, "uniform", lo=0.2, hi=0.5, T=T, B=B, w_std=0.1, bias_std=0.1, state_std=0.3)
+    mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in w.layers]
+    x, bias, y = torch.from_numpy(w.x).cuda(), [torch.from_numpy(b).cuda() for b in w.bias], torch.empty((T, B, H), device="cuda")
+
+    def run():
+        binding.csb_lstm_forward(mats, bias, x, None, None, y, None, None, 0)
+        return y.clone()
+    want = run()
+    binding.lib.csb_test_barrier_hook(2 + step, 200_000)
+    try:
+        with pytest.raises(binding.CsbError) as e:
+            run()
+        assert e.value.status == -7
+    finally:
+        binding.lib.csb_test_barrier_hook(0, 0)
+    assert torch.equal(run(), want)
+    for m in mats:
+        m.free()
