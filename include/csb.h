@@ -176,10 +176,10 @@ int csb_spmv(const csb_matrix_t* A, const float* x, float* y, void* stream);
  * With batch >= 8, fp16 values and block_r <= 64 the product runs on tensor cores (the kernel
  * matrix times the gathered inputs is then a dense contraction), up to 64 batch columns per pass: the
  * inputs are split into two binary16 halves (x = hi + lo, so no input precision is lost as long
- * as |x| < 65504; larger or non-finite inputs give inf / NaN in the outputs of their batch column), fp32
+ * as |x| < 65504; larger or non-finite inputs give NaN in the outputs that a block keeps them for), fp32
  * accumulation.  Blocks of 16, 32 or a multiple of 64 columns are expanded into dense tiles for tcgen05.mma,
- * with one device layout for all batch sizes; the others go through mma.sync.m16n8k16, with a layout per class
- * of batch sizes (<= 16, <= 32, more).  The first such call on a handle builds the layout and a
+ * with one device layout for all batch sizes; the others go through mma.sync.m16n8k16 (where such an input gives NaN
+ * in all rows of the block-rows that keep it), with a layout per class of batch sizes (<= 16, <= 32, more).  The first such call on a handle builds the layout and a
  * staging buffer for the packed inputs (allocates and synchronises once; make it outside of any stream
  * capture, where the second form serves more than 16 vectors by the layout of either of the larger classes).
  * The two kernels of this path are launched

@@ -273,7 +273,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
                 np->uids.push_back(W[l]->uid);
                 np->in_size[l] = in_size[l];
                 // (what is read of the packed inputs is written on the call's stream first, so they need no clearing here)
-                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], np->umma ? (size_t)np->umma->plan[l].windows * kUmmaImage : (size_t)(in_size[l] + H) * pitch));
+                CSB_CUDA(cudaMalloc((void**)&np->d_xp[l], np->umma ? umma_xp_bytes(np->umma->plan[l].windows) : (size_t)(in_size[l] + H) * pitch));
                 if (!packed_path) CSB_CUDA(cudaMalloc((void**)&np->d_v[l], (size_t)rows_v * (in_size[l] + H) * 4));
             }
             const int rc = np->umma ? (int)CSB_OK : prepare_spmm_stack(L, W, std::min(rows_v, 32), &np->stack);

@@ -11,20 +11,21 @@ namespace csb {
 
 // Packs fp32 inputs [nb][cols] into the operand images: one CTA per window, a thread per batch column and 8 matrix columns.
 template <int NB>
-__global__ void __launch_bounds__(NB * 8) csb_umma_pack_kernel(const float* __restrict__ X, long long ldx, int nb, int cols, int vec, uint8_t* __restrict__ xp) {
+__global__ void __launch_bounds__(NB * 8) csb_umma_pack_kernel(const float* __restrict__ X, long long ldx, int nb, int cols, int vec, uint8_t* __restrict__ xp,
+                                                               uint32_t* __restrict__ bad) {
     pdl_launch_dependents();
     pdl_wait();                                           // X may come from the kernel in front; xp may still be read by it
     const int b = threadIdx.x >> 3, c = (int)blockIdx.x * kUmmaWindow + (threadIdx.x & 7) * 8;
-    if (b < nb && c + 8 <= cols) { put_eight<NB>(xp, b, c, cols, X + (long long)b * ldx + c, vec != 0); return; }
-    float x[8];
+    bool large = false;
+    if (b < nb && c + 8 <= cols) large = put_eight<NB>(xp, b, c, cols, X + (long long)b * ldx + c, vec != 0);
+    else {
+        float x[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = b < nb && c + i < cols ? X[(long long)b * ldx + c + i] : 0.f;
-    uint4 hi, lo;
-    hi.x = split_pair(x[0], x[1], lo.x); hi.y = split_pair(x[2], x[3], lo.y);
-    hi.z = split_pair(x[4], x[5], lo.z); hi.w = split_pair(x[6], x[7], lo.w);
-    uint8_t* at = xp + image_at<NB>(b, c);
-    *reinterpret_cast<uint4*>(at) = hi;
-    *reinterpret_cast<uint4*>(at + NB * 128) = lo;
+        for (int i = 0; i < 8; ++i) x[i] = b < nb && c + i < cols ? X[(long long)b * ldx + c + i] : 0.f;
+        large = put_split<NB>(xp, b, c, x);
+    }
+    large = __any_sync(0xffffffffu, large);
+    if ((threadIdx.x & 31) == 0) bad[blockIdx.x * (NB / 4) + (threadIdx.x >> 5)] = large;
 }
 
 #define CSB_CUDA(call)                                                                     \
@@ -93,6 +94,8 @@ int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]) {
 
 int umma_nb(int batch) { return batch <= 16 ? 16 : batch <= 32 ? 32 : 64; }
 
+static uint32_t* bad_words(uint8_t* xp, int windows) { return reinterpret_cast<uint32_t*>(xp + (size_t)windows * kUmmaImage); }
+
 // Y = A . (packed inputs) with the plan's output rows.
 int launch_umma_packed(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, float* Y, int NB, int nb, int64_t ldy, cudaStream_t st) {
     UmmaArgs a{};
@@ -101,7 +104,7 @@ int launch_umma_packed(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, floa
     UmmaStages g;
     if (!umma_stages(0, NB, P->MT, P->max_round, A->smem_optin, &g)) { set_error("the batched product's stages do not fit"); return CSB_ERR_LAUNCH; }
     a.x_depth = g.x_depth; a.w_bytes = g.w_bytes;
-    p.stream = P->d_stream; p.ctas = P->d_ctas; p.rounds = P->d_rounds; p.quads = P->d_quads; p.xp = xp; p.Y = Y;
+    p.stream = P->d_stream; p.ctas = P->d_ctas; p.rounds = P->d_rounds; p.quads = P->d_quads; p.xp = xp; p.bad = bad_words(xp, P->windows); p.Y = Y;
     p.block_r = A->block_r; p.seg_words = P->seg_words; p.windows = P->windows; p.cta_end = P->n_ctas;
     cudaLaunchAttribute attr[2];
     const cudaLaunchConfig_t cfg = umma_config(P->n_ctas, P->S, g.smem, st, attr);
@@ -117,13 +120,14 @@ int launch_umma_pack(const float* X, int64_t ldx, int nb, int cols, int NB, uint
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = 1;
-    cfg.gridDim = dim3((unsigned)((cols + kUmmaWindow - 1) / kUmmaWindow)); cfg.blockDim = dim3((unsigned)NB * 8);
+    const int windows = (cols + kUmmaWindow - 1) / kUmmaWindow;
+    cfg.gridDim = dim3((unsigned)windows); cfg.blockDim = dim3((unsigned)NB * 8);
     CSB_CUDA(cudaLaunchKernelEx(&cfg, NB == 16 ? csb_umma_pack_kernel<16> : NB == 32 ? csb_umma_pack_kernel<32> : csb_umma_pack_kernel<64>, X, (long long)ldx, nb,
-                                cols, vec, xp));
+                                cols, vec, xp, bad_words(xp, windows)));
     return CSB_OK;
 }
 
-// Packs fp32 inputs into xp (windows * kUmmaImage bytes) and launches, 64 batch columns at a time.
+// Packs fp32 inputs into xp (umma_xp_bytes) and launches, 64 batch columns at a time.
 int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st) {
     for (int b0 = 0; b0 < batch; b0 += 64) {
         const int nb = std::min(64, batch - b0), NB = umma_nb(nb);

@@ -9,6 +9,7 @@
 //   header  uint4 per (row segment, column segment), row segments first:
 //             x  bit l: lane l's row is kept (zero outside of the segment's rows, and where no column is kept)
 //             y  where the segment's values start, bytes from the item
+//             z, w  bit c: the segment's column c is kept
 //   values  16 bytes per eight columns and kept row, [eight columns][row], binary16, zero where a column is not kept
 //
 // A row segment is the part of one block-row that lies in the quadrant, a column segment 16, 32 or 64 columns, the
@@ -35,6 +36,8 @@ struct UmmaQuad {             // 32 lanes of a tile
     int32_t out0, pad[3];     // the first one's place in a product's output
 };
 static_assert(sizeof(UmmaQuad) == 32, "two 16-byte words");
+// Bytes of packed inputs: the images of 64 batch columns, then 16 words per window (are there inputs that binary16 cannot hold?).
+inline size_t umma_xp_bytes(int windows) { return (size_t)windows * (kUmmaImage + 64); }
 struct UmmaCta {
     uint32_t off128;          // where its rounds start, 128-byte units
     int32_t table;            // its first entry in the table of rounds

@@ -10,7 +10,9 @@
 //     passes through shared memory in its dense form, whose bandwidth the B operand needs;
 //   * the inputs are packed into binary16 pairs x = hi + lo (no input precision is lost as long as |x| < 65504) as 128-byte
 //     swizzled, K-major operand images, 64 columns each, the hi rows of all batch columns, then the lo rows; a
-//     bulk copy brings an image as it is;
+//     bulk copy brings an image as it is.  An input that binary16 cannot hold (NaN, infinite, from 65520 on) would make
+//     NaN of its column's zeros too: it is left out of the product, marked, and where there is a mark the sums of
+//     the rows that keep its column are set to NaN behind the product (spoil_sums);
 //   * one warp issues the tcgen05.mma, one thread the copies of the inputs, one those of the values;
 //   * the tensor cores add into TMEM with truncation, so the hi rows' sums of a unit (a tile over `flush` windows) start
 //     from zero and are taken out by the same sixteen warps, which add them in registers with rounding.  The units' buffers
@@ -45,6 +47,7 @@ struct UmmaPart {
     const UmmaRound* rounds;
     const UmmaQuad* quads;
     uint8_t* xp;               // packed inputs: per window an image of 2 * NB rows of 128 bytes (time loop: two such buffers)
+    uint32_t* bad;             // NB / 4 words per window: are there marks in it?  (time loop: 16 bytes a buffer, the call and tick of the latest mark)
     float* Y;
     int cta_end;               // the part's CTAs end here in the grid
     int block_r, seg_words, windows;
@@ -65,6 +68,7 @@ struct UmmaArgs {
     uint32_t never;                                        // test hook: arrivals that never come,
     int never_step;                                        // and the step at which they are missing for the warps that pack x alone
     int T, H, x_vec;                                       // x_vec: rows of x start at multiples of 16 bytes
+    uint32_t call;                                         // this call's number
 };
 
 // ---- tcgen05 -----------------------------------------------------------------------------------------
@@ -199,20 +203,42 @@ __device__ __forceinline__ void add_pair(float2& a, uint32_t b0, uint32_t b1) {
 template <int NB> __device__ __forceinline__ size_t image_at(int n, int c) {
     return (size_t)(c >> 6) * (NB * 256) + (size_t)(n * 128 + ((((c >> 3) & 7) ^ (n & 7)) << 4) + (c & 7) * 2);
 }
-__device__ __forceinline__ uint32_t split_pair(float a, float b, uint32_t& lo) {
+// The mark of an input that binary16 cannot hold: +0 above, -0 below, which no other input gives (what rounds to +0 is not
+// negative, and -0 leaves a remainder of +0).
+constexpr uint32_t kBadLo = 0x8000u;
+__device__ __forceinline__ bool too_large(float x) { return !(fabsf(x) < 65520.f); }
+__device__ __forceinline__ uint32_t split_pair(float a, float b, uint32_t& lo, bool& large) {
+    const bool la = too_large(a), lb = too_large(b);
+    if (la) a = 0.f;
+    if (lb) b = 0.f;
+    large = large || la || lb;
     const __half h0 = __float2half_rn(a), h1 = __float2half_rn(b);
     const __half l0 = __float2half_rn(a - __half2float(h0)), l1 = __float2half_rn(b - __half2float(h1));
-    lo = (uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16);
+    lo = (uint32_t)__half_as_ushort(l0) | ((uint32_t)__half_as_ushort(l1) << 16) | (la ? kBadLo : 0u) | (lb ? kBadLo << 16 : 0u);
     return (uint32_t)__half_as_ushort(h0) | ((uint32_t)__half_as_ushort(h1) << 16);
 }
-template <int NB> __device__ __forceinline__ void put_value(uint8_t* images, int b, int c, float x) {
-    const __half hi = __float2half_rn(x);
+// These write inputs into the images; true where one of them is marked.
+template <int NB> __device__ __forceinline__ bool put_value(uint8_t* images, int b, int c, float x) {
+    const bool large = too_large(x);
+    if (large) x = 0.f;
+    const __half hi = __float2half_rn(x), lo = __float2half_rn(x - __half2float(hi));
     uint8_t* at = images + image_at<NB>(b, c);
     *reinterpret_cast<__half*>(at) = hi;
-    *reinterpret_cast<__half*>(at + NB * 128) = __float2half_rn(x - __half2float(hi));
+    *reinterpret_cast<__half*>(at + NB * 128) = large ? __ushort_as_half((unsigned short)kBadLo) : lo;
+    return large;
+}
+template <int NB> __device__ __forceinline__ bool put_split(uint8_t* images, int b, int c, const float (&x)[8]) {
+    bool large = false;
+    uint4 hi, lo;
+    hi.x = split_pair(x[0], x[1], lo.x, large); hi.y = split_pair(x[2], x[3], lo.y, large);
+    hi.z = split_pair(x[4], x[5], lo.z, large); hi.w = split_pair(x[6], x[7], lo.w, large);
+    uint8_t* at = images + image_at<NB>(b, c);
+    *reinterpret_cast<uint4*>(at) = hi;
+    *reinterpret_cast<uint4*>(at + NB * 128) = lo;
+    return large;
 }
 // Columns c .. c + 7 (those below n) of batch column b; src points at column c.
-template <int NB> __device__ __forceinline__ void put_eight(uint8_t* images, int b, int c, int n, const float* src, bool vec) {
+template <int NB> __device__ __forceinline__ bool put_eight(uint8_t* images, int b, int c, int n, const float* src, bool vec) {
     if (c + 8 <= n) {
         float x[8];
         if (vec) {
@@ -222,14 +248,49 @@ template <int NB> __device__ __forceinline__ void put_eight(uint8_t* images, int
 #pragma unroll
             for (int i = 0; i < 8; ++i) x[i] = src[i];
         }
-        uint4 hi, lo;
-        hi.x = split_pair(x[0], x[1], lo.x); hi.y = split_pair(x[2], x[3], lo.y);
-        hi.z = split_pair(x[4], x[5], lo.z); hi.w = split_pair(x[6], x[7], lo.w);
-        uint8_t* at = images + image_at<NB>(b, c);
-        *reinterpret_cast<uint4*>(at) = hi;
-        *reinterpret_cast<uint4*>(at + NB * 128) = lo;
-    } else {
-        for (int i = 0; c + i < n; ++i) put_value<NB>(images, b, c + i, src[i]);
+        return put_split<NB>(images, b, c, x);
+    }
+    bool large = false;
+    for (int i = 0; c + i < n; ++i) large |= put_value<NB>(images, b, c + i, src[i]);
+    return large;
+}
+
+// Sets those of an expanding warp's sums to NaN that have a marked input in a column that the lane's row keeps: out[b * ld] for the batch
+// columns b from b0 on.  Marks are rare, so the images and the items' headers are simply read again, and the sums are
+// overwritten where they lie.
+// buffer: which of a time loop's buffers of images, whose sums lie [batch column][row of the group]; -1: a product's.
+template <int NB, int MT>
+__device__ __noinline__ void spoil_sums(const UmmaArgs& a, int p_idx, int cta, int warp, int buffer, float* out, long long ld) {
+    constexpr int CN = NB * MT / 4, kPer = 4 / MT;         // windows of a round
+    const UmmaPart& pt = a.part[p_idx];
+    const UmmaCta me = pt.ctas[cta];
+    const int lane = threadIdx.x & 31, quad = warp & 3, slot = warp >> 2, mt = MT == 2 ? slot >> 1 : 0, b0 = (MT == 2 ? slot & 1 : slot) * CN;
+    const int w0 = me.w0, nw = me.nw, seg_words = pt.seg_words;
+    const UmmaQuad q = pt.quads[((size_t)me.group * MT + mt) * 4 + quad];
+    const uint32_t seg_off = lane < q.nrows ? (uint32_t)((q.row0 + lane) / pt.block_r - q.row0 / pt.block_r) * (uint32_t)(32 / seg_words * 16) : 0u;
+    const uint8_t *stream = pt.stream + (size_t)me.off128 * 128, *images = pt.xp + (size_t)max(buffer, 0) * pt.windows * (NB * 256);
+    const uint2* rounds = reinterpret_cast<const uint2*>(pt.rounds) + me.table;
+    out += (buffer < 0 ? q.out0 : mt * 128 + quad * 32) + lane;
+    for (int w = 0; w < nw; ++w) {
+        const int rd = w / kPer, nj = min(4, nw * MT - 4 * rd), len = umma_unit_len(MT, a.flush, nj);
+        int j = 0;
+        while (j < 3 && (umma_place(MT, len, j).mt != mt || umma_place(MT, len, j).window != w % kPer)) ++j;
+        const uint8_t* round = stream + (size_t)__ldg(rounds + rd).x * 16;
+        const uint8_t* header = round + __ldg(reinterpret_cast<const uint32_t*>(round) + j * 4 + quad) + seg_off;
+        const uint8_t* image = images + (size_t)(w0 + w) * (NB * 256);
+        for (int i = 0; i < CN && b0 + i < a.nb; ++i) {
+            const uint8_t* at = image + image_at<NB>(b0 + i, 2 * lane);
+            const uint32_t hi = __ldcg(reinterpret_cast<const uint32_t*>(at)), lo = __ldcg(reinterpret_cast<const uint32_t*>(at + NB * 128));
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                uint32_t marks = __ballot_sync(0xffffffffu, ((hi >> (16 * p)) & 0xffffu) == 0u && ((lo >> (16 * p)) & 0xffffu) == kBadLo);
+                for (; marks; marks &= marks - 1u) {
+                    const int c = 2 * (__ffs(marks) - 1) + p, k = c % (2 * seg_words);
+                    const uint4 h = __ldg(reinterpret_cast<const uint4*>(header + 16 * (c / (2 * seg_words))));
+                    if ((h.x >> lane) & ((k < 32 ? h.z : h.w) >> (k & 31)) & 1u) out[(b0 + i) * ld] = __int_as_float(0x7fffffff);
+                }
+            }
+        }
     }
 }
 
@@ -284,9 +345,14 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L.bars);
     uint64_t *xfull = bars, *xempty = xfull + kMaxXDepth, *wfull = xempty + kMaxXDepth, *wempty = wfull + kWRounds;
     uint64_t *afull = wempty + kWRounds, *aempty = afull + 2, *dfull = aempty + 2, *dempty = dfull + DB, *pfull = dempty + DB, *xdone = pfull + 1;
-    volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(xdone + 1);
-    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(xdone + 1) + 1;
-    volatile uint32_t* w_at = reinterpret_cast<volatile uint32_t*>(xdone + 2);       // where a round of values lies in its ring
+    uint64_t *sums = xdone + 1, *spoilt = sums + 1;
+    volatile uint32_t* s_dead = reinterpret_cast<volatile uint32_t*>(spoilt + 1);
+    uint32_t* s_tmem = reinterpret_cast<uint32_t*>(spoilt + 1) + 1;
+    volatile uint32_t* w_at = reinterpret_cast<volatile uint32_t*>(spoilt + 2);       // where a round of values lies in its ring
+    // Are there marks in the CTA's windows?  Time loop: the call and tick of the latest mark in the images (a copy, 16 bytes); then
+    // whether a state of the CTA's own is marked; then the number of ticks whose sums have been gone through.
+    volatile uint32_t* s_bad = reinterpret_cast<volatile uint32_t*>(smem + L.bars + 384);
+    static_assert((2 * kMaxXDepth + 2 * kWRounds + 4 + 2 * DB + 5) * 8 + kWRounds * 4 <= 384, "the barriers end before");
     float* part = reinterpret_cast<float*>(smem + L.part);        // the CTA's sums: [batch column][row of the group]
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -304,7 +370,10 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         for (int i = 0; i < DB; ++i) { mbar_init(dfull + i, 1); mbar_init(dempty + i, kUmmaExpandWarps / MT); }
         mbar_init(pfull, (uint32_t)a.S);
         mbar_init(xdone, 1);
+        mbar_init(sums, kUmmaExpandWarps);
+        mbar_init(spoilt, 1);
         *s_dead = 0u;
+        s_bad[0] = s_bad[1] = s_bad[4] = s_bad[5] = 0u;
         mbar_fence_init();
     }
     if (warp == kUmmaExpandWarps) tc_alloc(smem_u32(s_tmem), 512);
@@ -346,13 +415,16 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         while ((int32_t)(ld_acquire_gpu(a.count) - need) < 0) if (gave_up(spins, t0, a.limit_ns, kDevBarrierTimeout)) return false;
         return true;
     };
+    // Time loop: there is a marked input in what the part reads in that tick.
+    auto mark = [&](const UmmaPart& part_of, int tick) {
+        *reinterpret_cast<uint2*>(part_of.bad + 4 * (tick & 1)) = make_uint2(a.call, (uint32_t)tick + 1u);
+    };
     float2 acc[CN / 2];
 #pragma unroll
     for (int i = 0; i < CN / 2; ++i) acc[i] = make_float2(0.f, 0.f);
     const int quad = warp & 3, slot = warp >> 2;          // expanding warps: lanes of the tile, which tile-window of a round
     const int my_mt = MT == 2 ? slot >> 1 : 0, my_b0 = MT == 2 ? (slot & 1) * CN : slot * CN;      // and whose sums the warp keeps
     const UmmaQuad* quads = pt.quads + (size_t)me->group * MT * 4;
-
     if (warp < kUmmaExpandWarps) {
         const int seg_words = pt.seg_words, segs = 32 / seg_words;
         uint32_t seg_off[MT];                             // the lane's row segment: where its headers start in an item
@@ -449,6 +521,12 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 at[0] = acc[i].x; at[kRows] = acc[i].y;
                 acc[i] = make_float2(0.f, 0.f);
             }
+            if (ok && s_bad[0] == a.call && s_bad[1] == (uint32_t)(t + p_idx + 1)) {
+                const uint32_t par = s_bad[5] & 1u;       // the copying warp goes through them
+                __syncwarp();
+                if (lane == 0) mbar_arrive(sums);
+                ok = __all_sync(0xffffffffu, wait(spoilt, par));
+            }
             ok = expand_barrier(ok);
             if (!ok) break;
             if (a.S > 1 && (int)threadIdx.x < a.S) arrive_peer(pfull, threadIdx.x);
@@ -505,6 +583,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                     if (MODE == 1) h = lstm_cell(z[p][0], z[p][1], z[p][2], z[p][3], st);
                     else st = h = gru_cell(z[p][0], z[p][1], z[p][2], z[p][3], st);
                     *state = st;
+                    if (too_large(h)) s_bad[4] = 1u;
                     if (more) put_value<NB>(pt.xp + (size_t)next * pt.windows * kWin, b[p], a.in_size[p_idx] + u[p], h);
                     if (p_idx + 1 < a.n_parts) {
                         const UmmaPart& above = a.part[p_idx + 1];
@@ -521,7 +600,15 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
             if (warp == 0 && p_idx == 0 && more && ok) ok = __all_sync(0xffffffffu, wait(xdone, (uint32_t)t & 1u));
             ok = expand_barrier(ok);
             if (!ok) break;
-            if (threadIdx.x == 0) { __threadfence(); add_release_gpu(a.count, 1u); }
+            if (threadIdx.x == 0) {
+                if (s_bad[4]) {
+                    s_bad[4] = 0u;
+                    mark(pt, t + p_idx + 1);
+                    if (p_idx + 1 < a.n_parts) mark(a.part[p_idx + 1], t + p_idx + 1);
+                }
+                __threadfence();
+                add_release_gpu(a.count, 1u);
+            }
             }
         }
     } else if (warp == kUmmaExpandWarps) {
@@ -535,7 +622,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         for (int t = 0; t < T_ && ok; ++t)
             for (int rd = 0; rd < rounds && ok; ++rd) {
                 const int nj = min(4, ntw - 4 * rd), len = umma_unit_len(MT, F, nj);
-                ok = __all_sync(0xffffffffu, wait(xfull + xs, x_par) && wait(afull + half, a_par));
+                ok = __all_sync(0xffffffffu, wait(afull + half, a_par) && wait(xfull + xs, x_par));
                 uint64_t x = x_desc + (uint64_t)((xs * kXStage) >> 4);
                 for (int j0 = 0; j0 < nj && ok; j0 += len) {
                     if (XW < 4 / MT && j0 == XW) {        // the second stage of the round
@@ -573,12 +660,14 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 a_par ^= half ^ 1u;
             }
     } else if (warp == kUmmaExpandWarps + 1) {
-        if (lane == 0) {
-            if (!MODE) pdl_wait();                        // the packed inputs belong to the work in front on the stream
-            bool ok = true;
-            uint32_t at = 0, par = 1;
-            for (int t = 0; t < T_ && ok; ++t) {
+        if (!MODE) pdl_wait();                            // the packed inputs belong to the work in front on the stream
+        bool ok = true;
+        uint32_t at = 0, par = 1;
+        for (int t = 0; t < T_; ++t) {
+            bool marked = false;
+            if (lane == 0) {
                 const uint8_t* src = pt.xp + (size_t)w0 * kWin;
+                const uint32_t* marks = pt.bad + 4 * ((t + p_idx) & 1);
                 if (MODE) {
                     src += (size_t)((t + p_idx) & 1) * pt.windows * kWin;
                     ok = wait_tick(t, a.never);
@@ -588,10 +677,24 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                     ok = wait(xempty + at, par);
                     if (!ok) break;
                     const uint32_t bytes = (uint32_t)min(XW, nw - w) * kWin;
-                    mbar_expect_tx(xfull + at, bytes);
+                    if (MODE && w == 0) {                 // (with the tick's first images: the tick in front has been read)
+                        mbar_expect_tx(xfull + at, bytes + 16u);
+                        bulk_g2s(const_cast<uint32_t*>(s_bad), marks, 16u, xfull + at);
+                    } else mbar_expect_tx(xfull + at, bytes);
                     bulk_g2s(smem + at * kXStage, src + (size_t)w * kWin, bytes, xfull + at);
                     if (++at == (uint32_t)XD) { at = 0; par ^= 1u; }
                 }
+                if (MODE && ok) marked = __ldcg(marks) == a.call && __ldcg(marks + 1) == (uint32_t)(t + p_idx + 1);
+            }
+            if (MODE) {
+                if (!__shfl_sync(0xffffffffu, ok, 0)) break;
+                if (!__shfl_sync(0xffffffffu, marked, 0)) continue;
+                if (!__all_sync(0xffffffffu, wait(sums, s_bad[5] & 1u))) break;
+#pragma unroll 1
+                for (int v = 0; v < kUmmaExpandWarps; ++v) spoil_sums<NB, MT>(a, p_idx, (int)blockIdx.x - cta0, v, (t + p_idx) & 1, part, kRows);
+                __syncwarp();
+                if (lane == 0) { s_bad[5] = s_bad[5] + 1u; mbar_arrive(spoilt); }
+                __syncwarp();
             }
         }
     } else if (warp == kUmmaExpandWarps + 2) {
@@ -632,8 +735,17 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                     if (++at == kWRounds) at = 0;
                 }
         }
-    }
-    if (MODE != 0 && warp == kUmmaExpandWarps + 3 && p_idx == 0) {
+    } else if (MODE == 0) {                               // (as a block of its own behind these roles it cost 8192 x 8192 at batch 64 2.6 of 28 us)
+        pdl_wait();
+        const uint4* words = reinterpret_cast<const uint4*>(pt.bad) + w0 * (NB / 16);
+        uint32_t any = 0;
+#pragma unroll 4
+        for (int i = lane; i < nw * (NB / 16); i += 32) {
+            const uint4 u = __ldcg(words + i);
+            any |= u.x | u.y | u.z | u.w;
+        }
+        if (any) s_bad[0] = 1u;
+    } else if (p_idx == 0) {
         // x_{t+1}, shared between the CTAs of the first layer, while step t runs
         const int I = a.in_size[0], chunks = (I + 7) / 8;
         bool ok = true;
@@ -643,7 +755,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
             uint8_t* images = pt.xp + (size_t)((t + 1) & 1) * pt.windows * kWin;
             for (int i = (int)blockIdx.x * 32 + lane; i < chunks * a.nb; i += pt.cta_end * 32) {
                 const int b = i / chunks, c = (i - b * chunks) * 8;
-                put_eight<NB>(images, b, c, I, a.x + ((size_t)(t + 1) * a.nb + b) * I + c, a.x_vec != 0);
+                if (put_eight<NB>(images, b, c, I, a.x + ((size_t)(t + 1) * a.nb + b) * I + c, a.x_vec != 0)) mark(pt, t + 1);
             }
             __syncwarp();
             if (lane == 0) { __threadfence(); mbar_arrive(xdone); }
@@ -666,6 +778,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
         return;
     }
     pdl_wait();                                           // Y belongs to the work in front
+    const bool marked = s_bad[0] != 0u && !dead && warp < kUmmaExpandWarps;
     if (a.S == 1) {
         if (!dead && warp < kUmmaExpandWarps) {
             const UmmaQuad q = quads[my_mt * 4 + quad];
@@ -674,6 +787,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 for (int i = 0; i < CN; ++i)
                     if (my_b0 + i < a.nb) pt.Y[(long long)(my_b0 + i) * a.ldy + q.out0 + lane] = i & 1 ? acc[i / 2].y : acc[i / 2].x;
         }
+        if (marked) spoil_sums<NB, MT>(a, 0, (int)blockIdx.x, warp, -1, pt.Y, a.ldy);
         return;
     }
     if (warp < kUmmaExpandWarps)
@@ -711,6 +825,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     }
     __syncthreads();
     umma_cluster_barrier();                               // nobody leaves before everybody has read
+    if (marked) spoil_sums<NB, MT>(a, 0, (int)blockIdx.x, warp, -1, pt.Y, a.ldy);
 }
 
 }  // namespace csb

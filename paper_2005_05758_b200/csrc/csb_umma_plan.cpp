@@ -53,8 +53,8 @@ struct ItemWriter {
 
     int segments(const UmmaQuad& q) const { return q.nrows ? (int)((q.row0 + q.nrows - 1) / A->block_r - q.row0 / A->block_r) + 1 : 1; }
 
-    // One (row segment, column segment), the columns from `col` on: appends its values, returns the mask of its kept rows.
-    uint32_t segment(const UmmaQuad& q, int g, int64_t col, std::vector<uint8_t>& out) const {
+    // One (row segment, column segment), the columns from `col` on: appends its values, returns the masks of its kept rows and columns.
+    uint32_t segment(const UmmaQuad& q, int g, int64_t col, std::vector<uint8_t>& out, uint64_t* columns) const {
         if (!q.nrows || col >= A->cols) return 0;
         const int64_t bi = q.row0 / A->block_r + g, bj = col / A->block_c, b = bi * A->nbc + bj;
         const int m = A->m[b], n = A->n[b], base = (int)(col - bj * A->block_c);
@@ -80,7 +80,11 @@ struct ItemWriter {
         uint16_t* v = reinterpret_cast<uint16_t*>(out.data() + at);
         const uint16_t* src = reinterpret_cast<const uint16_t*>(A->val.data()) + A->val_off[b] + (size_t)first * n;
         uint16_t place[64];                                    // of the kept columns, in the first row
-        for (int k = k0; k < k1; ++k) { const int c = ci[k] - base; place[k - k0] = (uint16_t)((c >> 3) * kr * 8 + (c & 7)); }
+        for (int k = k0; k < k1; ++k) {
+            const int c = ci[k] - base;
+            place[k - k0] = (uint16_t)((c >> 3) * kr * 8 + (c & 7));
+            *columns |= 1ull << c;
+        }
         for (int i = 0; i < kr; ++i, src += n, v += 8)
             for (int k = k0; k < k1; ++k) v[place[k - k0]] = src[k];
         return rows;
@@ -93,7 +97,9 @@ struct ItemWriter {
         for (int g = 0; g < ng; ++g)
             for (int s = 0; s < ns; ++s) {
                 uint32_t h[4] = {0u, (uint32_t)(out.size() - start), 0u, 0u};
-                h[0] = segment(q, g, w0 + (int64_t)s * 2 * seg_words, out);
+                uint64_t columns = 0;
+                h[0] = segment(q, g, w0 + (int64_t)s * 2 * seg_words, out, &columns);
+                h[2] = (uint32_t)columns; h[3] = (uint32_t)(columns >> 32);
                 std::memcpy(out.data() + start + (size_t)(g * ns + s) * 16, h, 16);
             }
     }

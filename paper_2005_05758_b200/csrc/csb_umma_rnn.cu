@@ -29,10 +29,11 @@ UmmaStack::~UmmaStack() { for (UmmaPlan& p : plan) drop_umma_plan(p); }
 struct UmmaRnnPlan {
     std::shared_ptr<UmmaStack> stack;
     int B = 0, NB = 0;
-    uint8_t* d_xp[kMaxLayers] = {};    // two buffers of operand images per layer
+    uint8_t* d_xp[kMaxLayers] = {};    // two buffers of operand images per layer, and 16 bytes of marks for each
     float* d_state = nullptr;          // [L, B, H] c (LSTM) or h (GRU) at the start
     float* d_ends = nullptr;           // [4][L, B, H] h0 and c0 from the host; hT and cT where the caller's arrays cannot be written directly
     uint32_t* d_count = nullptr;
+    uint32_t calls = 0;                // counted, so that a mark of an earlier call is told from this one's
     uint32_t* h_status = nullptr; uint32_t* d_status = nullptr;
     float* d_stage = nullptr;          // host-I/O staging of x and y
     size_t stage_cap = 0;
@@ -150,24 +151,27 @@ struct UmmaBeginArgs {
     const float* x; const float* h0; const float* c0;     // h0, c0: null = zeros
     float* state; uint32_t* count;
     uint8_t* xp[kMaxLayers];
+    uint32_t* bad[kMaxLayers];
     int in_size[kMaxLayers], windows[kMaxLayers];
     int L, B, H, lstm, x_vec;
+    uint32_t call;
 };
 template <int NB>
 __global__ void __launch_bounds__(256) csb_umma_begin_kernel(const __grid_constant__ UmmaBeginArgs a) {
     const int chunks = (a.in_size[0] + 7) / 8, n = a.L * a.B * a.H;
     const long long all = (long long)n + (long long)chunks * a.B;
+    auto mark = [&](int l) { *reinterpret_cast<uint2*>(a.bad[l] + 4 * (l & 1)) = make_uint2(a.call, (uint32_t)l + 1u); };
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.count = 0u;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < all; i += (long long)gridDim.x * blockDim.x) {
         if (i < n) {
             const int u = (int)(i % a.H), b = (int)(i / a.H % a.B), l = (int)(i / a.H / a.B);
             const float h = a.h0 ? a.h0[i] : 0.f;
             // (layer l reads its first step in tick l)
-            put_value<NB>(a.xp[l] + (size_t)(l & 1) * a.windows[l] * (NB * 256), b, a.in_size[l] + u, h);
+            if (put_value<NB>(a.xp[l] + (size_t)(l & 1) * a.windows[l] * (NB * 256), b, a.in_size[l] + u, h)) mark(l);
             a.state[i] = !a.lstm ? h : a.c0 ? a.c0[i] : 0.f;
         } else {
             const int j = (int)(i - n), b = j / chunks, c = (j - b * chunks) * 8;
-            put_eight<NB>(a.xp[0], b, c, a.in_size[0], a.x + (size_t)b * a.in_size[0] + c, a.x_vec != 0);
+            if (put_eight<NB>(a.xp[0], b, c, a.in_size[0], a.x + (size_t)b * a.in_size[0] + c, a.x_vec != 0)) mark(0);
         }
     }
 }
@@ -177,7 +181,7 @@ static int build_plan(UmmaRnnPlan* P) {
     const size_t ns = (size_t)K.L * P->B * K.H * 4;
     for (int l = 0; l < K.L; ++l) {
         // what is not written (columns past the last, batch columns past B) stays zero
-        const size_t bytes = (size_t)2 * K.plan[l].windows * P->NB * 256;
+        const size_t bytes = (size_t)2 * K.plan[l].windows * P->NB * 256 + 32;
         CSB_CUDA(cudaMalloc((void**)&P->d_xp[l], bytes));
         CSB_CUDA(cudaMemsetAsync(P->d_xp[l], 0, bytes, cudaStreamPerThread));
     }
@@ -209,6 +213,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
             P = np.get();
             g_umma_plans.push_back(std::move(np));
         }
+        ++P->calls;
     }
     UmmaStages g;
     if (!umma_stages(1, P->NB, K->plan[0].MT, K->max_round, W[0]->smem_optin, &g)) return 1;
@@ -251,6 +256,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
         const UmmaPlan& Q = K->plan[l];
         UmmaPart& p = a.part[l];
         p.stream = Q.d_stream; p.ctas = Q.d_ctas; p.rounds = Q.d_rounds; p.quads = Q.d_quads; p.xp = P->d_xp[l];
+        p.bad = ba.bad[l] = reinterpret_cast<uint32_t*>(P->d_xp[l] + (size_t)2 * Q.windows * NB * 256);
         p.block_r = W[l]->block_r; p.seg_words = Q.seg_words; p.windows = Q.windows;
         ctas += Q.n_ctas;
         p.cta_end = ctas;
@@ -261,7 +267,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
     a.x = dx; a.y = dy; a.state0 = P->d_state;
     a.hT = move_hT ? P->d_ends + 2 * ns : hT;
     a.cT = move_cT ? P->d_ends + 3 * ns : cT;
-    a.count = P->d_count; a.T = (int)T; a.H = H; a.x_vec = ba.x_vec;
+    a.count = P->d_count; a.T = (int)T; a.H = H; a.x_vec = ba.x_vec; a.call = ba.call = P->calls;
     uint32_t extra = 0;
     barrier_test_hook(&extra, &a.limit_ns);
     a.never = extra == 1 ? kNever : 0u;

@@ -63,7 +63,7 @@ int make_umma_plan(const csb_matrix* A, UmmaPlan* P) {
             H.quads = umma_row_quads(A, H.MT);
             H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
             plan_umma_host(A, &H);
-            CSB_CUDA(cudaMalloc((void**)&P->d_xp, (size_t)H.windows * kUmmaImage));
+            CSB_CUDA(cudaMalloc((void**)&P->d_xp, umma_xp_bytes(H.windows)));
             return upload_umma(A, H, P);
         } catch (const std::bad_alloc&) { return CSB_ERR_ALLOC; }
     }();

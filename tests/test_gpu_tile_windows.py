@@ -121,3 +121,90 @@ def test_one_warp_that_gives_up_takes_the_sequence_along(I, H, L, step):
     assert torch.equal(run(), want)
     for m in mats:
         m.free()
+
+
+def kept(m):
+    """[rows, cols]: is the weight stored?"""
+    nbr, nbc = -(-m.rows // m.block_r), -(-m.cols // m.block_c)
+    both = m.row_keep.reshape(nbr, nbc, m.block_r, 1).astype(bool) & m.col_keep.reshape(nbr, nbc, 1, m.block_c).astype(bool)
+    return both.transpose(0, 2, 1, 3).reshape(nbr * m.block_r, nbc * m.block_c)[:m.rows, :m.cols]
+
+
+LARGE = [float("nan"), float("inf"), -float("inf"), 65520.0, -1e30]
+
+
+@pytest.mark.parametrize("rows,cols,br,bc,batch", [(127, 63, 32, 32, 9), (300, 1177, 16, 16, 17), (513, 2049, 64, 64, 64), (200, 130, 24, 128, 70), (4096, 700, 32, 32, 8),
+                                                   (8192, 1000, 64, 64, 33), (130, 2100, 64, 64, 40)])
+def test_an_input_past_binary16_touches_the_rows_that_keep_it(rows, cols, br, bc, batch):
+    # NaN where a block keeps the column for the row, and the bits of the same inputs without it everywhere else
+    w = workloads.make_spmv_workload(rows + cols, rows, cols, br, bc, "uniform", lo=0.1, hi=0.6, batch=batch, w_std=0.05)
+    m = w.matrix
+    A = binding.csb_encode(m.dense, br, bc, m.row_keep, m.col_keep, "f16", 0)
+    rng = np.random.default_rng(rows)
+    for n in (1, 5, batch * cols // 3):
+        bad = np.zeros((batch, cols), bool)
+        bad.reshape(-1)[rng.choice(batch * cols, n, replace=False)] = True
+        bad[batch - 1, cols - 1] = True
+        clean, x = np.where(bad, np.float32(0), w.X), w.X.copy()
+        x[bad] = np.resize(np.array(LARGE, np.float32), int(bad.sum()))
+        got, want = torch.empty((batch, rows), device="cuda"), torch.empty((batch, rows), device="cuda")
+        binding.csb_spmm(A, torch.from_numpy(x).cuda(), got)
+        binding.csb_spmm(A, torch.from_numpy(clean).cuda(), want)
+        torch.cuda.synchronize()
+        got, want, hit = got.cpu().numpy(), want.cpu().numpy(), bad.astype(np.float32) @ kept(m).T.astype(np.float32) > 0
+        assert np.array_equal(np.isnan(got), hit) and np.array_equal(got[~hit], want[~hit])
+    x = torch.from_numpy(w.X).cuda()
+    x[0, 0], x[batch - 1, cols - 1] = 65519.0, -65504.0          # binary16 still holds these
+    y = torch.empty((batch, rows), device="cuda")
+    binding.csb_spmm(A, x, y)
+    assert torch.isfinite(y).all()
+    A.free()
+
+
+@pytest.mark.parametrize("cell,B,I,H,L,br", [("lstm", 16, 39, 100, 3, 32), ("lstm", 32, 70, 96, 1, 16), ("gru", 17, 70, 96, 2, 32), ("gru", 32, 153, 160, 1, 64), ("lstm", 40, 39, 64, 2, 16),
+                                             ("gru", 40, 39, 64, 2, 32), ("lstm", 20, 600, 512, 2, 64)])
+def test_an_input_past_binary16_spreads_through_a_sequence_where_it_is_kept(cell, B, I, H, L, br):
+    T = 5
+    w = workloads.make_rnn_workload(61, cell, I, H, L, br, br, "uniform", lo=0.05, hi=0.3, T=T, B=B, w_std=0.15, bias_std=0.2, state_std=0.4)
+    mats = [binding.csb_encode(m.dense, m.block_r, m.block_c, m.row_keep, m.col_keep, m.val_dtype, 0) for m in w.layers]
+    bias = [torch.from_numpy(b).cuda() for b in w.bias]
+    rng = np.random.default_rng(B)
+    x, h0 = w.x.copy(), w.h0.copy()
+    # sequence 0 stays clean, 1 gets one at the start, 2 at the end, 3 in an upper state, 4 in the second step, 5 everywhere
+    bad_x, bad_h = np.zeros(x.shape, bool), np.zeros(h0.shape, bool)
+    bad_x[0, 1, rng.integers(I)] = bad_x[T - 1, 2, rng.integers(I)] = bad_x[1, 4, rng.integers(I)] = bad_h[L - 1, 3, rng.integers(H)] = True
+    bad_x[:, 5] = True
+    x[bad_x], h0[bad_h] = 0, 0
+
+    def run(x, h0):
+        y, hT, cT = (torch.full(s, float("nan"), device="cuda") for s in ((T, B, H), (L, B, H), (L, B, H)))
+        if cell == "gru":
+            binding.csb_gru_forward(mats, bias, torch.from_numpy(x).cuda(), torch.from_numpy(h0).cuda(), y, hT, 0)
+            cT.zero_()
+        else:
+            binding.csb_lstm_forward(mats, bias, torch.from_numpy(x).cuda(), torch.from_numpy(h0).cuda(), torch.from_numpy(w.c0).cuda(), y, hT, cT, 0)
+        return [t.cpu().numpy() for t in (y, hT, cT)]
+    want = run(x, h0)
+    assert all(np.isfinite(a).all() for a in want)
+    x[bad_x], h0[bad_h] = np.resize(np.array(LARGE, np.float32), int(bad_x.sum())), np.float32("inf") if cell == "lstm" else np.float32("nan")
+    got = run(x, h0)
+    K = [kept(m).astype(np.float32) for m in w.layers]
+    h, c, top = bad_h.copy(), np.zeros((L, B, H), bool), np.zeros((T, B, H), bool)
+    for t in range(T):
+        u = bad_x[t]
+        for l in range(L):
+            z = (np.concatenate([u, h[l]], 1).astype(np.float32) @ K[l].T > 0).reshape(B, -1, H)
+            if cell == "lstm":
+                c[l] |= z[:, 0] | z[:, 1] | z[:, 2]
+                h[l] = c[l] | z[:, 3]
+            else:
+                h[l] |= z[:, 0] | z[:, 1] | z[:, 2]
+            u = h[l]
+        top[t] = u
+    for a, b, hit in zip(got, want, (top, h, c)):
+        assert np.array_equal(np.isnan(a), hit) and np.array_equal(a[~hit], b[~hit])
+    assert top.any() and not top[:, 0].any()
+    for a, b in zip(run(np.where(bad_x, np.float32(0), x), np.where(bad_h, np.float32(0), h0)), want):       # nothing stays behind
+        assert np.array_equal(a, b)
+    for m in mats:
+        m.free()
