@@ -78,7 +78,7 @@ static cudaLaunchConfig_t umma_config(int ctas, int S, size_t smem, cudaStream_t
 // Clusters of S CTAs that the device holds at a time, S = 1 .. kUmmaMaxS (SMs that a processing cluster's size leaves over
 // are lost: 4 x 37 SMs do not make 37 clusters of four).
 int umma_clusters(const csb_matrix* A, int (&n)[kUmmaMaxS + 1]) {
-    const int sms = A->opts.ctas > 0 ? A->opts.ctas : A->sm_count;
+    const int sms = A->opts.ctas > 0 ? std::min(A->opts.ctas, A->sm_count) : A->sm_count;
     n[0] = 0; n[1] = sms;
     const void* kernel = pick_umma(0, 64, 2);
     const size_t smem = A->smem_optin;                     // (one CTA an SM in any case)

@@ -139,7 +139,10 @@ int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size,
     s->gates = gates; s->L = L; s->H = H; s->device = W[0]->device;
     for (int l = 0; l < L; ++l) { s->uids.push_back(W[l]->uid); s->in_size[l] = in_size[l]; }
     const int rc = build_stack(W, s.get());
-    if (rc != CSB_OK && rc != 1) return rc;
+    if (rc != CSB_OK && rc != 1 && rc != CSB_ERR_ALLOC) return rc;
+    // (where memory does not reach for these layouts, those of the step-by-step form may still fit; for good, so that a
+    // stack keeps its bits)
+    if (rc == CSB_ERR_ALLOC) for (UmmaPlan& p : s->plan) drop_umma_plan(p);
     s->taken = rc == CSB_OK;
     g_stacks.push_back(s);
     if (s->taken) *out = s;
@@ -209,7 +212,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
         if (!P) {
             std::unique_ptr<UmmaRnnPlan> np(new UmmaRnnPlan());
             np->stack = K; np->B = B; np->NB = B <= 16 ? 16 : 32;
-            if ((rc = build_plan(np.get())) != CSB_OK) { cudaGetLastError(); return rc; }
+            if ((rc = build_plan(np.get())) != CSB_OK) { cudaGetLastError(); return rc == CSB_ERR_ALLOC ? 1 : rc; }
             P = np.get();
             g_umma_plans.push_back(std::move(np));
         }
@@ -287,7 +290,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
     cfg.stream = st; cfg.attrs = attr; cfg.numAttrs = a.S > 1 ? 2 : 1;
     void* params[] = {&a};
     const cudaError_t e = cudaLaunchKernelExC(&cfg, pick_umma(lstm ? 1 : 2, NB, K->plan[0].MT), params);
-    if (e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); set_error("cooperative launch too large"); return CSB_ERR_LAUNCH; }
+    if (e == cudaErrorCooperativeLaunchTooLarge) { cudaGetLastError(); return 1; }     // a device that others share; nothing of the caller's has been written
     CSB_CUDA(e);
     const cudaMemcpyKind kind = host_io ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if (host_io && y) CSB_CUDA(cudaMemcpyAsync(y, dy, ny * 4, kind, st));

@@ -1,0 +1,71 @@
+// The host side of the batched recurrent calls (csb_umma_rnn.cu) on the CUDA runtime of fake_runtime.hpp: where the time loop
+// cannot run, the call has to be left to the step-by-step form.  Exit code 0: every rule below held.
+#include "../paper_2005_05758_b200/csrc/csb_umma_rnn.hpp"
+#include "fake_runtime.hpp"
+
+using namespace csb;
+
+static int g_clusters = 148;                               // CTAs that the device holds at a time
+namespace csb {
+void set_error(const char*, ...) {}
+void clear_error() {}
+int umma_clusters(const csb_matrix*, int (&n)[kUmmaMaxS + 1]) {
+    for (int s = 0; s <= kUmmaMaxS; ++s) n[s] = s ? g_clusters / s : 0;
+    return CSB_OK;
+}
+const void* pick_umma(int, int, int) { return nullptr; }
+bool umma_stages(int, int, int, int max_round, size_t room, UmmaStages* out) { *out = UmmaStages{2, max_round, room}; return true; }
+void note_recurrent_path(RecurrentPath) {}
+void barrier_test_hook(unsigned int* extra, unsigned long long* ns) { *extra = 0; *ns = 1; }
+}
+
+static const int I = 70, H = 96, L = 2, T = 3, B = 20, block = 32;
+static csb_matrix* layer(int cols, uint64_t uid) {
+    std::vector<float> W((size_t)4 * H * cols, 1.f);
+    const size_t blocks = (size_t)(4 * H / block) * ((cols + block - 1) / block);
+    std::vector<uint8_t> rk(blocks * block, 1), ck(rk.size(), 1);
+    csb_matrix* A = new csb_matrix();
+    A->device = 0; A->smem_optin = 232448; A->uid = uid;
+    if (encode_host(W.data(), 4 * H, cols, cols, block, block, rk.data(), ck.data(), CSB_F16, A) != CSB_OK) std::exit(3);
+    return A;
+}
+
+int main() {
+    csb_matrix* W[L] = {layer(I + H, 1), layer(2 * H, 2)};
+    const int in_size[L] = {I, H};
+    std::vector<float> x((size_t)T * B * I), y((size_t)T * B * H), s((size_t)L * B * H);
+    auto call = [&](unsigned flags) {
+        return rnn_forward_umma(4, L, W, nullptr, x.data(), T, B, H, in_size, s.data(), s.data(), y.data(), nullptr, nullptr, flags, nullptr);
+    };
+    auto forget = [&](const char* what, long n) {
+        for (csb_matrix* A : W) drop_umma_rnn_plans(A);
+        const int left = (int)g_live.size();
+        if (left) printf("%s, call %ld: %d arrays left\n", what, n, left);
+        g_live.clear();
+        return left != 0;
+    };
+    int bad = 0;
+    for (int onwards = 0; onwards < 2; ++onwards)
+        for (long n = 0;; ++n) {
+            g_calls = 0; g_fails = n; g_onwards = onwards;
+            const int rc = call(0);
+            const bool failed = g_calls > n;
+            // (the last call that can fail is the one that waits for the result)
+            if (failed ? rc != 1 && rc != CSB_ERR_ALLOC : rc != CSB_OK) { printf("call %ld: status %d\n", n, rc); ++bad; }
+            if (rc == CSB_ERR_ALLOC && g_launches < 2) { printf("call %ld: refused before anything ran\n", n); ++bad; }
+            g_fails = -1;
+            const int again = call(0);
+            if (again != CSB_OK && again != 1) { printf("call %ld: then status %d\n", n, again); ++bad; }
+            bad += forget("out of memory", n);
+            g_launches = 0;
+            if (!failed) break;
+        }
+    g_cooperative = cudaErrorCooperativeLaunchTooLarge;
+    const int large = call(0);
+    if (large != 1) { printf("a grid that does not fit: status %d\n", large); ++bad; }
+    g_cooperative = cudaSuccess;
+    if (call(0) != CSB_OK) { puts("and then"); ++bad; }
+    bad += forget("grid", 0);
+    puts(bad ? "failed" : "ok");
+    return bad != 0;
+}

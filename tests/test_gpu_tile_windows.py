@@ -208,3 +208,18 @@ def test_an_input_past_binary16_spreads_through_a_sequence_where_it_is_kept(cell
         assert np.array_equal(a, b)
     for m in mats:
         m.free()
+
+
+def test_more_ctas_than_the_device_holds_are_not_asked_for():
+    # csb_plan_opts may name any number of CTAs; eight layers of 640 units would then make a grid of 160
+    w = workloads.make_rnn_workload(31, "lstm", 640, 640, 8, 32, 32, "uniform", lo=0.2, hi=0.5, T=2, B=16, w_std=0.05)
+    outs = []
+    for ctas in (0, 400):
+        opts = dict(ctas=ctas, warps_per_cta=0, stage_bytes=0, stages=0)
+        mats = [binding.csb_encode(m.dense, 32, 32, m.row_keep, m.col_keep, "f16", 0, opts) for m in w.layers]
+        y = torch.full((2, 16, 640), float("nan"), device="cuda")
+        binding.csb_lstm_forward(mats, None, torch.from_numpy(w.x).cuda(), None, None, y, None, None, 0)
+        outs.append(y)
+        for m in mats:
+            m.free()
+    assert torch.equal(outs[0], outs[1])

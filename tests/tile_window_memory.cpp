@@ -1,43 +1,9 @@
-// The device side of a plan of the batched product (csb_umma_upload.cpp) on a CUDA runtime of this file's own, whose n-th
-// call that can fail does so, once or from then on, for every n.  Exit code 0: every rule below held.
-#include <cstdarg>
-#include <cstdio>
-#include <cstdlib>
-#include <cstring>
-#include <set>
-
+// The device side of a plan of the batched product (csb_umma_upload.cpp) on the CUDA runtime of fake_runtime.hpp, whose
+// n-th call that can fail does so, once or from then on, for every n.  Exit code 0: every rule below held.
 #include "../paper_2005_05758_b200/csrc/csb_umma_rnn.hpp"
+#include "fake_runtime.hpp"
 
 using namespace csb;
-
-static long g_calls = 0, g_fails = -1;                     // calls so far; the one that fails (< 0: none)
-static bool g_onwards = false;                             // and all behind it
-static cudaError_t g_error = cudaErrorMemoryAllocation;
-static std::set<void*> g_live;
-static bool fails() { const long n = g_calls++; return g_fails >= 0 && (n == g_fails || (g_onwards && n > g_fails)); }
-
-extern "C" {
-cudaError_t cudaMalloc(void** p, size_t n) {
-    *p = nullptr;
-    if (fails()) return g_error;
-    g_live.insert(*p = std::malloc(n));
-    return cudaSuccess;
-}
-cudaError_t cudaFree(void* p) {
-    if (p && !g_live.erase(p)) { puts("freed what was not allocated"); std::exit(2); }
-    std::free(p);
-    return cudaSuccess;
-}
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
-    if (fails()) return g_error;
-    std::memcpy(d, s, n);
-    return cudaSuccess;
-}
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return fails() ? g_error : cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return fails() ? g_error : cudaSuccess; }
-cudaError_t cudaGetLastError() { return cudaSuccess; }
-const char* cudaGetErrorString(cudaError_t) { return "failed on purpose"; }
-}
 
 namespace csb {
 void set_error(const char*, ...) {}
