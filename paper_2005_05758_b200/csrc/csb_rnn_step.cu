@@ -262,7 +262,7 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
             // speed of the bare product.
             const bool small = (gates == 3 ? 2 : 1) * B <= 32, unpacked = env_flag("CSB_RNN_STEP_UNPACKED");
             if (!small || unpacked) {
-                const int urc = umma_stack(gates, L, W, in_size, H, &np->umma);
+                const int urc = umma_stack(gates, L, W, in_size, H, false, &np->umma);
                 if (urc != CSB_OK) return urc;
             }
             const int rows_v = (gates == 3 && !np->umma ? 2 : 1) * B;

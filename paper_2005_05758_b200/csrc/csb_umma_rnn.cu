@@ -64,29 +64,34 @@ void drop_umma_rnn_plans(const csb_matrix* A) {
     cudaSetDevice(prev);
 }
 
-// Fills K; 1 when the layout does not take a layer.
-static int build_stack(const csb_matrix* const* W, UmmaStack* K) {
-    int clusters[kUmmaMaxS + 1];
-    int rc = umma_clusters(W[0], clusters);
+static int stack_windows(const UmmaStack& K, int l) { return (K.in_size[l] + K.H + kUmmaWindow - 1) / kUmmaWindow; }
+
+// Does one grid hold the stack, and in which shape?  1 when the device takes none.
+static int shape_stack(const csb_matrix* const* W, UmmaStack* K) {
+    int* clusters = K->clusters;
+    const int rc = umma_clusters(W[0], K->clusters);
     if (rc != CSB_OK) return rc;
     if (clusters[1] < 1) return 1;
     const int tiles = (K->H + 31) / 32;
-    int windows[kMaxLayers], most = 0, least = 0x7fffffff;
-    for (int l = 0; l < K->L; ++l) {
-        windows[l] = (K->in_size[l] + K->H + kUmmaWindow - 1) / kUmmaWindow;
-        most = std::max(most, windows[l]); least = std::min(least, windows[l]);
-    }
+    int most = 0, least = 0x7fffffff;
+    for (int l = 0; l < K->L; ++l) { most = std::max(most, stack_windows(*K, l)); least = std::min(least, stack_windows(*K, l)); }
     // One grid for all layers, every CTA there for the whole sequence: the shape whose slowest layer costs least (as in
     // umma_shape, with a step's cluster and counter on top whatever the shape).
     double best = 1e300;
-    int MT = 1, S = 1;
     for (int mt = kUmmaMaxMT; mt >= 1; --mt)
         for (int s = 1; s <= std::min<int>(kUmmaMaxS, least); ++s) {
             if (K->L * ((tiles + mt - 1) / mt) > clusters[s]) continue;
             const double cost = umma_cost(mt, s, most);
-            if (cost < best) { best = cost; MT = mt; S = s; }
+            if (cost < best) { best = cost; K->MT = mt; K->S = s; }
         }
     K->resident = best < 1e300;
+    K->flush = umma_flush(most);
+    return CSB_OK;
+}
+
+// The layouts of the layers; 1 when the layout does not take one.
+static int lay_out_stack(const csb_matrix* const* W, UmmaStack* K) {
+    const int tiles = (K->H + 31) / 32;
     // the layers side by side: planning one and uploading it take about as long as each other
     std::atomic<int> next{0};
     int layer_rc[kMaxLayers] = {};
@@ -95,11 +100,11 @@ static int build_stack(const csb_matrix* const* W, UmmaStack* K) {
             layer_rc[l] = guarded([&]() -> int {
                 CSB_CUDA(cudaSetDevice(K->device));
                 UmmaHostPlan H;
-                H.windows = windows[l];
+                H.windows = stack_windows(*K, l);
                 H.seg_words = umma_seg_words(W[l]->block_c);
-                H.flush = umma_flush(most);
-                if (K->resident) { H.MT = MT; H.S = S; }
-                else umma_shape(tiles, windows[l], clusters, &H.MT, &H.S);
+                H.flush = K->flush;
+                if (K->resident) { H.MT = K->MT; H.S = K->S; }
+                else umma_shape(tiles, H.windows, K->clusters, &H.MT, &H.S);
                 H.quads = umma_gate_quads(K->gates, K->in_size[l], K->H, H.MT);
                 H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
                 plan_umma_host(W[l], &H);
@@ -117,35 +122,42 @@ static int build_stack(const csb_matrix* const* W, UmmaStack* K) {
     UmmaStages g;
     if (K->resident)
         for (int NB = 16; NB <= 32; NB *= 2) {
-            if (!umma_stages(1, NB, MT, K->max_round, W[0]->smem_optin, &g)) { K->resident = false; break; }
-            CSB_CUDA(cudaFuncSetAttribute(pick_umma(K->gates == 4 ? 1 : 2, NB, MT), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W[0]->smem_optin));
+            if (!umma_stages(1, NB, K->MT, K->max_round, W[0]->smem_optin, &g)) { K->resident = false; break; }
+            CSB_CUDA(cudaFuncSetAttribute(pick_umma(K->gates == 4 ? 1 : 2, NB, K->MT), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)W[0]->smem_optin));
         }
     return CSB_OK;
 }
 
-int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size, int H, std::shared_ptr<UmmaStack>* out) {
+int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size, int H, bool for_loop, std::shared_ptr<UmmaStack>* out) {
     out->reset();
     for (int l = 0; l < L; ++l) if (!umma_applicable(W[l]) || W[l]->nnz == 0) return CSB_OK;
     std::lock_guard<std::mutex> lk(g_umma_mu);
+    std::shared_ptr<UmmaStack> K;
     for (auto& s : g_stacks) {
-        if (s->gates != gates || s->L != L || s->H != H) continue;
-        bool same = true;
-        for (int l = 0; l < L; ++l) same = same && s->uids[l] == W[l]->uid;
-        if (!same) continue;
-        if (s->taken) *out = s;
-        return CSB_OK;
+        bool same = s->gates == gates && s->L == L && s->H == H;
+        for (int l = 0; l < L && same; ++l) same = s->uids[l] == W[l]->uid;
+        if (same) { K = s; break; }
     }
-    auto s = std::make_shared<UmmaStack>();
-    s->gates = gates; s->L = L; s->H = H; s->device = W[0]->device;
-    for (int l = 0; l < L; ++l) { s->uids.push_back(W[l]->uid); s->in_size[l] = in_size[l]; }
-    const int rc = build_stack(W, s.get());
-    if (rc != CSB_OK && rc != 1 && rc != CSB_ERR_ALLOC) return rc;
-    // (where memory does not reach for these layouts, those of the step-by-step form may still fit; for good, so that a
-    // stack keeps its bits)
-    if (rc == CSB_ERR_ALLOC) for (UmmaPlan& p : s->plan) drop_umma_plan(p);
-    s->taken = rc == CSB_OK;
-    g_stacks.push_back(s);
-    if (s->taken) *out = s;
+    if (!K) {
+        K = std::make_shared<UmmaStack>();
+        K->gates = gates; K->L = L; K->H = H; K->device = W[0]->device;
+        for (int l = 0; l < L; ++l) { K->uids.push_back(W[l]->uid); K->in_size[l] = in_size[l]; }
+        const int rc = shape_stack(W, K.get());
+        if (rc != CSB_OK && rc != 1) return rc;
+        K->refused = rc == 1;
+        g_stacks.push_back(K);
+    }
+    if (K->refused || (for_loop && !K->resident)) return CSB_OK;
+    if (!K->laid_out) {
+        const int rc = lay_out_stack(W, K.get());
+        K->laid_out = rc == CSB_OK && (K->resident || !for_loop);
+        if (!K->laid_out) for (UmmaPlan& p : K->plan) drop_umma_plan(p);
+        if (rc != CSB_OK && rc != 1 && rc != CSB_ERR_ALLOC) return rc;
+        // (where memory does not reach for these layouts, those of the step-by-step form may still fit; for good, so that a
+        // stack keeps its bits)
+        K->refused = rc != CSB_OK;
+    }
+    if (K->laid_out) *out = K;
     return CSB_OK;
 }
 
@@ -202,9 +214,9 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
                      const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags, void* stream) {
     if (B > 32 || T > 0x3fffffff || (getenv("CSB_RNN_STEP_UNPACKED") && atoi(getenv("CSB_RNN_STEP_UNPACKED")))) return 1;
     std::shared_ptr<UmmaStack> K;
-    int rc = umma_stack(gates, L, W, in_size, H, &K);
+    int rc = umma_stack(gates, L, W, in_size, H, true, &K);
     if (rc != CSB_OK) return rc;
-    if (!K || !K->resident) return 1;
+    if (!K) return 1;
     UmmaRnnPlan* P = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_umma_mu);

@@ -25,12 +25,16 @@ struct UmmaStack {
     std::vector<uint64_t> uids;
     int gates = 0, L = 0, H = 0, device = -1;
     int in_size[kMaxLayers] = {};
-    bool taken = false;                // false: a layer does not suit the layout
+    bool refused = false;              // a layer does not suit the layout
     bool resident = false;             // one grid holds all layers: the time loop serves it
+    bool laid_out = false;             // only then are there plans
+    int clusters[kUmmaMaxS + 1] = {};
+    int MT = 1, S = 1, flush = 1;      // shape of a resident stack
     int max_round = 0;
     UmmaPlan plan[kMaxLayers];
     ~UmmaStack();
 };
-int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size, int H, std::shared_ptr<UmmaStack>* out);   // csb_umma_rnn.cu; null: not taken
+// csb_umma_rnn.cu.  for_loop: for the time loop, so that a stack that one grid does not hold is not laid out; *out null: not taken
+int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size, int H, bool for_loop, std::shared_ptr<UmmaStack>* out);
 
 }  // namespace csb

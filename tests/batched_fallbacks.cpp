@@ -66,6 +66,14 @@ int main() {
     g_cooperative = cudaSuccess;
     if (call(0) != CSB_OK) { puts("and then"); ++bad; }
     bad += forget("grid", 0);
+    // a stack that one grid does not hold: nothing is laid out for a loop that never runs
+    g_clusters = 2; g_bytes = 0;
+    if (call(0) != 1 || g_bytes) { printf("a stack past the grid: %zu bytes\n", g_bytes); ++bad; }
+    std::shared_ptr<UmmaStack> stack;                      // but for fp32 buffers, which use the layouts step by step
+    if (umma_stack(4, L, W, in_size, H, false, &stack) != CSB_OK || !stack || !stack->plan[L - 1].d_stream) { puts("no layouts for the fp32 buffers"); ++bad; }
+    if (call(0) != 1) { puts("a stack past the grid, laid out"); ++bad; }
+    stack.reset();
+    bad += forget("past the grid", 0);
     puts(bad ? "failed" : "ok");
     return bad != 0;
 }
