@@ -262,6 +262,7 @@ struct UmmaPlan {                          // device side
     bool built = false, unusable = false;
     int MT = 1, S = 1, flush = 1, n_ctas = 0, windows = 0, seg_words = 32;
     int max_round = 0;                     // bytes of the largest round of values
+    uint8_t* d_all = nullptr;              // the allocation that the arrays lie in (a stack's layers: the first one's)
     uint8_t* d_stream = nullptr; UmmaCta* d_ctas = nullptr; UmmaQuad* d_quads = nullptr; UmmaRound* d_rounds = nullptr;
     uint8_t* d_xp = nullptr;               // packed inputs of a bare product
 };

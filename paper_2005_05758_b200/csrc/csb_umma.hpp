@@ -50,6 +50,7 @@ struct UmmaRound { uint32_t off16, bytes; };   // a round of a CTA, from its sta
 
 struct UmmaHostPlan {
     int MT = 1, S = 1, flush = 1, n_groups = 0, windows = 0, seg_words = 32;   // seg_words: 32-bit words of a row of a column segment
+    int threads = 16;                     // to plan with, at most
     std::vector<UmmaQuad> quads;          // [n_groups][MT][4]
     std::vector<UmmaCta> ctas;            // [n_groups][S]
     std::vector<UmmaRound> rounds;        // CTA after CTA

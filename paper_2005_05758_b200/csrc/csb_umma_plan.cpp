@@ -108,7 +108,7 @@ struct ItemWriter {
 void plan_cta(const csb_matrix* A, const UmmaHostPlan& P, const UmmaCta& cta, UmmaRound* rounds, std::vector<uint8_t>* out) {
     const ItemWriter w{A, P.seg_words};
     const int ntw = cta.nw * P.MT, per = 4 / P.MT;         // windows of a round
-    out->reserve((size_t)ntw * 128 * 128 + (size_t)ntw * 1024);     // every row kept: pages that are not written cost nothing
+    out->clear();
     for (int r = 0; 4 * r < ntw; ++r) {
         const int nj = std::min(4, ntw - 4 * r), len = umma_unit_len(P.MT, P.flush, nj);
         const size_t start = out->size();
@@ -144,10 +144,13 @@ void plan_umma_host(const csb_matrix* A, UmmaHostPlan* P) {
     // the CTAs' streams are independent of one another
     std::atomic<size_t> next{0};
     std::atomic<bool> failed{false};
-    run_on_threads(A->nnz < 100000 ? 1 : (int)std::min<size_t>(16, P->ctas.size()), [&]() {
+    run_on_threads(A->nnz < 100000 ? 1 : (int)std::min<size_t>((size_t)P->threads, P->ctas.size()), [&]() {
         try {
-            for (size_t i; (i = next.fetch_add(1)) < P->ctas.size() && !failed;)
-                plan_cta(A, *P, P->ctas[i], P->rounds.data() + P->ctas[i].table, &P->streams[i]);
+            std::vector<uint8_t> scratch;                  // (room for the worst case for each CTA took a third to a half longer)
+            for (size_t i; (i = next.fetch_add(1)) < P->ctas.size() && !failed;) {
+                plan_cta(A, *P, P->ctas[i], P->rounds.data() + P->ctas[i].table, &scratch);
+                P->streams[i].assign(scratch.begin(), scratch.end());
+            }
         } catch (const std::bad_alloc&) { failed = true; }
     });
     if (failed) throw std::bad_alloc();

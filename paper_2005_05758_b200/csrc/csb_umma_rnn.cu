@@ -6,6 +6,7 @@
 #include <list>
 #include <memory>
 #include <mutex>
+#include <vector>
 
 #include "csb_host.hpp"
 #include "csb_rnn1.hpp"
@@ -37,9 +38,9 @@ struct UmmaRnnPlan {
     uint32_t* h_status = nullptr; uint32_t* d_status = nullptr;
     float* d_stage = nullptr;          // host-I/O staging of x and y
     size_t stage_cap = 0;
+    uint8_t* d_all = nullptr;          // the allocation that all of them but the staging lie in
     ~UmmaRnnPlan() {
-        for (uint8_t* p : d_xp) cudaFree(p);
-        cudaFree(d_state); cudaFree(d_ends); cudaFree(d_count); cudaFree(d_stage);
+        cudaFree(d_all); cudaFree(d_stage);
         if (h_status) cudaFreeHost(h_status);
     }
 };
@@ -92,33 +93,29 @@ static int shape_stack(const csb_matrix* const* W, UmmaStack* K) {
 // The layouts of the layers; 1 when the layout does not take one.
 static int lay_out_stack(const csb_matrix* const* W, UmmaStack* K) {
     const int tiles = (K->H + 31) / 32;
-    // the layers side by side: planning one and uploading it take about as long as each other
+    std::vector<UmmaHostPlan> H((size_t)K->L);
     std::atomic<int> next{0};
-    int layer_rc[kMaxLayers] = {};
-    run_on_threads(K->L, [&]() {
-        for (int l; (l = next.fetch_add(1)) < K->L;) {
-            layer_rc[l] = guarded([&]() -> int {
-                CSB_CUDA(cudaSetDevice(K->device));
-                UmmaHostPlan H;
-                H.windows = stack_windows(*K, l);
-                H.seg_words = umma_seg_words(W[l]->block_c);
-                H.flush = K->flush;
-                if (K->resident) { H.MT = K->MT; H.S = K->S; }
-                else umma_shape(tiles, H.windows, K->clusters, &H.MT, &H.S);
-                H.quads = umma_gate_quads(K->gates, K->in_size[l], K->H, H.MT);
-                H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
-                plan_umma_host(W[l], &H);
-                return upload_umma(W[l], H, &K->plan[l]);
-            });
+    std::atomic<bool> failed{false};
+    run_on_threads(K->L, [&]() {                           // the layers side by side
+        for (int l; (l = next.fetch_add(1)) < K->L && !failed;) {
+            try {
+                UmmaHostPlan& h = H[(size_t)l];
+                h.windows = stack_windows(*K, l);
+                h.seg_words = umma_seg_words(W[l]->block_c);
+                h.flush = K->flush;
+                h.threads = std::max(1, 16 / K->L);
+                if (K->resident) { h.MT = K->MT; h.S = K->S; }
+                else umma_shape(tiles, h.windows, K->clusters, &h.MT, &h.S);
+                h.quads = umma_gate_quads(K->gates, K->in_size[l], K->H, h.MT);
+                h.n_groups = (int)(h.quads.size() / (size_t)(4 * h.MT));
+                plan_umma_host(W[l], &h);
+            } catch (const std::bad_alloc&) { failed = true; }
         }
     });
-    for (int l = 0; l < K->L; ++l) {
-        if (layer_rc[l] == 1) return 1;
-        if (layer_rc[l] == CSB_ERR_ALLOC) set_error("out of memory");            // (another thread's error text is its own)
-        else if (layer_rc[l] != CSB_OK) set_error("uploading layer %d of the batched time loop failed", l);
-        if (layer_rc[l] != CSB_OK) { cudaGetLastError(); return layer_rc[l]; }
-        K->max_round = std::max(K->max_round, K->plan[l].max_round);
-    }
+    if (failed) return CSB_ERR_ALLOC;
+    const int rc = upload_umma(W[0], K->L, H.data(), false, K->plan);
+    if (rc != CSB_OK) { cudaGetLastError(); return rc; }
+    for (int l = 0; l < K->L; ++l) K->max_round = std::max(K->max_round, K->plan[l].max_round);
     UmmaStages g;
     if (K->resident)
         for (int NB = 16; NB <= 32; NB *= 2) {
@@ -149,7 +146,7 @@ int umma_stack(int gates, int L, const csb_matrix* const* W, const int* in_size,
     }
     if (K->refused || (for_loop && !K->resident)) return CSB_OK;
     if (!K->laid_out) {
-        const int rc = lay_out_stack(W, K.get());
+        const int rc = guarded([&] { return lay_out_stack(W, K.get()); });
         K->laid_out = rc == CSB_OK && (K->resident || !for_loop);
         if (!K->laid_out) for (UmmaPlan& p : K->plan) drop_umma_plan(p);
         if (rc != CSB_OK && rc != 1 && rc != CSB_ERR_ALLOC) return rc;
@@ -194,15 +191,17 @@ __global__ void __launch_bounds__(256) csb_umma_begin_kernel(const __grid_consta
 static int build_plan(UmmaRnnPlan* P) {
     const UmmaStack& K = *P->stack;
     const size_t ns = (size_t)K.L * P->B * K.H * 4;
-    for (int l = 0; l < K.L; ++l) {
-        // what is not written (columns past the last, batch columns past B) stays zero
-        const size_t bytes = (size_t)2 * K.plan[l].windows * P->NB * 256 + 32;
-        CSB_CUDA(cudaMalloc((void**)&P->d_xp[l], bytes));
-        CSB_CUDA(cudaMemsetAsync(P->d_xp[l], 0, bytes, cudaStreamPerThread));
-    }
-    CSB_CUDA(cudaMalloc((void**)&P->d_state, ns));
-    CSB_CUDA(cudaMalloc((void**)&P->d_ends, 4 * ns));
-    CSB_CUDA(cudaMalloc((void**)&P->d_count, 4));
+    size_t bytes = 0, xp[kMaxLayers];
+    auto room = [&bytes](size_t more) { const size_t here = bytes; bytes += (more + 255) / 256 * 256; return here; };
+    for (int l = 0; l < K.L; ++l) xp[l] = room((size_t)2 * K.plan[l].windows * P->NB * 256 + 32);
+    const size_t images = bytes, state = room(ns), ends = room(4 * ns), count = room(4);
+    CSB_CUDA(cudaMalloc((void**)&P->d_all, bytes));
+    // what is not written (columns past the last, batch columns past B) stays zero
+    CSB_CUDA(cudaMemsetAsync(P->d_all, 0, images, cudaStreamPerThread));
+    for (int l = 0; l < K.L; ++l) P->d_xp[l] = P->d_all + xp[l];
+    P->d_state = reinterpret_cast<float*>(P->d_all + state);
+    P->d_ends = reinterpret_cast<float*>(P->d_all + ends);
+    P->d_count = reinterpret_cast<uint32_t*>(P->d_all + count);
     CSB_CUDA(cudaHostAlloc((void**)&P->h_status, 4, cudaHostAllocMapped));
     *P->h_status = 0;
     CSB_CUDA(cudaHostGetDevicePointer((void**)&P->d_status, P->h_status, 0));

@@ -17,7 +17,7 @@ bool umma_stages(int mode, int NB, int MT, int max_round, size_t room, UmmaStage
 int launch_umma_fp32(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, cudaStream_t st);
 
 // csb_umma_upload.cpp
-int upload_umma(const csb_matrix* A, const UmmaHostPlan& H, UmmaPlan* P);
+int upload_umma(const csb_matrix* A, int n, const UmmaHostPlan* H, bool with_xp, UmmaPlan* P);
 int make_umma_plan(const csb_matrix* A, UmmaPlan* P);   // 1: the path does not take the matrix
 
 // The layouts of a stack's layers, for every batch size.
