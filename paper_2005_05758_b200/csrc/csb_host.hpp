@@ -1,4 +1,4 @@
-// Host-side helpers: planning work on a few threads, and the guard of the C entry points.
+// Host-side helpers: planning work on a few threads, the guard of the C entry points, and that of a product's handle.
 #pragma once
 
 #include <algorithm>
@@ -31,6 +31,14 @@ template <typename F>
 int guarded(F&& f) {
     try { return f(); }
     catch (const std::exception&) { set_error("out of host memory"); return CSB_ERR_ALLOC; }   // allocations are all that throws here
+}
+
+// What a product leaves behind when a wait of its kernel ran out stays with the handle.
+inline int product_gave_up(const csb_matrix* A) {
+    const ProductPlan& PP = A->product;
+    if (!PP.h_status || *PP.h_status == 0) return CSB_OK;
+    set_error("an earlier product on this handle gave up waiting on the device (code %u)", *PP.h_status);
+    return CSB_ERR_TIMEOUT;
 }
 
 }  // namespace csb

@@ -28,6 +28,7 @@
 #include <memory>
 #include <mutex>
 
+#include "csb_host.hpp"
 #include "csb_internal.hpp"
 #include "csb_device.cuh"
 #include "csb_gates.cuh"
@@ -399,8 +400,10 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
     for (int64_t t = 0; t < T; ++t) {
         for (int l = 0; l < L; ++l) {
             const int ld = in_size[l] + H;
-            const int rc = P->umma ? launch_umma_fp32(W[l], &P->umma->plan[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)4 * H, st)
-                                   : launch_spmm_stack_fp32(P->stack, l, W[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
+            int rc = product_gave_up(W[l]);
+            if (rc != CSB_OK) return rc;
+            rc = P->umma ? launch_umma_fp32(W[l], &P->umma->plan[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)4 * H, st)
+                         : launch_spmm_stack_fp32(P->stack, l, W[l], P->d_xp[l], P->d_v[l], ld, vrows, P->d_z, (int64_t)gates * H, stream);
             if (rc != CSB_OK) return rc;
             const bool top = l == L - 1;
             const float* x_next = (l == 0 && t + 1 < T) ? dx + (size_t)(t + 1) * B * I0 : nullptr;

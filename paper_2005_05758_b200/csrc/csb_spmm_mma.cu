@@ -34,6 +34,7 @@
 #include <cstdio>
 #include <mutex>
 
+#include "csb_host.hpp"
 #include "csb_internal.hpp"
 #include "csb_device.cuh"
 
@@ -669,13 +670,6 @@ static int ensure_mma(const csb_matrix* A) {
     return CSB_ERR_ALLOC;
 }
 
-static int gave_up(const csb_matrix* A) {
-    const ProductPlan& PP = A->product;
-    if (!PP.h_status || *PP.h_status == 0) return CSB_OK;
-    set_error("an earlier product on this handle gave up waiting on the device (code %u)", *PP.h_status);
-    return CSB_ERR_TIMEOUT;
-}
-
 // Launches the tile kernel over the products (P[i], xp[i], Y[i]) of matrices with the same block shape.
 static int launch_parts(int n, const csb_matrix* const* A, const MmaPlan::PerClass* const* P, const uint8_t* const* xp, float* const* Y, int NT, int nb,
                         int64_t ldy, cudaStream_t st) {
@@ -746,7 +740,7 @@ static bool capturing(cudaStream_t st) {
 
 // Returns CSB_OK after launching, or 1 when the caller should use the CUDA-core path.
 int launch_spmm_mma(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
-    int rc = gave_up(A);
+    int rc = product_gave_up(A);
     if (rc != CSB_OK) return rc;
     int prev = 0;
     CSB_CUDA(cudaGetDevice(&prev));
@@ -824,15 +818,13 @@ int prepare_spmm_stack(int L, const csb_matrix* const* A, int batch, SpmmStack* 
 
 int launch_spmm_stack_fp32(const SpmmStack& K, int l, const csb_matrix* A, uint8_t* xp, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy,
                            void* stream) {
-    const int rc = gave_up(A);
-    if (rc != CSB_OK) return rc;
     return pack_and_launch(A, K.plan[l], K.NT, xp, X, ldx, batch, Y, ldy, (cudaStream_t)stream);
 }
 
 int launch_spmm_stack(const SpmmStack& K, int l0, int l1, const csb_matrix* const* A, uint8_t* const* xp, float* const* Y, int nb, int64_t ldy, void* stream) {
     const uint8_t* x[kMaxLayers];
     for (int l = l0; l < l1; ++l) {
-        const int rc = gave_up(A[l]);
+        const int rc = product_gave_up(A[l]);
         if (rc != CSB_OK) return rc;
         x[l] = xp[l];
     }

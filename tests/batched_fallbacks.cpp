@@ -1,5 +1,6 @@
-// The host side of the batched recurrent calls (csb_umma_rnn.cu) on the CUDA runtime of fake_runtime.hpp: where the time loop
-// cannot run, the call has to be left to the step-by-step form.  Exit code 0: every rule below held.
+// The host side of the batched recurrent calls (csb_umma_rnn.cu, csb_rnn_step.cu) on the CUDA runtime of fake_runtime.hpp: where
+// the time loop cannot run, the call has to be left to the step-by-step form, and that form has to refuse a handle
+// whose product gave up.  Exit code 0: every rule below held.
 #include "../paper_2005_05758_b200/csrc/csb_umma_rnn.hpp"
 #include "fake_runtime.hpp"
 
@@ -15,6 +16,12 @@ int umma_clusters(const csb_matrix*, int (&n)[kUmmaMaxS + 1]) {
 }
 const void* pick_umma(int, int, int) { return nullptr; }
 bool umma_stages(int, int, int, int max_round, size_t room, UmmaStages* out) { *out = UmmaStages{2, max_round, room}; return true; }
+static int g_products = 0;
+int launch_umma_fp32(const csb_matrix*, const UmmaPlan*, uint8_t*, const float*, int64_t, int, float*, int64_t, cudaStream_t) { ++g_products; return CSB_OK; }
+bool spmm_mma_applicable(const csb_matrix*, int) { return true; }
+int prepare_spmm_stack(int, const csb_matrix* const*, int, SpmmStack*) { return 1; }
+int launch_spmm_stack(const SpmmStack&, int, int, const csb_matrix* const*, uint8_t* const*, float* const*, int, int64_t, void*) { return CSB_ERR_LAUNCH; }
+int launch_spmm_stack_fp32(const SpmmStack&, int, const csb_matrix*, uint8_t*, const float*, int64_t, int, float*, int64_t, void*) { return CSB_ERR_LAUNCH; }
 void note_recurrent_path(RecurrentPath) {}
 void barrier_test_hook(unsigned int* extra, unsigned long long* ns) { *extra = 0; *ns = 1; }
 }
@@ -74,6 +81,21 @@ int main() {
     if (call(0) != 1) { puts("a stack past the grid, laid out"); ++bad; }
     stack.reset();
     bad += forget("past the grid", 0);
+    // more sequences than the loop takes: step by step, and no step with a handle whose product has given up
+    g_clusters = 148;
+    const int many = 40;
+    std::vector<float> xs((size_t)T * many * I), ys((size_t)T * many * H), ss((size_t)L * many * H);
+    auto steps = [&]() {
+        g_products = 0;
+        return rnn_forward_stepwise(4, L, W, nullptr, xs.data(), T, many, H, in_size, ss.data(), ss.data(), ys.data(), nullptr, nullptr, CSB_FLAG_ASYNC, nullptr);
+    };
+    if (steps() != CSB_OK || g_products != T * L) { printf("steps: %d products\n", g_products); ++bad; }
+    uint32_t word = 1;
+    W[0]->product.h_status = &word;
+    if (steps() != CSB_ERR_TIMEOUT || g_products) { printf("steps of a handle that gave up: %d products\n", g_products); ++bad; }
+    W[0]->product.h_status = nullptr;
+    for (csb_matrix* A : W) drop_step_plans(A);
+    bad += forget("steps", 0);
     puts(bad ? "failed" : "ok");
     return bad != 0;
 }
