@@ -48,6 +48,7 @@ namespace csb {
 struct StepPlan {
     std::vector<uint64_t> uids;
     int L = 0, B = 0, H = 0, gates = 0, device = -1;
+    bool tiles = false, unpacked = false;   // what the environment asked for: the products on tcgen05, fp32 buffers for any batch
     int in_size[kMaxLayers] = {};
     float* d_v[kMaxLayers] = {};       // [B, in_size[l] + H] per layer (GRU: [2B, ...], input rows then recurrent rows)
     float* d_z = nullptr;              // [B, 4H] (GRU: [2B, 3H]) pre-activations; packed path: one such per layer
@@ -248,20 +249,23 @@ int rnn_forward_stepwise(int gates, int L, const csb_matrix* const* W, const flo
                          const int* in_size, const float* h0, const float* c0, float* y, float* hT, float* cT, unsigned flags,
                          void* stream) {
     StepPlan* P = nullptr;
+    bool tiles = true;
+    const bool unpacked = env_flag("CSB_RNN_STEP_UNPACKED") != 0;
+    for (int l = 0; l < L; ++l) tiles = tiles && umma_applicable(W[l]);
     {
         std::lock_guard<std::mutex> lk(g_step_mu);
         for (auto& p : g_step_plans) {
-            if (p->L != L || p->B != B || p->gates != gates) continue;
+            if (p->L != L || p->B != B || p->gates != gates || p->tiles != tiles || p->unpacked != unpacked) continue;
             bool same = true;
             for (int l = 0; l < L; ++l) same = same && p->uids[l] == W[l]->uid;
             if (same) { P = p.get(); break; }
         }
         if (!P) {
             std::unique_ptr<StepPlan> np(new StepPlan());
-            np->L = L; np->B = B; np->H = H; np->gates = gates; np->device = W[0]->device;
+            np->L = L; np->B = B; np->H = H; np->gates = gates; np->device = W[0]->device; np->tiles = tiles; np->unpacked = unpacked;
             // The layouts of the time loop serve the fp32 buffers as well: its numbers bit for bit, and batches past 32 at the
             // speed of the bare product.
-            const bool small = (gates == 3 ? 2 : 1) * B <= 32, unpacked = env_flag("CSB_RNN_STEP_UNPACKED");
+            const bool small = (gates == 3 ? 2 : 1) * B <= 32;
             if (!small || unpacked) {
                 const int urc = umma_stack(gates, L, W, in_size, H, false, &np->umma);
                 if (urc != CSB_OK) return urc;

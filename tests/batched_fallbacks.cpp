@@ -16,12 +16,12 @@ int umma_clusters(const csb_matrix*, int (&n)[kUmmaMaxS + 1]) {
 }
 const void* pick_umma(int, int, int) { return nullptr; }
 bool umma_stages(int, int, int, int max_round, size_t room, UmmaStages* out) { *out = UmmaStages{2, max_round, room}; return true; }
-static int g_products = 0;
+static int g_products = 0, g_other_products = 0;
 int launch_umma_fp32(const csb_matrix*, const UmmaPlan*, uint8_t*, const float*, int64_t, int, float*, int64_t, cudaStream_t) { ++g_products; return CSB_OK; }
 bool spmm_mma_applicable(const csb_matrix*, int) { return true; }
-int prepare_spmm_stack(int, const csb_matrix* const*, int, SpmmStack*) { return 1; }
+int prepare_spmm_stack(int, const csb_matrix* const*, int, SpmmStack*) { return CSB_OK; }
 int launch_spmm_stack(const SpmmStack&, int, int, const csb_matrix* const*, uint8_t* const*, float* const*, int, int64_t, void*) { return CSB_ERR_LAUNCH; }
-int launch_spmm_stack_fp32(const SpmmStack&, int, const csb_matrix*, uint8_t*, const float*, int64_t, int, float*, int64_t, void*) { return CSB_ERR_LAUNCH; }
+int launch_spmm_stack_fp32(const SpmmStack&, int, const csb_matrix*, uint8_t*, const float*, int64_t, int, float*, int64_t, void*) { ++g_other_products; return CSB_OK; }
 void note_recurrent_path(RecurrentPath) {}
 void barrier_test_hook(unsigned int* extra, unsigned long long* ns) { *extra = 0; *ns = 1; }
 }
@@ -86,7 +86,7 @@ int main() {
     const int many = 40;
     std::vector<float> xs((size_t)T * many * I), ys((size_t)T * many * H), ss((size_t)L * many * H);
     auto steps = [&]() {
-        g_products = 0;
+        g_products = g_other_products = 0;
         return rnn_forward_stepwise(4, L, W, nullptr, xs.data(), T, many, H, in_size, ss.data(), ss.data(), ys.data(), nullptr, nullptr, CSB_FLAG_ASYNC, nullptr);
     };
     if (steps() != CSB_OK || g_products != T * L) { printf("steps: %d products\n", g_products); ++bad; }
@@ -94,6 +94,11 @@ int main() {
     W[0]->product.h_status = &word;
     if (steps() != CSB_ERR_TIMEOUT || g_products) { printf("steps of a handle that gave up: %d products\n", g_products); ++bad; }
     W[0]->product.h_status = nullptr;
+    // the environment is read at every call: a plan of one form does not serve the other
+    setenv("CSB_NO_UMMA", "1", 1);
+    if (steps() != CSB_OK || g_products || g_other_products != T * L) { printf("steps by mma.sync: %d products, %d others\n", g_products, g_other_products); ++bad; }
+    unsetenv("CSB_NO_UMMA");
+    if (steps() != CSB_OK || g_products != T * L || g_other_products) { printf("steps again: %d products, %d others\n", g_products, g_other_products); ++bad; }
     for (csb_matrix* A : W) drop_step_plans(A);
     bad += forget("steps", 0);
     puts(bad ? "failed" : "ok");
