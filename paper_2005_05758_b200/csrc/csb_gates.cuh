@@ -12,9 +12,7 @@
 
 namespace csb {
 
-__device__ __forceinline__ float gate_logistic(float a) { return 1.f / (1.f + expf(-a)); }
-
-// The same arithmetic with every rounding spelled out, for kernels that have to give the same bits.
+// The arithmetic of the cells, every rounding spelled out: kernels that inline it differently have to give the same bits.
 __device__ __forceinline__ float cell_logistic(float a) { return __frcp_rn(__fadd_rn(1.f, expf(-a))); }
 __device__ __forceinline__ float lstm_cell(float zi, float zf, float zg, float zo, float& c) {
     c = __fmaf_rn(cell_logistic(zf), c, __fmul_rn(cell_logistic(zi), tanhf(zg)));
@@ -72,8 +70,8 @@ __device__ __forceinline__ void lstm_gates_tile(float (*tile)[33], const float* 
             float zi = __ldcg(z + j), zf = __ldcg(z + H + j), zg = __ldcg(z + 2 * H + j), zo = __ldcg(z + 3 * H + j);
             if (bias) { zi += bias[j]; zf += bias[H + j]; zg += bias[2 * H + j]; zo += bias[3 * H + j]; }
             const size_t e = (size_t)b * H + j;
-            const float cn = gate_logistic(zf) * __ldcg(c + e) + gate_logistic(zi) * tanhf(zg);
-            h = gate_logistic(zo) * tanhf(cn);
+            float cn = __ldcg(c + e);
+            h = lstm_cell(zi, zf, zg, zo, cn);
             c[e] = cn;
             hs[e] = h;
             if (y_t) y_t[e] = h;
@@ -100,10 +98,8 @@ __device__ __forceinline__ void gru_gates_tile(float (*tile)[33], const float* _
             float ar = __ldcg(zx + j) + __ldcg(zh + j), au = __ldcg(zx + H + j) + __ldcg(zh + H + j);
             float nx = __ldcg(zx + 2 * H + j), nh = __ldcg(zh + 2 * H + j);
             if (bias) { ar += bias[j]; au += bias[H + j]; nx += bias[2 * H + j]; nh += bias[3 * H + j]; }
-            const float r = gate_logistic(ar), u = gate_logistic(au);
-            const float cand = tanhf(nx + r * nh);
             const size_t e = (size_t)b * H + j;
-            h = (1.f - u) * cand + u * __ldcg(hs + e);
+            h = gru_cell(ar, au, nx, nh, __ldcg(hs + e));
             hs[e] = h;
             if (y_t) y_t[e] = h;
         }
