@@ -348,10 +348,17 @@ void csb_test_barrier_hook(unsigned int extra_arrivals, unsigned long long limit
 
 /*
  * csb_last_recurrent_path -- testing aid (the paper has no counterpart): which kernels served the calling thread's most
- * recent recurrent call: 1 the unit loop, 2 the block loop (both resident), 3 and 4 batched steps on tensor cores (up to 32 and more
- * rows of the step-by-step product, which has B rows, for the GRU 2B), 5 the persistent kernel, 6 steps of a cell variant; 0 before the first call.
+ * recent recurrent call: 1 the unit loop, 2 the block loop (both resident), 3 and 4 batched steps on tensor cores, in one launch or
+ * many (up to 32 and more rows of the step-by-step product, which has B rows, for the GRU 2B), 5 the persistent kernel, 6 steps of a cell variant; 0 before the first call.
  */
 int csb_last_recurrent_path(void);
+
+/*
+ * csb_last_tensor_kernel -- testing aid (the paper has no counterpart): which tensor-core kernel the calling thread's most
+ * recent csb_spmv, csb_spmm, csb_lstm_forward or csb_gru_forward launched last: 0 none, 1 the mma.sync product, 2 the tcgen05
+ * product, 3 the tcgen05 time loop.
+ */
+int csb_last_tensor_kernel(void);
 
 /*
  * csb_plan_dump -- inspection / testing aid (the paper has no counterpart): plan the bare product

@@ -18,9 +18,13 @@ void set_error(const char* fmt, ...) {
 }
 void clear_error() { g_err[0] = 0; }
 
+static thread_local int g_tensor_kernel = kTensorNone;
+void note_tensor_kernel(TensorKernel kernel) { g_tensor_kernel = kernel; }
+
 static std::atomic<uint64_t> g_uid{1};
 
 int product_any(const csb_matrix* A, const float* X, int64_t ldx, int batch, float* Y, int64_t ldy, void* stream) {
+    note_tensor_kernel(kTensorNone);
     if (spmm_mma_applicable(A, batch)) {
         const int rc = launch_spmm_mma(A, X, ldx, batch, Y, ldy, stream);
         if (rc != 1) return rc;                       // 1: the tensor-core plan does not fit this matrix
@@ -104,6 +108,8 @@ const char* csb_strerror(int status) {
 }
 
 const char* csb_last_error(void) { return g_err; }
+
+int csb_last_tensor_kernel(void) { return g_tensor_kernel; }
 
 static int encode_common(const float* dense, int64_t rows, int64_t cols, int64_t ld, int block_r, int block_c,
                          const uint8_t* row_keep, const uint8_t* col_keep, int val_dtype, int frac_bits, int device,

@@ -381,6 +381,8 @@ void drop_cell_plans(const csb_matrix* A); // forget cached plans of the cell va
 
 // csb_rnn.cu
 enum RecurrentPath { kPathUnitLoop = 1, kPathBlockLoop, kPathStepsPacked, kPathSteps, kPathPersistent, kPathCellSteps };
+enum TensorKernel { kTensorNone = 0, kTensorMma = 1, kTensorTiles = 2, kTensorLoop = 3 };
+void note_tensor_kernel(TensorKernel kernel);   // for csb_last_tensor_kernel
 void note_recurrent_path(RecurrentPath path);   // for csb_last_recurrent_path
 void drop_rnn_plans(const csb_matrix* A);  // forget cached time-loop plans that use A
 

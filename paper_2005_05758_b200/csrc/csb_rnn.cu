@@ -823,6 +823,7 @@ static int rnn_forward(int gates, int L, const csb_matrix_t* const* W, const flo
     }
     if (T == 0 || B == 0) return CSB_OK;
     if (!x) { set_error("x is NULL"); return CSB_ERR_INVALID_ARG; }
+    note_tensor_kernel(kTensorNone);
     const int I0 = in_size[0];
     int prev = 0;
     CSB_CUDA(cudaGetDevice(&prev));

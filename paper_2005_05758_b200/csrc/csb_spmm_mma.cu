@@ -673,6 +673,7 @@ static int ensure_mma(const csb_matrix* A) {
 // Launches the tile kernel over the products (P[i], xp[i], Y[i]) of matrices with the same block shape.
 static int launch_parts(int n, const csb_matrix* const* A, const MmaPlan::PerClass* const* P, const uint8_t* const* xp, float* const* Y, int NT, int nb,
                         int64_t ldy, cudaStream_t st) {
+    note_tensor_kernel(kTensorMma);
     const int MT = mt_of(A[0]);
     SpmmArgs a{};
     a.n_parts = n; a.nb = nb; a.ldy = ldy; a.status = A[0]->product.d_status;

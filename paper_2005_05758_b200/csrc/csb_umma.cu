@@ -98,6 +98,7 @@ static uint32_t* bad_words(uint8_t* xp, int windows) { return reinterpret_cast<u
 
 // Y = A . (packed inputs) with the plan's output rows.
 int launch_umma_packed(const csb_matrix* A, const UmmaPlan* P, uint8_t* xp, float* Y, int NB, int nb, int64_t ldy, cudaStream_t st) {
+    note_tensor_kernel(kTensorTiles);
     UmmaArgs a{};
     a.n_parts = 1; a.nb = nb; a.ldy = ldy; a.status = A->product.d_status; a.S = P->S; a.flush = P->flush;
     UmmaPart& p = a.part[0];

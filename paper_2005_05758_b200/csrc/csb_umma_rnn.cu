@@ -232,6 +232,7 @@ int rnn_forward_umma(int gates, int L, const csb_matrix* const* W, const float* 
     UmmaStages g;
     if (!umma_stages(1, P->NB, K->plan[0].MT, K->max_round, W[0]->smem_optin, &g)) return 1;
     // (as the step-by-step forms count: rows of their product, two per sequence for the GRU)
+    note_tensor_kernel(kTensorLoop);
     note_recurrent_path((gates == 3 ? 2 : 1) * B <= 32 ? kPathStepsPacked : kPathSteps);
     cudaStream_t st = (cudaStream_t)stream;
     const bool host_io = (flags & CSB_FLAG_HOST_IO) != 0, lstm = gates == 4;

@@ -23,6 +23,7 @@ int prepare_spmm_stack(int, const csb_matrix* const*, int, SpmmStack*) { return 
 int launch_spmm_stack(const SpmmStack&, int, int, const csb_matrix* const*, uint8_t* const*, float* const*, int, int64_t, void*) { return CSB_ERR_LAUNCH; }
 int launch_spmm_stack_fp32(const SpmmStack&, int, const csb_matrix*, uint8_t*, const float*, int64_t, int, float*, int64_t, void*) { ++g_other_products; return CSB_OK; }
 void note_recurrent_path(RecurrentPath) {}
+void note_tensor_kernel(TensorKernel) {}
 void barrier_test_hook(unsigned int* extra, unsigned long long* ns) { *extra = 0; *ns = 1; }
 }
 

@@ -135,9 +135,9 @@ def test_resume_equals_one_call_bitwise_and_host_io():
 
 @pytest.mark.parametrize("B,I,H,L,br,bc", [(16, 40, 48, 2, 16, 16), (32, 153, 160, 1, 32, 32), (40, 70, 192, 2, 64, 32), (8, 200, 512, 1, 32, 32)])
 def test_lstm_large_batch_runs_step_by_step_on_tensor_cores(monkeypatch, B, I, H, L, br, bc):
-    # batches of 16 and more take the path of one product (tensor cores) + one gate kernel per layer
-    # and step (8 where no resident loop holds the layers); bias, initial states, resumption and host I/O
-    # as for the persistent kernel
+    # batches of 16 and more (8 where no resident loop holds the layers) run on tensor cores, up to 32 in one launch,
+    # beyond it with a product and a gate kernel per layer and step; bias, initial states, resumption and host
+    # I/O as for the persistent kernel
     if B <= 8:
         monkeypatch.setenv("CSB_RNN_NO_RNN1", "1")
     w = workloads.make_rnn_workload(31, "lstm", I, H, L, br, bc, "lognormal", rate=4.0, T=6, B=B, w_std=0.15,
@@ -161,8 +161,9 @@ def test_lstm_large_batch_both_paths_agree(monkeypatch):
 
 @pytest.mark.parametrize("cell,B,I", [("lstm", 32, 153), ("lstm", 9, 40), ("gru", 16, 70), ("gru", 11, 33)])
 def test_step_by_step_packed_inputs_equal_the_fp32_buffers(monkeypatch, cell, B, I):
-    # up to 32 product rows the gate kernels write h_t and x_{t+1} straight into the products' packed
-    # binary16 (hi, lo) inputs; the same numbers as packing the fp32 buffers in a kernel of its own
+    # states and inputs written straight into the products' packed binary16 (hi, lo) inputs, here by the time loop on
+    # tcgen05, and the same products over fp32 buffers, packed by a kernel of its own: the same numbers
+    # (test_gpu_other_widths.py has the packed steps on mma.sync)
     w = workloads.make_rnn_workload(33, cell, I, 512, 2, 32, 32, "lognormal", rate=4.0, T=5, B=B, w_std=0.15,
                                     bias_std=0.2, state_std=0.4)
     ya, ha, ca = check(w)
@@ -191,8 +192,8 @@ def test_wavefront_of_layers_resumes_bitwise(monkeypatch, cell, B, I, H, L, br):
 
 @pytest.mark.parametrize("B,I,H,L,br,bc", [(16, 40, 48, 2, 16, 16), (20, 39, 100, 1, 32, 32), (33, 70, 192, 2, 64, 32), (8, 300, 512, 1, 32, 32)])
 def test_gru_batch_runs_step_by_step_on_tensor_cores(monkeypatch, B, I, H, L, br, bc):
-    # GRU from batch 16 (from batch 8 for layers of 100 k weights and more, where no resident loop holds them): one
-    # product over 2B rows ([u ; 0] and [0 ; h]) keeps the candidate's two parts apart
+    # GRU from batch 16 (from batch 8 for layers of 100 k weights and more, where no resident loop holds them): the
+    # candidate's two parts stay apart, as output rows of their own
     if B <= 8:
         monkeypatch.setenv("CSB_RNN_NO_RNN1", "1")
     w = workloads.make_rnn_workload(41, "gru", I, H, L, br, bc, "lognormal", rate=4.0, T=6, B=B, w_std=0.15,

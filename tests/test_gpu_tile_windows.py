@@ -14,6 +14,8 @@ from paper_2005_05758_b200 import binding
 
 pytestmark = pytest.mark.gpu
 
+TILES, LOOP = 2, 3                                         # csb_last_tensor_kernel
+
 # Error of an output in units of sum |w| |x|: the split x = hi + lo (2^-22), a chain of at most 8 truncated sums in the
 # tensor cores (2^-23 each), then one rounded sum per flush group and column range, at most 64 here (2^-24 each).
 TOL = 2.0 ** -22 + 8 * 2.0 ** -23 + 64 * 2.0 ** -24
@@ -35,6 +37,7 @@ def test_product_against_the_oracle(rows, cols, br, bc, batch):
         torch.cuda.synchronize()
         got = y.cpu().numpy()
         assert np.all(np.abs(got[:, :rows] - want) <= TOL * scale)
+        assert binding.lib.csb_last_tensor_kernel() == TILES
         assert np.isnan(got[:, rows:]).all()
     A.free()
 
@@ -53,6 +56,7 @@ def test_time_loop_against_the_oracle(cell, B, I, H, L, T):
         else:
             binding.csb_lstm_forward(mats, bias, x, h0, torch.from_numpy(w.c0).cuda(), y, hT, None, 0)
     run()
+    assert binding.lib.csb_last_tensor_kernel() == LOOP
     want = R.gru_forward(lay, w.bias, w.x, w.h0) if cell == "gru" else R.lstm_forward(lay, w.bias, w.x, w.h0, w.c0)
     # fp32 sums of fp16 weights: an absolute error of 1e-6 of a pre-activation of size 1 a step (TOL and the activations'), which
     # the recurrence carries on; 5 steps of up to 3 layers
@@ -185,7 +189,7 @@ def test_an_input_past_binary16_spreads_through_a_sequence_where_it_is_kept(cell
             binding.csb_lstm_forward(mats, bias, torch.from_numpy(x).cuda(), torch.from_numpy(h0).cuda(), torch.from_numpy(w.c0).cuda(), y, hT, cT, 0)
         return [t.cpu().numpy() for t in (y, hT, cT)]
     want = run(x, h0)
-    assert all(np.isfinite(a).all() for a in want)
+    assert all(np.isfinite(a).all() for a in want) and binding.lib.csb_last_tensor_kernel() == (LOOP if B <= 32 else TILES)
     x[bad_x], h0[bad_h] = np.resize(np.array(LARGE, np.float32), int(bad_x.sum())), np.float32("inf") if cell == "lstm" else np.float32("nan")
     got = run(x, h0)
     K = [kept(m).astype(np.float32) for m in w.layers]
