@@ -82,11 +82,16 @@ __host__ __device__
 inline UmmaPlace umma_place(int MT, int len, int j) {
     return MT == 1 ? UmmaPlace{0, j} : len == 2 ? UmmaPlace{j >> 1, j & 1} : UmmaPlace{j & 1, j >> 1};
 }
-// Windows per flush group.  The tensor cores truncate each sum, so the error follows the number of steps between two flushes;
-// the bounds are those at which it stays below what mma.sync gave, whose chains grow with the number of columns
-// (2-norm of the error against 64 bits, mma.sync / 1 / 2 windows: 1024 x 1536 at 4x 1.40e-7 / 1.30e-7 / 1.52e-7, 700 x
-// 2050 at 6x 1.75 / 1.08 / 1.27, 8192 x 8192 at 4x 8.37 / 1.45 / 1.73, 25x 2.07 / 1.23 / 1.32).
-inline int umma_flush(int windows) { return windows < 32 ? 1 : 2; }
+// Windows per flush group.  The tensor cores truncate each sum, so the error follows the number of steps between two flushes.
+// Two windows take 7 to 15 % less time from 4096 x 4096 on, and are taken where the error stays no larger than what
+// mma.sync gave, whose chains grow with the number of blocks (they are a CTA's share of a block-row): from 6000 blocks on.
+// 2-norm of the error against 64 bits, 1e-7, mma.sync / 1 / 2 windows, batch 8:
+//   blocks of 64 x 64:  512 x 4096 at 4x 1.49 / 1.38 / 1.71, 4096 x 4096 at 25x 1.26 / 1.15 / 1.27, 8192 x 3072 at 25x (6144
+//     blocks) 1.33 / 1.14 / 1.26, 8192 x 8192 at 4x 4.78 / 1.46 / 1.75, at 25x 1.70 / 1.20 / 1.32;
+//   blocks of 32 x 32:  512 x 4096 at 9x 1.23 / 1.12 / 1.30, 2048 x 4096 at 4x (8192 blocks) 2.24 / 1.26 / 1.51;
+//   of 64 x 128:  4096 x 4096 at 9x 1.70 / 1.28 / 1.87, 8192 x 8192 at 9x (8192 blocks) 2.87 / 1.36 / 1.91;
+//   of 16 x 16:  512 x 2049 at 4x 1.41 / 1.14 / 1.37, 8192 x 8192 at 4x 24.8 / 1.43 / 1.54.
+inline int umma_flush(int windows, int64_t blocks = 0x7fffffff) { return windows < 32 || blocks < 6000 ? 1 : 2; }
 // Fills streams, rounds, ctas (the other members are set); throws std::bad_alloc.
 void plan_umma_host(const csb_matrix* A, UmmaHostPlan* P);
 

@@ -75,7 +75,8 @@ static int shape_stack(const csb_matrix* const* W, UmmaStack* K) {
     if (clusters[1] < 1) return 1;
     const int tiles = (K->H + 31) / 32;
     int most = 0, least = 0x7fffffff;
-    for (int l = 0; l < K->L; ++l) { most = std::max(most, stack_windows(*K, l)); least = std::min(least, stack_windows(*K, l)); }
+    int64_t blocks = 0x7fffffff;
+    for (int l = 0; l < K->L; ++l) { most = std::max(most, stack_windows(*K, l)); least = std::min(least, stack_windows(*K, l)); blocks = std::min(blocks, W[l]->nblk); }
     // One grid for all layers, every CTA there for the whole sequence: the shape whose slowest layer costs least (as in
     // umma_shape, with a step's cluster and counter on top whatever the shape).
     double best = 1e300;
@@ -86,7 +87,7 @@ static int shape_stack(const csb_matrix* const* W, UmmaStack* K) {
             if (cost < best) { best = cost; K->MT = mt; K->S = s; }
         }
     K->resident = best < 1e300;
-    K->flush = umma_flush(most);
+    K->flush = umma_flush(most, blocks);
     return CSB_OK;
 }
 

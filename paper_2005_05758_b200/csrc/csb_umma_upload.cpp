@@ -77,7 +77,7 @@ int make_umma_plan(const csb_matrix* A, UmmaPlan* P) {
             if (crc != CSB_OK) return crc;
             if (clusters[1] < 1) return 1;
             umma_shape((int)((A->rows + 127) / 128), H.windows, clusters, &H.MT, &H.S);
-            H.flush = umma_flush(H.windows);
+            H.flush = umma_flush(H.windows, A->nblk);
             H.quads = umma_row_quads(A, H.MT);
             H.n_groups = (int)(H.quads.size() / (size_t)(4 * H.MT));
             plan_umma_host(A, &H);

@@ -227,3 +227,25 @@ def test_more_ctas_than_the_device_holds_are_not_asked_for():
         for m in mats:
             m.free()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("rows,cols,br,bc,rate", [(513, 2049, 64, 64, 2.5), (70, 4200, 64, 64, 3.0), (512, 4096, 64, 64, 4.0), (1024, 2049, 64, 64, 25.0), (512, 4096, 32, 32, 9.0),
+                                                  (2048, 4096, 64, 128, 9.0), (4096, 4096, 64, 64, 25.0), (8192, 3072, 64, 64, 25.0), (1024, 1536, 16, 16, 4.0)])
+def test_the_error_is_no_larger_than_that_of_mma_sync(monkeypatch, rows, cols, br, bc, rate):
+    # 2-norm of the error against 64 bits over that of the result; 3 % is what other inputs of the same size change
+    f = rate ** -0.5
+    w = workloads.make_spmv_workload(rows, rows, cols, br, bc, "uniform", lo=0.7 * f, hi=min(1.0, 1.3 * f), batch=64, w_std=0.05)
+    m = w.matrix
+    A = binding.csb_encode(m.dense, br, bc, m.row_keep, m.col_keep, "f16", 0)
+    x = torch.from_numpy(w.X).cuda()
+    want = x.double() @ torch.from_numpy(np.where(kept(m), m.dense.astype(np.float16), np.float16(0))).cuda().double().T
+    for batch in (8, 32, 64):
+        err = {}
+        for other in ("1", "0"):
+            monkeypatch.setenv("CSB_NO_UMMA", other)
+            y = torch.empty((batch, rows), device="cuda")
+            binding.csb_spmm(A, x[:batch], y)
+            assert binding.lib.csb_last_tensor_kernel() == (1 if other == "1" else TILES)
+            err[other] = float((y.double() - want[:batch]).norm() / want[:batch].norm())
+        assert err["0"] <= 1.03 * err["1"] and err["0"] < 2e-7, err
+    A.free()
