@@ -1,6 +1,7 @@
 // Tensor-core CSB-SpMM (batch >= 8, fp16 values, fp32 accumulation) for blocks whose width is not 16, 32 or a multiple of 64;
-// those go through csb_umma_kernel.cuh, whose column segments need such widths (at 20 sizes from 512 x 256 to 8192 x 8192, 8 to
-// 64 columns, 4x to 25x, that kernel was the faster one at each).
+// those go through csb_umma_kernel.cuh, whose column segments need such widths (at 8 sizes from 512 x 512 to 8192 x 8192, 8 to
+// 64 columns, 25x to 1000x, that kernel was the faster one at each, though its time does not fall with the kept weights, but for
+// 8192 x 8192 at 1000x with 8 and 16 columns, 17.3 us here and 17.7 there).
 //
 // With a batch of vectors the product of a block's kernel matrix (m kept rows x n kept columns)
 // with the gathered inputs (n x batch) of Section 4.3.1 is a small dense contraction, the one place

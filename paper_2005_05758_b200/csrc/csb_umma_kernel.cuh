@@ -3,7 +3,7 @@
 //
 // The kernel matrices of the blocks (Section 4.3.1) are small and all different, and with rows and columns put back in their
 // places a block is mostly zeros.  Tensor instructions for those zeros are cheap on this chip (8192 x 8192 dense, 64 columns as
-// hi and lo halves: 7.5 us of all SMs), so a warp expands the kept values into the dense tile and the contraction is a dense one:
+// hi and lo halves: 10.5 us at the measured rate), so a warp expands the kept values into the dense tile and the contraction is a dense one:
 //
 //   * sixteen warps expand: lane = output row, eight 16-byte loads of its row's 64 columns, zeros where the row is not
 //     kept, and one tcgen05.st puts the 32 words into TMEM as the A operand (128 rows x 64 columns per tile-window).  A never

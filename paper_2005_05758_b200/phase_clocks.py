@@ -10,7 +10,8 @@ build.py), loads it instead of libcsb.so and prints
          (mean / min / max over the CTAs);
   panel: wall-clock stamps of csb_panel_kernel per CTA, in microseconds from the earliest CTA start;
   spmm:  cycles per phase of csb_spmm_tile_kernel, summed per warp (mean / max over the warps, and the
-         same for the slowest CTA, and the warp that finishes its items last).
+         same for the slowest CTA, and the warp that finishes its items last); that kernel serves block
+         widths other than 16, 32 and multiples of 64, and here the matrices of the configs by CSB_NO_UMMA=1.
 The instrumented kernels are slower than the product ones (thread 0 reads the clock between phases),
 so these figures say where the time goes, never how long a call takes.
 """
@@ -111,7 +112,7 @@ SPMM_PHASES = ["set-up, first copies, wait for the work in front", "waiting for 
 
 def spmm(cases):
     import workloads
-    os.environ["CSB_NO_UMMA"] = "1"                # (blocks of these sizes take the kernel without such counters)
+    os.environ["CSB_NO_UMMA"] = "1"                # (csb_umma_kernel, which serves blocks of these sizes, has no such counters)
     torch, binding = _load()
     for case in cases:
         rate, B = case.split(":")
