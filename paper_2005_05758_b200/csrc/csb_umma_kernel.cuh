@@ -255,39 +255,58 @@ template <int NB> __device__ __forceinline__ bool put_eight(uint8_t* images, int
     return large;
 }
 
-// Sets those of an expanding warp's sums to NaN that have a marked input in a column that the lane's row keeps: out[b * ld] for the batch
-// columns b from b0 on.  Marks are rare, so the images and the items' headers are simply read again, and the sums are
-// overwritten where they lie.
-// buffer: which of a time loop's buffers of images, whose sums lie [batch column][row of the group]; -1: a product's.
-template <int NB, int MT>
-__device__ __noinline__ void spoil_sums(const UmmaArgs& a, int p_idx, int cta, int warp, int buffer, float* out, long long ld) {
-    constexpr int CN = NB * MT / 4, kPer = 4 / MT;         // windows of a round
+// Sets those sums to NaN, where they lie, that have a marked input in a column that their row keeps: out[b * ld] for the batch
+// columns b.  Marks are rare, so the images and the items' headers are simply read again: first which columns of each window and
+// batch column are marked, into shared memory that is free at the time (scratch), then each header once.  WARPS: the
+// expanding warps of a product together, or the one that copies a time loop's inputs (the former cost two 2048-unit
+// LSTM layers 2 % without any marks).  buffer: which of a time loop's buffers of images, whose sums lie [batch column][row
+// of the group]; -1: a product's.
+template <int NB, int MT, int WARPS>
+__device__ __noinline__ void spoil_sums(const UmmaArgs& a, int p_idx, int cta, int warp, int buffer, uint8_t* scratch, int scratch_bytes, float* out, long long ld) {
+    constexpr int kPer = 4 / MT;                           // windows of a round
     const UmmaPart& pt = a.part[p_idx];
     const UmmaCta me = pt.ctas[cta];
-    const int lane = threadIdx.x & 31, quad = warp & 3, slot = warp >> 2, mt = MT == 2 ? slot >> 1 : 0, b0 = (MT == 2 ? slot & 1 : slot) * CN;
-    const int w0 = me.w0, nw = me.nw, seg_words = pt.seg_words;
-    const UmmaQuad q = pt.quads[((size_t)me.group * MT + mt) * 4 + quad];
-    const uint32_t seg_off = lane < q.nrows ? (uint32_t)((q.row0 + lane) / pt.block_r - q.row0 / pt.block_r) * (uint32_t)(32 / seg_words * 16) : 0u;
-    const uint8_t *stream = pt.stream + (size_t)me.off128 * 128, *images = pt.xp + (size_t)max(buffer, 0) * pt.windows * (NB * 256);
+    const int lane = threadIdx.x & 31, nw = me.nw, seg_words = pt.seg_words, segs = 32 / seg_words, chunk = scratch_bytes / (NB * 8);
+    const uint8_t *stream = pt.stream + (size_t)me.off128 * 128, *images = pt.xp + ((size_t)max(buffer, 0) * pt.windows + me.w0) * (NB * 256);
     const uint2* rounds = reinterpret_cast<const uint2*>(pt.rounds) + me.table;
-    out += (buffer < 0 ? q.out0 : mt * 128 + quad * 32) + lane;
-    for (int w = 0; w < nw; ++w) {
-        const int rd = w / kPer, nj = min(4, nw * MT - 4 * rd), len = umma_unit_len(MT, a.flush, nj);
-        int j = 0;
-        while (j < 3 && (umma_place(MT, len, j).mt != mt || umma_place(MT, len, j).window != w % kPer)) ++j;
-        const uint8_t* round = stream + (size_t)__ldg(rounds + rd).x * 16;
-        const uint8_t* header = round + __ldg(reinterpret_cast<const uint32_t*>(round) + j * 4 + quad) + seg_off;
-        const uint8_t* image = images + (size_t)(w0 + w) * (NB * 256);
-        for (int i = 0; i < CN && b0 + i < a.nb; ++i) {
-            const uint8_t* at = image + image_at<NB>(b0 + i, 2 * lane);
-            const uint32_t hi = __ldcg(reinterpret_cast<const uint32_t*>(at)), lo = __ldcg(reinterpret_cast<const uint32_t*>(at + NB * 128));
+    auto sync = [] { if (WARPS > 1) expand_barrier(true); else __syncwarp(); };
+    for (int c0 = 0; c0 < nw; c0 += chunk) {
+        const int n = min(chunk, nw - c0);
+        sync();
+#pragma unroll 4
+        for (int i = warp * 32 + lane; i < n * a.nb * 8; i += WARPS * 32) {        // eight columns of a batch column
+            const int w = (i >> 3) / a.nb, b = (i >> 3) - w * a.nb;
+            const uint8_t* at = images + (size_t)(c0 + w) * (NB * 256) + b * 128 + (i & 7) * 16;
+            const uint4 h = __ldcg(reinterpret_cast<const uint4*>(at)), l = __ldcg(reinterpret_cast<const uint4*>(at + NB * 128));
+            auto pair = [](uint32_t hi, uint32_t lo) {
+                return (uint32_t)((hi & 0xffffu) == 0u && (lo & 0xffffu) == kBadLo) | (uint32_t)(hi >> 16 == 0u && lo >> 16 == kBadLo) << 1;
+            };
+            scratch[(w * NB + b) * 8 + ((i & 7) ^ (b & 7))] = (uint8_t)(pair(h.x, l.x) | pair(h.y, l.y) << 2 | pair(h.z, l.z) << 4 | pair(h.w, l.w) << 6);
+        }
+        sync();
+#pragma unroll 1
+        for (int i = warp; i < n * MT; i += WARPS) {
+            const int w = i / MT, mt = i - w * MT, rd = (c0 + w) / kPer, nj = min(4, nw * MT - 4 * rd), len = umma_unit_len(MT, a.flush, nj);
+            int j = 0;
+            while (j < 3 && (umma_place(MT, len, j).mt != mt || umma_place(MT, len, j).window != (c0 + w) % kPer)) ++j;
+            const uint8_t* round = stream + (size_t)__ldg(rounds + rd).x * 16;
+            const uint4 items = __ldg(reinterpret_cast<const uint4*>(round) + j);
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-                uint32_t marks = __ballot_sync(0xffffffffu, ((hi >> (16 * p)) & 0xffffu) == 0u && ((lo >> (16 * p)) & 0xffffu) == kBadLo);
-                for (; marks; marks &= marks - 1u) {
-                    const int c = 2 * (__ffs(marks) - 1) + p, k = c % (2 * seg_words);
-                    const uint4 h = __ldg(reinterpret_cast<const uint4*>(header + 16 * (c / (2 * seg_words))));
-                    if ((h.x >> lane) & ((k < 32 ? h.z : h.w) >> (k & 31)) & 1u) out[(b0 + i) * ld] = __int_as_float(0x7fffffff);
+            for (int quad = 0; quad < 4; ++quad) {
+                const UmmaQuad q = pt.quads[((size_t)me.group * MT + mt) * 4 + quad];
+                const uint32_t seg = lane < q.nrows ? (uint32_t)((q.row0 + lane) / pt.block_r - q.row0 / pt.block_r) * (uint32_t)(segs * 16) : 0u;
+                const uint8_t* header = round + (quad == 0 ? items.x : quad == 1 ? items.y : quad == 2 ? items.z : items.w) + seg;
+                float* to = out + (buffer < 0 ? q.out0 : mt * 128 + quad * 32) + lane;
+#pragma unroll 1
+                for (int s = 0; s < segs; ++s) {
+                    const uint4 h = __ldg(reinterpret_cast<const uint4*>(header) + s);
+                    const bool row = (h.x >> lane) & 1u;
+#pragma unroll 8
+                    for (int b = 0; b < a.nb; ++b) {
+                        const uint32_t m = smem_u32(scratch) + (uint32_t)((w * NB + b) * 8);
+                        const uint32_t hit = segs == 1 ? (lds32(m) & h.z) | (lds32(m + 4) & h.w) : segs == 2 ? lds32(m + 4 * s) & h.z : (lds32(m + 4 * (s >> 1)) >> (16 * (s & 1))) & h.z;
+                        if (row && hit) to[b * ld] = __int_as_float(0x7fffffff);
+                    }
                 }
             }
         }
@@ -690,8 +709,9 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 if (!__shfl_sync(0xffffffffu, ok, 0)) break;
                 if (!__shfl_sync(0xffffffffu, marked, 0)) continue;
                 if (!__all_sync(0xffffffffu, wait(sums, s_bad[5] & 1u))) break;
-#pragma unroll 1
-                for (int v = 0; v < kUmmaExpandWarps; ++v) spoil_sums<NB, MT>(a, p_idx, (int)blockIdx.x - cta0, v, (t + p_idx) & 1, part, kRows);
+                // (the inputs' ring is free: this warp fills it, and every product of the step is done)
+                spoil_sums<NB, MT, 1>(a, p_idx, (int)blockIdx.x - cta0, 0, (t + p_idx) & 1, smem, (int)L.w, part, kRows);
+                fence_proxy_async_all();                  // (the next tick's copies go over the scratch)
                 __syncwarp();
                 if (lane == 0) { s_bad[5] = s_bad[5] + 1u; mbar_arrive(spoilt); }
                 __syncwarp();
@@ -787,7 +807,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
                 for (int i = 0; i < CN; ++i)
                     if (my_b0 + i < a.nb) pt.Y[(long long)(my_b0 + i) * a.ldy + q.out0 + lane] = i & 1 ? acc[i / 2].y : acc[i / 2].x;
         }
-        if (marked) spoil_sums<NB, MT>(a, 0, (int)blockIdx.x, warp, -1, pt.Y, a.ldy);
+        if (marked) spoil_sums<NB, MT, kUmmaExpandWarps>(a, 0, (int)blockIdx.x, warp, -1, smem, (int)L.w, pt.Y, a.ldy);
         return;
     }
     if (warp < kUmmaExpandWarps)
@@ -825,7 +845,7 @@ __global__ void __launch_bounds__(kUmmaThreads, 1) csb_umma_kernel(const __grid_
     }
     __syncthreads();
     umma_cluster_barrier();                               // nobody leaves before everybody has read
-    if (marked) spoil_sums<NB, MT>(a, 0, (int)blockIdx.x, warp, -1, pt.Y, a.ldy);
+    if (marked) spoil_sums<NB, MT, kUmmaExpandWarps>(a, 0, (int)blockIdx.x, warp, -1, smem, (int)L.w, pt.Y, a.ldy);
 }
 
 }  // namespace csb
