@@ -269,6 +269,14 @@ __device__ __noinline__ void spoil_sums(const UmmaArgs& a, int p_idx, int cta, i
     const int lane = threadIdx.x & 31, nw = me.nw, seg_words = pt.seg_words, segs = 32 / seg_words, chunk = scratch_bytes / (NB * 8);
     const uint8_t *stream = pt.stream + (size_t)me.off128 * 128, *images = pt.xp + ((size_t)max(buffer, 0) * pt.windows + me.w0) * (NB * 256);
     const uint2* rounds = reinterpret_cast<const uint2*>(pt.rounds) + me.table;
+    uint32_t seg_off[4 * MT];                              // the lane's row segment in each quadrant: where its headers start in an item
+    int to[4 * MT];                                        // and its row in `out`
+#pragma unroll
+    for (int i = 0; i < 4 * MT; ++i) {
+        const UmmaQuad q = pt.quads[(size_t)me.group * MT * 4 + i];
+        seg_off[i] = lane < q.nrows ? (uint32_t)((q.row0 + lane) / pt.block_r - q.row0 / pt.block_r) * (uint32_t)(segs * 16) : 0u;
+        to[i] = (buffer < 0 ? q.out0 : i * 32) + lane;
+    }
     auto sync = [] { if (WARPS > 1) expand_barrier(true); else __syncwarp(); };
     for (int c0 = 0; c0 < nw; c0 += chunk) {
         const int n = min(chunk, nw - c0);
@@ -284,28 +292,27 @@ __device__ __noinline__ void spoil_sums(const UmmaArgs& a, int p_idx, int cta, i
             scratch[(w * NB + b) * 8 + ((i & 7) ^ (b & 7))] = (uint8_t)(pair(h.x, l.x) | pair(h.y, l.y) << 2 | pair(h.z, l.z) << 4 | pair(h.w, l.w) << 6);
         }
         sync();
-#pragma unroll 1
+#pragma unroll 2
         for (int i = warp; i < n * MT; i += WARPS) {
             const int w = i / MT, mt = i - w * MT, rd = (c0 + w) / kPer, nj = min(4, nw * MT - 4 * rd), len = umma_unit_len(MT, a.flush, nj);
             int j = 0;
             while (j < 3 && (umma_place(MT, len, j).mt != mt || umma_place(MT, len, j).window != (c0 + w) % kPer)) ++j;
             const uint8_t* round = stream + (size_t)__ldg(rounds + rd).x * 16;
             const uint4 items = __ldg(reinterpret_cast<const uint4*>(round) + j);
-#pragma unroll
-            for (int quad = 0; quad < 4; ++quad) {
-                const UmmaQuad q = pt.quads[((size_t)me.group * MT + mt) * 4 + quad];
-                const uint32_t seg = lane < q.nrows ? (uint32_t)((q.row0 + lane) / pt.block_r - q.row0 / pt.block_r) * (uint32_t)(segs * 16) : 0u;
-                const uint8_t* header = round + (quad == 0 ? items.x : quad == 1 ? items.y : quad == 2 ? items.z : items.w) + seg;
-                float* to = out + (buffer < 0 ? q.out0 : mt * 128 + quad * 32) + lane;
+            const uint32_t item[4] = {items.x, items.y, items.z, items.w};
 #pragma unroll 1
-                for (int s = 0; s < segs; ++s) {
-                    const uint4 h = __ldg(reinterpret_cast<const uint4*>(header) + s);
-                    const bool row = (h.x >> lane) & 1u;
-#pragma unroll 8
-                    for (int b = 0; b < a.nb; ++b) {
-                        const uint32_t m = smem_u32(scratch) + (uint32_t)((w * NB + b) * 8);
-                        const uint32_t hit = segs == 1 ? (lds32(m) & h.z) | (lds32(m + 4) & h.w) : segs == 2 ? lds32(m + 4 * s) & h.z : (lds32(m + 4 * (s >> 1)) >> (16 * (s & 1))) & h.z;
-                        if (row && hit) to[b * ld] = __int_as_float(0x7fffffff);
+            for (int s = 0; s < segs; ++s) {
+                uint4 h[4];                                // (all four loaded in front of the stores)
+#pragma unroll
+                for (int quad = 0; quad < 4; ++quad) h[quad] = __ldg(reinterpret_cast<const uint4*>(round + item[quad] + seg_off[MT == 2 ? mt * 4 + quad : quad]) + s);
+#pragma unroll 2
+                for (int b = 0; b < a.nb; ++b) {
+                    const uint32_t m = smem_u32(scratch) + (uint32_t)((w * NB + b) * 8), m0 = lds32(m), m1 = lds32(m + 4);
+                    if ((m0 | m1) == 0u) continue;
+#pragma unroll
+                    for (int quad = 0; quad < 4; ++quad) {
+                        const uint32_t hit = segs == 1 ? (m0 & h[quad].z) | (m1 & h[quad].w) : segs == 2 ? (s ? m1 : m0) & h[quad].z : ((s < 2 ? m0 : m1) >> (16 * (s & 1))) & h[quad].z;
+                        if (((h[quad].x >> lane) & 1u) && hit) out[to[MT == 2 ? mt * 4 + quad : quad] + b * ld] = __int_as_float(0x7fffffff);
                     }
                 }
             }
